@@ -350,10 +350,11 @@ int helm_precond_apply_noalloc(const helm_grid* grid, double k, double theta_bet
  * --------------------------------------------------------------------------------- */
 
 /* Tune the launch choices of one problem's V-cycle on the current device: the tiles
- * per CTA of the 2D passes (Arnoldi steps, residual + restriction, prolongation), and
- * for 3D complex64 levels of pitch 128..1024 the TMA-fed Arnoldi pass of each step
- * (off, or on with 2..8 plane slots in flight, 2 or 4 points per thread in y, and the
- * level shared as one piece per resident CTA or as 1, 2 or 4 z pieces per column).
+ * per CTA of the 2D passes (residual + restriction, prolongation, complex128 Arnoldi
+ * steps), and for 3D complex64 levels of pitch 128..1024 the TMA-fed restriction and
+ * post-smoothing residual (off, or on with 2..8 plane slots in flight, 2 or 4 points per
+ * thread in y, and the level shared as one piece per resident CTA or as 1, 2 or 4 z
+ * pieces per column).  The complex64 smoothing sweeps have no tuned choice.
  * Every candidate is timed over whole V-cycles (reps cycles, best of three trials) by
  * coordinate descent from the defaults, finest level first, and kept when it makes the
  * V-cycle more than 0.5% faster.  grid, phi, k, theta_beta, opts as for helm_setup
@@ -374,8 +375,8 @@ int helm_tuning_load(const char* path);
  * level of dimension dim and pitch P in precision prec (HELM_C64 / HELM_C128) for Arnoldi
  * step J (0 for the other passes): writes its 4 integers into v and returns 1, or
  * returns 0 when the table has none (the built-in default applies).  v: 2D passes
- * {tiles per CTA}; 3D Arnoldi {TMA-fed pass on, plane slots, z pieces per column (0: one
- * share per resident CTA), points per thread in y}; "persist" {persistent segment on};
+ * {tiles per CTA}; 3D restrict and prolong {TMA-fed pass on, plane slots, z pieces per
+ * column (0: one share per resident CTA), points per thread in y}; "persist" {persistent segment on};
  * "zplanes" (3D levels without the TMA-fed passes) {planes each CTA marches: 2, 4, 8 or
  * 16}.  Host only. */
 int helm_tuning_get(const char* pass, int dim, int P, int prec, int J, int* v);

@@ -5,14 +5,15 @@
 // coordinate descent from the built-in defaults, finest level first.  A candidate
 // replaces the current choice when the V-cycle gets faster by more than 0.5%, which
 // keeps run-to-run noise from deciding.  Choices:
-//   2D levels: tiles per CTA of the Arnoldi passes (each step J), of the residual +
-//     restriction pass and of the prolongation pass (1, 2, 4, 8);
+//   2D levels: tiles per CTA of the residual + restriction pass, of the prolongation pass
+//     and (complex128) of the Arnoldi passes of each step J (1, 2, 4, 8);
 //   3D levels without the TMA-fed passes (pitch below 128, or complex128): the planes
 //     each CTA of the plain passes marches (2, 4, 8, 16);
-//   3D complex64 levels of pitch 128..1024: the TMA-fed Arnoldi pass of each step J
-//     off, or on with 2..8 plane slots in flight, 2 or 4 points per thread in y, and
-//     the level shared as one piece per resident CTA or as 1, 2 or 4 z pieces per
-//     column.
+//   3D complex64 levels of pitch 128..1024: the TMA-fed restriction and post-smoothing
+//     residual off, or on with 2..8 plane slots in flight, 2 or 4 points per thread in y
+//     (the residual), and the level shared as one piece per resident CTA or as 1, 2 or 4
+//     z pieces per column.
+// The complex64 sweep passes (sweep.cuh) take their launch shape from the level size alone.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -130,21 +131,11 @@ int autotune(const helm_grid* grid, const float* phi, double k, double theta_bet
       knobs.push_back(kz);
     }
     if (dim == 2) {
-      for (int J = 1; J <= h->s; ++J) knobs.push_back({TP_ARNOLDI, 2, P, eb, J, {tc(1), tc(2), tc(4), tc(8)}});
+      if (eb == 16)
+        for (int J = 1; J <= h->s; ++J) knobs.push_back({TP_ARNOLDI, 2, P, eb, J, {tc(1), tc(2), tc(4), tc(8)}});
       knobs.push_back({TP_RESTRICT, 2, P, eb, 0, {tc(1), tc(2), tc(4), tc(8)}});
       knobs.push_back({TP_PROLONG, 2, P, eb, 0, {tc(1), tc(2), tc(4), tc(8)}});
     } else if (eb == 8 && L.tm && P >= 128 && P <= 1024 && P % 32 == 0) {
-      for (int J = 1; J <= h->s; ++J) {
-        Knob kb{TP_ARNOLDI, 3, P, eb, J, {tc(0, 2, 0, 2)}};
-        for (int qy : {2, 4}) {
-          if (qy == 4 && J > 2) continue;
-          for (int stg : {2, 3, 4, 6, 8}) {
-            if (!tma3_fits(J, qy, stg)) continue;
-            for (int pieces : {0, 1, 2, 4}) kb.cands.push_back(tc(1, stg, pieces, qy));
-          }
-        }
-        knobs.push_back(kb);
-      }
       Knob kr{TP_RESTRICT, 3, P, eb, 0, {tc(0, 2, 0, 2)}};
       for (int stg : {2, 3, 4})
         if (tma3_fits(h->s + 1, 2, stg))

@@ -1,0 +1,375 @@
+// The coarse sub-cycle of the complex64 V-cycle: every level of at most 31^2 or 7^3 points,
+// down to the coarsest and up again, by one CTA per problem.
+//
+// Bound by latency: a level is one or two points per thread, and a sweep is a chain of
+// stencils, one Gram reduction and one small minimisation (gram.cuh), each behind a
+// barrier.  So every thread keeps the stencil coefficients of its points and its values of
+// k_0..k_S in registers for the whole sweep; shared memory only carries what neighbours
+// read, in the padded layout (row pitch P = n + 1, ghosts zero), whose ghosts and the ghost
+// rows of the vector before make the stencil free of bounds checks.  The coarsest system is
+// solved with its inverse, formed in binary64 at set-up and held as double-floats: a matrix
+// times vector, all rows at once, instead of 2 m dependent elimination steps on the FP64
+// pipe.  Everything that does not depend on the previous kernel is loaded before the wait.
+#pragma once
+#include "gram.cuh"
+
+namespace helm {
+
+constexpr int CG_THREADS = 512, CG_NW = CG_THREADS / 32, CG_PT = 2;
+constexpr int CG_COARSE_POINTS = CG_THREADS * CG_PT;  // most interior points of a level
+constexpr int CG_INV = 1024;                          // entries of the inverse staged in shared memory
+constexpr int CG_COEF = 3 * 64;                       // 1D coefficients of all levels (31 + 15 + 7 + 3 per array)
+
+HELM_HD constexpr int cg_vectors(int S) { return 3 + (S > 1 ? S - 1 : 0); }  // b, x, r, k_1..k_{S-1}
+
+// One thread's points of a level and the level's vectors.
+template <int S, int DIM>
+struct CgLevel {
+  int n, P;
+  float t, it;                         // basis scale and its reciprocal
+  float2 *b, *x, *r, *k[S > 1 ? S - 1 : 1];
+  int off[CG_PT], cx[CG_PT], cy[CG_PT], cz[CG_PT];
+  bool on[CG_PT];
+  float2 ax[CG_PT], qx[CG_PT], ay[CG_PT], qy[CG_PT], az[CG_PT], qz[CG_PT], dg[CG_PT], dz[CG_PT];
+
+  __device__ __forceinline__ void stencil_setup(const LevelDev<float2>& L, const float2* coef, int tid) {
+    n = L.n;
+    P = L.P;
+    t = L.kt;
+    it = 1.0f / t;
+    const int np = DIM == 3 ? n * n * n : n * n;
+    const float phc = L.phir * t;
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) {
+      const int i = tid + q * CG_THREADS;
+      on[q] = i < np;
+      const int ii = on[q] ? i : 0;
+      const int yy = ii / n;
+      cx[q] = ii - yy * n;
+      cz[q] = DIM == 3 ? yy / n : 0;
+      cy[q] = yy - cz[q] * n;
+      off[q] = (cz[q] * P + cy[q]) * P + cx[q];
+      auto sc = [&](float2 v) { return make_float2(v.x * t, v.y * t); };
+      ax[q] = sc(coef[cx[q]]);
+      qx[q] = sc(coef[2 * n + cx[q]]);
+      ay[q] = sc(coef[cy[q]]);
+      qy[q] = sc(coef[2 * n + cy[q]]);
+      dg[q] = cadd(sc(coef[n + cx[q]]), sc(coef[n + cy[q]]));
+      if (DIM == 3) {
+        az[q] = sc(coef[cz[q]]);
+        qz[q] = sc(coef[2 * n + cz[q]]);
+        dz[q] = sc(coef[n + cz[q]]);
+      }
+      dg[q].x -= L.phi ? __ldg(L.phi + off[q]) * t : phc;
+    }
+  }
+  // t (M - sigma) v at point q; v0 the point's own value
+  __device__ __forceinline__ float2 apply(const float2* v, float2 v0, int q, float2 sg) const {
+    float2 d = dg[q];
+    d.x -= sg.x;
+    d.y -= sg.y;
+    float2 p = cmul(d, v0);
+    const float2* s = v + off[q];
+    p = cfma(ax[q], s[-1], p);
+    p = cfma(qx[q], s[1], p);
+    p = cfma(ay[q], s[-P], p);
+    p = cfma(qy[q], s[P], p);
+    if (DIM == 3) {
+      p = cfma(dz[q], v0, p);  // apart: the sum of the three diagonals would be rounded
+      p = cfma(az[q], s[-P * P], p);
+      p = cfma(qz[q], s[P * P], p);
+    }
+    return p;
+  }
+};
+
+struct CgShared {
+  float wsum[CG_NW * 32];
+  float2 gs[CG_NW * gram_nv(SMAX)];
+  float2 xc[SMAX], rc[SMAX + 1];
+};
+
+// One sweep: k0 (this thread's values of R_0, already in shared memory at R0 and visible to
+// the CTA) -> x += dx and k0 = the new residual.
+template <int S, int DIM>
+__device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2* R0, float2 (&k0)[CG_PT],
+                                         float2 (&x)[CG_PT], const float2 (&sg)[S], CgShared& sh) {
+  constexpr int NV = gram_nv(S), NS = gram_ns(S), H = NS == 16 ? 2 : 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float2 k[CG_PT][S + 1];
+#pragma unroll
+  for (int q = 0; q < CG_PT; ++q) k[q][0] = k0[q];
+#pragma unroll
+  for (int j = 1; j <= S; ++j) {
+    const float2* src = j == 1 ? R0 : V.k[j >= 2 ? j - 2 : 0];
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) {
+      k[q][j] = make_float2(0.f, 0.f);
+      if (V.on[q]) {
+        k[q][j] = V.apply(src, k[q][j - 1], q, sg[j - 1]);
+        if (j < S) V.k[j >= 1 && j < S ? j - 1 : 0][V.off[q]] = k[q][j];
+      }
+    }
+    if (j < S) __syncthreads();
+  }
+  float acc[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
+#pragma unroll
+  for (int q = 0; q < CG_PT; ++q) gram_point<S>(k[q], acc);
+  const float tot = warp_transpose_sum_f<NS>(acc, lane);
+  if (NS == 32) sh.wsum[warp * NS + lane] = tot;
+  else if ((lane & 1) == 0) sh.wsum[warp * NS + (lane >> 1)] = tot;
+  __syncthreads();
+  if (warp == 0) {
+    const int v = NS == 16 ? (lane & 15) : lane, h = NS == 16 ? lane >> 4 : 0;
+    float s = 0.f, c = 0.f;
+#pragma unroll
+    for (int q = h; q < CG_NW; q += H) {
+      float t, r;
+      df_two_sum(s, sh.wsum[q * NS + v], t, r);
+      s = t;
+      c += r;
+    }
+    if (H == 2) {
+      const float s2 = __shfl_xor_sync(0xffffffffu, s, 16), c2 = __shfl_xor_sync(0xffffffffu, c, 16);
+      float t, r;
+      df_two_sum(s, s2, t, r);
+      c = (c + c2) + r;
+      s = t;
+    }
+    if (h == 0 && v < NV) sh.gs[v] = df_fast2(s, c);
+    __syncwarp();
+    float2 xc[S], rc[S + 1];
+    gram_solve<S>(sh.gs, sg, V.t, xc, rc);
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < S; ++i) sh.xc[i] = xc[i];
+#pragma unroll
+      for (int i = 0; i <= S; ++i) sh.rc[i] = rc[i];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < CG_PT; ++q) {
+    float2 dx = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < S; ++i) dx = cfma(sh.xc[i], k[q][i], dx);
+#pragma unroll
+    for (int i = 0; i <= S; ++i) r = cfma(sh.rc[i], k[q][i], r);
+    x[q] = cadd(x[q], dx);
+    k0[q] = r;
+  }
+}
+
+template <int S, int DIM>
+__global__ void __launch_bounds__(CG_THREADS, 1)
+k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, const CoarseLU* __restrict__ lus,
+              int nu1, int nu2) {
+  extern __shared__ __align__(16) float2 cgsm[];
+  __shared__ LevelDev<float2> Ls[MAX_COARSE_LEVELS_HOST];
+  __shared__ int s_base[MAX_COARSE_LEVELS_HOST], s_cof[MAX_COARSE_LEVELS_HOST];
+  __shared__ float2 coef[CG_COEF];
+  __shared__ float4 inv_sm[CG_INV];
+  __shared__ CgShared sh;
+  constexpr int NVEC = cg_vectors(S);
+  const int tid = threadIdx.x, prob = blockIdx.x;
+  const LevelDev<float2>* G = levs_all + (size_t)prob * lev_stride;
+  const CoarseLU lu = lus[prob];
+  const int nlev = lu.nlev;
+  {  // descriptors (a word per thread)
+    constexpr int W = (int)(sizeof(LevelDev<float2>) / sizeof(int));
+    for (int i = tid; i < nlev * W; i += CG_THREADS)
+      reinterpret_cast<int*>(Ls)[i] = reinterpret_cast<const int*>(G)[i];
+  }
+  __syncthreads();
+  int total = 0, ctot = 0;
+  for (int l = 0; l < nlev; ++l) {
+    const int P = Ls[l].P, np = DIM == 3 ? P * P * P : P * P;
+    if (tid == 0) {
+      s_base[l] = total + np / P;  // a guard row (plane) of zeros before the level's first vector
+      s_cof[l] = ctot;
+    }
+    total += np / P + NVEC * np;
+    ctot += 3 * Ls[l].n;
+  }
+  for (int i = tid; i < total; i += CG_THREADS) cgsm[i] = make_float2(0.f, 0.f);
+  __syncthreads();
+  for (int l = 0; l < nlev; ++l)
+    for (int i = tid; i < 3 * Ls[l].n; i += CG_THREADS) coef[s_cof[l] + i] = __ldg(Ls[l].ca + i);
+  const bool staged = lu.m * lu.m <= CG_INV;
+  if (staged)
+    for (int i = tid; i < lu.m * lu.m; i += CG_THREADS) inv_sm[i] = __ldg(lu.inv + i);
+  __syncthreads();
+  CgLevel<S, DIM> V;
+  auto enter = [&](int l) {
+    const int P = Ls[l].P, np = DIM == 3 ? P * P * P : P * P;
+    float2* v = cgsm + s_base[l];
+    V.b = v;
+    V.x = v + np;
+    V.r = v + 2 * np;
+#pragma unroll
+    for (int j = 0; j + 1 < S; ++j) V.k[j] = v + (3 + j) * np;
+    V.stencil_setup(Ls[l], coef + s_cof[l], tid);
+  };
+  enter(0);
+  pdl_wait();
+  pdl_trigger();
+#pragma unroll
+  for (int q = 0; q < CG_PT; ++q)
+    if (V.on[q]) V.b[V.off[q]] = G[0].b[V.off[q]];
+  __syncthreads();
+  // descent
+  for (int l = 0; l < nlev - 1; ++l) {
+    if (l > 0) enter(l);
+    float2 k0[CG_PT], x[CG_PT];
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) {
+      k0[q] = V.on[q] ? V.b[V.off[q]] : make_float2(0.f, 0.f);
+      x[q] = make_float2(0.f, 0.f);
+    }
+    const float2* R0 = V.b;
+    for (int sw = 0; sw < nu1; ++sw) {
+      float2 sg[S];
+      gram_shifts<S>(Ls[l], sw == 0, sg);
+      cg_sweep<S, DIM>(V, R0, k0, x, sg, sh);
+      R0 = V.r;
+#pragma unroll
+      for (int q = 0; q < CG_PT; ++q)
+        if (V.on[q]) V.r[V.off[q]] = k0[q];
+      __syncthreads();
+    }
+    const float2* rr = nu1 > 0 ? V.r : V.b;
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q)
+      if (V.on[q]) V.x[V.off[q]] = x[q];
+    // b_c = full weighting of the residual
+    const int nc = Ls[l + 1].n, Pc = Ls[l + 1].P, P = V.P;
+    const int ncp = DIM == 3 ? nc * nc * nc : nc * nc;
+    float2* bc = cgsm + s_base[l + 1];
+    for (int i = tid; i < ncp; i += CG_THREADS) {
+      const int yy = i / nc, X = i - yy * nc, Z = DIM == 3 ? yy / nc : 0, Y = yy - Z * nc;
+      const float2* f = rr + (DIM == 3 ? (2 * Z + 1) * P * P : 0) + (2 * Y + 1) * P + 2 * X + 1;
+      float2 out = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int dz = (DIM == 3 ? -1 : 0); dz <= (DIM == 3 ? 1 : 0); ++dz)
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+          for (int dx = -1; dx <= 1; ++dx) {
+            const float wgt = (dx == 0 ? 0.5f : 0.25f) * (dy == 0 ? 0.5f : 0.25f) * (DIM == 3 ? (dz == 0 ? 0.5f : 0.25f) : 1.0f);
+            const float2 v = f[(dz * P + dy) * P + dx];
+            out.x = fmaf(wgt, v.x, out.x);
+            out.y = fmaf(wgt, v.y, out.y);
+          }
+      bc[((DIM == 3 ? Z * Pc : 0) + Y) * Pc + X] = out;
+    }
+    __syncthreads();
+  }
+  // coarsest: x = A^{-1} b, sixteen lanes per row, double-float sums
+  {
+    const LevelDev<float2>& L = Ls[nlev - 1];
+    const int m = lu.m, n = L.n, P = L.P, np = DIM == 3 ? P * P * P : P * P;
+    const float2* b = cgsm + s_base[nlev - 1];
+    float2* x = cgsm + s_base[nlev - 1] + np;
+    const float4* inv = staged ? inv_sm : lu.inv;
+    const int l16 = tid & 15;
+    auto at = [&](int i) {
+      const int yy = i / n, X = i - yy * n, Z = DIM == 3 ? yy / n : 0, Y = yy - Z * n;
+      return (Z * P + Y) * P + X;
+    };
+    for (int r0 = 0; r0 < m; r0 += CG_THREADS / 16) {  // the same trips for every thread
+      const int row = r0 + (tid >> 4);
+      float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
+      if (row < m)
+        for (int j = l16; j < m; j += 16) {
+          const float4 a = inv[(size_t)row * m + j];
+          const float2 v = b[at(j)];
+          df_mac1(sr, cr, a.x, a.y, v.x);
+          df_mac1(sr, cr, -a.z, -a.w, v.y);
+          df_mac1(si, ci, a.x, a.y, v.y);
+          df_mac1(si, ci, a.z, a.w, v.x);
+        }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        float t, r;
+        const float s2 = __shfl_xor_sync(0xffffffffu, sr, o), c2 = __shfl_xor_sync(0xffffffffu, cr, o);
+        df_two_sum(sr, s2, t, r);
+        cr = (cr + c2) + r;
+        sr = t;
+        const float s3 = __shfl_xor_sync(0xffffffffu, si, o), c3 = __shfl_xor_sync(0xffffffffu, ci, o);
+        df_two_sum(si, s3, t, r);
+        ci = (ci + c3) + r;
+        si = t;
+      }
+      if (row < m && l16 == 0) x[at(row)] = make_float2(sr + cr, si + ci);
+    }
+    __syncthreads();
+  }
+  // ascent
+  for (int l = nlev - 2; l >= 0; --l) {
+    enter(l);
+    const int Pc = Ls[l + 1].P, npc = DIM == 3 ? Pc * Pc * Pc : Pc * Pc;
+    const float2* xcv = cgsm + s_base[l + 1] + npc;  // ghosts zero, and zeros before it (b's ghosts)
+    float2 k0[CG_PT], x[CG_PT];
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) {
+      x[q] = make_float2(0.f, 0.f);
+      if (!V.on[q]) continue;
+      // odd i: coarse (i - 1) / 2; even i: the mean of i / 2 - 1 and i / 2
+      const int X = V.cx[q] >> 1, Y = V.cy[q] >> 1, Z = V.cz[q] >> 1;
+      const int dx = (V.cx[q] & 1) ? 0 : 1, dy = (V.cy[q] & 1) ? 0 : Pc, dz = (DIM == 3 && !(V.cz[q] & 1)) ? Pc * Pc : 0;
+      const float2* f = xcv + ((DIM == 3 ? Z * Pc : 0) + Y) * Pc + X;
+      float2 e = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < (DIM == 3 ? 2 : 1); ++c)
+#pragma unroll
+        for (int bq = 0; bq < 2; ++bq) {
+          const float2 v0 = f[-(c ? dz : 0) - (bq ? dy : 0)], v1 = f[-(c ? dz : 0) - (bq ? dy : 0) - dx];
+          e = cadd(e, cadd(v0, v1));
+        }
+      const float w = DIM == 3 ? 0.125f : 0.25f;
+      x[q] = cadd(V.x[V.off[q]], make_float2(e.x * w, e.y * w));
+    }
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q)
+      if (V.on[q]) V.x[V.off[q]] = x[q];
+    __syncthreads();
+    if (nu2 > 0) {
+      float2 z0 = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < CG_PT; ++q) {
+        k0[q] = make_float2(0.f, 0.f);
+        if (V.on[q]) {
+          const float2 p = V.apply(V.x, x[q], q, z0);
+          k0[q] = csub(V.b[V.off[q]], make_float2(p.x * V.it, p.y * V.it));
+          V.r[V.off[q]] = k0[q];
+        }
+      }
+      __syncthreads();
+      for (int sw = 0; sw < nu2; ++sw) {
+        float2 sg[S];
+        gram_shifts<S>(Ls[l], false, sg);
+        cg_sweep<S, DIM>(V, V.r, k0, x, sg, sh);
+        if (sw + 1 < nu2) {
+#pragma unroll
+          for (int q = 0; q < CG_PT; ++q)
+            if (V.on[q]) V.r[V.off[q]] = k0[q];
+          __syncthreads();
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < CG_PT; ++q)
+        if (V.on[q]) V.x[V.off[q]] = x[q];
+      __syncthreads();
+    }
+  }
+  {  // the top level's result, ghosts included
+    const int P = Ls[0].P, np = DIM == 3 ? P * P * P : P * P;
+    const float2* x = cgsm + s_base[0] + np;
+    float2* out = Ls[0].xb;
+    for (int i = tid; i < np; i += CG_THREADS) out[i] = x[i];
+  }
+}
+
+}  // namespace helm

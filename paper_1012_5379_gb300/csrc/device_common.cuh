@@ -488,4 +488,17 @@ __device__ inline void grid_sum_sweep(T (&v)[2 * J + 1], void* partv, int tile, 
   for (int i = tid; i < words; i += nt) gsrc[i] = sdst[i];
 }
 
+// ------------------------------------------------------------------ first shift of a Gram sweep (gram.cuh)
+// v rounded to 8 significant bits (towards zero).
+__device__ __forceinline__ float bits8(float v) { return __uint_as_float(__float_as_uint(v) & 0xffff0000u); }
+
+// The finest level's first shift from diff2 = sum |b_{x+1} - b_x|^2 over the pairs of
+// neighbours counted and norm2 = sum |b|^2: the Rayleigh quotient of the Laplacian's
+// isotropic estimate, minus the constant wavenumber term.  klap = (d / h^2) e^{-2 i theta}.
+__device__ __forceinline__ float2 sweep_first_shift(float2 klap, float phic, float diff2, float norm2) {
+  const float e = norm2 > 0.0f ? fminf(diff2 / norm2, 2.0f) : 0.0f;
+  if (!isfinite(e)) return make_float2(0.f, 0.f);
+  return make_float2(bits8(klap.x * e - phic), bits8(klap.y * e));
+}
+
 }  // namespace helm

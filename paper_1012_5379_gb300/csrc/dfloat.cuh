@@ -29,7 +29,7 @@ namespace helm {
 // Kept out of line: inlined, the compiler predicates it into every split, and its FP64
 // instructions then occupy the FP64 pipe for every point (measured: the cycle-start pass
 // at 85% of that pipe).
-__device__ __noinline__ float2 df_split_rare(double x) {
+static __device__ __noinline__ float2 df_split_rare(double x) {
   const float h = __double2float_rn(x);
   return make_float2(h, __double2float_rn(x - (double)h));
 }

@@ -81,6 +81,21 @@ static int upload_level_coefficients(Handle* h, int l, double theta_beta, cudaSt
     const cplx per_axis(0.0, -h->csl_eps * h->k * h->k / h->dim);
     for (auto& v : d) v += per_axis;
   }
+  if (h->prec == HELM_C64) {
+    // basis of the Gram sweeps (gram.cuh): the interior's Laplacian scale and diagonal, and a
+    // power of two near the reciprocal of half the spectrum's width
+    const int mid = L.n / 2;
+    const cplx lap = -0.5 * (double)h->dim * (a[mid] + c[mid]);
+    const cplx diag = (double)h->dim * d[mid] - (L.phi ? 0.0 : L.phic);
+    auto bits8 = [](double v) {
+      int e = 0;
+      const double m = std::frexp(v, &e);
+      return (float)std::ldexp(std::trunc(m * 256.0) / 256.0, e);
+    };
+    L.kt = (float)std::ldexp(1.0, -(int)std::lround(std::log2(2.0 * std::abs(lap))));
+    L.ksh = make_float2(bits8(diag.real()), bits8(diag.imag()));
+    L.klap = make_float2((float)lap.real(), (float)lap.imag());
+  }
   double2* c64 = reinterpret_cast<double2*>(h->stage + h->stage_coef[l]);
   for (int i = 0; i < L.n; ++i) {
     c64[i] = make_double2(a[i].real(), a[i].imag());
@@ -116,6 +131,30 @@ static int factor_coarsest(Handle* h, double theta_beta, cudaStream_t st) {
   std::vector<cplx> A = dense_operator(h->dim, Lc.n, a, d, c, phic, cplx(1.0, h->csl_eps));
   std::vector<int> perm;
   if (!lu_factor(A, cm, perm)) { set_error("coarsest operator is singular"); return HELM_ENUMERIC; }
+  if (h->prec == HELM_C64) {
+    // the inverse, column by column from the factors (binary64), as double-floats
+    float4* iv = reinterpret_cast<float4*>(h->stage + h->stage_inv);
+    std::vector<cplx> y(cm);
+    auto split = [](double v, float* hi, float* lo) {
+      *hi = (float)v;
+      *lo = (float)(v - (double)*hi);
+    };
+    for (int j = 0; j < cm; ++j) {
+      for (int i = 0; i < cm; ++i) y[i] = perm[i] == j ? 1.0 : 0.0;
+      for (int i = 0; i < cm; ++i)
+        for (int q = 0; q < i; ++q) y[i] -= A[(size_t)i * cm + q] * y[q];
+      for (int i = cm - 1; i >= 0; --i) {
+        for (int q = i + 1; q < cm; ++q) y[i] -= A[(size_t)i * cm + q] * y[q];
+        y[i] /= A[(size_t)i * cm + i];
+      }
+      for (int i = 0; i < cm; ++i) {
+        float4& o = iv[(size_t)i * cm + j];
+        split(y[i].real(), &o.x, &o.y);
+        split(y[i].imag(), &o.z, &o.w);
+      }
+    }
+    CUDA_TRY(cudaMemcpyAsync(h->inv, iv, A.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
+  }
   double2* Ad = reinterpret_cast<double2*>(h->stage + h->stage_lu);
   int* pv = reinterpret_cast<int*>(h->stage + h->stage_piv);
   for (size_t i = 0; i < A.size(); ++i) Ad[i] = make_double2(A[i].real(), A[i].imag());
@@ -229,6 +268,8 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     off += r256((size_t)cm * cm * sizeof(double2));
     h->stage_piv = off;
     off += r256((size_t)cm * sizeof(int));
+    h->stage_inv = off;
+    if (h->prec == HELM_C64) off += r256((size_t)cm * cm * sizeof(float4));
     h->stage_coef.resize(nlev);
     for (int l = 0; l < nlev; ++l) {
       h->stage_coef[l] = off;
@@ -261,39 +302,40 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     const size_t scb = h->prec == HELM_C128 ? sizeof(SweepScalarsT<double>) : sizeof(SweepScalarsT<float>);
     TRY(dev_alloc(h.get(), &L.sc, scb));
     CUDA_TRY(cudaMemsetAsync(L.sc, 0, scb, st));
-    // partial slots: one per tile of the marching passes, per flat-pass CTA, and per
-    // share of the 3D TMA-fed pass
+    // partial slots: one per tile of the marching passes and per flat-pass CTA (complex128:
+    // NPART sums each), or per CTA of the sweep pass (complex64: GRAM_SLOT double-floats)
     size_t nparts = std::max<size_t>(std::max(L.ntiles, L.nflat), 1);
     if (h->dim == 3) {
       TileCfg finest;  // the most tiles a tuned plane count (2) gives
       finest.rows = 2;
-      nparts = std::max<size_t>(nparts, std::max<size_t>(TMA3_MAX_UNITS, tiles_per_problem(3, L.P, finest)));
+      nparts = std::max<size_t>(nparts, tiles_per_problem(3, L.P, finest));
     }
-    TRY(dev_alloc(h.get(), &L.part, nparts * NPART * sizeof(double)));
-    // TMA maps of the raw vectors the complex64 Arnoldi passes stream
-    // (3D: two sets, for column tiles of 16 and of 32 rows)
-    if (h->prec == HELM_C64 && L.P >= 64 && (h->dim == 2 || L.P % 32 == 0)) {
-      const int nmaps = h->dim == 2 ? TM_COUNT : 2 * TM_COUNT;
-      std::vector<CUtensorMap> maps(nmaps);
+    size_t part_bytes = nparts * NPART * sizeof(double);
+    if (h->prec == HELM_C64) {
+      L.sweep = sweep_cfg(h->dim, L.n, h->s, sm_count_host());
+      part_bytes = std::max(part_bytes, (size_t)L.sweep.units * GRAM_SLOT * sizeof(float2));
+    }
+    TRY(dev_alloc(h.get(), &L.part, part_bytes));
+    // TMA maps of the vectors the large 3D complex64 levels' passes stream (two sets, for
+    // column tiles of 16 and of 32 rows)
+    if (h->prec == HELM_C64 && h->dim == 3 && L.P >= 64 && L.P % 32 == 0) {
+      std::vector<CUtensorMap> maps(2 * TM_COUNT);
       const void* vecs[TM_COUNT] = {};
       vecs[TM_B] = L.b;
       vecs[TM_R0] = L.r0;
       vecs[TM_XB] = L.xb;
       for (int j = 0; j < h->s; ++j) vecs[TM_P0 + j] = L.p[j];
-      const bool encoded = h->dim == 2 ? encode_level_tmaps(L.P, vecs, TM_COUNT, maps.data())
-                                       : encode_level_tmaps3(L.P, 18, vecs, TM_COUNT, maps.data()) &&
-                                             encode_level_tmaps3(L.P, 34, vecs, TM_COUNT, maps.data() + TM_COUNT);
-      if (encoded) {
+      if (encode_level_tmaps3(L.P, 18, vecs, TM_COUNT, maps.data()) &&
+          encode_level_tmaps3(L.P, 34, vecs, TM_COUNT, maps.data() + TM_COUNT)) {
         CUtensorMap* dtm = nullptr;
-        TRY(dev_alloc(h.get(), &dtm, nmaps * sizeof(CUtensorMap)));
-        CUDA_TRY(cudaMemcpyAsync(dtm, maps.data(), nmaps * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
+        TRY(dev_alloc(h.get(), &dtm, maps.size() * sizeof(CUtensorMap)));
+        CUDA_TRY(cudaMemcpyAsync(dtm, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
         L.tm = dtm;
       }
     }
     // coefficients of M on this level (rediscretisation with spacing 2^l h)
     TRY(dev_alloc(h.get(), &L.coef64, 3 * L.n * sizeof(double2)));
     TRY(dev_alloc(h.get(), &L.coef, 3 * L.n * eb));
-    TRY(upload_level_coefficients(h.get(), l, theta_beta, st));
     // phi sampled at this level's nodes (node x of level l is fine node (x+1) 2^l - 1)
     if (phi) {
       TRY(dev_alloc(h.get(), &L.phi, L.np * sizeof(float)));
@@ -302,11 +344,13 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     } else {
       L.phic = k * k;
     }
+    TRY(upload_level_coefficients(h.get(), l, theta_beta, st));
   }
   // ------------------------------------------------ coarsest LU (FP64)
   h->lu_m = cm;
   TRY(dev_alloc(h.get(), &h->lu, (size_t)cm * cm * sizeof(double2)));
   TRY(dev_alloc(h.get(), &h->piv, cm * sizeof(int)));
+  if (h->prec == HELM_C64) TRY(dev_alloc(h.get(), &h->inv, (size_t)cm * cm * sizeof(float4)));
   TRY(factor_coarsest(h.get(), theta_beta, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   // ------------------------------------------------ H and the outer storage
@@ -392,6 +436,10 @@ static LevelDev<C> make_leveldev(const Handle& h, int l) {
   d.sc = (SS*)L.sc;
   d.part = L.part;
   d.tm = L.tm;
+  d.kt = L.kt;
+  d.ksh = L.ksh;
+  d.klap = L.klap;
+  d.top = l == 0;
   if (l + 1 < (int)h.lev.size()) {
     const HostLevel& Lc = h.lev[l + 1];
     d.nc = Lc.n;
@@ -436,6 +484,8 @@ static OuterDev<C> make_outerdev(const Handle& h) {
   o.gcnt = h.dcnt;
   o.st = h.st;
   o.sc0 = (SweepScalarsT<typename RealOf<C>::T>*)h.lev[0].sc;
+  o.klap = h.lev[0].klap;
+  o.phir = (float)h.lev[0].phic;
   return o;
 }
 
@@ -448,6 +498,8 @@ struct Group {
   struct Depth {
     int n = 0, cnt = 0, ntiles = 0, nflat = 0;
     bool tma = true;  // every problem at this depth has TMA maps
+    SweepCfg sweep{}; // complex64: the sweep pass's launch choice
+    bool phi = false; // some problem at this depth has a wavenumber field
     TileCfg cfg{8};
     LevelDev<C>* d = nullptr;
     C* pw = nullptr;  // polynomial smoother: three Richardson weights per problem
@@ -552,6 +604,11 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     for (int p = 0; p < count; ++p) if (off[p] == 0) big = hs[p];
     size_t bytes = 0;
     for (int t = g->tc; t < g->Lmax; ++t) bytes += (size_t)(4 + g->s) * big->lev[t].np * sizeof(C);
+    if (sizeof(C) == 8) {
+      std::vector<int> ns;
+      for (int t = g->tc; t < g->Lmax; ++t) ns.push_back(big->lev[t].n);
+      bytes = coarse_gram_smem(g->dim, g->s, ns.data(), (int)ns.size());
+    }
     g->coarse_smem = (g->nlev_c <= MAX_COARSE_LEVELS_HOST && bytes <= 200 * 1024) ? bytes : 0;
   }
   // tile config of a group: the first problem's
@@ -581,6 +638,8 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
       D.cnt += 1;
       D.tma = D.tma && L.tm != nullptr;
       D.nflat = L.nflat;
+      D.sweep = L.sweep;
+      D.phi = D.phi || L.phi != nullptr;
       D.cfg.rows = g->dim == 3 ? tuned_zchunk(L.P, (int)sizeof(C)) : zchunk(L.P);
       D.cfg.P = L.P;
       D.ntiles = g->dim == 3 ? tiles_per_problem(3, L.P, D.cfg) : L.ntiles;
@@ -601,6 +660,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     c.m = hs[p]->lu_m;
     c.lu = hs[p]->lu;
     c.piv = hs[p]->piv;
+    c.inv = hs[p]->inv;
     lus.push_back(c);
   }
   std::vector<LevelDev<C>> lev0;
@@ -700,6 +760,15 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   return HELM_OK;
 }
 
+// The coarse sub-cycle of every problem, one CTA each.
+template <typename C>
+static void launch_coarse_part(const Group<C>& g, cudaStream_t st) {
+  if constexpr (sizeof(C) == 8)
+    launch_coarse_gram(g.dim, g.s, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
+  else
+    launch_coarse_smem<C>(g.dim, g.dcoarse, g.nlev_c, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
+}
+
 // One V(nu1, nu2) cycle from a zero guess on every problem of the group (Sec. 3.1).
 // Algorithmic bytes per launch count every vector the pass must read or write once
 // (E bytes per complex value), plus 4 bytes per point for a phi field.
@@ -737,10 +806,7 @@ static void run_vcycle_poly(const Group<C>& g, cudaStream_t st) {
   }
   {
     Launch L("vc.coarse", st, 0, 0);
-    if (g.coarse_smem > 0)
-      launch_coarse_smem<C>(dim, g.dcoarse, g.nlev_c, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
-    else
-      launch_coarse_cluster<C>(dim, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, st);
+    launch_coarse_part<C>(g, st);
   }
   for (int t = g.tc - 1; t >= 0; --t) {
     const auto& D = g.depth[t];
@@ -775,6 +841,34 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
     seq.npass = 0;
     seq_bytes = 0;
   };
+  // One sweep's Krylov vectors and coefficients: complex64 in one pass (gram.cuh), complex128
+  // one Arnoldi step per pass; store_last: the last vector is read again.
+  auto arnoldi = [&](const typename Group<C>::Depth& D, bool first, bool store_last, bool fine, bool rec, double ph,
+                     double pts) {
+    const char* name = fine ? "vc.arnoldi.l0" : "vc.arnoldi.lc";
+    if constexpr (sizeof(C) == 8) {
+      const double bytes = pts * (E * (g.s + (store_last ? 1 : 0)) + ph);
+      if (rec) {
+        record_sweep(seq, g.s, D.d, D.cnt, D.sweep, first, store_last);
+        seq_bytes += bytes;
+        return;
+      }
+      Launch L(name, st, bytes, pts * (8.0 * (2 * dim + 1) * g.s + 4.0 * (g.s + 1) * (g.s + 1)));
+      launch_sweep(dim, g.s, D.d, D.cnt, D.sweep, first, store_last, D.phi, st);
+    } else {
+      for (int J = 1; J <= g.s; ++J) {
+        const bool store = J < g.s || store_last;
+        const double bytes = pts * (E * (J + (store ? 1 : 0)) + ph);
+        if (rec) {
+          record_arnoldi<C>(seq, dim, J, D.d, D.cnt, D.ntiles, D.cfg, first, store);
+          seq_bytes += bytes;
+          continue;
+        }
+        Launch L(name, st, bytes, pts * (8.0 * (2 * dim + 1) + 8.0 * J + 4));
+        launch_arnoldi<C>(dim, J, D.d, D.cnt, D.ntiles, D.cfg, first, store, st);
+      }
+    }
+  };
   for (int t = 0; t < g.tc; ++t) {
     const auto& D = g.depth[t];
     const double pts = (double)D.cnt * (dim == 3 ? (double)(D.n + 1) * (D.n + 1) * (D.n + 1) : (double)(D.n + 1) * (D.n + 1));
@@ -792,15 +886,7 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
       continue;
     }
     for (int sw = 0; sw < g.nu1; ++sw) {
-      for (int J = 1; J <= g.s; ++J) {
-        if (rec) {
-          record_arnoldi<C>(seq, dim, J, D.d, D.cnt, D.ntiles, D.cfg, sw == 0, true);
-          seq_bytes += pts * (E * (J + 1) + ph);
-          continue;
-        }
-        Launch L(fine ? "vc.arnoldi.l0" : "vc.arnoldi.lc", st, pts * (E * (J + 1) + ph), pts * (8.0 * (2 * dim + 1) + 8.0 * J + 4));
-        launch_arnoldi<C>(dim, J, D.d, D.cnt, D.ntiles, D.cfg, sw == 0, true, D.tma, st);
-      }
+      arnoldi(D, sw == 0, true, fine, rec, ph, pts);
       if (sw < g.nu1 - 1) {
         if (rec) {
           record_update<C>(seq, dim, UPD_RESIDUAL, D.d, D.cnt, D.nflat, sw == 0, 0, sw == 0);
@@ -823,10 +909,7 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
   flush("vc.seq.down");
   {
     Launch L("vc.coarse", st, 0, 0);
-    if (g.coarse_smem > 0)
-      launch_coarse_smem<C>(dim, g.dcoarse, g.nlev_c, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
-    else
-      launch_coarse_cluster<C>(dim, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, st);
+    launch_coarse_part<C>(g, st);
   }
   for (int t = g.tc - 1; t >= 0; --t) {
     const auto& D = g.depth[t];
@@ -846,17 +929,7 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
     }
     for (int sw = 0; sw < g.nu2; ++sw) {
       const bool last = (sw == g.nu2 - 1);
-      for (int J = 1; J <= g.s; ++J) {
-        const bool store = J < g.s || !last;
-        if (rec) {
-          record_arnoldi<C>(seq, dim, J, D.d, D.cnt, D.ntiles, D.cfg, false, store);
-          seq_bytes += pts * (E * (J + (store ? 1 : 0)) + ph);
-          continue;
-        }
-        Launch L(fine ? "vc.arnoldi.l0" : "vc.arnoldi.lc", st, pts * (E * (J + (store ? 1 : 0)) + ph),
-                 pts * (8.0 * (2 * dim + 1) + 8.0 * J + 4));
-        launch_arnoldi<C>(dim, J, D.d, D.cnt, D.ntiles, D.cfg, false, store, D.tma, st);
-      }
+      arnoldi(D, false, !last, fine, rec, ph, pts);
       if (rec) {
         record_update<C>(seq, dim, last ? UPD_XONLY : UPD_RESIDUAL, D.d, D.cnt, D.nflat, false, 1, false);
         seq_bytes += pts * E * (last ? g.s + 2.0 : g.s + 4.0);
@@ -1461,6 +1534,8 @@ size_t estimate_handle_bytes(int dim, int n, int prec, int s, int restart, int m
   bytes += 3 * vs * sizeof(double2) + (m + 1) * vs * sizeof(double2) + m * vs * eb + (m + 1) * (m + 8) * 16;
   bytes += outer_part_doubles(outer_chunks(vs), (int)m) * sizeof(double);
   bytes += (size_t)outer_dot_counters(outer_chunks(vs)) * sizeof(unsigned);
+  if (prec == HELM_C64)
+    for (int nl : sizes) bytes += (size_t)sweep_cfg(dim, nl, s, sm_count_host()).units * GRAM_SLOT * sizeof(float2);
   return bytes;
 }
 

@@ -49,7 +49,10 @@ struct HostLevel {
   float* phi = nullptr;     // padded phi or nullptr
   double phic = 0.0;
   void* sc = nullptr;          // SweepScalarsT<R> of the preconditioner precision
-  const CUtensorMap* tm = nullptr;  // TMA maps (2D complex64 grid-wide levels), device memory
+  const CUtensorMap* tm = nullptr;  // TMA maps (3D complex64 grid-wide levels), device memory
+  float kt = 0;                // Gram sweeps (complex64): basis scale, shift, Laplacian scale
+  float2 ksh{}, klap{};
+  SweepCfg sweep{};            // the sweep pass's launch choice
   double* part = nullptr;
 };
 
@@ -68,6 +71,7 @@ struct Handle {
   double2* lu = nullptr;
   int* piv = nullptr;
   int lu_m = 0;
+  float4* inv = nullptr;      // complex64: the coarsest inverse as double-floats
   double2* hcoef = nullptr;   // 3n FP64 coefficients of H
   float4* hcoef_df = nullptr; // the same as double-floats (hi + lo, rounded to nearest)
   // outer FGMRES storage
@@ -98,7 +102,7 @@ struct Handle {
   // the outer state, the coarsest LU and pivots, each level's coefficients (FP64 and
   // the preconditioner precision), at fixed offsets
   char* stage = nullptr;
-  size_t stage_lu = 0, stage_piv = 0;
+  size_t stage_lu = 0, stage_piv = 0, stage_inv = 0;
   std::vector<size_t> stage_coef;  // per level: FP64 block, then the level-precision block
   ~Handle();
 };

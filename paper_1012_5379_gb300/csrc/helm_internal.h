@@ -24,6 +24,7 @@ namespace helm {
 
 constexpr int SMAX = 4;            // max GMRES(s) steps per smoothing sweep
 constexpr int NPART = 2 * SMAX + 4;  // doubles per partial-sum slot of a sweep pass
+constexpr int GRAM_SLOT = 32;        // double-floats per partial slot of a Gram sweep pass (gram.cuh)
 
 // Real and complex scalar types of a preconditioner precision.
 template <typename C> struct RealOf;
@@ -50,6 +51,7 @@ struct SweepScalarsT {
   CR rcoef[SMAX + 1];             // r_new = sum_k rcoef[k] R_k
   int status;                     // nonzero: NaN/Inf seen
   int pad0;
+  CR sig0;                        // complex64: first basis shift of the finest level's first sweep (gram.cuh)
   // everything above is the sweep algebra's state (staged through shared memory);
   // the reduction counter below is never part of that copy
   unsigned int counter;           // last-block-done counter
@@ -79,7 +81,12 @@ struct LevelDev {
   SweepScalarsT<typename RealOf<C>::T>* sc;   // this level's sweep state
   SweepScalarsT<typename RealOf<C>::T>* scc;  // coarser level's sweep state
   double* part;           // partial sums: ntiles * NPART slots (R or double)
-  const CUtensorMap* tm;  // 2D complex64 levels: TMA maps of b, r0, p_1..p_SMAX (else nullptr)
+  const CUtensorMap* tm;  // 3D complex64 levels: TMA maps of b, r0, p_1..p_SMAX, xb (else nullptr)
+  // Gram sweeps (complex64, gram.cuh)
+  float kt;               // basis scale: a power of two near 1 / (spectral half width)
+  float2 ksh;             // the stencil's diagonal in the interior, to 8 significant bits
+  float2 klap;            // d / h^2 of the interior spacing (the Laplacian's scale)
+  int top;                // 1: the problem's finest level
 };
 
 // TMA maps per level: b, r0, p_1..p_SMAX (in this order).
@@ -93,6 +100,7 @@ struct CoarseLU {
   int nlev;               // levels of the problem's coarse sub-cycle
   const double2* lu;      // m*m
   const int* piv;         // m
+  const float4* inv;      // complex64: m*m entries of the inverse as double-floats (re hi, lo, im hi, lo)
 };
 
 // Outer FGMRES state of one problem (FP64, device memory).
@@ -144,6 +152,7 @@ struct OuterDev {
   unsigned* gcnt;         // the multi-dot's group counters (zero between calls)
   OuterState* st;
   SweepScalarsT<typename RealOf<C>::T>* sc0;  // level-0 sweep state (set by the kernel that writes b0)
+  float2 klap; float phir;  // level 0's Laplacian scale and constant wavenumber term (first basis shift)
 };
 
 // Tile configuration: rows (2D) or planes (3D) marched per warp / CTA (even).
@@ -163,6 +172,15 @@ HELM_HD inline int zchunk(int P) { return P >= 128 ? 32 : (P >= 64 ? 4 : 2); }
 HELM_HD inline int vtiles(int dim, int P) {
   return dim == 2 ? ceil_div(P, 64) * ceil_div(P, 16) : ceil_div(P, 32) * ceil_div(P, 8) * ceil_div(P, zchunk(P));
 }
+
+// Launch choice of a complex64 level's sweep pass (sweep.cuh): 2D rows per warp `geo`; 3D
+// small levels (march = 0) the own rows `geo` of a CTA in y and z, large levels planes `geo`
+// per march; `units` CTAs per problem.  A function of the level size, the sweep's steps and
+// the device's SM count only.
+struct SweepCfg {
+  int march, geo, units;
+};
+SweepCfg sweep_cfg(int dim, int n, int S, int sms);
 
 // Marching FP64 stencil of the outer solve: 2D warps march cfg.rows rows, 3D CTAs
 // march cfg.rows planes.
@@ -201,7 +219,16 @@ enum UpdateMode { UPD_RESTRICT = 0, UPD_RESIDUAL = 1, UPD_XONLY = 2 };
 // V-cycle passes (vcycle_c64.cu / vcycle_c128.cu), C = float2 or double2.
 template <typename C>
 void launch_arnoldi(int dim, int J, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
-                    bool store_p, bool tma, cudaStream_t st);
+                    bool store_p, cudaStream_t st);
+// the complex64 sweep's basis and minimisation (first: R_0 = b, else r0; store_last: keep k_S)
+void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
+                  bool store_last, bool phi, cudaStream_t st);
+void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
+                  bool store_last);
+// the complex64 coarse sub-cycle; smem from coarse_gram_smem over its level sizes
+void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
+                        int nu1, int nu2, size_t smem, cudaStream_t st);
+size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev);
 template <typename C>
 void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
                      bool x_from_zero, bool nosmooth, cudaStream_t st, bool tma = false, int nraw = SMAX + 1);
@@ -229,10 +256,7 @@ int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_
 template <typename C>
 void launch_coarse(int dim, const LevelDev<C>* levs, int nlev, int lev_stride, const CoarseLU* lus, int nprob,
                    int nu1, int nu2, cudaStream_t st);
-// coarse sub-cycle staged in shared memory (smem_bytes: all levels' vectors)
-template <typename C>
-void launch_coarse_cluster(int dim, const LevelDev<C>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                           int nu1, int nu2, cudaStream_t st);
+// complex128 coarse sub-cycle staged in shared memory (smem_bytes: all levels' vectors)
 template <typename C>
 void launch_coarse_smem(int dim, const LevelDev<C>* levs, int nlev, int lev_stride, const CoarseLU* lus, int nprob,
                         int nu1, int nu2, size_t smem_bytes, cudaStream_t st);
@@ -247,20 +271,16 @@ template <typename C>
 void outer_residual(int dim, const OuterDev<C>* od, int nprob, int ntiles, TileCfg cfg, cudaStream_t st);
 template <typename C>
 void outer_apply_h(int dim, const OuterDev<C>* od, int nprob, int ntiles, TileCfg cfg, cudaStream_t st);
-// TMA maps of a 2D complex64 level (tma.cpp): a 136 x 18 float box (64 x 16 complex
-// points plus halo) over a P x P complex field.  False when the driver has no
-// tensor-map encoder or the layout does not meet its rules.
-bool encode_level_tmaps(int P, const void* const* vectors, int count, CUtensorMap* out);
 // TMA maps of a 3D complex64 level (tma.cpp): 72 x box_rows x 1 float boxes (a 32-point
 // wide column tile plus halo, one plane) over a P^3 complex field; P a multiple of 32.
 bool encode_level_tmaps3(int P, int box_rows, const void* const* vectors, int count, CUtensorMap* out);
 // ---------------------------------------------------------------- tuned launch choices
 // (tune.cpp) keyed by pass, dimension, level pitch P, precision (bytes per complex
 // value) and Arnoldi step J (0 for the other passes); TUNE_NV integers per choice:
-//   arnoldi (step J) and prolong (J = 0), 3D, complex64: {TMA-fed pass on, plane slots
-//                            in flight, z pieces per column (0: one equal share per
-//                            resident CTA), points per thread in y (2 or 4; 0: 2)}
-//   arnoldi / restrict / prolong, 2D: {tiles per CTA}
+//   restrict and prolong, 3D, complex64: {TMA-fed pass on, plane slots in flight, z pieces
+//                            per column (0: one equal share per resident CTA), points per
+//                            thread in y (2 or 4; 0: 2; the restriction always takes 2)}
+//   restrict / prolong, 2D, and arnoldi (step J, complex128), 2D: {tiles per CTA}
 //   persist, 2D/3D: {grid-wide level run inside the persistent segments (1) or by its
 //                    own launches (0)}
 enum TunePass { TP_ARNOLDI = 0, TP_RESTRICT = 1, TP_PROLONG = 2, TP_PERSIST = 3, TP_ZPLANES = 4 };
@@ -290,15 +310,15 @@ bool persist_level(int dim, int P, int prec_bytes);
 unsigned long long barrier_limit_ns();
 void set_barrier_limit_ns(unsigned long long ns);
 
-// The 3D TMA-fed Arnoldi pass of step J on a level of pitch P: whether it runs (else
-// the plain pass), plane slots in flight, how the level is shared among CTAs (pieces
+// A 3D TMA-fed pass (pass TP_RESTRICT, or TP_PROLONG: the post-smoothing residual) on a
+// level of pitch P: whether it runs (else the plain pass), plane slots in flight, how the level is shared among CTAs (pieces
 // > 0: every column in that many equal z pieces, one per CTA; 0: one equal share of
 // the (column, plane) sequence per resident CTA), and points per thread in y (2, 4).
 struct Tma3Params {
   bool enabled;
   int stages, pieces, qy;
 };
-Tma3Params tma3_params(int pass, int J, int P);  // pass TP_ARNOLDI (step J) or TP_PROLONG (J = 0)
+Tma3Params tma3_params(int pass, int P);
 constexpr int TMA3_MAX_UNITS = 2048;  // shares per problem (partial-sum slots of a 3D level)
 constexpr int TMA3_MIN_P = 128;       // the 3D TMA-fed passes run on levels of 127^3 and larger
 constexpr int TMA3_MAX_P = 1024;      // (32-bit point indices)
@@ -306,7 +326,7 @@ constexpr int TMA3_MAX_P = 1024;      // (32-bit point indices)
 // into the row-wise prolongation and the TMA-fed residual pass, else 1.
 inline int prolong_kernels(int dim, bool with_residual, int prec_bytes, bool tma, int P) {
   return dim == 3 && with_residual && prec_bytes == 8 && tma && P >= TMA3_MIN_P && P <= TMA3_MAX_P &&
-                 tma3_params(TP_PROLONG, 0, P).enabled
+                 tma3_params(TP_PROLONG, P).enabled
              ? 2
              : 1;
 }

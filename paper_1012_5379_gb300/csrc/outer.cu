@@ -676,6 +676,15 @@ HELM_HD constexpr size_t vnew_smem_bytes(int m) {
   return 2 * (size_t)(m + 1) * 16 + (size_t)(m + 1) * 16 + (size_t)m * 16 + (size_t)m * 8;
 }
 
+// |c - (the next lane's c)|^2 where a warp's 32 consecutive points are all below `end` (else
+// zero: the test is uniform over the warp); 31 of 32 neighbours are counted.
+__device__ __forceinline__ float warp_diff2(float2 c, size_t idx, size_t end) {
+  const int lane = threadIdx.x & 31;
+  if (idx - lane + 31 >= end) return 0.0f;
+  const float2 d = csub(shfl_down_c(c, 1), c);
+  return lane < 31 ? cabs2(d) : 0.0f;
+}
+
 // u = w - sum_{i<=j} h_i v_i stored as V[j+1] with ||u|| reduced here; the last block
 // sets h_{j+1,j} = ||u||, vscale[j+1] = 1/||u||, performs the Givens update and decides
 // whether the cycle ends.  Writes the next V-cycle input b0 (precision C) and starts
@@ -684,7 +693,7 @@ template <typename C>
 __global__ void __launch_bounds__(256, 4)
 k_vnew(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
   extern __shared__ double2 sh[];  // m+1
-  __shared__ double sm[64];
+  __shared__ double sm[96];
   const int tid = threadIdx.x;
   for (int g = blockIdx.x; g < nprob * chunks; g += gridDim.x) {
     const int prob = g / chunks, unit = g - prob * chunks;
@@ -714,6 +723,7 @@ k_vnew(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
     double2* vout = O.V + (size_t)jn * O.vs;
     double accu = 0.0;
     typename CT<C>::R accb = 0;
+    float accd = 0.0f;  // complex64: differences of neighbouring values (the first sweep's shift)
     const size_t end = unit_begin(O.vs, unit + 1, chunks);
     if (df) {
       // u = w - sum h_i v_i in double-float: four multiply-adds per vector on the FP32
@@ -778,6 +788,7 @@ k_vnew(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
         else c = from_d<C>(make_double2(df_value(ur, lr) * bsc, df_value(ui, li) * bsc));
         O.b0[idx] = c;
         accb += cabs2(c);
+        if constexpr (sizeof(C) == 8) accd += warp_diff2(c, idx, end);
       }
       accu = df_value(ns, nc);
     } else
@@ -798,9 +809,14 @@ k_vnew(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
       C c = from_d<C>(make_double2(wv.x * bsc, wv.y * bsc));
       O.b0[idx] = c;
       accb += cabs2(c);
+      if constexpr (sizeof(C) == 8) accd += warp_diff2(c, idx, end);
     }
-    double red[2] = {accu, (double)accb}, tot[2];
-    if (grid_sum_last<2>(red, O.part, unit, chunks, &st->counter, sm, tot)) {
+    constexpr int NR = sizeof(C) == 8 ? 3 : 2;
+    double red[NR], tot[NR];
+    red[0] = accu;
+    red[1] = (double)accb;
+    if (NR == 3) red[NR - 1] = (double)accd;
+    if (grid_sum_last<NR>(red, O.part, unit, chunks, &st->counter, sm, tot)) {
       const int mm = st->m;
       double2* hc = sh + 2 * (mm + 1);
       double2* sn_prev = hc + (mm + 1);
@@ -818,6 +834,8 @@ k_vnew(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
       if (tid < 32) givens_step_warp(O, st, j, tid == 0 ? sqrt(tot[0]) : 0.0, hc, cs, sn_prev, &t_last);
       if (tid == 0) {
         sweep_begin(O.sc0, (typename CT<C>::R)tot[1], O.s);
+        if constexpr (sizeof(C) == 8)
+          O.sc0->sig0 = sweep_first_shift(O.klap, O.phir, (float)tot[NR - 1] * (32.0f / 31.0f), (float)tot[1]);
         const double hn = sqrt(tot[0]);
         O.vscale[jn] = hn > 0.0 ? 1.0 / hn : 0.0;
         st->iters += 1;
@@ -857,6 +875,7 @@ k_vstart(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
     const double inv = s_inv;
     double2* vout = O.V;
     typename CT<C>::R accb = 0;
+    float accd = 0.0f;  // complex64: differences of neighbouring values (the first sweep's shift)
     const size_t end = unit_begin(O.vs, unit + 1, chunks);
     if (df && sizeof(C) == 8) {
       const float2 sinv = df_split(inv);
@@ -873,6 +892,7 @@ k_vstart(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
         const C c = CT<C>::make((typename CT<C>::R)__fadd_rn(ur, lr), (typename CT<C>::R)__fadd_rn(ui, li));
         O.b0[idx] = c;
         accb += cabs2(c);
+        if constexpr (sizeof(C) == 8) accd += warp_diff2(c, idx, end);
       }
     } else {
       for (size_t idx = unit_begin(O.vs, unit, chunks) + tid; idx < end; idx += blockDim.x) {
@@ -883,12 +903,18 @@ k_vstart(const OuterDev<C>* __restrict__ ods, int nprob, int chunks) {
         const C c = from_d<C>(wv);
         O.b0[idx] = c;
         accb += cabs2(c);
+        if constexpr (sizeof(C) == 8) accd += warp_diff2(c, idx, end);
       }
     }
-    double red[1] = {(double)accb}, tot[1];
-    if (grid_sum_last<1>(red, O.part, unit, chunks, &st->counter, sm, tot)) {
+    constexpr int NR = sizeof(C) == 8 ? 2 : 1;
+    double red[NR], tot[NR];
+    red[0] = (double)accb;
+    if (NR == 2) red[NR - 1] = (double)accd;
+    if (grid_sum_last<NR>(red, O.part, unit, chunks, &st->counter, sm, tot)) {
       if (tid == 0) {
         sweep_begin(O.sc0, (typename CT<C>::R)tot[0], O.s);
+        if constexpr (sizeof(C) == 8)
+          O.sc0->sig0 = sweep_first_shift(O.klap, O.phir, (float)tot[NR - 1] * (32.0f / 31.0f), (float)tot[0]);
         O.vscale[0] = 1.0;
         st->fresh = 0;
         st->j = 0;

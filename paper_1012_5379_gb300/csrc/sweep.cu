@@ -1,0 +1,128 @@
+// Launchers of the complex64 sweep passes (sweep.cuh) and of the complex64 coarse sub-cycle
+// (coarse.cuh).
+#include "sweep.cuh"
+#include "coarse.cuh"
+#include "launch.cuh"
+
+#include <algorithm>
+
+namespace helm {
+
+SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
+  SweepCfg c{0, 0, 1};
+  if (dim == 2) {
+    c.geo = n <= 255 ? 2 : (n <= 1023 || S > 3 ? 4 : 8);
+    c.units = sw2_units(S, c.geo, n);
+    return c;
+  }
+  if (n < 96 || S > 3) {
+    c.geo = n < 64 ? 4 : 8;
+    c.units = sw3_units(S, c.geo, n);
+    return c;
+  }
+  // planes per march: the fewest plane steps of the CTA that takes the most, one CTA per SM
+  c.march = 1;
+  long long best = -1;
+  for (int pieces = 1; pieces <= 32 && pieces <= n; ++pieces) {
+    const int zc = ceil_div(n, pieces);
+    const long long units = sm3_units(S, n, zc);
+    const long long steps = (units + sms - 1) / sms * (zc + 2 * S + 2);
+    if (best < 0 || steps < best) {
+      best = steps;
+      c.geo = zc;
+      c.units = (int)units;
+    }
+  }
+  return c;
+}
+
+template <int S>
+static void launch_sweep_s(int dim, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
+                           bool store_last, bool phi, cudaStream_t st) {
+  const dim3 grid(nprob * cfg.units);
+  const int f = first ? 1 : 0, sl = store_last ? 1 : 0;
+  if (dim == 2) {
+    const dim3 block(32, SW2_NW);
+    if (cfg.geo == 2) pdl_launch(k_sweep2<S, 2>, grid, block, 0, st, levs, cfg.units, f, sl);
+    else if (cfg.geo == 4 || S > 3) pdl_launch(k_sweep2<S, 4>, grid, block, 0, st, levs, cfg.units, f, sl);
+    else if constexpr (S <= 3) pdl_launch(k_sweep2<S, 8>, grid, block, 0, st, levs, cfg.units, f, sl);
+    return;
+  }
+  if (!cfg.march) {
+    const dim3 block(32, SW3_NW);
+    thread_local bool configured = false;  // per host thread; setting the attribute again is harmless
+    if (!configured) {
+      cudaFuncSetAttribute(k_sweep3<S, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw3_smem(S, 4));
+      cudaFuncSetAttribute(k_sweep3<S, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw3_smem(S, 8));
+      configured = true;
+    }
+    if (cfg.geo == 4) pdl_launch(k_sweep3<S, 4>, grid, block, sw3_smem(S, 4), st, levs, cfg.units, f, sl);
+    else pdl_launch(k_sweep3<S, 8>, grid, block, sw3_smem(S, 8), st, levs, cfg.units, f, sl);
+    return;
+  }
+  if constexpr (S <= 3) {
+    const dim3 block(32, SM3_NW);
+    const size_t smem = sm3_smem(S, cfg.geo);
+    thread_local size_t configured = 0;
+    if (configured < smem) {
+      cudaFuncSetAttribute(k_sweep3_march<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_sweep3_march<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      configured = smem;
+    }
+    if (phi) pdl_launch(k_sweep3_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
+    else pdl_launch(k_sweep3_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
+  }
+}
+
+void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
+                  bool store_last, bool phi, cudaStream_t st) {
+  switch (S) {
+    case 1: launch_sweep_s<1>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
+    case 2: launch_sweep_s<2>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
+    case 3: launch_sweep_s<3>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
+    default: launch_sweep_s<4>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
+  }
+}
+
+void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
+                  bool store_last) {
+  seq_push(q, levs, PK_ARNOLDI, S, cfg.units, cfg.geo, first, store_last, 0, 0, nprob * cfg.units);
+}
+
+size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {
+  size_t total = 0;
+  for (int l = 0; l < nlev; ++l) {
+    const size_t P = sizes[l] + 1, np = dim == 3 ? P * P * P : P * P;
+    total += np / P + cg_vectors(S) * np;
+  }
+  return total * sizeof(float2);
+}
+
+template <int S, int DIM>
+static void launch_coarse_gram_sd(const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
+                                  int nu1, int nu2, size_t smem, cudaStream_t st) {
+  thread_local size_t configured = 0;
+  if (configured < smem) {
+    cudaFuncSetAttribute(k_coarse_gram<S, DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    configured = smem;
+  }
+  pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, nu1, nu2);
+}
+
+void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
+                        int nu1, int nu2, size_t smem, cudaStream_t st) {
+#define HELM_CG(SS)                                                                                   \
+  case SS:                                                                                            \
+    if (dim == 2) launch_coarse_gram_sd<SS, 2>(levs, lev_stride, lus, nprob, nu1, nu2, smem, st);     \
+    else launch_coarse_gram_sd<SS, 3>(levs, lev_stride, lus, nprob, nu1, nu2, smem, st);              \
+    break;
+  switch (S) {
+    HELM_CG(1)
+    HELM_CG(2)
+    HELM_CG(3)
+    HELM_CG(4)
+  }
+#undef HELM_CG
+}
+
+}  // namespace helm

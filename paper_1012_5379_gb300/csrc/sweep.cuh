@@ -1,0 +1,431 @@
+// The grid-wide sweep passes of the complex64 V-cycle: k_1..k_S of a GMRES(S) sweep and the
+// Gram matrix of k_0..k_S from one read of R_0 (gram.cuh).
+//
+// A point of k_S depends on R_0 within S points in every direction, so a CTA forms k_j on
+// its own points plus S - j points around them, redundantly with its neighbours, and no
+// CTA waits for another.  In all three kernels a warp's 32 lanes are 32 neighbouring x
+// positions, of which the inner 32 - 2S are the CTA's own: x neighbours come from shuffles
+// or shared memory, and lanes at the rim hold values that are wrong beyond S - j points
+// and are never used.  Outside the domain every value is zero without a test: R_0 is
+// loaded as zero there and the 1D coefficients are zero.
+#pragma once
+#include <type_traits>
+
+#include "gram.cuh"
+
+namespace helm {
+
+HELM_HD constexpr int sw_ox(int S) { return 32 - 2 * S; }  // own points of a warp row
+
+// 1D coefficients of one axis position times the basis scale t (exact: a power of two).
+struct SwCoef {
+  float2 a, d, c;
+};
+__device__ __forceinline__ SwCoef sw_coef(const float2* ca, int i, int n, float t) {
+  SwCoef r;
+  r.a = r.d = r.c = make_float2(0.f, 0.f);
+  if ((unsigned)i < (unsigned)n) {
+    const float2 a = __ldg(ca + i), d = __ldg(ca + n + i), c = __ldg(ca + 2 * n + i);
+    r.a = make_float2(a.x * t, a.y * t);
+    r.d = make_float2(d.x * t, d.y * t);
+    r.c = make_float2(c.x * t, c.y * t);
+  }
+  return r;
+}
+
+// ------------------------------------------------------------------ 2D
+// A CTA of 8 warps holds a 32 x 8 QY region in registers, QY consecutive rows per warp;
+// only the rows at a warp's edges pass through shared memory.  Its own points are the
+// inner (32 - 2S) x (8 QY - 2S).
+constexpr int SW2_NW = 8;
+HELM_HD constexpr int sw2_oy(int S, int QY) { return SW2_NW * QY - 2 * S; }
+HELM_HD inline int sw2_units(int S, int QY, int n) { return ceil_div(n, sw_ox(S)) * ceil_div(n, sw2_oy(S, QY)); }
+
+template <int S, int QY>
+struct Sw2Shared {
+  float4 yac[SW2_NW * QY];                // y coefficients a, c of the region's rows
+  float2 yd[SW2_NW * QY];
+  float2 edge[2][SW2_NW + 2][2][32];      // [parity][warp + 1][first / last row][lane]
+  float2 gs[SW2_NW * gram_nv(S)];
+  float wsum[SW2_NW * gram_ns(S)];
+};
+
+template <int S, int QY, bool NC = true>
+__device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
+                                            int store_last, int vblk, Sw2Shared<S, QY>& sh) {
+  constexpr int NS = gram_ns(S), RY = SW2_NW * QY;
+  auto& edge = sh.edge;
+  auto& yac = sh.yac;
+  auto& yd = sh.yd;
+  const int prob = vblk / nunits, unit = vblk - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+  const int n = L.n, P = L.P;
+  const float t = L.kt;
+  const int ntx = ceil_div(n, sw_ox(S));
+  const int tx = unit % ntx, ty = unit / ntx;
+  const int x = tx * sw_ox(S) - S + lane, yr = ty * sw2_oy(S, QY) - S, y0 = yr + warp * QY;
+  const SwCoef cx = sw_coef(L.ca, x, n, t);
+  if (tid < RY) {
+    const SwCoef c = sw_coef(L.ca, yr + tid, n, t);
+    yac[tid] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
+    yd[tid] = c.d;
+  }
+  if (warp < 2) {  // the rows beyond the region
+    edge[warp][0][1][lane] = make_float2(0.f, 0.f);
+    edge[warp][SW2_NW + 1][0][lane] = make_float2(0.f, 0.f);
+  }
+  float ph[QY];
+  const float phc = L.phir * t;
+#pragma unroll
+  for (int q = 0; q < QY; ++q)
+    ph[q] = (L.phi && inside(x, y0 + q, 0, n)) ? __ldg(L.phi + pidx(x, y0 + q, 0, P)) * t : phc;
+  pdl_wait();
+  float2 sg[S];
+  gram_shifts<S>(L, first != 0, sg);
+  const float2* R0 = first ? L.b : L.r0;
+  float2 k[S + 1][QY];
+#pragma unroll
+  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2, NC>(R0, x, y0 + q, 0, n, P);
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    edge[j & 1][warp + 1][0][lane] = k[j][0];
+    edge[j & 1][warp + 1][1][lane] = k[j][QY - 1];
+    __syncthreads();
+    const float2 up = edge[j & 1][warp][1][lane], dn = edge[j & 1][warp + 2][0][lane];
+#pragma unroll
+    for (int q = 0; q < QY; ++q) {
+      const float4 ac = yac[warp * QY + q];
+      float2 dg = cadd(cx.d, yd[warp * QY + q]);
+      dg.x = (dg.x - ph[q]) - sg[j].x;
+      dg.y -= sg[j].y;
+      const float2 v = k[j][q];
+      float2 p = cmul(dg, v);
+      p = cfma(cx.a, shfl_up_c(v, 1), p);
+      p = cfma(cx.c, shfl_down_c(v, 1), p);
+      p = cfma(make_float2(ac.x, ac.y), q > 0 ? k[j][q - 1] : up, p);
+      p = cfma(make_float2(ac.z, ac.w), q < QY - 1 ? k[j][q + 1] : dn, p);
+      k[j + 1][q] = p;
+    }
+  }
+  float acc[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
+  const bool ownx = lane >= S && lane < 32 - S && x < n;
+#pragma unroll
+  for (int q = 0; q < QY; ++q) {
+    const int ry = warp * QY + q, y = y0 + q;
+    if (ry < S || ry >= RY - S || y >= n) continue;  // uniform over the warp
+    if (ownx) {
+      float2 kk[S + 1];
+#pragma unroll
+      for (int j = 0; j <= S; ++j) kk[j] = k[j][q];
+      gram_point<S>(kk, acc);
+#pragma unroll
+      for (int j = 1; j <= S; ++j)
+        if (j < S || store_last) L.p[j - 1][pidx(x, y, 0, P)] = kk[j];
+    }
+  }
+  pdl_trigger();  // the main work is done: let the next pass launch
+  gram_finish<S, SW2_NW>(acc, L, sg, unit, nunits, sh.wsum, sh.gs);
+}
+template <int S, int QY>
+__global__ void __launch_bounds__(256, 2)
+k_sweep2(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int store_last) {
+  __shared__ Sw2Shared<S, QY> sh;
+  sweep2_body<S, QY>(levs, nunits, first, store_last, blockIdx.x, sh);
+}
+
+// ------------------------------------------------------------------ 3D, small levels
+// A CTA of 8 warps owns (32 - 2S) x O x O points and keeps k_0..k_{S-1} on the region
+// around them in shared memory, one warp per (y, z) row at a time.  Every row of a stage is
+// independent, so a level of a few thousand points finishes in S short stages.
+constexpr int SW3_NW = 8;
+HELM_HD inline int sw3_units(int S, int O, int n) {
+  return ceil_div(n, sw_ox(S)) * ceil_div(n, O) * ceil_div(n, O);
+}
+HELM_HD constexpr int sw3_rows(int S, int O) {
+  int r = 0;
+  for (int j = 0; j < S; ++j) r += (O + 2 * S - 2 * j) * (O + 2 * S - 2 * j);
+  return r;
+}
+HELM_HD constexpr unsigned sw3_smem(int S, int O) { return (unsigned)sw3_rows(S, O) * 256u; }
+
+template <int S, int O, int J>
+__device__ __forceinline__ int sw3_base() {  // first row of k_J in the shared array
+  int r = 0;
+#pragma unroll
+  for (int j = 0; j < J; ++j) r += (O + 2 * S - 2 * j) * (O + 2 * S - 2 * j);
+  return r;
+}
+
+// Row (ry, rz) of stage J (its region O + 2 (S - J) rows wide) of the basis.
+template <int S, int O, int J>
+__device__ __forceinline__ float2 sw3_row(const float2* sm, const SwCoef& cx, const float4* yac, const float2* yd,
+                                          const float4* zac, const float2* zd, const float2 sg, float ph, int ry,
+                                          int rz, int lane) {
+  constexpr int Hp = O + 2 * (S - J) + 2;  // rows of stage J - 1
+  const float2* src = sm + (size_t)(sw3_base<S, O, J - 1>() + (rz + 1) * Hp + ry + 1) * 32 + lane;
+  const float2 v = src[0], vs = src[-32], vn = src[32], vb = src[-32 * Hp], vt = src[32 * Hp];
+  const float4 ya = yac[ry + J], za = zac[rz + J];
+  float2 dg = cadd(cx.d, yd[ry + J]);
+  dg.x = (dg.x - ph) - sg.x;
+  dg.y -= sg.y;
+  float2 p = cmul(dg, v);
+  p = cfma(zd[rz + J], v, p);
+  p = cfma(cx.a, shfl_up_c(v, 1), p);
+  p = cfma(cx.c, shfl_down_c(v, 1), p);
+  p = cfma(make_float2(ya.x, ya.y), vs, p);
+  p = cfma(make_float2(ya.z, ya.w), vn, p);
+  p = cfma(make_float2(za.x, za.y), vb, p);
+  return cfma(make_float2(za.z, za.w), vt, p);
+}
+
+template <int S, int O, bool NC = true>
+__device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
+                                            int store_last, int vblk, float2* sm) {
+  constexpr int NS = gram_ns(S), NV = gram_nv(S), R = O + 2 * S;
+  __shared__ float4 yac[R], zac[R];
+  __shared__ float2 yd[R], zd[R];
+  __shared__ float wsum[SW3_NW * NS];
+  __shared__ float2 gs[SW3_NW * NV];
+  const int prob = vblk / nunits, unit = vblk - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+  const int n = L.n, P = L.P;
+  const float t = L.kt, phc = L.phir * t;
+  const float* const phi = L.phi;
+  const int ntx = ceil_div(n, sw_ox(S)), nty = ceil_div(n, O);
+  const int x = (unit % ntx) * sw_ox(S) - S + lane;
+  const int y0 = ((unit / ntx) % nty) * O - S, z0 = (unit / (ntx * nty)) * O - S;
+  const SwCoef cx = sw_coef(L.ca, x, n, t);
+  for (int i = tid; i < 2 * R; i += 256) {
+    const int q = i < R ? i : i - R;
+    const SwCoef c = sw_coef(L.ca, (i < R ? y0 : z0) + q, n, t);
+    (i < R ? yac : zac)[q] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
+    (i < R ? yd : zd)[q] = c.d;
+  }
+  pdl_wait();
+  float2 sg[S];
+  gram_shifts<S>(L, first != 0, sg);
+  const float2* R0 = first ? L.b : L.r0;
+#pragma unroll 4
+  for (int r = warp; r < R * R; r += SW3_NW)
+    sm[r * 32 + lane] = ldc<float2, NC>(R0, x, y0 + r % R, z0 + r / R, n, P);
+  __syncthreads();
+  auto phi_of = [&](int y, int z) -> float {
+    return phi ? (inside(x, y, z, n) ? __ldg(phi + pidx(x, y, z, P)) * t : 0.f) : phc;
+  };
+  // stages 1 .. S - 1 into shared memory
+  auto stage = [&](auto jc) {
+    constexpr int J = decltype(jc)::value;
+    constexpr int H = O + 2 * (S - J);
+    for (int r = warp; r < H * H; r += SW3_NW) {
+      const int ry = r % H, rz = r / H;
+      sm[(sw3_base<S, O, J>() + r) * 32 + lane] = sw3_row<S, O, J>(
+          sm, cx, yac, yd, zac, zd, sg[J - 1], phi_of(y0 + ry + J, z0 + rz + J), ry, rz, lane);
+    }
+    __syncthreads();
+  };
+  if constexpr (S >= 2) stage(std::integral_constant<int, 1>());
+  if constexpr (S >= 3) stage(std::integral_constant<int, 2>());
+  if constexpr (S >= 4) stage(std::integral_constant<int, 3>());
+  float acc[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
+  const bool ownx = lane >= S && lane < 32 - S && x < n;
+  for (int r = warp; r < O * O; r += SW3_NW) {
+    const int ry = r % O, rz = r / O, y = y0 + ry + S, z = z0 + rz + S;
+    if (y >= n || z >= n) continue;  // uniform over the warp
+    float2 kk[S + 1];
+    kk[S] = sw3_row<S, O, S>(sm, cx, yac, yd, zac, zd, sg[S - 1], phi_of(y, z), ry, rz, lane);
+    kk[0] = sm[((rz + S) * R + ry + S) * 32 + lane];
+    if constexpr (S >= 2) kk[1] = sm[(sw3_base<S, O, 1>() + (rz + S - 1) * (R - 2) + ry + S - 1) * 32 + lane];
+    if constexpr (S >= 3) kk[2] = sm[(sw3_base<S, O, 2>() + (rz + S - 2) * (R - 4) + ry + S - 2) * 32 + lane];
+    if constexpr (S >= 4) kk[3] = sm[(sw3_base<S, O, 3>() + (rz + S - 3) * (R - 6) + ry + S - 3) * 32 + lane];
+    if (ownx) {
+      gram_point<S>(kk, acc);
+#pragma unroll
+      for (int j = 1; j <= S; ++j)
+        if (j < S || store_last) L.p[j - 1][pidx(x, y, z, P)] = kk[j];
+    }
+  }
+  pdl_trigger();  // the main work is done: let the next pass launch
+  gram_finish<S, SW3_NW>(acc, L, sg, unit, nunits, wsum, gs);
+}
+template <int S, int O>
+__global__ void __launch_bounds__(256)
+k_sweep3(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int store_last) {
+  extern __shared__ __align__(16) float2 swsm[];
+  sweep3_body<S, O>(levs, nunits, first, store_last, blockIdx.x, swsm);
+}
+
+// ------------------------------------------------------------------ 3D, large levels
+// A CTA of 16 warps holds a 32 x 32 column of the level (two rows per warp) and marches in
+// z.  In the step that loads plane z of R_0 it forms k_j of plane z - j for every j: the z
+// neighbours are in registers (four planes of each vector), the x and y neighbours were
+// published to shared memory in the previous step, so one barrier per step suffices.  R_0
+// of the next planes is loaded ahead.  Own points: (32 - 2S)^2 columns of `zc` planes.
+constexpr int SM3_NW = 16, SM3_R = 32;
+HELM_HD inline int sm3_units(int S, int n, int zc) {
+  return ceil_div(n, sw_ox(S)) * ceil_div(n, sw_ox(S)) * ceil_div(n, zc);
+}
+// published planes: [parity][vector][row][lane], one guard row at either end
+HELM_HD constexpr unsigned sm3_plane() { return (SM3_R + 2) * 32; }
+HELM_HD constexpr unsigned sm3_smem(int S, int zc) {
+  return 2u * S * sm3_plane() * 8u + (unsigned)(zc + 2 * S) * 24u;
+}
+
+template <int S, bool PHI>
+__global__ void __launch_bounds__(SM3_NW * 32, 1)
+k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, int first, int store_last) {
+  constexpr int NS = gram_ns(S), NV = gram_nv(S), W = 4;
+  static_assert(S <= 3, "register windows hold four planes");
+  extern __shared__ __align__(16) float2 swsm[];
+  __shared__ float wsum[SM3_NW * NS];
+  __shared__ float2 gs[SM3_NW * NV];
+  const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+  const int n = L.n, P = L.P;
+  const float t = L.kt, phir = L.phir, phc = phir * t;
+  const float* const phi = L.phi;
+  const int nt = ceil_div(n, sw_ox(S));
+  const int x = (unit % nt) * sw_ox(S) - S + lane;
+  const int ry = 2 * warp, y = ((unit / nt) % nt) * sw_ox(S) - S + ry;  // rows y, y + 1
+  const int zb = (unit / (nt * nt)) * zc, ze = min(zb + zc, n);
+  float2* const pub = swsm;                                              // 2 S planes
+  float4* const zac = reinterpret_cast<float4*>(swsm + 2 * S * sm3_plane());
+  float2* const zd = reinterpret_cast<float2*>(zac + (zc + 2 * S));
+  const SwCoef cx = sw_coef(L.ca, x, n, t), cy0 = sw_coef(L.ca, y, n, t), cy1 = sw_coef(L.ca, y + 1, n, t);
+  const float2 dxy[2] = {cadd(cx.d, cy0.d), cadd(cx.d, cy1.d)};
+  for (int i = tid; i < ze - zb + 2 * S; i += SM3_NW * 32) {
+    const SwCoef c = sw_coef(L.ca, zb - S + i, n, t);
+    zac[i] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
+    zd[i] = c.d;
+  }
+  for (int i = tid; i < 2 * S * (int)sm3_plane(); i += SM3_NW * 32) pub[i] = make_float2(0.f, 0.f);
+  pdl_wait();
+  float2 sg[S];
+  gram_shifts<S>(L, first != 0, sg);
+  const float2* R0 = first ? L.b : L.r0;
+  const bool in0 = (unsigned)x < (unsigned)n && (unsigned)y < (unsigned)n;
+  const bool in1 = (unsigned)x < (unsigned)n && (unsigned)(y + 1) < (unsigned)n;
+  const long long col = (long long)y * P + x;
+  const size_t PP = (size_t)P * P;
+  float2 win[S][W][2];  // k_j of the last planes, slot = plane & 3
+#pragma unroll
+  for (int j = 0; j < S; ++j)
+#pragma unroll
+    for (int w = 0; w < W; ++w) win[j][w][0] = win[j][w][1] = make_float2(0.f, 0.f);
+  float phw[W][2];
+  float2 nxt[W][2];
+  float phn[W][2];
+  auto fetch = [&](int z, float2 (&v)[2], float (&f)[2]) {
+    const bool zin = (unsigned)z < (unsigned)n;
+    v[0] = (zin && in0) ? __ldg(R0 + (col + (long long)(z * PP))) : make_float2(0.f, 0.f);
+    v[1] = (zin && in1) ? __ldg(R0 + (col + P + (long long)(z * PP))) : make_float2(0.f, 0.f);
+    if (PHI) {  // some problem of the launch has a field; this one may not
+      f[0] = (phi && zin && in0) ? __ldg(phi + (col + (long long)(z * PP))) : phir;
+      f[1] = (phi && zin && in1) ? __ldg(phi + (col + P + (long long)(z * PP))) : phir;
+    }
+  };
+  float acc[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
+  const bool ox = lane >= S && lane < 32 - S && x < n;
+  const bool own0 = ox && ry >= S && ry < SM3_R - S && y < n;
+  const bool own1 = ox && ry + 1 >= S && ry + 1 < SM3_R - S && y + 1 < n;
+  const int zf = zb - S, zl = ze + S;  // planes loaded: zf .. zl - 1
+  constexpr int AHEAD = 2;             // planes of loads in flight beyond the current one
+#pragma unroll
+  for (int u = 0; u < AHEAD; ++u) fetch(zf + u, nxt[u], phn[u]);
+  __syncthreads();
+  // step i loads plane zf + i; slots are indexed by i & 3, which the unrolling by four
+  // makes static
+#pragma unroll 1
+  for (int i0 = 0; i0 < zl - zf; i0 += W) {
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      const int i = i0 + u;
+      if (i >= zl - zf) break;  // uniform
+      const int z = zf + i;
+      float2 k0[2];
+      k0[0] = nxt[u][0];
+      k0[1] = nxt[u][1];
+      if (PHI) {
+        phw[u][0] = phn[u][0] * t;
+        phw[u][1] = phn[u][1] * t;
+      }
+      if (z + AHEAD < zl) fetch(z + AHEAD, nxt[(u + AHEAD) & 3], phn[(u + AHEAD) & 3]);
+      const float2* rd = pub + (size_t)((u & 1) ^ 1) * S * sm3_plane() + (ry + 1) * 32 + lane;
+      float2* wr = pub + (size_t)(u & 1) * S * sm3_plane() + (ry + 1) * 32 + lane;
+      win[0][u][0] = k0[0];
+      win[0][u][1] = k0[1];
+      wr[0] = k0[0];
+      wr[32] = k0[1];
+      float2 last[2];
+#pragma unroll
+      for (int j = 1; j <= S; ++j) {
+        // k_j at plane z - j from k_{j-1} at planes z - j - 1 .. z - j + 1
+        const int c = (u - j) & 3, b = (u - j - 1) & 3, f = (u - j + 1) & 3;
+        float2 r[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        const int iz = i - j;  // index into the staged z coefficients
+        if (iz >= 0) {         // uniform
+          const float4 za = zac[iz];
+          const float2 zdd = zd[iz];
+          const float2* s = rd + (size_t)(j - 1) * sm3_plane();
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            float2 dg = dxy[q];
+            dg.x = (dg.x - (PHI ? phw[c][q] : phc)) - sg[j - 1].x;
+            dg.y -= sg[j - 1].y;
+            const float2 v = win[j - 1][c][q];
+            float2 p = cmul(dg, v);
+            p = cfma(zdd, v, p);
+            p = cfma(cx.a, s[32 * q - 1], p);
+            p = cfma(cx.c, s[32 * q + 1], p);
+            const SwCoef& cy = q ? cy1 : cy0;
+            p = cfma(cy.a, q ? win[j - 1][c][0] : s[-32], p);
+            p = cfma(cy.c, q ? s[64] : win[j - 1][c][1], p);
+            p = cfma(make_float2(za.x, za.y), win[j - 1][b][q], p);
+            p = cfma(make_float2(za.z, za.w), win[j - 1][f][q], p);
+            r[q] = p;
+          }
+        }
+        if (j < S) {
+          win[j][c][0] = r[0];
+          win[j][c][1] = r[1];
+          wr[(size_t)j * sm3_plane()] = r[0];
+          wr[(size_t)j * sm3_plane() + 32] = r[1];
+        } else {
+          last[0] = r[0];
+          last[1] = r[1];
+        }
+      }
+      const int zo = z - S;
+      if (i >= 2 * S) {  // uniform: zo is one of the CTA's planes
+        const int c = (u - S) & 3;
+        const size_t at = (size_t)(col + (long long)(zo * PP));
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          if (q ? own1 : own0) {
+            float2 kk[S + 1];
+#pragma unroll
+            for (int j = 0; j < S; ++j) kk[j] = win[j][c][q];
+            kk[S] = last[q];
+            gram_point<S>(kk, acc);
+#pragma unroll
+            for (int j = 1; j <= S; ++j)
+              if (j < S || store_last) L.p[j - 1][at + (q ? P : 0)] = kk[j];
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+  pdl_trigger();  // the main work is done: let the next pass launch
+  gram_finish<S, SM3_NW>(acc, L, sg, unit, nunits, wsum, gs);
+}
+
+}  // namespace helm

@@ -12,6 +12,7 @@
 //     z+2, after iteration z+1's barrier, so one __syncthreads per plane suffices.
 #pragma once
 #include "vcycle.cuh"
+#include "sweep.cuh"
 
 namespace helm {
 
@@ -132,145 +133,6 @@ k_arnoldi_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_i
   arnoldi_t2_body<C, J>(levs, ntiles, tpc, r0_is_b, store_p, blockIdx.x);
 }
 
-// ------------------------------------------------------------------ Arnoldi step J, TMA (2D, complex64)
-// The same pass with the raw vectors streamed by the tensor memory accelerator: a
-// 136 x 18 float box per raw vector (the 64 x 16 tile plus halo, from x0 - 2 so that
-// the box starts on a 16-byte boundary; out-of-range rows and columns arrive as
-// zero, which is the boundary value) lands in shared memory, TMA_STAGES deep: while
-// the CTA works on one tile, the next tiles' boxes are in flight.  Every wait is
-// bounded; on a timeout the CTA records the error, waits (bounded) for its own copies
-// and returns.
-constexpr int TMA_BX = T2X + 4, TMA_BY = T2Y + 2;                        // box in complex points
-constexpr unsigned TMA_BOX_BYTES = TMA_BX * TMA_BY * 8;                    // 9792
-constexpr unsigned TMA_BOX_STRIDE = (TMA_BOX_BYTES + 127) / 128 * 128;     // 9856
-constexpr int TMA_STAGES = 2;                                             // tiles in flight per CTA
-HELM_HD constexpr unsigned tma_arnoldi_smem(int J) { return (unsigned)TMA_STAGES * J * TMA_BOX_STRIDE; }
-
-template <int J>
-__global__ void __launch_bounds__(256, J <= 2 ? 4 : 3)
-k_arnoldi_tma2(const LevelDev<float2>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int store_p) {
-  typedef float R;
-  typedef float2 C;
-  extern __shared__ __align__(128) unsigned char tsm[];
-  __shared__ C vt[T2Y + 2][T2X + 2];
-  __shared__ R sm[32 * (2 * J + 1)];
-  __shared__ __align__(8) uint64_t bar[TMA_STAGES];
-  const int nunits = ceil_div(ntiles, tpc);
-  const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
-  const LevelDev<C>& L = levs[prob];
-  auto* sc = L.sc;
-  const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
-  if (tid == 0) {
-#pragma unroll
-    for (int q = 0; q < TMA_STAGES; ++q) mbar_init(&bar[q], 1);
-    mbar_fence_init();
-  }
-  pdl_wait();
-  if (sc->m < J) return;  // earlier breakdown or empty sweep: uniform for the problem
-  const int n = L.n, P = L.P;
-  const int ntx = ceil_div(P, T2X);
-  const StencilRegs<C> S(L);
-  C* const pJ = L.p[J - 1];
-  const CUtensorMap* tm[J];
-  C cf[J];
-#pragma unroll
-  for (int k = 0; k < J; ++k) {
-    tm[k] = L.tm + (k == 0 ? (r0_is_b ? TM_B : TM_R0) : TM_P0 + k - 1);
-    cf[k] = sc->Cf[J][k];
-  }
-  if (tid == 0)
-#pragma unroll
-    for (int k = 0; k < J; ++k) tmap_acquire(tm[k]);
-  __syncthreads();  // initialised barriers
-  const int t_beg = unit * tpc, t_end = min(ntiles, (unit + 1) * tpc);
-  auto issue = [&](int t, int stage) {
-    const int x0 = (t % ntx) * T2X, y0 = (t / ntx) * T2Y;
-    mbar_expect_tx(&bar[stage], J * TMA_BOX_BYTES);
-#pragma unroll
-    for (int k = 0; k < J; ++k)
-      tma_load_2d(tsm + (stage * J + k) * TMA_BOX_STRIDE, tm[k], 2 * (x0 - 2), y0 - 1, &bar[stage]);
-  };
-  if (tid == 0)
-    for (int q = 0; q < TMA_STAGES - 1 && t_beg + q < t_end; ++q) issue(t_beg + q, q);
-  C acc[J];
-#pragma unroll
-  for (int k = 0; k < J; ++k) acc[k] = czero<C>();
-  R accn = 0;
-  bool ok = true;
-  int it = 0;
-#pragma unroll 1
-  for (int tile = t_beg; tile < t_end; ++tile, ++it) {
-    const int stage = it % TMA_STAGES;
-    // the stage of tile it + STAGES - 1 is the one tile it - 1 released at its end
-    if (tid == 0 && tile + TMA_STAGES - 1 < t_end)
-      issue(tile + TMA_STAGES - 1, (it + TMA_STAGES - 1) % TMA_STAGES);
-    const bool mine = mbar_wait(&bar[stage], (unsigned)((it / TMA_STAGES) & 1));
-    if (!__syncthreads_and(mine)) { ok = false; break; }
-    const C* box[J];
-#pragma unroll
-    for (int k = 0; k < J; ++k) box[k] = reinterpret_cast<const C*>(tsm + (stage * J + k) * TMA_BOX_STRIDE);
-    // v_J on the tile plus halo: vt[r][c] is the point (x0 - 1 + c, y0 - 1 + r), box
-    // column c + 1.  Each thread forms its own four points and keeps their raw values
-    // for the dot products; the first HALO2 threads form the halo.
-    C raw[4][J];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
-      C v = czero<C>();
-#pragma unroll
-      for (int k = 0; k < J; ++k) {
-        raw[q][k] = box[k][(oy + 1) * TMA_BX + ox + 2];
-        v = cfma(cf[k], raw[q][k], v);
-      }
-      vt[oy + 1][ox + 1] = v;
-    }
-    if (tid < HALO2) {
-      int hx, hy;
-      halo_coord<T2X, T2Y>(tid, hx, hy);
-      C v = czero<C>();
-#pragma unroll
-      for (int k = 0; k < J; ++k) v = cfma(cf[k], box[k][(hy + 1) * TMA_BX + hx + 2], v);
-      vt[hy + 1][hx + 1] = v;
-    }
-    __syncthreads();
-    const int x0 = (tile % ntx) * T2X, y0 = (tile / ntx) * T2Y;
-    const Coef3<C> cx0 = S.coef(x0 + lx), cx1 = S.coef(x0 + lx + 32);
-    Coef3<C> cy;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
-      const int x = x0 + ox, y = y0 + oy;
-      if ((q & 1) == 0) cy = S.coef(y);  // one row per pair of points
-      C p = czero<C>();
-      if (x < n && y < n) {
-        p = stencil5((q & 1) ? cx1 : cx0, cy, S.phi_at(x, y, 0), vt[oy + 1][ox + 1], vt[oy + 1][ox],
-                     vt[oy + 1][ox + 2], vt[oy][ox + 1], vt[oy + 2][ox + 1]);
-#pragma unroll
-        for (int k = 0; k < J; ++k) acc[k] = cdotacc(raw[q][k], p, acc[k]);
-        accn += cabs2(p);
-      }
-      if (store_p && x < P && y < P) pJ[pidx(x, y, 0, P)] = p;
-    }
-    __syncthreads();  // vt and this stage are free for reuse
-  }
-  if (!ok) {
-    if (tid == 0) {
-      atomicExch(&g_vcycle_error, 1);
-      // the copies of this CTA that may still be landing (bounded)
-      for (int u = it; u < it + TMA_STAGES && t_beg + u < t_end; ++u)
-        mbar_wait(&bar[u % TMA_STAGES], (unsigned)((u / TMA_STAGES) & 1));
-    }
-    __syncthreads();
-    return;
-  }
-  R red[2 * J + 1];
-#pragma unroll
-  for (int k = 0; k < J; ++k) { red[2 * k] = acc[k].x; red[2 * k + 1] = acc[k].y; }
-  red[2 * J] = accn;
-  pdl_trigger();  // the main work is done: let the next pass launch
-  grid_sum_sweep<R, J>(red, L.part, unit, nunits, sc, sm);
-}
-
 template <typename C, int J, bool NC = true>
 __device__ __forceinline__ void arnoldi_t3_body(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_is_b, int store_p, int vblk) {
   typedef typename CT<C>::R R;
@@ -371,8 +233,8 @@ k_arnoldi_t3(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_is
   arnoldi_t3_body<C, J>(levs, ntiles, zc, r0_is_b, store_p, blockIdx.x);
 }
 
-// ------------------------------------------------------------------ Arnoldi step J, TMA (3D, complex64)
-// The 3D pass with the raw vectors streamed by the tensor memory accelerator.  A CTA of
+// ------------------------------------------------------------------ post-smoothing residual, TMA (3D, complex64)
+// r0 = b - M x_b with x_b streamed by the tensor memory accelerator.  A CTA of
 // 32 x 8 threads works on columns of 32 x 8 QY points (QY points per thread, rows ly,
 // ly + 8, ...).  The level's work is the sequence of (column, plane) pairs, column by
 // column in z order, and CTA `unit` of a problem takes the `unit`-th of `nunits`
@@ -380,24 +242,23 @@ k_arnoldi_t3(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_is
 // multiple of the column count every share is one piece of one column, and CTAs on
 // neighbouring columns march the same planes at the same time, so a tile's halo is
 // read from L2).  For every plane z - 1 .. z_end of each column piece, one 72 x
-// (8 QY + 2) x 1 float box per raw vector (the columns plus a one-point halo in x and
+// (8 QY + 2) x 1 float box (the columns plus a one-point halo in x and
 // y, starting two points left of the tile so that the box starts on a 16-byte
 // boundary; out-of-range parts arrive as zero, the boundary value) lands in a ring of
-// `stages` plane slots, so several planes' copies are in flight while the CTA forms
-// v_J of the newest plane.  Each thread keeps v_J of its own points on three
-// consecutive planes in registers (the stencil's z neighbours) and writes the newest
-// plane into a 3-slot shared ring for the x and y neighbours: the slot written in
-// iteration f was last read in iteration f - 2, before iteration f - 1's barrier, so
-// one barrier per plane suffices.  Every wait is bounded; on a timeout the CTA records
-// the error, waits (bounded) for its own copies and returns.
+// `stages` plane slots, so several planes' copies are in flight.  Each thread keeps its
+// own points on three consecutive planes in registers (the stencil's z neighbours) and
+// writes the newest plane into a 3-slot shared ring for the x and y
+// neighbours: the slot written in iteration f was last read in iteration f - 2, before
+// iteration f - 1's barrier, so one barrier per plane suffices.  Every wait is bounded; on
+// a timeout the CTA records the error, waits (bounded) for its own copies and returns.
 constexpr int TM3_TX = 32;
 constexpr int TM3_TY2 = 16;                                                  // tile height at two points per thread
 constexpr int TM3_BX = TM3_TX + 4;                                          // box width in complex points
 HELM_HD constexpr int tm3_ty(int QY) { return 8 * QY; }
 HELM_HD constexpr unsigned tm3_box_bytes(int QY) { return TM3_BX * (8 * QY + 2) * 8; }
 HELM_HD constexpr unsigned tm3_box_stride(int QY) { return (tm3_box_bytes(QY) + 127) / 128 * 128; }
-HELM_HD constexpr unsigned tma3_arnoldi_smem(int J, int QY, int stages) {
-  return (unsigned)stages * J * tm3_box_stride(QY);
+HELM_HD constexpr unsigned tma3_smem(int nvec, int QY, int stages) {
+  return (unsigned)stages * nvec * tm3_box_stride(QY);
 }
 // (column, plane) pairs and columns of a level of pitch P (a multiple of 32)
 HELM_HD inline int tma3_cols(int P, int QY) { return (P / TM3_TX) * (P / tm3_ty(QY)); }
@@ -423,10 +284,9 @@ struct Tma3Cursor {
   }
 };
 
-template <int J, int QY, bool RESID>
-__global__ void __launch_bounds__(256, (J == 1 && QY == 2) ? 3 : 2)
-k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages, int r0_is_b, int store_p) {
-  typedef float R;
+template <int QY>
+__global__ void __launch_bounds__(256, QY == 2 ? 3 : 2)
+k_resid_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages) {
   typedef float2 C;
   constexpr int TY = 8 * QY;
   constexpr int BY = TY + 2;
@@ -434,40 +294,22 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
   constexpr int HALO = 2 * (TM3_TX + 2) + 2 * TY;
   extern __shared__ __align__(128) unsigned char tsm[];
   __shared__ C vr[3][BY][TM3_TX + 2];
-  __shared__ R sm[32 * (2 * J + 1)];
   __shared__ __align__(8) uint64_t bar[TM3_STAGES_MAX];
   const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
   const LevelDev<C>& L = levs[prob];
-  auto* sc = L.sc;
   const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
   if (tid == 0) {
     for (int q = 0; q < stages; ++q) mbar_init(&bar[q], 1);
     mbar_fence_init();
   }
   pdl_wait();
-  if (!RESID && sc->m < J) return;  // earlier breakdown or empty sweep: uniform for the problem
   const int n = L.n, P = L.P;
   const int ntx = P / TM3_TX;
   const long long work = tma3_work(P, QY);
   const int g0 = (int)(work * unit / nunits), g1 = (int)(work * (unit + 1) / nunits);
   const StencilRegs<C> S(L);
-  C* const pJ = L.p[J - 1];
-  const CUtensorMap* tm[J];
-  C cf[J];
-  const CUtensorMap* maps = L.tm + (QY == 4 ? TM_COUNT : 0);
-#pragma unroll
-  for (int k = 0; k < J; ++k) {
-    if (RESID) {
-      tm[k] = maps + TM_XB;
-      cf[k] = make_float2(1.f, 0.f);
-    } else {
-      tm[k] = maps + (k == 0 ? (r0_is_b ? TM_B : TM_R0) : TM_P0 + k - 1);
-      cf[k] = sc->Cf[J][k];
-    }
-  }
-  if (tid == 0)
-#pragma unroll
-    for (int k = 0; k < J; ++k) tmap_acquire(tm[k]);
+  const CUtensorMap* const tm = L.tm + (QY == 4 ? TM_COUNT : 0) + TM_XB;
+  if (tid == 0) tmap_acquire(tm);
   __syncthreads();  // initialised barriers
   // producer (thread 0): issues the planes of the share in order into the stage ring
   Tma3Cursor pc;
@@ -476,10 +318,8 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
   int pstage = 0, issued = 0;
   auto issue_next = [&]() {
     const int x0 = (pc.col % ntx) * TM3_TX, y0 = (pc.col / ntx) * TY;
-    mbar_expect_tx(&bar[pstage], J * BOX);
-#pragma unroll
-    for (int k = 0; k < J; ++k)
-      tma_load_3d(tsm + (pstage * J + k) * STRIDE, tm[k], 2 * (x0 - 2), y0 - 1, pc.z, &bar[pstage]);
+    mbar_expect_tx(&bar[pstage], BOX);
+    tma_load_3d(tsm + pstage * STRIDE, tm, 2 * (x0 - 2), y0 - 1, pc.z, &bar[pstage]);
     pstage = pstage + 1 == stages ? 0 : pstage + 1;
     ++issued;
     pmore = pc.advance(g1, P) != 0;
@@ -489,12 +329,7 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
   int hx = 0, hy = 0;
   const bool halo = tid < HALO;
   if (halo) halo_coord<TM3_TX, TY>(tid, hx, hy);
-  C acc[J];
-#pragma unroll
-  for (int k = 0; k < J; ++k) acc[k] = czero<C>();
-  R accn = 0;
-  C rawp[QY][J];          // own raw values of the previous plane
-  C vprev[QY], vcur[QY];  // own v_J two planes and one plane back
+  C vprev[QY], vcur[QY];  // own points two planes and one plane back
   Coef3<C> cx, cy[QY];
   int x0 = 0, y0 = 0;
   unsigned off = 0;       // padded index of the thread's first point in plane 0
@@ -515,40 +350,27 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
       off = (unsigned)(y0 + ly) * P + x0 + lx;
     }
     // the stencil of this iteration works on plane z = cc.z - 1 (from the third plane
-    // of a piece on); its phi is fetched before the wait (in bounds: z < P)
+    // of a piece on); its phi and b are fetched before the wait (in bounds: z < P)
     const int z = cc.z - 1;
     const unsigned pz = off + (unsigned)z * P * P;
-    R ph[QY];
-    C bq[QY];  // residual mode: b at the stencil plane, fetched with phi
+    float ph[QY];
+    C bq[QY];
 #pragma unroll
     for (int q = 0; q < QY; ++q) {
       ph[q] = (u >= 2 && S.phi) ? __ldg(S.phi + pz + 8 * q * P) : S.phic;
-      if (RESID) bq[q] = u >= 2 ? __ldg(L.b + pz + 8 * q * P) : czero<C>();
+      bq[q] = u >= 2 ? __ldg(L.b + pz + 8 * q * P) : czero<C>();
     }
     const bool mine = mbar_wait(&bar[cstage], cphase);
-    const C* box[J];
-#pragma unroll
-    for (int k = 0; k < J; ++k) box[k] = reinterpret_cast<const C*>(tsm + (cstage * J + k) * STRIDE);
+    const C* box = reinterpret_cast<const C*>(tsm + cstage * STRIDE);
     C (*vs)[TM3_TX + 2] = vr[rslot];
-    C rawn[QY][J], vnew[QY];
+    C vnew[QY];
 #pragma unroll
     for (int q = 0; q < QY; ++q) {
       const int oy = ly + 8 * q;
-      C v = czero<C>();
-#pragma unroll
-      for (int k = 0; k < J; ++k) {
-        rawn[q][k] = box[k][(oy + 1) * TM3_BX + lx + 2];
-        v = cfma(cf[k], rawn[q][k], v);
-      }
-      vnew[q] = v;
-      vs[oy + 1][lx + 1] = v;
+      vnew[q] = box[(oy + 1) * TM3_BX + lx + 2];
+      vs[oy + 1][lx + 1] = vnew[q];
     }
-    if (halo) {
-      C v = czero<C>();
-#pragma unroll
-      for (int k = 0; k < J; ++k) v = cfma(cf[k], box[k][(hy + 1) * TM3_BX + hx + 2], v);
-      vs[hy + 1][hx + 1] = v;
-    }
+    if (halo) vs[hy + 1][hx + 1] = box[(hy + 1) * TM3_BX + hx + 2];
     if (!__syncthreads_and(mine)) { ok = false; break; }
     ++consumed;
     // every thread is done with this stage: refill it with the next plane
@@ -567,25 +389,15 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
           p = cfma(cz.d, vcur[q], p);
           p = cfma(cz.a, vprev[q], p);
           p = cfma(cz.c, vnew[q], p);
-          if (RESID) {
-            p = csub(bq[q], p);  // r0 = b - M x_b
-            accn += cabs2(p);
-          } else {
-#pragma unroll
-            for (int k = 0; k < J; ++k) acc[k] = cdotacc(rawp[q][k], p, acc[k]);
-            accn += cabs2(p);
-          }
+          p = csub(bq[q], p);  // r0 = b - M x_b
         }
-        if (RESID) L.r0[pz + 8 * q * P] = p;
-        else if (store_p) pJ[pz + 8 * q * P] = p;
+        L.r0[pz + 8 * q * P] = p;
       }
     }
 #pragma unroll
     for (int q = 0; q < QY; ++q) {
       vprev[q] = vcur[q];
       vcur[q] = vnew[q];
-#pragma unroll
-      for (int k = 0; k < J; ++k) rawp[q][k] = rawn[q][k];
     }
     rslot = rslot == 2 ? 0 : rslot + 1;
     if (++cstage == stages) { cstage = 0; cphase ^= 1u; }
@@ -593,34 +405,18 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
     more = step != 0;
     u = step == 2 ? 0 : u + 1;
   }
-  if (!ok) {
-    if (tid == 0) {
-      atomicExch(&g_vcycle_error, 1);
-      // the copies of this CTA that may still be landing (bounded)
-      int st = cstage;
-      unsigned ph = cphase;
-      for (int g = consumed; g < issued; ++g) {
-        mbar_wait(&bar[st], ph);
-        if (++st == stages) { st = 0; ph ^= 1u; }
-      }
+  if (!ok && tid == 0) {
+    atomicExch(&g_vcycle_error, 1);
+    // the copies of this CTA that may still be landing (bounded)
+    int st = cstage;
+    unsigned ph = cphase;
+    for (int g = consumed; g < issued; ++g) {
+      mbar_wait(&bar[st], ph);
+      if (++st == stages) { st = 0; ph ^= 1u; }
     }
-    __syncthreads();
-    return;
   }
+  __syncthreads();
   pdl_trigger();  // the main work is done: let the next pass launch
-  if (RESID) {
-    // ||r0||^2 starts the post-smoothing sweep
-    R red[1] = {accn}, tot[1];
-    if (grid_sum_last<1>(red, L.part, unit, nunits, &sc->counter, sm, tot)) {
-      if (flat_tid() == 0) sweep_begin(sc, tot[0], L.s);
-    }
-    return;
-  }
-  R red[2 * J + 1];
-#pragma unroll
-  for (int k = 0; k < J; ++k) { red[2 * k] = acc[k].x; red[2 * k + 1] = acc[k].y; }
-  red[2 * J] = accn;
-  grid_sum_sweep<R, J>(red, L.part, unit, nunits, sc, sm);
 }
 
 // ------------------------------------------------------------------ end of pre-smoothing, TMA (3D, complex64)
@@ -637,8 +433,7 @@ k_stencil_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages
 template <typename C, int M>
 __device__ __forceinline__ void restrict_tma3_run(const LevelDev<C>& L, const UpdCoef<C>& u, int g0, int g1, int stages,
                                                   int x_from_zero, const CUtensorMap* const* tm, unsigned char* tsm,
-                                                  uint64_t* bar, C (*rr)[TM3_TY2 + 1][TM3_TX + 1], typename CT<C>::R& acc,
-                                                  bool& ok) {
+                                                  uint64_t* bar, C (*rr)[TM3_TY2 + 1][TM3_TX + 1]) {
   typedef typename CT<C>::R R;
   constexpr int NR = M + 1;  // raw vectors
   constexpr unsigned BOX = tm3_box_bytes(2), STRIDE = tm3_box_stride(2);
@@ -674,7 +469,7 @@ __device__ __forceinline__ void restrict_tma3_run(const LevelDev<C>& L, const Up
   int u_ = 0, cstage = 0, f = 0, consumed = 0;
   unsigned cphase = 0;
   int x0 = 0, y0 = 0;
-  bool more = true;
+  bool more = true, ok = true;
 #pragma unroll 1
   while (more) {
     if (u_ == 0) {
@@ -737,7 +532,6 @@ __device__ __forceinline__ void restrict_tma3_run(const LevelDev<C>& L, const Up
       if (Ix < Pc && Iy < Pc && Iz < Pc) {
         const bool valid = Ix < nc && Iy < nc && Iz < nc;
         bc[pidx(Ix, Iy, Iz, Pc)] = valid ? out : czero<C>();
-        if (valid) acc += cabs2(out);
       }
     }
     if (++cstage == stages) { cstage = 0; cphase ^= 1u; }
@@ -765,7 +559,6 @@ k_restrict_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stage
   typedef float2 C;
   extern __shared__ __align__(128) unsigned char tsm[];
   __shared__ C rr[4][TM3_TY2 + 1][TM3_TX + 1];
-  __shared__ R sm[32];
   __shared__ __align__(8) uint64_t bar[TM3_STAGES_MAX];
   const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
   const LevelDev<C>& L = levs[prob];
@@ -787,21 +580,14 @@ k_restrict_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stage
   if (tid == 0)
     for (int k = 0; k <= u.m; ++k) tmap_acquire(tm[k]);
   __syncthreads();  // initialised barriers
-  R acc = 0;
-  bool ok = true;
   switch (u.m) {  // uniform over the grid
-    case 0: restrict_tma3_run<C, 0>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr, acc, ok); break;
-    case 1: restrict_tma3_run<C, 1>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr, acc, ok); break;
-    case 2: restrict_tma3_run<C, 2>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr, acc, ok); break;
-    case 3: restrict_tma3_run<C, 3>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr, acc, ok); break;
-    default: restrict_tma3_run<C, 4>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr, acc, ok); break;
+    case 0: restrict_tma3_run<C, 0>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr); break;
+    case 1: restrict_tma3_run<C, 1>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr); break;
+    case 2: restrict_tma3_run<C, 2>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr); break;
+    case 3: restrict_tma3_run<C, 3>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr); break;
+    default: restrict_tma3_run<C, 4>(L, u, g0, g1, stages, x_from_zero, tm, tsm, bar, rr); break;
   }
-  if (!__syncthreads_and(ok)) return;
-  R red[1] = {acc}, tot[1];
   pdl_trigger();  // the main work is done: let the next pass launch
-  if (grid_sum_last<1>(red, L.part, unit, nunits, &L.sc->counter, sm, tot)) {
-    if (flat_tid() == 0) sweep_begin(L.scc, tot[0], L.s);
-  }
 }
 
 // x_b = x_a + P e_c on a 3D level, in tiles of PR_ROWS full rows at one z: every
@@ -809,7 +595,7 @@ k_restrict_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stage
 // coarse rows the tile's trilinear interpolation reads (Y = y0/2 - 1 .. y0/2 + 3),
 // each already combined over the one or two coarse planes of z with their weight,
 // are staged in shared memory, from which every point takes its y and x neighbours.
-// The stencil and residual follow in k_stencil_tma3<1, QY, true>.
+// The stencil and residual follow in k_resid_tma3.
 constexpr int PR_ROWS = 8;
 template <typename C, int PR_XPT>  // points per thread per row: P <= 256 PR_XPT
 __global__ void __launch_bounds__(256)
@@ -965,10 +751,12 @@ __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__
     default: break;
   }
   static_assert(SMAX == 4, "restrict_tiles is instantiated for m = 0..4");
-  R red[1] = {acc}, tot[1];
   pdl_trigger();  // the main work is done: let the next pass launch
-  if (grid_sum_last<1>(red, L.part, unit, nunits, &L.sc->counter, sm, tot)) {
-    if (flat_tid() == 0) sweep_begin(L.scc, tot[0], L.s);
+  if constexpr (sizeof(C) == 16) {  // complex64 sweeps take the norm from their Gram matrix
+    R red[1] = {acc}, tot[1];
+    if (grid_sum_last<1>(red, L.part, unit, nunits, &L.sc->counter, sm, tot)) {
+      if (flat_tid() == 0) sweep_begin(L.scc, tot[0], L.s);
+    }
   }
 }
 template <typename C>
@@ -1074,10 +862,12 @@ __device__ __forceinline__ void restrict_t3_body(const LevelDev<C>* __restrict__
       default: break;
     }
   }
-  R red[1] = {acc}, tot[1];
   pdl_trigger();  // the main work is done: let the next pass launch
-  if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
-    if (flat_tid() == 0) sweep_begin(L.scc, tot[0], L.s);
+  if constexpr (sizeof(C) == 16) {  // complex64 sweeps take the norm from their Gram matrix
+    R red[1] = {acc}, tot[1];
+    if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
+      if (flat_tid() == 0) sweep_begin(L.scc, tot[0], L.s);
+    }
   }
 }
 template <typename C>
@@ -1150,10 +940,12 @@ __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ 
     }
     __syncthreads();  // the next tile rewrites vt
   }
-  R red[1] = {acc}, tot[1];
   pdl_trigger();  // the main work is done: let the next pass launch
-  if (grid_sum_last<1>(red, L.part, unit, nunits, &L.sc->counter, sm, tot)) {
-    if (flat_tid() == 0) sweep_begin(L.sc, tot[0], L.s);
+  if constexpr (sizeof(C) == 16) {  // complex64 sweeps take the norm from their Gram matrix
+    R red[1] = {acc}, tot[1];
+    if (grid_sum_last<1>(red, L.part, unit, nunits, &L.sc->counter, sm, tot)) {
+      if (flat_tid() == 0) sweep_begin(L.sc, tot[0], L.s);
+    }
   }
 }
 template <typename C>
@@ -1216,10 +1008,12 @@ __device__ __forceinline__ void prolong_t3_body(const LevelDev<C>* __restrict__ 
       }
     }
   }
-  R red[1] = {acc}, tot[1];
   pdl_trigger();  // the main work is done: let the next pass launch
-  if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
-    if (flat_tid() == 0) sweep_begin(L.sc, tot[0], L.s);
+  if constexpr (sizeof(C) == 16) {  // complex64 sweeps take the norm from their Gram matrix
+    R red[1] = {acc}, tot[1];
+    if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
+      if (flat_tid() == 0) sweep_begin(L.sc, tot[0], L.s);
+    }
   }
 }
 template <typename C>
@@ -1275,12 +1069,23 @@ __device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned nblocks, unsi
   return ok != 0;
 }
 
+constexpr int SEQ_O3 = 4;  // own rows of the 3D sweep pass on levels the segments may hold
+
 // Each pass body is called as a separate function, so the persistent kernel needs the
 // registers of its largest body only, not of all of them inlined together.
+// (complex64: J is the sweep's step count S and the pass the whole basis, gram.cuh)
 template <typename C, int DIM, int J>
-__device__ __noinline__ void seq_arnoldi(const PassDesc d, const LevelDev<C>* levs, int v) {
-  if constexpr (DIM == 2) arnoldi_t2_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
-  else arnoldi_t3_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
+__device__ __noinline__ void seq_arnoldi(const PassDesc d, const LevelDev<C>* levs, int v, float2* sm) {
+  if constexpr (sizeof(C) == 8 && DIM == 2) {
+    if (d.geo == 2) sweep2_body<J, 2, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 2>*>(sm));
+    else sweep2_body<J, 4, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 4>*>(sm));
+  } else if constexpr (sizeof(C) == 8) {
+    sweep3_body<J, SEQ_O3, false>(levs, d.ntiles, d.f0, d.f1, v, sm);
+  } else if constexpr (DIM == 2) {
+    arnoldi_t2_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
+  } else {
+    arnoldi_t3_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
+  }
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_restrict(const PassDesc d, const LevelDev<C>* levs, int v) {
@@ -1304,14 +1109,14 @@ __device__ __noinline__ void seq_prolong_flat(const PassDesc d, const LevelDev<C
 // flags: arnoldi f0 = R_0 is b, f1 = store p_J; restrict f0 = R_0 is b, f1 = x from zero,
 // f2 = no smoothing; update f0 = mode, f1 = R_0 is b, f2 = x selection, f3 = x from zero
 template <typename C, int DIM>
-__device__ __forceinline__ void run_pass(const PassDesc& d, const LevelDev<C>* levs, int v) {
+__device__ __forceinline__ void run_pass(const PassDesc& d, const LevelDev<C>* levs, int v, float2* sm) {
   switch (d.kind) {
     case PK_ARNOLDI:
       switch (d.J) {
-        case 1: seq_arnoldi<C, DIM, 1>(d, levs, v); break;
-        case 2: seq_arnoldi<C, DIM, 2>(d, levs, v); break;
-        case 3: seq_arnoldi<C, DIM, 3>(d, levs, v); break;
-        default: seq_arnoldi<C, DIM, 4>(d, levs, v); break;
+        case 1: seq_arnoldi<C, DIM, 1>(d, levs, v, sm); break;
+        case 2: seq_arnoldi<C, DIM, 2>(d, levs, v, sm); break;
+        case 3: seq_arnoldi<C, DIM, 3>(d, levs, v, sm); break;
+        default: seq_arnoldi<C, DIM, 4>(d, levs, v, sm); break;
       }
       break;
     case PK_RESTRICT: seq_restrict<C, DIM>(d, levs, v); break;
@@ -1326,11 +1131,12 @@ __device__ __forceinline__ void run_pass(const PassDesc& d, const LevelDev<C>* l
 template <typename C, int DIM>
 __global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1)
 k_vcycle_seq(const __grid_constant__ PassSeq seq, GridBar* gb, unsigned long long limit_ns) {
+  extern __shared__ __align__(16) float2 seqsm[];
   for (int q = 0; q < seq.npass; ++q) {
     const PassDesc& d = seq.p[q];
     const LevelDev<C>* levs = reinterpret_cast<const LevelDev<C>*>(d.levs);
     for (int v = blockIdx.x; v < d.nvblk; v += gridDim.x) {
-      run_pass<C, DIM>(d, levs, v);
+      run_pass<C, DIM>(d, levs, v, seqsm);
       __syncthreads();  // the next virtual block reuses the pass's shared memory
     }
     if (q + 1 < seq.npass && !grid_barrier(gb, gridDim.x, limit_ns)) return;

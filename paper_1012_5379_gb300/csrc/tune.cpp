@@ -313,24 +313,22 @@ int tune_write(const char* path, const std::string& run_record, std::string* err
   return f ? HELM_OK : HELM_EINVAL;
 }
 
-// 3D TMA-fed passes (Arnoldi step J; the prolongation's residual and the restriction,
-// J = 0): tuned (on, plane slots, z pieces per column, points per thread in y), else on
-// with as many plane slots in flight as leave the kernel its CTAs per SM (Arnoldi: 3, 2,
-// 2, 2 for J = 1..4; restriction of four raw vectors: 2), one equal share of the level
-// per resident CTA, two points per thread (the restriction always takes two).
-Tma3Params tma3_params(int pass, int J, int P) {
+// 3D TMA-fed passes (the post-smoothing residual and the restriction): tuned (on, plane
+// slots, z pieces per column, points per thread in y), else on with as many plane slots in
+// flight as leave the kernel its CTAs per SM (residual 3, restriction of four vectors 2),
+// one equal share of the level per resident CTA, two points per thread.
+Tma3Params tma3_params(int pass, int P) {
   Tma3Params p;
   TuneChoice c;
-  const int maxj = pass == TP_PROLONG ? 1 : J;
-  if (tune_get(pass, 3, P, 8, J, &c)) {
+  if (tune_get(pass, 3, P, 8, 0, &c)) {
     p.enabled = c.v[0] != 0;
     p.stages = std::max(2, std::min(c.v[1], TM3_STAGES_MAX));
     p.pieces = std::max(0, c.v[2]);
-    p.qy = c.v[3] == 4 && maxj <= 2 ? 4 : 2;
+    p.qy = c.v[3] == 4 ? 4 : 2;
     return p;
   }
   p.enabled = true;
-  p.stages = pass == TP_RESTRICT ? 3 : (maxj <= 2 ? 6 : (maxj == 3 ? 4 : 3));
+  p.stages = pass == TP_RESTRICT ? 3 : 6;
   p.pieces = 0;
   p.qy = 2;
   return p;

@@ -212,7 +212,7 @@ __device__ __forceinline__ void update_pass_body(const LevelDev<C>* __restrict__
     default: break;
   }
   static_assert(SMAX == 4, "update_flat_body is instantiated for m = 0..4");
-  if (!want_r) return;
+  if (!want_r || sizeof(C) == 8) return;  // complex64: the next sweep takes ||r||^2 from its Gram matrix
   typename CT<C>::R red[1] = {acc}, tot[1];
   pdl_trigger();  // the main work is done: let the next pass launch
   if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
@@ -231,7 +231,7 @@ k_update_flat(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, int mod
 template <typename Cin, typename C>
 __global__ void __launch_bounds__(256)
 k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Cin* __restrict__ src) {
-  __shared__ typename CT<C>::R sm[32];
+  __shared__ typename CT<C>::R sm[64];
   const int prob = blockIdx.x / ntiles, tile = blockIdx.x - prob * ntiles;
   const LevelDev<C>& L = levs[prob];
   const int n = L.n, P = L.P;
@@ -239,7 +239,8 @@ k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Ci
   // CTAs take rows (z, y) of the padded layout in turn; threads stride along x
   const int nrows = dim == 3 ? P * P : P;
   C* const b = L.b;
-  typename CT<C>::R acc = 0;
+  constexpr bool GRAM = sizeof(C) == 8;  // complex64: the first sweep's shift from neighbour differences
+  typename CT<C>::R acc = 0, accd = 0;
   for (int row = tile; row < nrows; row += ntiles) {
     const int y = dim == 3 ? row % P : row, z = dim == 3 ? row / P : 0;
     const bool rin = y < n && z < n;
@@ -249,12 +250,24 @@ k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Ci
       if (rin && x < n) v = to_c<C>(src[sbase + x]);
       b[base + x] = v;
       acc += cabs2(v);
+      if (GRAM && rin && x + 1 < n) accd += cabs2(csub(to_c<C>(src[sbase + x + 1]), v));
     }
   }
-  typename CT<C>::R red[1] = {acc}, tot[1];
-  pdl_trigger();  // the main work is done: let the next pass launch
-  if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
-    if (flat_tid() == 0) sweep_begin(L.sc, tot[0], L.s);
+  if constexpr (GRAM) {
+    typename CT<C>::R red[2] = {acc, accd}, tot[2];
+    pdl_trigger();  // the main work is done: let the next pass launch
+    if (grid_sum_last<2>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
+      if (flat_tid() == 0) {
+        sweep_begin(L.sc, tot[0], L.s);
+        L.sc->sig0 = sweep_first_shift(L.klap, L.phir, tot[1], tot[0]);
+      }
+    }
+  } else {
+    typename CT<C>::R red[1] = {acc}, tot[1];
+    pdl_trigger();  // the main work is done: let the next pass launch
+    if (grid_sum_last<1>(red, L.part, tile, ntiles, &L.sc->counter, sm, tot)) {
+      if (flat_tid() == 0) sweep_begin(L.sc, tot[0], L.s);
+    }
   }
 }
 
@@ -317,72 +330,7 @@ struct CtaTeam {
   __device__ __forceinline__ void sum(T (&v)[NV], T* sm) { block_sum<NV, T>(v, sm); }
 };
 
-constexpr int CLUSTER_MAX = 16;
-constexpr int TEAM_NV = 2 * SMAX + 1;  // most values one team sum carries
 constexpr int CB_U = 4;                // points per thread per step of the team loops
-
-__device__ __forceinline__ unsigned cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ unsigned cluster_size() {
-  unsigned n;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
-  return n;
-}
-// Every thread of every CTA of the cluster; release/acquire at cluster scope.
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Load a word of CTA `rank`'s shared memory at the address of `p` in this CTA's.
-__device__ __forceinline__ float ld_dsmem(const float* p, unsigned rank) {
-  unsigned a = (unsigned)__cvta_generic_to_shared(p), ra;
-  float v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
-  return v;
-}
-__device__ __forceinline__ double ld_dsmem(const double* p, unsigned rank) {
-  unsigned a = (unsigned)__cvta_generic_to_shared(p), ra;
-  double v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ra) : "memory");
-  return v;
-}
-
-// `slots` is this CTA's [2][CLUSTER_MAX][TEAM_NV] doubles of shared memory.  The two
-// halves alternate between sums: a CTA can only rewrite a half after every CTA has
-// passed the barrier that follows the reads of the previous sum in it.
-struct ClusterTeam {
-  unsigned r, n;
-  double* slots;
-  int buf;
-  __device__ __forceinline__ explicit ClusterTeam(double* s) : r(cluster_rank()), n(cluster_size()), slots(s), buf(0) {}
-  __device__ __forceinline__ int rank() const { return (int)r; }
-  __device__ __forceinline__ unsigned gtid() const { return r * (unsigned)block_threads() + (unsigned)flat_tid(); }
-  __device__ __forceinline__ unsigned gnth() const { return n * (unsigned)block_threads(); }
-  __device__ __forceinline__ void sync() const { cluster_sync(); }
-  template <int NV, typename T>
-  __device__ __forceinline__ void sum(T (&v)[NV], T* sm) {
-    block_sum<NV, T>(v, sm);
-    T* half = reinterpret_cast<T*>(slots + (size_t)buf * CLUSTER_MAX * TEAM_NV);
-    if (flat_tid() == 0)
-#pragma unroll
-      for (int i = 0; i < NV; ++i) half[r * NV + i] = v[i];
-    cluster_sync();
-    if (flat_tid() < 32) {  // lane q reads rank q's sums, a fixed butterfly adds them
-      const unsigned q = (unsigned)flat_tid();
-#pragma unroll
-      for (int i = 0; i < NV; ++i) v[i] = q < n ? ld_dsmem(half + q * NV + i, q) : (T)0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    }
-    buf ^= 1;
-  }
-};
 
 template <typename C>
 __device__ void cblock_stencil_apply(const LevelDev<C>& L, const C* v, int x, int y, int z, int dim, C& out) {
@@ -868,44 +816,6 @@ k_coarse_smem(const LevelDev<C>* __restrict__ levs_all, int nlev, int lev_stride
     const size_t np0 = dim == 3 ? (size_t)G[0].P * G[0].P * G[0].P : (size_t)G[0].P * G[0].P;
     for (size_t i = tid; i < np0; i += nth) G[0].xb[i] = Ls[0].xb[i];
   }
-}
-
-// Coarse sub-cycle on one thread-block cluster per problem (clusters are consecutive
-// blocks along x): the level vectors stay in global memory, every CTA holds its own
-// copy of the descriptors and sweep scalars.  Problem p runs lus[p].nlev levels.
-constexpr int CLUSTER_THREADS = 512;
-template <typename C>
-__global__ void __launch_bounds__(CLUSTER_THREADS)
-k_coarse_cluster(const LevelDev<C>* __restrict__ levs_all, int lev_stride, const CoarseLU* __restrict__ lus,
-                 int nu1, int nu2, int dim) {
-  __shared__ double sm[32 * (2 * SMAX + 1)];
-  __shared__ double slots[2 * CLUSTER_MAX * TEAM_NV];
-  __shared__ LevelDev<C> Ls[MAX_COARSE_LEVELS];
-  __shared__ SweepScalarsT<typename CT<C>::R> Ss[MAX_COARSE_LEVELS];
-  pdl_trigger();
-  ClusterTeam team(slots);
-  const int prob = blockIdx.x / (int)team.n;
-  const CoarseLU lu = lus[prob];
-  const int nlev = lu.nlev;
-  const LevelDev<C>* G = levs_all + (size_t)prob * lev_stride;
-  const int tid = flat_tid(), nth = block_threads();
-  pdl_wait();
-  if (tid == 0) {
-    for (int l = 0; l < nlev; ++l) {
-      Ls[l] = G[l];
-      Ls[l].sc = &Ss[l];
-    }
-    for (int l = 0; l + 1 < nlev; ++l) Ls[l].scc = &Ss[l + 1];
-  }
-  {
-    const int* src = reinterpret_cast<const int*>(G[0].sc);
-    int* dst = reinterpret_cast<int*>(&Ss[0]);
-    const int words = sweep_words<typename CT<C>::R>();
-    for (int i = tid; i < words; i += nth) dst[i] = __ldcg(src + i);
-  }
-  __syncthreads();
-  coarse_cycle<C>(team, Ls, nlev, lu, nu1, nu2, dim, sm);
-  team.sync();  // no CTA leaves while another may still read its shared memory
 }
 
 }  // namespace helm

@@ -2,44 +2,13 @@
 // vcycle_c64.cu and vcycle_c128.cu (two translation units compile in parallel).
 #pragma once
 #include "tiles.cuh"
+#include "launch.cuh"
 #include <algorithm>
 #include <type_traits>
 #include "../../include/helm.h"
 #include "poly.h"
 
 namespace helm {
-
-// Launch with programmatic stream serialisation: the kernel may start while its
-// predecessor finishes and synchronises with it through griddepcontrol.wait.  The
-// passes that end in a grid reduction signal their dependents only after their main
-// work, so waiting dependents never hold SM slots the predecessor's later waves need;
-// the launch latency and the dependent's prologue then overlap the predecessor's
-// reduction tail.
-static inline int sm_count() {
-  // initialised once, thread-safely (serving and callers' threads launch concurrently)
-  static const int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 1;
-    return v;
-  }();
-  return n;
-}
-template <typename... KArgs, typename... Args>
-static inline void pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args... args) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
 
 // Tiles per CTA of a 2D pass for one problem of `ntiles` tiles: each CTA pays a fixed
 // cost (its reduction, the atomic, the ramp; about half a tile's time on GB300) plus
@@ -67,71 +36,34 @@ static int tiles_per_cta(K kernel, int ntiles, size_t smem = 0) {
   return best;
 }
 
-constexpr int TMA_MIN_TILES = 16384;  // 2D levels of 4095^2 and larger
-
-template <int J>
-static void arnoldi_tma2(const LevelDev<float2>* levs, int nprob, int ntiles, int P, bool r0_is_b, bool store_p,
-                         cudaStream_t st) {
-  const size_t smem = tma_arnoldi_smem(J);
-  thread_local bool configured = false;  // the attribute is per function; setting it again is harmless
-  if (!configured) {
-    cudaFuncSetAttribute(k_arnoldi_tma2<J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
-  const int t = tuned_tpc(TP_ARNOLDI, P, 8, J, tiles_per_cta(k_arnoldi_tma2<J>, ntiles, smem));
-  pdl_launch(k_arnoldi_tma2<J>, dim3(nprob * ceil_div(ntiles, t)), dim3(32, 8), smem, st, levs, ntiles, t,
-             r0_is_b ? 1 : 0, store_p ? 1 : 0);
-}
-
-// The 3D TMA-fed Arnoldi pass: planes per z-march, plane slots in flight and tiles per
-// CTA of a level of pitch P (tuned table, else these defaults).
-
-template <int J, int QY, bool RESID>
-static void stencil_tma3_q(const LevelDev<float2>* levs, int nprob, int P, const Tma3Params& tp, bool r0_is_b,
-                           bool store_p, cudaStream_t st) {
-  const size_t smem = tma3_arnoldi_smem(J, QY, tp.stages);
+// The post-smoothing residual of a 3D complex64 level, x_b streamed by TMA.
+template <int QY>
+static void resid_tma3(const LevelDev<float2>* levs, int nprob, int P, const Tma3Params& tp, cudaStream_t st) {
+  const size_t smem = tma3_smem(1, QY, tp.stages);
   // per host thread: the largest dynamic shared memory set so far, and the residency
   // of the last configuration
   thread_local size_t configured = 0;
   thread_local int occ_stages = -1, occ = 1;
   if (configured < smem) {
-    cudaFuncSetAttribute(k_stencil_tma3<J, QY, RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_resid_tma3<QY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     configured = smem;
   }
   if (occ_stages != tp.stages) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_stencil_tma3<J, QY, RESID>, 256, smem) != cudaSuccess ||
-        occ < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_resid_tma3<QY>, 256, smem) != cudaSuccess || occ < 1)
       occ = 1;
     occ_stages = tp.stages;
   }
-  // shares of the level's (column, plane) sequence: column pieces, or one per resident
-  // CTA (a function of the level size and the device only: it fixes the order of the
-  // partial sums)
+  // shares of the level's (column, plane) sequence: column pieces, or one per resident CTA
   const long long cols = tma3_cols(P, QY);
   long long units = tp.pieces > 0 ? cols * std::min(tp.pieces, P) : (long long)occ * sm_count();
   units = std::max<long long>(1, std::min<long long>(units, std::min<long long>(TMA3_MAX_UNITS, cols * P)));
-  const int nunits = (int)units;
-  pdl_launch(k_stencil_tma3<J, QY, RESID>, dim3(nprob * nunits), dim3(32, 8), smem, st, levs, nunits, tp.stages,
-             r0_is_b ? 1 : 0, store_p ? 1 : 0);
-}
-
-template <int J>
-static void arnoldi_tma3(const LevelDev<float2>* levs, int nprob, int P, bool r0_is_b, bool store_p,
-                         cudaStream_t st) {
-  const Tma3Params tp = tma3_params(TP_ARNOLDI, J, P);
-  if constexpr (J <= 2) {
-    if (tp.qy == 4) {
-      stencil_tma3_q<J, 4, false>(levs, nprob, P, tp, r0_is_b, store_p, st);
-      return;
-    }
-  }
-  stencil_tma3_q<J, 2, false>(levs, nprob, P, tp, r0_is_b, store_p, st);
+  pdl_launch(k_resid_tma3<QY>, dim3(nprob * (int)units), dim3(32, 8), smem, st, levs, (int)units, tp.stages);
 }
 
 // Coarse correction and post-smoothing residual of a 3D complex64 level in two passes:
 // x_b = x_a + P e_c row by row, then r0 = b - M x_b with x_b streamed by TMA.
 static void prolong_tma3(const LevelDev<float2>* levs, int nprob, int P, cudaStream_t st) {
-  const Tma3Params tp = tma3_params(TP_PROLONG, 0, P);
+  const Tma3Params tp = tma3_params(TP_PROLONG, P);
   const int nblk = std::max(1, std::min(8 * sm_count() / std::max(nprob, 1), (P / PR_ROWS) * P));
   if (P <= 256)
     pdl_launch(k_prolong3_rows<float2, 1>, dim3(nprob * nblk), dim3(256), 0, st, levs, nblk);
@@ -140,26 +72,15 @@ static void prolong_tma3(const LevelDev<float2>* levs, int nprob, int P, cudaStr
   else
     pdl_launch(k_prolong3_rows<float2, 4>, dim3(nprob * nblk), dim3(256), 0, st, levs, nblk);
   if (tp.qy == 4)
-    stencil_tma3_q<1, 4, true>(levs, nprob, P, tp, false, false, st);
+    resid_tma3<4>(levs, nprob, P, tp, st);
   else
-    stencil_tma3_q<1, 2, true>(levs, nprob, P, tp, false, false, st);
+    resid_tma3<2>(levs, nprob, P, tp, st);
 }
 
+// Arnoldi steps one pass at a time (complex128; complex64 sweeps: sweep.cu).
 template <typename C, int J>
 static void arnoldi_J(int dim, const LevelDev<C>* levs, int grid, int ntiles, TileCfg cfg, bool r0_is_b,
-                      bool store_p, bool tma, cudaStream_t st) {
-  if constexpr (std::is_same<C, float2>::value) {
-    // the TMA pipeline pays off on levels that stream from HBM; smaller levels are
-    // latency-bound and L2-resident
-    if (dim == 2 && tma && ntiles >= TMA_MIN_TILES) {
-      arnoldi_tma2<J>(levs, grid / ntiles, ntiles, cfg.P, r0_is_b, store_p, st);
-      return;
-    }
-    if (dim == 3 && tma && cfg.P >= TMA3_MIN_P && cfg.P <= TMA3_MAX_P && tma3_params(TP_ARNOLDI, J, cfg.P).enabled) {
-      arnoldi_tma3<J>(levs, grid / ntiles, cfg.P, r0_is_b, store_p, st);
-      return;
-    }
-  }
+                      bool store_p, cudaStream_t st) {
   if (dim == 2) {
     const int t = tuned_tpc(TP_ARNOLDI, cfg.P, (int)sizeof(C), J, tiles_per_cta(k_arnoldi_t2<C, J>, ntiles));
     pdl_launch(k_arnoldi_t2<C, J>, dim3(grid / ntiles * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t,
@@ -171,20 +92,20 @@ static void arnoldi_J(int dim, const LevelDev<C>* levs, int grid, int ntiles, Ti
 
 template <typename C>
 void launch_arnoldi(int dim, int J, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
-                    bool store_p, bool tma, cudaStream_t st) {
+                    bool store_p, cudaStream_t st) {
   const int grid = nprob * ntiles;
   switch (J) {
-    case 1: arnoldi_J<C, 1>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, tma, st); break;
-    case 2: arnoldi_J<C, 2>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, tma, st); break;
-    case 3: arnoldi_J<C, 3>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, tma, st); break;
-    default: arnoldi_J<C, 4>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, tma, st); break;
+    case 1: arnoldi_J<C, 1>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, st); break;
+    case 2: arnoldi_J<C, 2>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, st); break;
+    case 3: arnoldi_J<C, 3>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, st); break;
+    default: arnoldi_J<C, 4>(dim, levs, grid, ntiles, cfg, r0_is_b, store_p, st); break;
   }
 }
 
 // The TMA-fed 3D restriction (complex64 levels of pitch 128..1024 with tensor maps).
 static void restrict_tma3(const LevelDev<float2>* levs, int nprob, int P, bool r0_is_b, bool x_from_zero,
                           bool nosmooth, int nraw, cudaStream_t st) {
-  const Tma3Params tp = tma3_params(TP_RESTRICT, 0, P);
+  const Tma3Params tp = tma3_params(TP_RESTRICT, P);
   const size_t smem = (size_t)tp.stages * nraw * tm3_box_stride(2);
   thread_local size_t configured = 0;
   thread_local int occ_key = -1, occ = 1;
@@ -209,7 +130,7 @@ template <typename C>
 void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
                      bool x_from_zero, bool nosmooth, cudaStream_t st, bool tma, int nraw) {
   if constexpr (std::is_same<C, float2>::value) {
-    if (dim == 3 && tma && cfg.P >= TMA3_MIN_P && cfg.P <= TMA3_MAX_P && tma3_params(TP_RESTRICT, 0, cfg.P).enabled) {
+    if (dim == 3 && tma && cfg.P >= TMA3_MIN_P && cfg.P <= TMA3_MAX_P && tma3_params(TP_RESTRICT, cfg.P).enabled) {
       restrict_tma3(levs, nprob, cfg.P, r0_is_b, x_from_zero, nosmooth, nraw, st);
       return;
     }
@@ -271,54 +192,6 @@ void launch_coarse_smem(int dim, const LevelDev<C>* levs, int nlev, int lev_stri
   pdl_launch(k_coarse_smem<C>, dim3(nprob), dim3(512), smem_bytes, st, levs, nlev, lev_stride, lus, nu1, nu2, dim);
 }
 
-// Cluster size of the coarse sub-cycle: the largest power of two up to CLUSTER_MAX
-// that the device can make resident (a constant of the device, so a problem's result
-// does not depend on the other problems of its launch).
-template <typename C>
-static int coarse_cluster_size() {
-  // the largest cluster the device can place, found once (thread-safe initialisation)
-  static const int csize = [] {
-    cudaFuncSetAttribute(k_coarse_cluster<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    int found = 0;
-    for (int c = CLUSTER_MAX; c >= 1 && found == 0; c >>= 1) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(c);
-      cfg.blockDim = dim3(CLUSTER_THREADS);
-      cudaLaunchAttribute at;
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = c;
-      at.val.clusterDim.y = 1;
-      at.val.clusterDim.z = 1;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      int nclusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_cluster<C>, &cfg) == cudaSuccess && nclusters > 0)
-        found = c;
-    }
-    cudaGetLastError();
-    return found == 0 ? 1 : found;
-  }();
-  return csize;
-}
-
-template <typename C>
-void launch_coarse_cluster(int dim, const LevelDev<C>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                           int nu1, int nu2, cudaStream_t st) {
-  const int c = coarse_cluster_size<C>();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nprob * c);
-  cfg.blockDim = dim3(CLUSTER_THREADS);
-  cfg.stream = st;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = c;
-  at.val.clusterDim.y = 1;
-  at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_coarse_cluster<C>, levs, lev_stride, lus, nu1, nu2, dim);
-}
-
 template <typename C>
 void launch_load_input(int dim, const LevelDev<C>* levs, int ntiles, const void* src, int in_prec, cudaStream_t st) {
   if (in_prec == HELM_C128)
@@ -352,22 +225,6 @@ void launch_poly_restrict(int dim, const LevelDev<C>* levs, int nprob, int nflat
 // ------------------------------------------------------------------ persistent segments
 // The recorders append the pass an ordinary launch would run (the same launch
 // parameters, so the same partial-sum order) to a pass list instead of launching it.
-static inline void seq_push(PassSeq& q, const void* levs, int kind, int J, int ntiles, int geo, int f0, int f1, int f2,
-                            int f3, int nvblk) {
-  if (q.npass >= SEQ_MAX) return;  // the caller sizes its lists (checked by the engine)
-  PassDesc& d = q.p[q.npass++];
-  d.levs = levs;
-  d.kind = kind;
-  d.J = J;
-  d.ntiles = ntiles;
-  d.geo = geo;
-  d.f0 = f0;
-  d.f1 = f1;
-  d.f2 = f2;
-  d.f3 = f3;
-  d.nvblk = nvblk;
-}
-
 template <typename C, int J>
 static void record_arnoldi_J(PassSeq& q, int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg,
                              bool r0_is_b, bool store_p) {
@@ -427,10 +284,13 @@ template <typename C>
 int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_ns, cudaStream_t st) {
   if (q.npass == 0) return 0;
   void (*kern)(const PassSeq, GridBar*, unsigned long long) = dim == 2 ? k_vcycle_seq<C, 2> : k_vcycle_seq<C, 3>;
+  // shared memory of the complex64 sweep pass
+  const size_t smem = sizeof(C) != 8 ? 0 : dim == 3 ? sw3_smem(SMAX, SEQ_O3) : sizeof(Sw2Shared<SMAX, 4>);
   thread_local void (*last)(const PassSeq, GridBar*, unsigned long long) = nullptr;
   thread_local int occ = 1;
   if (kern != last) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, 0) != cudaSuccess || occ < 1) occ = 1;
+    if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, smem) != cudaSuccess || occ < 1) occ = 1;
     last = kern;
   }
   int maxv = 1;
@@ -444,7 +304,7 @@ int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(32, 8);  // the tile passes' shape; the flat passes use the flat thread index
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
@@ -453,7 +313,6 @@ int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_
 }
 
 #define HELM_VCYCLE_INST(C)                                                                                   \
-  template void launch_arnoldi<C>(int, int, const LevelDev<C>*, int, int, TileCfg, bool, bool, bool, cudaStream_t); \
   template void launch_restrict<C>(int, const LevelDev<C>*, int, int, TileCfg, bool, bool, bool,           \
                                     cudaStream_t, bool, int);                                               \
   template void launch_update_flat<C>(int, UpdateMode, const LevelDev<C>*, int, int, bool, int, bool,         \
@@ -461,15 +320,10 @@ int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_
   template void launch_prolong<C>(int, bool, const LevelDev<C>*, int, int, TileCfg, bool, cudaStream_t);      \
   template void launch_coarse<C>(int, const LevelDev<C>*, int, int, const CoarseLU*, int, int, int,           \
                                  cudaStream_t);                                                               \
-  template void launch_coarse_smem<C>(int, const LevelDev<C>*, int, int, const CoarseLU*, int, int, int, size_t, \
-                                      cudaStream_t);                                                          \
-  template void launch_coarse_cluster<C>(int, const LevelDev<C>*, int, const CoarseLU*, int, int, int,       \
-                                         cudaStream_t);                                                       \
   template void launch_load_input<C>(int, const LevelDev<C>*, int, const void*, int, cudaStream_t);           \
   template void launch_store_output<C>(int, int, const LevelDev<C>*, void*, int, cudaStream_t);              \
   template void launch_poly_step<C>(int, const LevelDev<C>*, const C*, int, int, int, int, int, cudaStream_t); \
   template void launch_poly_restrict<C>(int, const LevelDev<C>*, int, int, int, cudaStream_t);                \
-  template void record_arnoldi<C>(PassSeq&, int, int, const LevelDev<C>*, int, int, TileCfg, bool, bool);      \
   template void record_restrict<C>(PassSeq&, int, const LevelDev<C>*, int, int, TileCfg, bool, bool, bool);    \
   template void record_update<C>(PassSeq&, int, UpdateMode, const LevelDev<C>*, int, int, bool, int, bool);    \
   template void record_prolong<C>(PassSeq&, int, bool, const LevelDev<C>*, int, int, TileCfg);                 \
