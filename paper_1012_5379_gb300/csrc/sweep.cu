@@ -8,11 +8,30 @@
 
 namespace helm {
 
+// 2D levels from this size on march: 639^2 20 us a sweep against 21.7 in register regions,
+// 1023^2 25 against 37; at 511^2 and below a march of few rows is mostly halo.
+constexpr int SWEEP2_MARCH_N = 600;
+
 SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
   SweepCfg c{0, 0, 1};
   if (dim == 2) {
-    c.geo = n <= 255 ? 2 : (n <= 1023 || S > 3 ? 4 : 8);
-    c.units = sw2_units(S, c.geo, n);
+    if (n < SWEEP2_MARCH_N || S > 3) {
+      c.geo = n <= 255 ? 2 : 4;
+      c.units = sw2_units(S, c.geo, n);
+      return c;
+    }
+    // rows per march: the fewest row steps of the SM that takes the most, four CTAs per SM
+    c.march = 1;
+    long long best = -1;
+    for (int rows = 4; rows <= 256; ++rows) {
+      const long long units = sv2_units(n, rows);
+      const long long steps = (units + 4LL * sms - 1) / (4LL * sms) * (rows + 2 * S + 2);
+      if (best < 0 || steps < best) {
+        best = steps;
+        c.geo = rows;
+        c.units = (int)units;
+      }
+    }
     return c;
   }
   if (n < 96 || S > 3) {
@@ -42,10 +61,16 @@ static void launch_sweep_s(int dim, const LevelDev<float2>* levs, int nprob, con
   const dim3 grid(nprob * cfg.units);
   const int f = first ? 1 : 0, sl = store_last ? 1 : 0;
   if (dim == 2) {
-    const dim3 block(32, SW2_NW);
-    if (cfg.geo == 2) pdl_launch(k_sweep2<S, 2>, grid, block, 0, st, levs, cfg.units, f, sl);
-    else if (cfg.geo == 4 || S > 3) pdl_launch(k_sweep2<S, 4>, grid, block, 0, st, levs, cfg.units, f, sl);
-    else if constexpr (S <= 3) pdl_launch(k_sweep2<S, 8>, grid, block, 0, st, levs, cfg.units, f, sl);
+    if (!cfg.march) {
+      const dim3 block(32, SW2_NW);
+      if (cfg.geo == 2) pdl_launch(k_sweep2<S, 2>, grid, block, 0, st, levs, cfg.units, f, sl);
+      else pdl_launch(k_sweep2<S, 4>, grid, block, 0, st, levs, cfg.units, f, sl);
+    } else if constexpr (S <= 3) {
+      const dim3 block(32, SV2_NW);
+      const size_t smem = sv2_smem(S, cfg.geo);  // at most 256 rows: below 48 KB
+      if (phi) pdl_launch(k_sweep2_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
+      else pdl_launch(k_sweep2_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
+    }
     return;
   }
   if (!cfg.march) {

@@ -136,6 +136,142 @@ k_sweep2(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int s
   sweep2_body<S, QY>(levs, nunits, first, store_last, blockIdx.x, sh);
 }
 
+// ------------------------------------------------------------------ 2D, large levels
+// Every warp marches in y on its own 64-column strip, two neighbouring columns per lane (own:
+// the inner 56): x neighbours by shuffle, y neighbours in registers (four rows of each
+// vector), rows of R_0 loaded four steps ahead; no barrier and no shared vector.  In the step
+// that takes row y of R_0 it forms k_j of row y - j for every j.  A CTA's four warps take
+// neighbouring strips of one chunk of `rows` rows and share its y coefficients.
+// Bound by instruction issue (68% active, 192 lane instructions a point, 16 warps per SM at
+// 128 registers).  4095^2, s = 3: 129 us a sweep, 3.7 TB/s; a register-region kernel like the
+// one above with 8 rows per warp took 303 us (259 instructions a point, 45% issue: its
+// barriers and exposed loads).
+constexpr int SV2_NW = 4, SV2_OX = 56;
+HELM_HD inline int sv2_groups(int n) { return ceil_div(ceil_div(n, SV2_OX), SV2_NW); }
+HELM_HD inline int sv2_units(int n, int rows) { return sv2_groups(n) * ceil_div(n, rows); }
+HELM_HD constexpr unsigned sv2_smem(int S, int rows) { return (unsigned)(rows + 2 * S) * 24u; }
+
+template <int S, bool PHI>
+__global__ void __launch_bounds__(SV2_NW * 32, 4)
+k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, int first, int store_last) {
+  constexpr int NS = gram_ns(S), NV = gram_nv(S), W = 4;
+  static_assert(S <= 3, "register windows hold four rows");
+  extern __shared__ __align__(16) float2 swsm[];
+  __shared__ float wsum[SV2_NW * NS];
+  __shared__ float2 gs[SV2_NW * NV];
+  const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+  const int n = L.n, P = L.P;
+  const float t = L.kt, phir = L.phir, phc = phir * t;
+  const float* const phi = L.phi;
+  const int ng = sv2_groups(n);
+  const int x = ((unit % ng) * SV2_NW + warp) * SV2_OX - 4 + 2 * lane;  // columns x, x + 1
+  const int yb = (unit / ng) * rows, ye = min(yb + rows, n);
+  float4* const yac = reinterpret_cast<float4*>(swsm);
+  float2* const yd = reinterpret_cast<float2*>(yac + rows + 2 * S);
+  const SwCoef cx[2] = {sw_coef(L.ca, x, n, t), sw_coef(L.ca, x + 1, n, t)};
+  for (int i = tid; i < ye - yb + 2 * S; i += SV2_NW * 32) {
+    const SwCoef c = sw_coef(L.ca, yb - S + i, n, t);
+    yac[i] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
+    yd[i] = c.d;
+  }
+  pdl_wait();
+  __syncthreads();
+  float2 sg[S];
+  gram_shifts<S>(L, first != 0, sg);
+  const float2* R0 = first ? L.b : L.r0;
+  const bool in = (unsigned)x < (unsigned)P;  // the pair lies in the row (P is even, x too)
+  float2 win[S][W][2];  // k_j of the last rows, slot = step & 3
+#pragma unroll
+  for (int j = 0; j < S; ++j)
+#pragma unroll
+    for (int w = 0; w < W; ++w) win[j][w][0] = win[j][w][1] = make_float2(0.f, 0.f);
+  float phw[W][2];
+  float4 nxt[W];
+  float2 phn[W];
+  auto fetch = [&](int y, float4& v, float2& f) {
+    const bool ok = in && (unsigned)y < (unsigned)n;
+    v = ok ? __ldg(reinterpret_cast<const float4*>(R0 + (size_t)y * P + x)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (PHI)  // some problem of the launch has a field; this one may not
+      f = (ok && phi) ? __ldg(reinterpret_cast<const float2*>(phi + (size_t)y * P + x)) : make_float2(phir, phir);
+  };
+  float acc[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
+  const bool own = lane >= 2 && lane < 30 && x < n;
+  const int yf = yb - S, steps = ye - yb + 2 * S;
+#pragma unroll
+  for (int u = 0; u < W; ++u) fetch(u < steps ? yf + u : -1, nxt[u], phn[u]);
+#pragma unroll 1
+  for (int i0 = 0; i0 < steps; i0 += W) {
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      const int i = i0 + u;
+      if (i >= steps) break;  // uniform
+      const int y = yf + i;
+      win[0][u][0] = make_float2(nxt[u].x, nxt[u].y);
+      win[0][u][1] = make_float2(nxt[u].z, nxt[u].w);
+      if (PHI) {
+        phw[u][0] = phn[u].x * t;
+        phw[u][1] = phn[u].y * t;
+      }
+      if (i + W < steps) fetch(y + W, nxt[u], phn[u]);
+      float2 last[2];
+#pragma unroll
+      for (int j = 1; j <= S; ++j) {
+        // k_j at row y - j from k_{j-1} at rows y - j - 1 .. y - j + 1
+        const int c = (u - j) & 3, b = (u - j - 1) & 3, f = (u - j + 1) & 3;
+        float2 r[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (i >= j) {  // uniform
+          const float4 ya = yac[i - j];
+          const float2 ydd = yd[i - j];
+          const float2 v0 = win[j - 1][c][0], v1 = win[j - 1][c][1];
+          const float2 vl = shfl_up_c(v1, 1), vr = shfl_down_c(v0, 1);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            float2 dg = cadd(cx[q].d, ydd);
+            dg.x = (dg.x - (PHI ? phw[c][q] : phc)) - sg[j - 1].x;
+            dg.y -= sg[j - 1].y;
+            float2 p = cmul(dg, q ? v1 : v0);
+            p = cfma(cx[q].a, q ? v0 : vl, p);
+            p = cfma(cx[q].c, q ? vr : v1, p);
+            p = cfma(make_float2(ya.x, ya.y), win[j - 1][b][q], p);
+            r[q] = cfma(make_float2(ya.z, ya.w), win[j - 1][f][q], p);
+          }
+        }
+        if (j < S) {
+          win[j][c][0] = r[0];
+          win[j][c][1] = r[1];
+        } else {
+          last[0] = r[0];
+          last[1] = r[1];
+        }
+      }
+      if (i >= 2 * S && own) {
+        const int c = (u - S) & 3;
+        const size_t at = (size_t)(y - S) * P + x;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float2 kk[S + 1];
+#pragma unroll
+          for (int j = 0; j < S; ++j) kk[j] = win[j][c][q];
+          kk[S] = last[q];
+          gram_point<S>(kk, acc);
+        }
+#pragma unroll
+        for (int j = 1; j <= S; ++j)
+          if (j < S || store_last) {
+            const float2 a = j < S ? win[j < S ? j : 0][c][0] : last[0], b = j < S ? win[j < S ? j : 0][c][1] : last[1];
+            *reinterpret_cast<float4*>(L.p[j - 1] + at) = make_float4(a.x, a.y, b.x, b.y);
+          }
+      }
+    }
+  }
+  pdl_trigger();  // the main work is done: let the next pass launch
+  gram_finish<S, SV2_NW>(acc, L, sg, unit, nunits, wsum, gs);
+}
+
 // ------------------------------------------------------------------ 3D, small levels
 // A CTA of 8 warps owns (32 - 2S) x O x O points and keeps k_0..k_{S-1} on the region
 // around them in shared memory, one warp per (y, z) row at a time.  Every row of a stage is

@@ -37,7 +37,7 @@ def vcycle(helm, dim, n, r, tb=0.3, k=None, phi=None, **kw):
 
 
 @pytest.mark.parametrize("dim,n,s", [(2, 23, 3), (2, 27, 3), (2, 39, 3), (2, 47, 4), (2, 55, 2), (2, 71, 1), (2, 87, 3),
-                                     (2, 143, 3), (2, 223, 4), (2, 319, 3), (2, 1279, 2), (3, 9, 3), (3, 11, 4),
+                                     (2, 143, 3), (2, 223, 4), (2, 319, 3), (2, 639, 3), (2, 703, 1), (2, 895, 3), (2, 1279, 2), (3, 9, 3), (3, 11, 4),
                                      (3, 19, 3), (3, 23, 2), (3, 39, 1), (3, 47, 4), (3, 79, 3), (3, 79, 2), (3, 95, 3),
                                      (3, 95, 4), (3, 159, 3)])
 def test_sizes_at_region_edges(helm, dim, n, s):
