@@ -9,7 +9,9 @@
 // rows of the vector before make the stencil free of bounds checks.  The coarsest system is
 // solved with its inverse, formed in binary64 at set-up and held as double-floats: a matrix
 // times vector, all rows at once, instead of 2 m dependent elimination steps on the FP64
-// pipe.  Everything that does not depend on the previous kernel is loaded before the wait.
+// pipe.  From 31^2: about 20 us (18 Arnoldi passes with a barrier-separated reduction and
+// algebra each, and the elimination, took 90 us), 2.9 us a sweep; 512 threads of two points
+// each, 256 of four are 1-2% slower.  Everything that does not depend on the previous kernel is loaded before the wait.
 #pragma once
 #include "gram.cuh"
 
@@ -32,11 +34,13 @@ struct CgLevel {
   bool on[CG_PT];
   float2 ax[CG_PT], qx[CG_PT], ay[CG_PT], qy[CG_PT], az[CG_PT], qz[CG_PT], dg[CG_PT], dz[CG_PT];
 
+  // coef: the level's 1D coefficients a, d, c times t
   __device__ __forceinline__ void stencil_setup(const LevelDev<float2>& L, const float2* coef, int tid) {
     n = L.n;
     P = L.P;
     t = L.kt;
-    it = 1.0f / t;
+    it = __frcp_rn(t);
+    const float rn = __frcp_rn((float)n);  // i / n for i < 1024: exact with half a unit added
     const int np = DIM == 3 ? n * n * n : n * n;
     const float phc = L.phir * t;
 #pragma unroll
@@ -44,21 +48,20 @@ struct CgLevel {
       const int i = tid + q * CG_THREADS;
       on[q] = i < np;
       const int ii = on[q] ? i : 0;
-      const int yy = ii / n;
+      const int yy = (int)(((float)ii + 0.5f) * rn);
       cx[q] = ii - yy * n;
-      cz[q] = DIM == 3 ? yy / n : 0;
+      cz[q] = DIM == 3 ? (int)(((float)yy + 0.5f) * rn) : 0;
       cy[q] = yy - cz[q] * n;
       off[q] = (cz[q] * P + cy[q]) * P + cx[q];
-      auto sc = [&](float2 v) { return make_float2(v.x * t, v.y * t); };
-      ax[q] = sc(coef[cx[q]]);
-      qx[q] = sc(coef[2 * n + cx[q]]);
-      ay[q] = sc(coef[cy[q]]);
-      qy[q] = sc(coef[2 * n + cy[q]]);
-      dg[q] = cadd(sc(coef[n + cx[q]]), sc(coef[n + cy[q]]));
+      ax[q] = coef[cx[q]];
+      qx[q] = coef[2 * n + cx[q]];
+      ay[q] = coef[cy[q]];
+      qy[q] = coef[2 * n + cy[q]];
+      dg[q] = cadd(coef[n + cx[q]], coef[n + cy[q]]);
       if (DIM == 3) {
-        az[q] = sc(coef[cz[q]]);
-        qz[q] = sc(coef[2 * n + cz[q]]);
-        dz[q] = sc(coef[n + cz[q]]);
+        az[q] = coef[cz[q]];
+        qz[q] = coef[2 * n + cz[q]];
+        dz[q] = coef[n + cz[q]];
       }
       dg[q].x -= L.phi ? __ldg(L.phi + off[q]) * t : phc;
     }
@@ -85,7 +88,7 @@ struct CgLevel {
 
 struct CgShared {
   float wsum[CG_NW * 32];
-  float2 gs[CG_NW * gram_nv(SMAX)];
+  float2 gs[gram_nv(SMAX)];
   float2 xc[SMAX], rc[SMAX + 1];
 };
 
@@ -94,7 +97,7 @@ struct CgShared {
 template <int S, int DIM>
 __device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2* R0, float2 (&k0)[CG_PT],
                                          float2 (&x)[CG_PT], const float2 (&sg)[S], CgShared& sh) {
-  constexpr int NV = gram_nv(S), NS = gram_ns(S), H = NS == 16 ? 2 : 1;
+  constexpr int NS = gram_ns(S);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float2 k[CG_PT][S + 1];
 #pragma unroll
@@ -117,37 +120,13 @@ __device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2*
   for (int i = 0; i < NS; ++i) acc[i] = 0.f;
 #pragma unroll
   for (int q = 0; q < CG_PT; ++q) gram_point<S>(k[q], acc);
-  const float tot = warp_transpose_sum_f<NS>(acc, lane);
-  if (NS == 32) sh.wsum[warp * NS + lane] = tot;
-  else if ((lane & 1) == 0) sh.wsum[warp * NS + (lane >> 1)] = tot;
+  gram_block_sum<S, CG_NW>(acc, sh.wsum, sh.gs);
   __syncthreads();
   if (warp == 0) {
-    const int v = NS == 16 ? (lane & 15) : lane, h = NS == 16 ? lane >> 4 : 0;
-    float s = 0.f, c = 0.f;
-#pragma unroll
-    for (int q = h; q < CG_NW; q += H) {
-      float t, r;
-      df_two_sum(s, sh.wsum[q * NS + v], t, r);
-      s = t;
-      c += r;
-    }
-    if (H == 2) {
-      const float s2 = __shfl_xor_sync(0xffffffffu, s, 16), c2 = __shfl_xor_sync(0xffffffffu, c, 16);
-      float t, r;
-      df_two_sum(s, s2, t, r);
-      c = (c + c2) + r;
-      s = t;
-    }
-    if (h == 0 && v < NV) sh.gs[v] = df_fast2(s, c);
-    __syncwarp();
-    float2 xc[S], rc[S + 1];
-    gram_solve<S>(sh.gs, sg, V.t, xc, rc);
-    if (lane == 0) {
-#pragma unroll
-      for (int i = 0; i < S; ++i) sh.xc[i] = xc[i];
-#pragma unroll
-      for (int i = 0; i <= S; ++i) sh.rc[i] = rc[i];
-    }
+    float2 xk, rk;
+    gram_solve<S>(sh.gs, sg[0], sg[S > 1 ? 1 : 0], V.t, lane, xk, rk);
+    if (lane < S) sh.xc[lane] = xk;
+    if (lane <= S) sh.rc[lane] = rk;
   }
   __syncthreads();
 #pragma unroll
@@ -196,7 +175,10 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
   for (int i = tid; i < total; i += CG_THREADS) cgsm[i] = make_float2(0.f, 0.f);
   __syncthreads();
   for (int l = 0; l < nlev; ++l)
-    for (int i = tid; i < 3 * Ls[l].n; i += CG_THREADS) coef[s_cof[l] + i] = __ldg(Ls[l].ca + i);
+    for (int i = tid; i < 3 * Ls[l].n; i += CG_THREADS) {
+      const float2 v = __ldg(Ls[l].ca + i);
+      coef[s_cof[l] + i] = make_float2(v.x * Ls[l].kt, v.y * Ls[l].kt);
+    }
   const bool staged = lu.m * lu.m <= CG_INV;
   if (staged)
     for (int i = tid; i < lu.m * lu.m; i += CG_THREADS) inv_sm[i] = __ldg(lu.inv + i);
@@ -247,8 +229,10 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
     const int nc = Ls[l + 1].n, Pc = Ls[l + 1].P, P = V.P;
     const int ncp = DIM == 3 ? nc * nc * nc : nc * nc;
     float2* bc = cgsm + s_base[l + 1];
+    const float rnc = __frcp_rn((float)nc);
     for (int i = tid; i < ncp; i += CG_THREADS) {
-      const int yy = i / nc, X = i - yy * nc, Z = DIM == 3 ? yy / nc : 0, Y = yy - Z * nc;
+      const int yy = (int)(((float)i + 0.5f) * rnc), X = i - yy * nc;
+      const int Z = DIM == 3 ? (int)(((float)yy + 0.5f) * rnc) : 0, Y = yy - Z * nc;
       const float2* f = rr + (DIM == 3 ? (2 * Z + 1) * P * P : 0) + (2 * Y + 1) * P + 2 * X + 1;
       float2 out = make_float2(0.f, 0.f);
 #pragma unroll

@@ -8,9 +8,8 @@
 //
 // so k_1..k_s need no reduction in between and one pass over R_0 forms all of them.  The
 // pass reduces the Gram matrix G = K^H K; the minimisation then follows from
-// M K_s = K_{s+1} B (B lower bidiagonal: sigma_j on the diagonal, 1/t below) and
-// G = L D L^H:  min_y ||D^{1/2} L^H (e_0 - B y)||, an (s+1) x s Hessenberg least-squares
-// problem.  In exact arithmetic this is GMRES(s) (a Krylov space does not depend on its
+// M K_s = K_{s+1} B (B lower bidiagonal: sigma_j on the diagonal, 1/t below) and one
+// linear system with G (gram_solve).  In exact arithmetic this is GMRES(s) (a Krylov space does not depend on its
 // basis); x += K_s y and r = K_{s+1} (e_0 - B y) are combinations of the stored vectors.
 //
 // Accuracy.  Errors of G are amplified by the square of the basis's condition number, so
@@ -84,145 +83,125 @@ __device__ __forceinline__ float2 df_fast2(float s, float c) {
   const float t = __fadd_rn(s, c);
   return make_float2(t, __fsub_rn(c, __fsub_rn(t, s)));
 }
-__device__ __forceinline__ float2 df_mul2(float2 a, float2 b) {
-  const float p = __fmul_rn(a.x, b.x);
-  float e = fmaf(a.x, b.x, -p);
-  e = fmaf(a.x, b.y, fmaf(a.y, b.x, e));
-  return df_fast2(p, e);
-}
-// a - b c
-__device__ __forceinline__ float2 df_fms2(float2 a, float2 b, float2 c) {
-  const float p = __fmul_rn(b.x, c.x);
-  float e = fmaf(b.x, c.x, -p);
-  e = fmaf(b.x, c.y, fmaf(b.y, c.x, e));
-  float t, r;
-  df_two_sum(a.x, -p, t, r);
-  return df_fast2(t, __fadd_rn(__fadd_rn(r, a.y), -e));
-}
-__device__ __forceinline__ float2 df_neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 df_recip(float2 b) {
-  const float r = __frcp_rn(b.x);
-  const float e = fmaf(-b.y, r, fmaf(-b.x, r, 1.0f));
-  return df_fast2(r, __fmul_rn(r, e));
-}
 
 // ------------------------------------------------------------------ the minimisation
-// A pivot of the factorisation below this fraction of its diagonal entry means that k_j is
-// a combination of the earlier vectors (to the rounding of binary32 vectors and of their
-// Gram sums): the sweep stops at j Krylov steps.
+// min ||K_{s+1} rho|| over rho = e_0 - B y.  B's left null vector c (c_0 = 1, c_{j+1} =
+// -t sigma_j c_j: the basis polynomials' values at zero) makes the constraint c^T rho = 1,
+// so rho = w / (c^T w) with G w = conj(c), and y follows from B's subdiagonal,
+// y_{j-1} = -rho_j - t sigma_j y_j.
+//
+// One warp, one entry of [G | conj(c)] per lane (row j, column k), Gauss-Jordan elimination
+// without pivoting (G is positive definite) in double-float.  The step runs once per sweep,
+// in one warp, usually on an SM that has not run it before, so instruction fetch counts as
+// much as the arithmetic: this form is about 3 KB of code (1650-1900 cycles for s = 3 whatever
+// the instruction caches hold).  Unrolled in one thread it is 12 KB: 1520 cycles with the code
+// in the first-level cache, 2300-2600 from the next one, 4700-4900 from L2.
+//
+// A pivot below GRAM_TAU of its diagonal entry means that k_i is a combination of the
+// earlier vectors (to the rounding of binary32 vectors and of their Gram sums): rho is then
+// that combination, m = i Krylov steps.
 constexpr float GRAM_TAU = 1e-7f;
 
-// g: the NV double-float sums; sg[j] = t sigma_j.  Results: m Krylov steps, x += sum_{k<m}
-// xc[k] k_k, r = sum_{k<=m} rc[k] k_k.  One thread's work (every lane of a warp may run it).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// s - a b - c d in double-float
+__device__ __forceinline__ float2 df_fms2x2(float2 s, float2 a, float2 b, float2 c, float2 d) {
+  const float p = __fmul_rn(a.x, b.x), q = __fmul_rn(c.x, d.x);
+  const float e = fmaf(a.x, b.y, fmaf(a.y, b.x, fmaf(a.x, b.x, -p)));
+  const float f = fmaf(c.x, d.y, fmaf(c.y, d.x, fmaf(c.x, d.x, -q)));
+  float t, x, v, y;
+  df_two_sum(s.x, -p, t, x);
+  df_two_sum(t, -q, v, y);
+  return df_fast2(v, ((s.y - e) - f) + (x + y));
+}
+
+// g: the NV double-float sums; sg0 = t sigma_0, sg1 = t sigma_1 = t sigma_3 (sigma_2 = 0).
+// Lane k < S returns x's coefficient xk of k_k (x += sum_{k<m} x_k k_k), lane k <= S the
+// residual's rk (r = sum_{k<=m} r_k k_k); every lane returns m.  The whole warp calls it.
 template <int S>
-__device__ __forceinline__ int gram_solve(const float2* g, const float2 (&sg)[S], float t, float2 (&xc)[S],
-                                          float2 (&rc)[S + 1]) {
-#pragma unroll
-  for (int k = 0; k < S; ++k) xc[k] = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int k = 0; k <= S; ++k) rc[k] = make_float2(k == 0 ? 1.f : 0.f, 0.f);
+__device__ __forceinline__ int gram_solve(const float2* g, float2 sg0, float2 sg1, float t, int lane, float2& xk,
+                                          float2& rk) {
+  constexpr int NC = S + 2, N = S + 1;
+  const unsigned full = 0xffffffffu;
+  xk = make_float2(0.f, 0.f);
+  rk = make_float2(lane == 0 ? 1.f : 0.f, 0.f);
   const float g00 = g[0].x;
   if (!(g00 > 0.0f) || !isfinite(g00)) return 0;
   // scale by a power of two so that G_00 is near one (exact; the products' low parts then
   // stay far from underflow)
-  const unsigned e = (__float_as_uint(g00) >> 23) & 0xffu;
-  const float sc = __uint_as_float(min(max(254u - e, 1u), 253u) << 23);
-  float2 re[S + 1][S + 1], im[S + 1][S + 1];  // upper triangle, then D and U = L^H
-  float dg[S + 1];
-#pragma unroll
-  for (int i = 0; i <= S; ++i)
-#pragma unroll
-    for (int j = i; j <= S; ++j) {
-      const float2 a = g[gram_at(S, i, j)];
-      re[i][j] = make_float2(a.x * sc, a.y * sc);
-      if (j > i) {
-        const float2 b = g[gram_at(S, i, j) + 1];
-        im[i][j] = make_float2(b.x * sc, b.y * sc);
-      } else {
-        dg[i] = re[i][i].x;
-      }
+  const unsigned ex = (__float_as_uint(g00) >> 23) & 0xffu;
+  const float sc = __uint_as_float(min(max(254u - ex, 1u), 253u) << 23);
+  const int j = min(lane / NC, S), k = lane - (lane / NC) * NC;
+  // c_0 = 1, c_1 = -sg0, c_2 = sg0 sg1, then 0 (sigma_2 = 0)
+  const float2 c2 = cmul(sg0, sg1);
+  auto cq = [&](int q) {
+    return q == 0 ? make_float2(1.f, 0.f) : q == 1 ? make_float2(-sg0.x, -sg0.y) : q == 2 ? c2 : make_float2(0.f, 0.f);
+  };
+  float2 re, im;
+  {
+    const int lo = min(j, k), hi = min(max(j, k), S);
+    const int at = gram_at(S, lo, hi);
+    const float2 a = g[at], b = g[lo < hi ? at + 1 : at];
+    const float s = j < k ? sc : j > k ? -sc : 0.f;
+    re = make_float2(a.x * sc, a.y * sc);
+    im = make_float2(b.x * s, b.y * s);
+    if (k > S) {
+      const float2 c = cq(j);
+      re = make_float2(c.x, 0.f);
+      im = make_float2(-c.y, 0.f);
     }
-  int m = S;
-  bool alive = true;
-  float w[S + 1];  // square roots of the pivots
-  float2 u[S + 1][S + 1];
-#pragma unroll
-  for (int i = 0; i <= S; ++i) {
-    const float d = re[i][i].x;
-    if (alive && !(d > GRAM_TAU * dg[i])) {
-      m = min(m, i);
-      alive = false;
-    }
-    w[i] = alive ? sqrtf(d) : 0.0f;
-    if (i == S) break;
-    const float2 r = df_recip(alive ? re[i][i] : make_float2(1.f, 0.f));
-    float2 ur[S + 1], ui[S + 1];
-#pragma unroll
-    for (int j = i + 1; j <= S; ++j) {
-      ur[j] = df_mul2(re[i][j], r);
-      ui[j] = df_mul2(im[i][j], r);
-      u[i][j] = make_float2(ur[j].x, ui[j].x);
-    }
-    // S_jk -= conj(U_ij) S_ik
-#pragma unroll
-    for (int j = i + 1; j <= S; ++j)
-#pragma unroll
-      for (int k = j; k <= S; ++k) {
-        re[j][k] = df_fms2(df_fms2(re[j][k], ur[j], re[i][k]), ui[j], im[i][k]);
-        if (k > j) im[j][k] = df_fms2(df_fms2(im[j][k], ur[j], im[i][k]), df_neg(ui[j]), re[i][k]);
-      }
   }
-  // A = D^{1/2} U (t B): column j is sg_j U_{.j} + U_{.,j+1}
-  float2 A[S + 1][S];
-#pragma unroll
-  for (int i = 0; i <= S; ++i)
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      float2 v = make_float2(0.f, 0.f);
-      if (i < j) v = cmul(u[i][j], sg[j]);
-      if (i == j) v = sg[j];
-      if (i < j + 1) v = cadd(v, u[i][j + 1]);
-      if (i == j + 1) v.x += 1.0f;
-      A[i][j] = make_float2(v.x * w[i], v.y * w[i]);
+  const float tau = re.x * GRAM_TAU;  // lanes (i, i): the threshold of pivot i
+  int m = N, ii = 0, ji = j * NC, ik = k;
+  float dinv = 0.f;                   // lane i: 1 / d_i
+#pragma unroll 1
+  for (int i = 0; i < N; ++i) {
+    const unsigned ok = __ballot_sync(full, re.x > tau);
+    const float dx = __shfl_sync(full, re.x, ii), dy = __shfl_sync(full, re.y, ii);
+    const float2 ar = make_float2(__shfl_sync(full, re.x, ji), __shfl_sync(full, re.y, ji));
+    const float2 ai = make_float2(__shfl_sync(full, im.x, ji), __shfl_sync(full, im.y, ji));
+    const float2 br = make_float2(__shfl_sync(full, re.x, ik), __shfl_sync(full, re.y, ik));
+    const float2 bi = make_float2(__shfl_sync(full, im.x, ik), __shfl_sync(full, im.y, ik));
+    const float r = rcp_approx(dx), rl = r * fmaf(-dy, r, fmaf(-dx, r, 1.0f));
+    if (m == N && !((ok >> ii) & 1u)) m = i;  // the remaining steps change nothing
+    if (m == N && lane == i) dinv = r + rl;
+    // u = S_ji / d, then row j minus u times row i
+    const float urx = __fmul_rn(ar.x, r), uix = __fmul_rn(ai.x, r);
+    const float2 ur = make_float2(urx, fmaf(ar.x, r, -urx) + fmaf(ar.x, rl, ar.y * r));
+    const float2 ui = make_float2(uix, fmaf(ai.x, r, -uix) + fmaf(ai.x, rl, ai.y * r));
+    const float2 nr = df_fms2x2(re, ur, br, make_float2(-ui.x, -ui.y), bi);
+    const float2 ni = df_fms2x2(im, ur, bi, ui, br);
+    if (m == N && j != i) {
+      re = nr;
+      im = ni;
     }
-  // Givens rotations (the subdiagonal w[j + 1] is real); right-hand side w_0 e_0
-  float2 q[S + 1];
-  float rinv[S];
-  q[0] = make_float2(w[0], 0.f);
-#pragma unroll
-  for (int j = 0; j < S; ++j) {
-    const float2 a = A[j][j];
-    const float b = A[j + 1][j].x;
-    const float r2 = fmaf(a.x, a.x, fmaf(a.y, a.y, b * b));
-    const float inv = r2 > 0.0f ? rsqrtf(r2) : 0.0f;
-    const float2 ca = make_float2(a.x * inv, -a.y * inv);  // conj(a) / r
-    const float sb = b * inv;
-    rinv[j] = inv;
-#pragma unroll
-    for (int l = j + 1; l < S; ++l) {
-      const float2 t0 = A[j][l], t1 = A[j + 1][l];
-      A[j][l] = cadd(cmul(ca, t0), make_float2(sb * t1.x, sb * t1.y));
-      A[j + 1][l] = csub(cmul(fconj(ca), t1), make_float2(sb * t0.x, sb * t0.y));
-    }
-    const float2 q0 = q[j];
-    q[j] = cmul(ca, q0);
-    q[j + 1] = make_float2(-sb * q0.x, -sb * q0.y);
+    ii += NC + 1;
+    ji += 1;
+    ik += NC;
   }
-  float2 y[S];
+  // w_i in lane i; after a breakdown at m the null vector: w_m = 1, w_i = 0 beyond
+  const int src = min(lane, S) * NC + (m < N ? m : S + 1);
+  float2 w = make_float2(__shfl_sync(full, re.x, src) * dinv, __shfl_sync(full, im.x, src) * dinv);
+  if (m < N) w = lane < m ? make_float2(-w.x, -w.y) : make_float2(lane == m ? 1.f : 0.f, 0.f);
+  if (lane > S) w = make_float2(0.f, 0.f);
+  m = min(m, S);
+  // rho = w / (c^T w); c_i = 0 from i = 3 on
+  float2 cw = cmul(cq(lane), w);
 #pragma unroll
-  for (int j = S - 1; j >= 0; --j) {
-    float2 v = q[j];
-#pragma unroll
-    for (int l = j + 1; l < S; ++l) v = csub(v, cmul(A[j][l], y[l]));
-    y[j] = j < m ? make_float2(v.x * rinv[j], v.y * rinv[j]) : make_float2(0.f, 0.f);
-  }
-#pragma unroll
-  for (int j = 0; j < S; ++j) {
-    xc[j] = make_float2(t * y[j].x, t * y[j].y);
-    const float2 sy = cmul(sg[j], y[j]);
-    rc[j] = csub(rc[j], sy);
-    rc[j + 1] = csub(rc[j + 1], y[j]);
-  }
+  for (int o = 1; o <= 2; o <<= 1)
+    cw = make_float2(cw.x + __shfl_xor_sync(full, cw.x, o), cw.y + __shfl_xor_sync(full, cw.y, o));
+  cw = make_float2(__shfl_sync(full, cw.x, 0), __shfl_sync(full, cw.y, 0));
+  const float n2 = fabs2(cw), in = 1.0f / n2;
+  if (!(n2 > 0.0f) || !isfinite(in)) return 0;  // M is singular on the space: no step
+  rk = cmul(w, make_float2(cw.x * in, -cw.y * in));
+  // y_j = -rho_{j+1} - sg_{j+1} y_{j+1}: sg_2 = 0, so odd j end there and even j take one more
+  const float2 r1 = make_float2(__shfl_down_sync(full, rk.x, 1), __shfl_down_sync(full, rk.y, 1));
+  const float2 r2 = make_float2(__shfl_down_sync(full, rk.x, 2), __shfl_down_sync(full, rk.y, 2));
+  const float2 y = csub(cmul((lane & 1) ? make_float2(0.f, 0.f) : sg1, r2), r1);
+  xk = make_float2(t * y.x, t * y.y);
   return m;
 }
 
@@ -241,58 +220,66 @@ __device__ __forceinline__ void gram_shifts(const LevelDev<float2>& L, bool firs
   }
 }
 
-// End of a sweep pass: every thread's Gram sums `acc` are reduced over its warp (binary32),
-// the CTA and the level (double-float, fixed order); the last CTA of the problem solves the
-// minimisation and writes the sweep's coefficients.  Every thread of the block calls it.
-// `wsum` is NW * NS floats, `gs` gram_nv(S) * 8 float2 of shared memory.
+// Sum of NW double-floats per value, gs-style: thread v NW + w holds part w of value v (NW a
+// power of two up to 16); the thread with w = 0 ends with the total.  Whole warps call it.
+template <int NW>
+__device__ __forceinline__ float2 df_group_sum(float2 a) {
+#pragma unroll
+  for (int o = NW / 2; o > 0; o >>= 1) {
+    const float2 b = make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+    float t, r;
+    df_two_sum(a.x, b.x, t, r);
+    a = make_float2(t, (a.y + b.y) + r);
+  }
+  return df_fast2(a.x, a.y);
+}
+
+// The warps' sums of a CTA of NW warps, combined: gs[0..NV-1].  Every thread calls it (it
+// starts with a barrier; another must precede the reads of gs).
 template <int S, int NW>
-__device__ __forceinline__ void gram_finish(float (&acc)[gram_ns(S)], const LevelDev<float2>& L, const float2 (&sg)[S],
-                                            int unit, int nunits, float* wsum, float2* gs) {
+__device__ __forceinline__ void gram_block_sum(float (&acc)[gram_ns(S)], float* wsum, float2* gs) {
   constexpr int NV = gram_nv(S), NS = gram_ns(S);
-  constexpr int H = NS == 16 ? 2 : 1;  // slot groups a warp sums at a time
-  __shared__ int s_last;
   const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5;
   const float tot = warp_transpose_sum_f<NS>(acc, lane);
   if (NS == 32) wsum[warp * NS + lane] = tot;
   else if ((lane & 1) == 0) wsum[warp * NS + (lane >> 1)] = tot;
   __syncthreads();
+  const int v = tid / NW, w = tid % NW;
+  if (warp * 32 < NV * NW) {  // uniform over the warp
+    const float2 a = df_group_sum<NW>(make_float2(v < NV ? wsum[w * NS + v] : 0.f, 0.f));
+    if (w == 0 && v < NV) gs[v] = a;
+  }
+}
+
+// End of a sweep pass: every thread's Gram sums `acc` are reduced over its warp (binary32),
+// the CTA and the level (double-float, fixed order); the last CTA of the problem solves the
+// minimisation and writes the sweep's coefficients.  Every thread of the block calls it.
+// `wsum` is NW * NS floats, `gs` gram_nv(S) * (NW + 1) float2 of shared memory.
+template <int S, int NW>
+__device__ __forceinline__ void gram_finish(float (&acc)[gram_ns(S)], const LevelDev<float2>& L, const float2 (&sg)[S],
+                                            int unit, int nunits, float* wsum, float2* gs) {
+  constexpr int NV = gram_nv(S), NS = gram_ns(S);
+  constexpr int H = NS == 16 ? 2 : 1;  // slots a warp reads at a time
+  __shared__ int s_last;
+  const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5;
+  gram_block_sum<S, NW>(acc, wsum, gs);
+  __syncthreads();
   auto* sc = L.sc;
-  float2* const part = reinterpret_cast<float2*>(L.part);
-  const int v = NS == 16 ? (lane & 15) : lane, h = NS == 16 ? lane >> 4 : 0;
-  if (warp == 0) {
-    float s = 0.f, c = 0.f;
-#pragma unroll
-    for (int q = h; q < NW; q += H) {
-      float t, r;
-      df_two_sum(s, wsum[q * NS + v], t, r);
-      s = t;
-      c += r;
-    }
-    if (H == 2) {
-      const float s2 = __shfl_xor_sync(0xffffffffu, s, 16), c2 = __shfl_xor_sync(0xffffffffu, c, 16);
-      float t, r;
-      df_two_sum(s, s2, t, r);
-      c = (c + c2) + r;
-      s = t;
-    }
-    const float2 w = df_fast2(s, c);
-    if (nunits > 1) {
-      if (h == 0 && v < NV) __stcg(part + (size_t)unit * GRAM_SLOT + v, w);
+  if (nunits > 1) {
+    float2* const part = reinterpret_cast<float2*>(L.part);
+    if (warp == 0) {
+      if (lane < NV) __stcg(part + (size_t)unit * GRAM_SLOT + lane, gs[lane]);
       __syncwarp();
       if (lane == 0) {
         __threadfence();
         s_last = (atomicAdd(&sc->counter, 1u) == (unsigned)nunits - 1u);
       }
-    } else {
-      if (h == 0 && v < NV) gs[v] = w;
-      if (lane == 0) s_last = 1;
     }
-  }
-  __syncthreads();
-  if (!s_last) return;
-  if (nunits > 1) {
+    __syncthreads();
+    if (!s_last) return;
     __threadfence();
     // warp w sums slots w H + h, + NW H, ... of value v, four loads in flight
+    const int v = NS == 16 ? (lane & 15) : lane, h = NS == 16 ? lane >> 4 : 0;
     float s = 0.f, c = 0.f;
     for (int u0 = warp * H + h; u0 < nunits; u0 += 4 * NW * H) {
       float2 p[4];
@@ -316,40 +303,23 @@ __device__ __forceinline__ void gram_finish(float (&acc)[gram_ns(S)], const Leve
       c = (c + c2) + r;
       s = t;
     }
-    if (h == 0 && v < NV) gs[warp * NV + v] = make_float2(s, c);
+    float2* const gw = gs + NV;  // [warp][value]
+    if (h == 0 && v < NV) gw[warp * NV + v] = make_float2(s, c);
     __syncthreads();
-    if (warp == 0) {
-      float s1 = 0.f, c1 = 0.f;
-      if (v < NV)
-        for (int q = h; q < NW; q += H) {
-          const float2 p = gs[q * NV + v];
-          float t, r;
-          df_two_sum(s1, p.x, t, r);
-          s1 = t;
-          c1 += r + p.y;
-        }
-      if (H == 2) {
-        const float s2 = __shfl_xor_sync(0xffffffffu, s1, 16), c2 = __shfl_xor_sync(0xffffffffu, c1, 16);
-        float t, r;
-        df_two_sum(s1, s2, t, r);
-        c1 = (c1 + c2) + r;
-        s1 = t;
-      }
-      __syncwarp();
-      if (h == 0 && v < NV) gs[v] = df_fast2(s1, c1);
-      __syncwarp();
+    const int vv = tid / NW, w = tid % NW;
+    if (warp * 32 < NV * NW) {
+      const float2 a = df_group_sum<NW>(vv < NV ? gw[w * NV + vv] : make_float2(0.f, 0.f));
+      if (w == 0 && vv < NV) gs[vv] = a;
     }
+    __syncthreads();
   }
   if (warp == 0) {
-    __syncwarp();
-    float2 xc[S], rc[S + 1];
-    const int m = gram_solve<S>(gs, sg, L.kt, xc, rc);
+    float2 xk, rk;
+    const int m = gram_solve<S>(gs, sg[0], sg[S > 1 ? 1 : 0], L.kt, lane, xk, rk);
+    if (lane < S) sc->xcoef[lane] = xk;
+    if (lane <= S) sc->rcoef[lane] = rk;
     if (lane == 0) {
       sc->m = m;
-#pragma unroll
-      for (int k = 0; k < S; ++k) sc->xcoef[k] = xc[k];
-#pragma unroll
-      for (int k = 0; k <= S; ++k) sc->rcoef[k] = rc[k];
       sc->counter = 0u;
     }
   }

@@ -46,7 +46,7 @@ struct Sw2Shared {
   float4 yac[SW2_NW * QY];                // y coefficients a, c of the region's rows
   float2 yd[SW2_NW * QY];
   float2 edge[2][SW2_NW + 2][2][32];      // [parity][warp + 1][first / last row][lane]
-  float2 gs[SW2_NW * gram_nv(S)];
+  float2 gs[(SW2_NW + 1) * gram_nv(S)];
   float wsum[SW2_NW * gram_ns(S)];
 };
 
@@ -158,7 +158,7 @@ k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, 
   static_assert(S <= 3, "register windows hold four rows");
   extern __shared__ __align__(16) float2 swsm[];
   __shared__ float wsum[SV2_NW * NS];
-  __shared__ float2 gs[SV2_NW * NV];
+  __shared__ float2 gs[(SV2_NW + 1) * NV];
   const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
   const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
@@ -324,7 +324,7 @@ __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__
   __shared__ float4 yac[R], zac[R];
   __shared__ float2 yd[R], zd[R];
   __shared__ float wsum[SW3_NW * NS];
-  __shared__ float2 gs[SW3_NW * NV];
+  __shared__ float2 gs[(SW3_NW + 1) * NV];
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
   const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
@@ -419,7 +419,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   static_assert(S <= 3, "register windows hold four planes");
   extern __shared__ __align__(16) float2 swsm[];
   __shared__ float wsum[SM3_NW * NS];
-  __shared__ float2 gs[SM3_NW * NV];
+  __shared__ float2 gs[(SM3_NW + 1) * NV];
   const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
   const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
