@@ -118,7 +118,7 @@ int autotune(const helm_grid* grid, const float* phi, double k, double theta_bet
   CUDA_TRY(cudaMemcpy(r, hr.data(), npts * sizeof(float2), cudaMemcpyHostToDevice));
 
   // the choices of this hierarchy's grid-wide levels
-  const int thr = dim == 2 ? 31 : 7;
+  const int thr = coarse_threshold(dim, h->prec);
   std::vector<Knob> knobs;
   for (const HostLevel& L : h->lev) {
     if (L.n <= thr) continue;

@@ -175,11 +175,56 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, in
 __device__ __forceinline__ int flat_tid() { return threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z); }
 __device__ __forceinline__ int block_threads() { return blockDim.x * blockDim.y * blockDim.z; }
 
-// Sum NV doubles over the block in a fixed order; thread 0 ends with the totals.
-// `sm` needs 32 * NV doubles.  Every thread of the block must call it.
+// Values a transposed sum carries: NV padded to a power of two.
+HELM_HD constexpr int sum_vp(int NV) { return NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : NV <= 8 ? 8 : 16; }
+
+// Totals of nw rows of VP binary64 values in shared memory (row w: warp w's sums), by warp 0:
+// lane l adds the rows l / VP, l / VP + 32 / VP, ... of value l % VP, then lanes are combined.
+// Thread 0 ends with all NV totals.
+template <int NV>
+__device__ __forceinline__ void warp_rows_total(const double* sm, int nw, double (&tot)[NV]) {
+  constexpr int VP = sum_vp(NV), G = 32 / VP;
+  const int lane = flat_tid() & 31, g = lane / VP;
+  double s = g < nw ? sm[lane] : 0.0;
+  for (int w = g + G; w < nw; w += G) s += sm[w * VP + (lane % VP)];
+#pragma unroll
+  for (int o = VP; o < 32; o <<= 1)
+    if (o / VP < nw) s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) tot[i] = __shfl_sync(0xffffffffu, s, i);
+}
+
+// Sum NV values over the block in a fixed order; thread 0 ends with the totals.
+// `sm` needs 32 * NV values.  Every thread of the block must call it.
 template <int NV, typename T>
 __device__ __forceinline__ void block_sum(T (&v)[NV], T* sm) {
   const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5, nw = (block_threads() + 31) >> 5;
+  if constexpr (sizeof(T) == 8) {
+    // binary64: an addition occupies the FP64 pipe for 64 cycles whatever the lanes do, so
+    // the warp halves the values kept at every butterfly (VP - 1 + 5 - log2 VP additions,
+    // 9 for seven values, instead of 5 NV = 35) and the cross-warp sum takes four more
+    constexpr int VP = sum_vp(NV);
+    double a[VP];
+#pragma unroll
+    for (int i = 0; i < VP; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : 0.0;
+    int o = 16;
+#pragma unroll
+    for (int c = VP / 2; c >= 1; c >>= 1, o >>= 1) {
+      const bool hi = lane & o;
+#pragma unroll
+      for (int k = 0; k < c; ++k) {
+        const double send = hi ? a[k] : a[k + c], keep = hi ? a[k + c] : a[k];
+        a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+#pragma unroll
+    for (int q = 16 / VP; q >= 1; q >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], q);
+    if ((lane & (32 / VP - 1)) == 0) sm[warp * VP + lane / (32 / VP)] = a[0];
+    __syncthreads();
+    if (warp == 0) warp_rows_total<NV>(sm, nw, v);
+    __syncthreads();
+    return;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -221,6 +266,38 @@ __device__ __forceinline__ void sum_partials(const T* part, int ntiles, T (&acc)
   }
 }
 
+// Totals of `ntiles` partial slots of NV values each in a fixed order, left with thread 0.
+// binary64: value t % VP of slots t / VP, t / VP + threads / VP, ... per thread.
+template <int NV, typename T>
+__device__ __forceinline__ void slots_total(const T* part, int ntiles, T (&acc)[NV], T* sm) {
+  if constexpr (sizeof(T) == 8) {
+    constexpr int VP = sum_vp(NV);
+    const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5, nt = block_threads();
+    const int v = tid % VP, G = nt / VP;
+    double s = 0.0;
+    for (int t0 = tid / VP; t0 < ntiles; t0 += 4 * G) {
+      double x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int t = t0 + u * G;
+        x[u] = (t < ntiles && v < NV) ? __ldcg(part + (size_t)t * NPART + v) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (t0 + u * G < ntiles) s += x[u];
+    }
+#pragma unroll
+    for (int o = VP; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < VP) sm[warp * VP + lane] = s;
+    __syncthreads();
+    if (warp == 0) warp_rows_total<NV>(sm, (nt + 31) >> 5, acc);
+    __syncthreads();
+  } else {
+    sum_partials<NV, T>(part, ntiles, acc);
+    block_sum<NV, T>(acc, sm);
+  }
+}
+
 // Write this block's NV partial sums to slot `tile`, then report whether this block
 // is the last of `ntiles` blocks of its problem to arrive.  If so, the returned
 // block reduces all slots in a fixed order (independent of arrival order) and
@@ -245,8 +322,7 @@ __device__ __forceinline__ bool grid_sum_last(T (&v)[NV], void* partv, int tile,
   if (!s_last) return false;
   __threadfence();
   T acc[NV];
-  sum_partials<NV, T>(part, ntiles, acc);
-  block_sum<NV, T>(acc, sm);
+  slots_total<NV, T>(part, ntiles, acc, sm);
 #pragma unroll
   for (int i = 0; i < NV; ++i) tot[i] = acc[i];
   if (tid == 0) *counter = 0u;
@@ -269,6 +345,8 @@ __device__ __forceinline__ float2 fdiv(float2 a, float2 b) {
   return make_float2((a.x * b.x + a.y * b.y) * d, (a.y * b.x - a.x * b.y) * d);
 }
 __device__ __forceinline__ double2 fdiv(double2 a, double2 b) { return ddiv(a, b); }
+__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 
 template <typename T>
 __device__ __forceinline__ int sweep_words() {
@@ -293,86 +371,20 @@ __device__ inline void sweep_begin(SweepScalarsT<T>* sc, T beta2, int s) {
     return;
   }
   sc->m = s;
-  sc->Cf[1][0] = CT<CR>::make((T)1 / sqrt(beta2), 0);
+  sc->z[0] = CT<CR>::make(1, 0);
+  sc->Cf[1][0] = CT<CR>::make(rsqrt_t(beta2), 0);
 }
 
 // The sweep algebra works on register copies: every field it reads is loaded before
 // anything is computed (one memory latency instead of a chain), and the results are
 // stored at the end.
 
-// min || beta e1 - Hbar y || for the (M+1) x M Hessenberg matrix hh, complex Givens.
-// M is a compile-time constant so every array stays in registers.
-template <typename T, int M>
-__device__ __forceinline__ void sweep_lstsq(const typename CplxOf<T>::T (&hh)[SMAX + 1][SMAX], T beta,
-                                            typename CplxOf<T>::T* y) {
-  typedef typename CplxOf<T>::T CR;
-  CR R[M + 1][M];
-  CR g[M + 1];
-#pragma unroll
-  for (int i = 0; i <= M; ++i) {
-    g[i] = CT<CR>::make(i == 0 ? beta : (T)0, 0);
-#pragma unroll
-    for (int j = 0; j < M; ++j) R[i][j] = (i <= j + 1) ? hh[i][j] : CT<CR>::make(0, 0);
-  }
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    const CR a = R[j][j], b = R[j + 1][j];
-    const T na = sqrt(fabs2(a)), nb = sqrt(fabs2(b));
-    const T r = sqrt(na * na + nb * nb);
-    T c;
-    CR s;
-    if (r == (T)0) { c = 1; s = CT<CR>::make(0, 0); }
-    else if (na == (T)0) { c = 0; s = CT<CR>::make(1, 0); }
-    else {
-      const T inv_na = (T)1 / na, inv_r = (T)1 / r;
-      c = na * inv_r;
-      s = cmul(CT<CR>::make(a.x * inv_na, a.y * inv_na), fconj(b));
-      s = CT<CR>::make(s.x * inv_r, s.y * inv_r);
-    }
-#pragma unroll
-    for (int l = j; l < M; ++l) {
-      const CR t0 = R[j][l], t1 = R[j + 1][l];
-      R[j][l] = cadd(CT<CR>::make(c * t0.x, c * t0.y), cmul(s, t1));
-      R[j + 1][l] = csub(CT<CR>::make(c * t1.x, c * t1.y), cmul(fconj(s), t0));
-    }
-    const CR g0 = g[j];
-    g[j] = CT<CR>::make(c * g0.x, c * g0.y);
-    g[j + 1] = cmul(CT<CR>::make(-s.x, s.y), g0);  // -conj(s) g0
-  }
-#pragma unroll
-  for (int j = M - 1; j >= 0; --j) {
-    CR acc = g[j];
-#pragma unroll
-    for (int l = j + 1; l < M; ++l) acc = csub(acc, cmul(R[j][l], y[l]));
-    y[j] = (fabs2(R[j][j]) > (T)0) ? fdiv(acc, R[j][j]) : CT<CR>::make(0, 0);
-  }
-}
-
-// Least-squares solution of the sweep and its update coefficients over the raw
-// vectors: x += sum_{k<M} xcoef[k] R_k, r = sum_{k<=M} rcoef[k] R_k.
-template <typename T, int M>
-__device__ __forceinline__ void sweep_finish(SweepScalarsT<T>* sc, const typename CplxOf<T>::T (&hh)[SMAX + 1][SMAX],
-                                             const typename CplxOf<T>::T (&cf)[SMAX + 1][SMAX], T beta2) {
-  typedef typename CplxOf<T>::T CR;
-  CR y[M];
-  sweep_lstsq<T, M>(hh, sqrt(beta2), y);
-  CR xc[SMAX + 1], rc[SMAX + 1];
-#pragma unroll
-  for (int k = 0; k <= SMAX; ++k) { xc[k] = CT<CR>::make(0, 0); rc[k] = CT<CR>::make(0, 0); }
-#pragma unroll
-  for (int k = 0; k < M; ++k) {
-    CR acc = CT<CR>::make(0, 0);
-#pragma unroll
-    for (int jj = k + 1; jj <= M; ++jj) acc = cadd(acc, cmul(y[jj - 1], cf[jj][k]));
-    xc[k] = acc;
-  }
-  rc[0] = CT<CR>::make(1, 0);
-#pragma unroll
-  for (int jj = 1; jj <= M; ++jj) rc[jj] = CT<CR>::make(-y[jj - 1].x, -y[jj - 1].y);
-  sc->m = M;
-#pragma unroll
-  for (int k = 0; k <= SMAX; ++k) { sc->xcoef[k] = xc[k]; sc->rcoef[k] = rc[k]; }
-}
+// The minimisation min ||beta e_1 - H y|| needs no rotations: the smallest residual is the
+// projection of beta e_1 onto H's left null vector z (z^H H = 0, z_0 = 1, grown by one entry
+// per column), rho = beta z / ||z||^2, and y follows from H's subdiagonal, last entry first.
+// No square root or quotient but 1 / h_{j+1,j} and 1 / ||z||^2 (in binary64 every instruction
+// of the one thread that runs this takes 64 cycles: about 110 of them for the third step,
+// 500 with Givens rotations).
 
 // After Arnoldi pass J: red[2k..2k+1] = <R_k, p_J> (k < J), red[2J] = ||p_J||^2.
 // Works on `sc` in any memory space (the kernels pass a shared-memory copy).
@@ -380,50 +392,95 @@ template <typename T, int J>
 __device__ __forceinline__ void sweep_after_pass(SweepScalarsT<T>* sc, const T* red) {
   typedef typename CplxOf<T>::T CR;
   // every field the algebra reads, loaded first
-  CR cf[SMAX + 1][SMAX], hh[SMAX + 1][SMAX];
+  CR cf[SMAX + 1][SMAX], hh[SMAX + 1][SMAX], z[SMAX + 1];
+  T inv[SMAX + 1];
 #pragma unroll
   for (int i = 1; i <= J; ++i)
 #pragma unroll
     for (int k = 0; k < i; ++k) cf[i][k] = sc->Cf[i][k];
 #pragma unroll
-  for (int j = 0; j + 1 < J; ++j)
+  for (int j = 0; j + 1 < J; ++j) {
+    inv[j] = sc->inv[j];
 #pragma unroll
-    for (int i = 0; i <= j + 1; ++i) hh[i][j] = sc->Hh[i][j];
+    for (int i = 1; i <= j + 1; ++i) hh[i][j] = sc->Hh[i][j];
+  }
+#pragma unroll
+  for (int i = 0; i < J; ++i) z[i] = sc->z[i];
   const int s = sc->s;
   const T beta2 = sc->beta2;
-  CR g[J];
-#pragma unroll
-  for (int k = 0; k < J; ++k) g[k] = CT<CR>::make(red[2 * k], red[2 * k + 1]);
   const T gg = red[2 * J];
   CR h[J + 1];
   T hs = 0;
+  CR zs = CT<CR>::make(0, 0);  // sum_i conj(z_i) h_i
 #pragma unroll
   for (int i = 1; i <= J; ++i) {
     CR acc = CT<CR>::make(0, 0);
 #pragma unroll
-    for (int k = 0; k < i; ++k) acc = cadd(acc, cmul(fconj(cf[i][k]), g[k]));
+    for (int k = 0; k < i; ++k) {
+      const CR g = CT<CR>::make(red[2 * k], red[2 * k + 1]);
+      acc = cdotacc(cf[i][k], g, acc);
+    }
     h[i] = acc;
     hh[i - 1][J - 1] = acc;
     hs += fabs2(acc);
+    zs = i == 1 ? acc : cdotacc(z[i - 1], acc, zs);
   }
   if (!isfinite(gg) || !isfinite(hs)) sc->status = 1;
   const T w2 = gg - hs;
-  const T hn = w2 > (T)0 ? sqrt(w2) : (T)0;
-  hh[J][J - 1] = CT<CR>::make(hn, 0);
   const bool breakdown = !(w2 > SweepTau<T>::v * gg);
+  const T in = breakdown ? (T)0 : rsqrt_t(w2);
+  hh[J][J - 1] = CT<CR>::make(w2 * in, 0);
+  const CR zn = CT<CR>::make(-zs.x * in, zs.y * in);  // z_J
   if (breakdown || J == s) {
-    sweep_finish<T, J>(sc, hh, cf, beta2);
+    const T beta = beta2 * cf[1][0].x;  // Cf[1][0] = 1 / beta
+    CR y[J], rho[J + 1];
+#pragma unroll
+    for (int i = 0; i <= J; ++i) rho[i] = CT<CR>::make(0, 0);
+    if (breakdown) {
+      y[J - 1] = fabs2(zs) > (T)0 ? fdiv(CT<CR>::make(beta, 0), zs) : CT<CR>::make(0, 0);
+    } else {
+      T nz = (T)1 + fabs2(zn);
+#pragma unroll
+      for (int i = 1; i < J; ++i) nz += fabs2(z[i]);
+      const T bz = beta / nz;
+#pragma unroll
+      for (int i = 1; i < J; ++i) rho[i] = CT<CR>::make(bz * z[i].x, bz * z[i].y);
+      const T f = -bz * in;
+      y[J - 1] = CT<CR>::make(f * zn.x, f * zn.y);
+    }
+#pragma unroll
+    for (int j = J - 2; j >= 0; --j) {
+      CR acc = rho[j + 1];
+#pragma unroll
+      for (int l = j + 1; l < J; ++l) acc = cfma(hh[j + 1][l], y[l], acc);
+      y[j] = CT<CR>::make(-acc.x * inv[j], -acc.y * inv[j]);
+    }
+    // x += sum_{k<J} xcoef[k] R_k, r = sum_{k<=J} rcoef[k] R_k
+#pragma unroll
+    for (int k = 0; k <= SMAX; ++k) {
+      CR x = CT<CR>::make(0, 0);
+      if (k < J) {
+#pragma unroll
+        for (int jj = k + 1; jj <= J; ++jj) x = cfma(y[jj - 1], cf[jj][k < J ? k : 0], x);
+      }
+      sc->xcoef[k] = x;
+      sc->rcoef[k] = k == 0 ? CT<CR>::make(1, 0)
+                            : k <= J ? CT<CR>::make(-y[k <= J && k > 0 ? k - 1 : 0].x, -y[k <= J && k > 0 ? k - 1 : 0].y)
+                                     : CT<CR>::make(0, 0);
+    }
+    sc->m = J;
   } else if (J < SMAX) {
-    const T inv = (T)1 / hn;
     CR cn[J + 1];
 #pragma unroll
     for (int k = 0; k < J; ++k) {
       CR acc = CT<CR>::make(0, 0);
 #pragma unroll
-      for (int i = k + 1; i <= J; ++i) acc = cadd(acc, cmul(h[i], cf[i][k]));
-      cn[k] = CT<CR>::make(-acc.x * inv, -acc.y * inv);
+      for (int i = k + 1; i <= J; ++i) acc = cfma(h[i], cf[i][k], acc);
+      cn[k] = CT<CR>::make(-acc.x * in, -acc.y * in);
     }
-    cn[J] = CT<CR>::make(inv, 0);
+    cn[J] = CT<CR>::make(in, 0);
+    sc->inv[J - 1] = in;
+    sc->z[J] = zn;
 #pragma unroll
     for (int i = 0; i <= J; ++i) sc->Hh[i][J - 1] = hh[i][J - 1];
 #pragma unroll
@@ -473,11 +530,10 @@ __device__ inline void grid_sum_sweep(T (&v)[2 * J + 1], void* partv, int tile, 
 #pragma unroll
   for (int q = 0; q < WPT; ++q) w[q] = tid + q * nt < words ? __ldcg(gsrc + tid + q * nt) : 0;
   T acc[NV];
-  sum_partials<NV, T>(part, ntiles, acc);
 #pragma unroll
   for (int q = 0; q < WPT; ++q)
     if (tid + q * nt < words) sdst[tid + q * nt] = w[q];
-  block_sum<NV, T>(acc, sm);
+  slots_total<NV, T>(part, ntiles, acc, sm);
   if (tid == 0) {
     sc->counter = 0u;
 #pragma unroll

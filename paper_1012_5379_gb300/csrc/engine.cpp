@@ -48,10 +48,6 @@ static TileCfg default_tiles(int dim, int P) {
   return c;
 }
 
-// Largest level size run by the coarse sub-cycle kernel (one CTA per problem with the
-// levels staged in shared memory) instead of grid-wide launches.
-static int coarse_threshold(int dim) { return dim == 2 ? 31 : 7; }
-
 // Tiles of the finest tile configuration (2 rows / planes per march).
 static int max_tiles(int dim, int P) {
   TileCfg c;
@@ -131,9 +127,9 @@ static int factor_coarsest(Handle* h, double theta_beta, cudaStream_t st) {
   std::vector<cplx> A = dense_operator(h->dim, Lc.n, a, d, c, phic, cplx(1.0, h->csl_eps));
   std::vector<int> perm;
   if (!lu_factor(A, cm, perm)) { set_error("coarsest operator is singular"); return HELM_ENUMERIC; }
-  if (h->prec == HELM_C64) {
-    // the inverse, column by column from the factors (binary64), as double-floats
-    float4* iv = reinterpret_cast<float4*>(h->stage + h->stage_inv);
+  {  // the inverse, column by column from the factors (binary64); complex64: as double-floats
+    double2* ivd = reinterpret_cast<double2*>(h->stage + h->stage_inv);
+    float4* iv = reinterpret_cast<float4*>(ivd);
     std::vector<cplx> y(cm);
     auto split = [](double v, float* hi, float* lo) {
       *hi = (float)v;
@@ -148,11 +144,16 @@ static int factor_coarsest(Handle* h, double theta_beta, cudaStream_t st) {
         y[i] /= A[(size_t)i * cm + i];
       }
       for (int i = 0; i < cm; ++i) {
-        float4& o = iv[(size_t)i * cm + j];
-        split(y[i].real(), &o.x, &o.y);
-        split(y[i].imag(), &o.z, &o.w);
+        const size_t at = (size_t)i * cm + j;
+        if (h->prec == HELM_C128) {
+          ivd[at] = make_double2(y[i].real(), y[i].imag());
+        } else {
+          split(y[i].real(), &iv[at].x, &iv[at].y);
+          split(y[i].imag(), &iv[at].z, &iv[at].w);
+        }
       }
     }
+    static_assert(sizeof(float4) == sizeof(double2), "one staging block for either form");
     CUDA_TRY(cudaMemcpyAsync(h->inv, iv, A.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
   }
   double2* Ad = reinterpret_cast<double2*>(h->stage + h->stage_lu);
@@ -269,7 +270,7 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     h->stage_piv = off;
     off += r256((size_t)cm * sizeof(int));
     h->stage_inv = off;
-    if (h->prec == HELM_C64) off += r256((size_t)cm * cm * sizeof(float4));
+    off += r256((size_t)cm * cm * sizeof(float4));
     h->stage_coef.resize(nlev);
     for (int l = 0; l < nlev; ++l) {
       h->stage_coef[l] = off;
@@ -350,7 +351,7 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
   h->lu_m = cm;
   TRY(dev_alloc(h.get(), &h->lu, (size_t)cm * cm * sizeof(double2)));
   TRY(dev_alloc(h.get(), &h->piv, cm * sizeof(int)));
-  if (h->prec == HELM_C64) TRY(dev_alloc(h.get(), &h->inv, (size_t)cm * cm * sizeof(float4)));
+  TRY(dev_alloc(h.get(), &h->inv, (size_t)cm * cm * sizeof(float4)));
   TRY(factor_coarsest(h.get(), theta_beta, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   // ------------------------------------------------ H and the outer storage
@@ -588,7 +589,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     const Handle* big = nullptr;
     for (int p = 0; p < count; ++p) if (off[p] == 0) big = hs[p];
     for (int t = 0; t < g->Lmax; ++t)
-      if (big->lev[t].n <= coarse_threshold(g->dim)) { tthr = t; break; }
+      if (big->lev[t].n <= coarse_threshold(g->dim, h0.prec)) { tthr = t; break; }
   }
   // the split depends on the level sizes only, never on the other problems: a problem
   // whose finest level is already coarse runs its whole cycle in the coarse kernel
@@ -660,7 +661,8 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     c.m = hs[p]->lu_m;
     c.lu = hs[p]->lu;
     c.piv = hs[p]->piv;
-    c.inv = hs[p]->inv;
+    c.inv = sizeof(C) == 8 ? hs[p]->inv : nullptr;
+    c.invd = sizeof(C) == 16 ? reinterpret_cast<const double2*>(hs[p]->inv) : nullptr;
     lus.push_back(c);
   }
   std::vector<LevelDev<C>> lev0;

@@ -71,7 +71,7 @@ struct Handle {
   double2* lu = nullptr;
   int* piv = nullptr;
   int lu_m = 0;
-  float4* inv = nullptr;      // complex64: the coarsest inverse as double-floats
+  float4* inv = nullptr;      // the coarsest inverse: double-floats (complex64) or binary64 (complex128)
   double2* hcoef = nullptr;   // 3n FP64 coefficients of H
   float4* hcoef_df = nullptr; // the same as double-floats (hi + lo, rounded to nearest)
   // outer FGMRES storage

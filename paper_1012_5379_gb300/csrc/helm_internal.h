@@ -47,6 +47,8 @@ struct SweepScalarsT {
   int s;                          // requested steps
   CR Cf[SMAX + 1][SMAX + 1];      // Arnoldi vectors over raw vectors
   CR Hh[SMAX + 1][SMAX];          // Hessenberg matrix of the sweep
+  CR z[SMAX + 1];                 // its left null vector: sum_i conj(z_i) Hh[i][j] = 0, z_0 = 1
+  R inv[SMAX + 1];                // 1 / Hh[j + 1][j]
   CR xcoef[SMAX + 1];             // x_new = x_old + sum_k xcoef[k] R_k
   CR rcoef[SMAX + 1];             // r_new = sum_k rcoef[k] R_k
   int status;                     // nonzero: NaN/Inf seen
@@ -101,6 +103,7 @@ struct CoarseLU {
   const double2* lu;      // m*m
   const int* piv;         // m
   const float4* inv;      // complex64: m*m entries of the inverse as double-floats (re hi, lo, im hi, lo)
+  const double2* invd;    // complex128: the inverse (null: solve with the factors)
 };
 
 // Outer FGMRES state of one problem (FP64, device memory).
@@ -166,11 +169,24 @@ constexpr int WY3 = 8;        // 3D: owned y rows per CTA (plus 2 halo warps)
 
 HELM_HD inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
-// V-cycle tile kernels: 2D tiles of 64 x 16 points; 3D blocks of 32 x 8 columns
-// marching zchunk(P) planes.
+// V-cycle tile kernels: 2D tiles of 32 Q x 8 Q points, Q = tile2_q(P); 3D blocks of 32 x 8
+// columns marching zchunk(P) planes.  Q = 1 where 64 x 16 tiles would be fewer than four per
+// SM of a 152-SM device: a complex128 Arnoldi pass on 127^2 takes 15.5 us instead of 32 (16
+// CTAs of 1024 points hold 16 SMs' FP64 pipes for 13 us), a complex64 restriction 6.9 instead
+// of 7.6; at 1023^2 and above the larger tile's thinner halo wins.
 HELM_HD inline int zchunk(int P) { return P >= 128 ? 32 : (P >= 64 ? 4 : 2); }
+// (The persistent segments' levels, P <= 512, have Q = 1.)
+HELM_HD inline int tile2_q(int P) { return ceil_div(P, 64) * ceil_div(P, 16) < 608 ? 1 : 2; }
 HELM_HD inline int vtiles(int dim, int P) {
-  return dim == 2 ? ceil_div(P, 64) * ceil_div(P, 16) : ceil_div(P, 32) * ceil_div(P, 8) * ceil_div(P, zchunk(P));
+  const int q = tile2_q(P);
+  return dim == 2 ? ceil_div(P, 32 * q) * ceil_div(P, 8 * q) : ceil_div(P, 32) * ceil_div(P, 8) * ceil_div(P, zchunk(P));
+}
+
+// Largest level size run by the coarse sub-cycle kernel (one CTA per problem) instead of
+// grid-wide launches.  Complex128 is bound by the FP64 pipe (2 lanes per SM and cycle): a
+// 31^2 Arnoldi step takes one SM 29,000 cycles, more than its launches on four.
+HELM_HD inline int coarse_threshold(int dim, int prec) {
+  return dim == 3 ? 7 : prec == 2 /* HELM_C128 */ ? 23 : 31;
 }
 
 // Launch choice of a complex64 level's sweep pass (sweep.cuh): 2D rows per warp `geo`; 3D

@@ -1,10 +1,10 @@
 // Shared-memory tile kernels of the grid-wide V-cycle passes (Sec. 3.1).
 //
-// 2D: a CTA of 32 x 8 threads owns a 64 x 16 tile; each thread owns four points
-//     (x0 + lx + 32a, y0 + ly + 8b).  Threads load the raw vectors at their own points
-//     (keeping them in registers for the dot products) and write the formed vector
-//     into a (16+2) x (64+2) shared tile; the 164 halo points are loaded by the first
-//     164 threads.  The stencil then reads shared memory only.
+// 2D: a CTA of 32 x 8 threads owns a 64 x 16 (or 32 x 8) tile; each thread owns four
+//     points (or one) (x0 + lx + 32a, y0 + ly + 8b).  Threads load the raw vectors at their
+//     own points (keeping them in registers for the dot products) and write the formed
+//     vector into a shared tile with a one-point halo; the 164 (84) halo points are loaded
+//     by the first threads.  The stencil then reads shared memory only.
 // 3D: a CTA of 32 x 8 threads owns a 32 x 8 column block and marches `zc` planes in
 //     z.  Plane tiles (8+2) x (32+2) live in a 4-slot shared ring: the plane loaded in
 //     iteration z sits in slot (z+1)&3, the stencil of plane z reads slots (z-1)&3,
@@ -16,9 +16,12 @@
 
 namespace helm {
 
-constexpr int T2X = 64, T2Y = 16;
+// 2D tiles are 32 Q x 8 Q points, Q x Q per thread: Q = 2 on large levels, Q = 1 where 64 x 16
+// tiles would leave SMs idle (tile2_q).
+HELM_HD constexpr int t2x(int Q) { return 32 * Q; }
+HELM_HD constexpr int t2y(int Q) { return 8 * Q; }
 constexpr int T3X = 32, T3Y = 8;
-constexpr int HALO2 = 2 * (T2X + 2) + 2 * T2Y;  // 164
+HELM_HD constexpr int halo2(int Q) { return 2 * (t2x(Q) + 2) + 2 * t2y(Q); }  // 164, 84
 constexpr int HALO3 = 2 * (T3X + 2) + 2 * T3Y;  // 84
 
 // h-th halo point of a TX x TY tile in local coordinates (-1..TX, -1..TY):
@@ -49,10 +52,10 @@ __device__ __forceinline__ C stencil5(const Coef3<C>& cx, const Coef3<C>& cy, ty
 
 // ------------------------------------------------------------------ Arnoldi step J
 // Complex128 holds twice the registers per raw vector: two CTAs per SM.
-template <typename C, int J, bool NC = true>
+template <typename C, int J, int Q, bool NC = true>
 __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int store_p, int vblk) {
   typedef typename CT<C>::R R;
-  __shared__ C vt[T2Y + 2][T2X + 2];
+  __shared__ C vt[t2y(Q) + 2][t2x(Q) + 2];
   __shared__ R sm[32 * (2 * J + 1)];
   const int nunits = ceil_div(ntiles, tpc);
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
@@ -61,7 +64,7 @@ __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ 
   pdl_wait();
   if (sc->m < J) return;  // earlier breakdown or empty sweep: uniform for the problem
   const int n = L.n, P = L.P;
-  const int ntx = ceil_div(P, T2X);
+  const int ntx = ceil_div(P, t2x(Q));
   const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
   const StencilRegs<C> S(L);
   C* const pJ = L.p[J - 1];
@@ -79,11 +82,11 @@ __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ 
   const int t_end = min(ntiles, (unit + 1) * tpc);
 #pragma unroll 1
   for (int tile = unit * tpc; tile < t_end; ++tile) {
-    const int x0 = (tile % ntx) * T2X, y0 = (tile / ntx) * T2Y;
-    C raw[4][J];
+    const int x0 = (tile % ntx) * t2x(Q), y0 = (tile / ntx) * t2y(Q);
+    C raw[Q * Q][J];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
+    for (int q = 0; q < Q * Q; ++q) {
+      const int ox = lx + 32 * (q % Q), oy = ly + 8 * (q / Q);
       C v = czero<C>();
 #pragma unroll
       for (int k = 0; k < J; ++k) {
@@ -92,25 +95,25 @@ __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ 
       }
       vt[oy + 1][ox + 1] = v;
     }
-    if (tid < HALO2) {
+    if (tid < halo2(Q)) {
       int hx, hy;
-      halo_coord<T2X, T2Y>(tid, hx, hy);
+      halo_coord<t2x(Q), t2y(Q)>(tid, hx, hy);
       C v = czero<C>();
 #pragma unroll
       for (int k = 0; k < J; ++k) v = cfma(cf[k], ldc<C, NC>(Rk[k], x0 + hx, y0 + hy, 0, n, P), v);
       vt[hy + 1][hx + 1] = v;
     }
     __syncthreads();
-    const Coef3<C> cx0 = S.coef(x0 + lx), cx1 = S.coef(x0 + lx + 32);
+    const Coef3<C> cx0 = S.coef(x0 + lx), cx1 = Q == 2 ? S.coef(x0 + lx + 32) : cx0;
     Coef3<C> cy;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
+    for (int q = 0; q < Q * Q; ++q) {
+      const int ox = lx + 32 * (q % Q), oy = ly + 8 * (q / Q);
       const int x = x0 + ox, y = y0 + oy;
-      if ((q & 1) == 0) cy = S.coef(y);  // one row per pair of points
+      if (q % Q == 0) cy = S.coef(y);  // one row per pair of points
       C p = czero<C>();
       if (x < n && y < n) {
-        p = stencil5((q & 1) ? cx1 : cx0, cy, S.phi_at(x, y, 0), vt[oy + 1][ox + 1], vt[oy + 1][ox],
+        p = stencil5(q % Q ? cx1 : cx0, cy, S.phi_at(x, y, 0), vt[oy + 1][ox + 1], vt[oy + 1][ox],
                      vt[oy + 1][ox + 2], vt[oy][ox + 1], vt[oy + 2][ox + 1]);
 #pragma unroll
         for (int k = 0; k < J; ++k) acc[k] = cdotacc(raw[q][k], p, acc[k]);
@@ -127,10 +130,10 @@ __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ 
   pdl_trigger();  // the main work is done: let the next pass launch
   grid_sum_sweep<R, J>(red, L.part, unit, nunits, sc, sm);
 }
-template <typename C, int J>
-__global__ void __launch_bounds__(256, sizeof(C) == 16 ? 2 : (J <= 2 ? 4 : 3))
+template <typename C, int J, int Q>
+__global__ void __launch_bounds__(256, 2)
 k_arnoldi_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int store_p) {
-  arnoldi_t2_body<C, J>(levs, ntiles, tpc, r0_is_b, store_p, blockIdx.x);
+  arnoldi_t2_body<C, J, Q>(levs, ntiles, tpc, r0_is_b, store_p, blockIdx.x);
 }
 
 template <typename C, int J, bool NC = true>
@@ -663,28 +666,28 @@ k_prolong3_rows(const LevelDev<C>* __restrict__ levs, int nblk) {
 // The tiles of one CTA with the sweep's raw-vector count M fixed, so that every load
 // of a tile (M + 1 raw vectors and x at four points per thread) is issued before the
 // first is used.
-template <typename C, int M, bool NC = true>
+template <typename C, int M, int Q, bool NC = true>
 __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCoef<C>& u, int unit, int tpc,
-                                               int ntiles, int x_from_zero, C (*rt)[T2X + 1],
+                                               int ntiles, int x_from_zero, C (*rt)[t2x(Q) + 1],
                                                typename CT<C>::R& acc) {
   typedef typename CT<C>::R R;
   const int n = L.n, P = L.P, nc = L.nc, Pc = L.Pc;
-  const int ntx = ceil_div(P, T2X);
+  const int ntx = ceil_div(P, t2x(Q));
   const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
   C* const xa = L.xa;
   C* const bc = L.bc;
   const int t_end = min(ntiles, (unit + 1) * tpc);
 #pragma unroll 1
   for (int tile = unit * tpc; tile < t_end; ++tile) {
-    const int x0 = (tile % ntx) * T2X, y0 = (tile / ntx) * T2Y;
-    constexpr int QB = M >= 3 ? 2 : 4;  // points whose loads are in flight together (registers)
+    const int x0 = (tile % ntx) * t2x(Q), y0 = (tile / ntx) * t2y(Q);
+    constexpr int QB = Q == 1 ? 1 : M >= 3 ? 2 : 4;  // points whose loads are in flight together (registers)
 #pragma unroll
-    for (int q0 = 0; q0 < 4; q0 += QB) {
+    for (int q0 = 0; q0 < Q * Q; q0 += QB) {
       C v[QB][M + 1], xv[QB];
 #pragma unroll
       for (int b = 0; b < QB; ++b) {
         const int q = q0 + b;
-        const int x = x0 + lx + 32 * (q & 1), y = y0 + ly + 8 * (q >> 1);
+        const int x = x0 + lx + 32 * (q % Q), y = y0 + ly + 8 * (q / Q);
 #pragma unroll
         for (int k = 0; k <= M; ++k) v[b][k] = ldc<C, NC>(u.Rk[k], x, y, 0, n, P);
         xv[b] = (x_from_zero || x >= n || y >= n) ? czero<C>() : xa[pidx(x, y, 0, P)];
@@ -692,7 +695,7 @@ __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCo
 #pragma unroll
       for (int b = 0; b < QB; ++b) {
         const int q = q0 + b;
-        const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
+        const int ox = lx + 32 * (q % Q), oy = ly + 8 * (q / Q);
         const int x = x0 + ox, y = y0 + oy;
         C dx = czero<C>(), r = czero<C>();
 #pragma unroll
@@ -703,37 +706,40 @@ __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCo
         rt[oy][ox] = r;
       }
     }
-    if (tid < T2X + 1 + T2Y) {
-      const int hx = tid < T2X + 1 ? tid : T2X;
-      const int hy = tid < T2X + 1 ? T2Y : tid - (T2X + 1);
+    if (tid < t2x(Q) + 1 + t2y(Q)) {
+      const int hx = tid < t2x(Q) + 1 ? tid : t2x(Q);
+      const int hy = tid < t2x(Q) + 1 ? t2y(Q) : tid - (t2x(Q) + 1);
       C r = czero<C>();
 #pragma unroll
       for (int k = 0; k <= M; ++k) r = cfma(u.rc[k], ldc<C, NC>(u.Rk[k], x0 + hx, y0 + hy, 0, n, P), r);
       rt[hy][hx] = r;
     }
     __syncthreads();
-    const int fx = 2 * lx + 1, fy = 2 * ly + 1;
-    C out = czero<C>();
+    if (tid < (t2x(Q) / 2) * (t2y(Q) / 2)) {  // one coarse point each
+      const int px = tid % (t2x(Q) / 2), py = tid / (t2x(Q) / 2);
+      const int fx = 2 * px + 1, fy = 2 * py + 1;
+      C out = czero<C>();
 #pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
+      for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
-      for (int dx = -1; dx <= 1; ++dx)
-        out = cadd(out, cscale(rt[fy + dy][fx + dx], (R)((dx == 0 ? 0.5 : 0.25) * (dy == 0 ? 0.5 : 0.25))));
-    const int Ix = x0 / 2 + lx, Iy = y0 / 2 + ly;
-    if (Ix < Pc && Iy < Pc) {
-      const bool valid = Ix < nc && Iy < nc;
-      bc[pidx(Ix, Iy, 0, Pc)] = valid ? out : czero<C>();
-      if (valid) acc += cabs2(out);
+        for (int dx = -1; dx <= 1; ++dx)
+          out = cadd(out, cscale(rt[fy + dy][fx + dx], (R)((dx == 0 ? 0.5 : 0.25) * (dy == 0 ? 0.5 : 0.25))));
+      const int Ix = x0 / 2 + px, Iy = y0 / 2 + py;
+      if (Ix < Pc && Iy < Pc) {
+        const bool valid = Ix < nc && Iy < nc;
+        bc[pidx(Ix, Iy, 0, Pc)] = valid ? out : czero<C>();
+        if (valid) acc += cabs2(out);
+      }
     }
     __syncthreads();  // the next tile rewrites rt
   }
 }
 
-template <typename C, bool NC = true>
+template <typename C, int Q, bool NC = true>
 __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int x_from_zero,
               int nosmooth, int vblk) {
   typedef typename CT<C>::R R;
-  __shared__ C rt[T2Y + 1][T2X + 1];
+  __shared__ C rt[t2y(Q) + 1][t2x(Q) + 1];
   __shared__ R sm[32];
   const int nunits = ceil_div(ntiles, tpc);
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
@@ -743,11 +749,11 @@ __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__
   if (nosmooth) { u.m = 0; u.rc[0] = CT<C>::make(1, 0); }
   R acc = 0;
   switch (u.m) {  // uniform over the grid
-    case 0: restrict_tiles<C, 0, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 1: restrict_tiles<C, 1, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 2: restrict_tiles<C, 2, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 3: restrict_tiles<C, 3, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 4: restrict_tiles<C, 4, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 0: restrict_tiles<C, 0, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 1: restrict_tiles<C, 1, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 2: restrict_tiles<C, 2, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 3: restrict_tiles<C, 3, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 4: restrict_tiles<C, 4, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
     default: break;
   }
   static_assert(SMAX == 4, "restrict_tiles is instantiated for m = 0..4");
@@ -759,11 +765,11 @@ __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__
     }
   }
 }
-template <typename C>
+template <typename C, int Q>
 __global__ void __launch_bounds__(256, sizeof(C) == 16 ? 2 : 3)
 k_restrict_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int x_from_zero,
               int nosmooth) {
-  restrict_t2_body<C>(levs, ntiles, tpc, r0_is_b, x_from_zero, nosmooth, blockIdx.x);
+  restrict_t2_body<C, Q>(levs, ntiles, tpc, r0_is_b, x_from_zero, nosmooth, blockIdx.x);
 }
 
 // The z-march of one 3D restriction tile with the sweep's raw-vector count M fixed:
@@ -878,17 +884,17 @@ k_restrict_t3(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_i
 
 // ------------------------------------------------------------------ coarse correction
 // x_b = x_a + P e_c, r0 = b - M x_b, ||r0||^2 starts post-smoothing.
-template <typename C, bool NC = true>
+template <typename C, int Q, bool NC = true>
 __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int vblk) {
   typedef typename CT<C>::R R;
-  __shared__ C vt[T2Y + 2][T2X + 2];
+  __shared__ C vt[t2y(Q) + 2][t2x(Q) + 2];
   __shared__ R sm[32];
   const int nunits = ceil_div(ntiles, tpc);
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
   const LevelDev<C>& L = levs[prob];
   const int n = L.n, P = L.P;
   pdl_wait();
-  const int ntx = ceil_div(P, T2X);
+  const int ntx = ceil_div(P, t2x(Q));
   const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
   const StencilRegs<C> S(L);
   const C* const xa = L.xa;
@@ -904,31 +910,31 @@ __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ 
   const int t_end = min(ntiles, (unit + 1) * tpc);
 #pragma unroll 1
   for (int tile = unit * tpc; tile < t_end; ++tile) {
-    const int x0 = (tile % ntx) * T2X, y0 = (tile / ntx) * T2Y;
-    C bq[4];  // b at the owned points, loaded with the first phase's reads
+    const int x0 = (tile % ntx) * t2x(Q), y0 = (tile / ntx) * t2y(Q);
+    C bq[Q * Q];  // b at the owned points, loaded with the first phase's reads
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
+    for (int q = 0; q < Q * Q; ++q) {
+      const int ox = lx + 32 * (q % Q), oy = ly + 8 * (q / Q);
       bq[q] = ldc<C, NC>(bv, x0 + ox, y0 + oy, 0, n, P);
       vt[oy + 1][ox + 1] = form(x0 + ox, y0 + oy);
     }
-    if (tid < HALO2) {
+    if (tid < halo2(Q)) {
       int hx, hy;
-      halo_coord<T2X, T2Y>(tid, hx, hy);
+      halo_coord<t2x(Q), t2y(Q)>(tid, hx, hy);
       vt[hy + 1][hx + 1] = form(x0 + hx, y0 + hy);
     }
     __syncthreads();
-    const Coef3<C> cx0 = S.coef(x0 + lx), cx1 = S.coef(x0 + lx + 32);
+    const Coef3<C> cx0 = S.coef(x0 + lx), cx1 = Q == 2 ? S.coef(x0 + lx + 32) : cx0;
     Coef3<C> cy;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
+    for (int q = 0; q < Q * Q; ++q) {
+      const int ox = lx + 32 * (q % Q), oy = ly + 8 * (q / Q);
       const int x = x0 + ox, y = y0 + oy;
-      if ((q & 1) == 0) cy = S.coef(y);  // one row per pair of points
+      if (q % Q == 0) cy = S.coef(y);  // one row per pair of points
       if (x < P && y < P) {
         C r = czero<C>(), xo = czero<C>();
         if (x < n && y < n) {
-          const C p = stencil5((q & 1) ? cx1 : cx0, cy, S.phi_at(x, y, 0), vt[oy + 1][ox + 1], vt[oy + 1][ox],
+          const C p = stencil5(q % Q ? cx1 : cx0, cy, S.phi_at(x, y, 0), vt[oy + 1][ox + 1], vt[oy + 1][ox],
                                vt[oy + 1][ox + 2], vt[oy][ox + 1], vt[oy + 2][ox + 1]);
           r = csub(bq[q], p);
           xo = vt[oy + 1][ox + 1];
@@ -948,10 +954,10 @@ __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ 
     }
   }
 }
-template <typename C>
+template <typename C, int Q>
 __global__ void __launch_bounds__(256)
 k_prolong_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc) {
-  prolong_t2_body<C>(levs, ntiles, tpc, blockIdx.x);
+  prolong_t2_body<C, Q>(levs, ntiles, tpc, blockIdx.x);
 }
 
 template <typename C, bool NC = true>
@@ -1082,19 +1088,19 @@ __device__ __noinline__ void seq_arnoldi(const PassDesc d, const LevelDev<C>* le
   } else if constexpr (sizeof(C) == 8) {
     sweep3_body<J, SEQ_O3, false>(levs, d.ntiles, d.f0, d.f1, v, sm);
   } else if constexpr (DIM == 2) {
-    arnoldi_t2_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
+    arnoldi_t2_body<C, J, 1, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
   } else {
     arnoldi_t3_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
   }
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_restrict(const PassDesc d, const LevelDev<C>* levs, int v) {
-  if constexpr (DIM == 2) restrict_t2_body<C, false>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
+  if constexpr (DIM == 2) restrict_t2_body<C, 1, false>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
   else restrict_t3_body<C, false>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_prolong(const PassDesc d, const LevelDev<C>* levs, int v) {
-  if constexpr (DIM == 2) prolong_t2_body<C, false>(levs, d.ntiles, d.geo, v);
+  if constexpr (DIM == 2) prolong_t2_body<C, 1, false>(levs, d.ntiles, d.geo, v);
   else prolong_t3_body<C, false>(levs, d.ntiles, d.geo, v);
 }
 template <typename C, int DIM>
@@ -1107,7 +1113,7 @@ __device__ __noinline__ void seq_prolong_flat(const PassDesc d, const LevelDev<C
 }
 
 // flags: arnoldi f0 = R_0 is b, f1 = store p_J; restrict f0 = R_0 is b, f1 = x from zero,
-// f2 = no smoothing; update f0 = mode, f1 = R_0 is b, f2 = x selection, f3 = x from zero
+// f2 = no smoothing; 2D levels here have tiles of Q = 1; update f0 = mode, f1 = R_0 is b, f2 = x selection, f3 = x from zero
 template <typename C, int DIM>
 __device__ __forceinline__ void run_pass(const PassDesc& d, const LevelDev<C>* levs, int v, float2* sm) {
   switch (d.kind) {

@@ -370,6 +370,17 @@ __device__ __forceinline__ unsigned cblock_npts(int P, int dim) {
   return dim == 3 ? (unsigned)P * P * P : (unsigned)P * P;
 }
 
+// The first NV of a pass's sums over the team (a step carries 2 J + 1 of them).
+template <int NV, typename T, typename Team>
+__device__ __forceinline__ void team_sum_first(Team& team, T (&red)[2 * SMAX + 1], T* sm) {
+  T v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] = red[i];
+  team.sum(v, sm);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) red[i] = v[i];
+}
+
 // One GMRES(s) sweep on level L by the team.  R_0 is b (r0_is_b) or r0; x is updated
 // in place in xo (or written from zero).  `tmp` holds v_J.  At the end, in residual
 // mode r0 <- r_new and the next sweep starts; in restrict mode the residual is left in
@@ -431,7 +442,13 @@ __device__ void cblock_sweep(Team& team, const LevelDev<C>& L, int dim, int r0_i
     }
     for (int k = 0; k < J; ++k) { red[2 * k] = acc[k].x; red[2 * k + 1] = acc[k].y; }
     red[2 * J] = accn;
-    team.sum(red, sm);  // also separates this pass's reads of tmp from the next pass's writes
+    // also separates this pass's reads of tmp from the next pass's writes
+    switch (J) {
+      case 1: team_sum_first<3>(team, red, sm); break;
+      case 2: team_sum_first<5>(team, red, sm); break;
+      case 3: team_sum_first<7>(team, red, sm); break;
+      default: team_sum_first<9>(team, red, sm); break;
+    }
     if (flat_tid() == 0) sweep_after_pass_rt<R>(sc, J, red);
   }
   __syncthreads();
@@ -488,7 +505,7 @@ __device__ void coarse_cycle(Team& team, const LevelDev<C>* Ls, int nlev, const 
   R* sm = reinterpret_cast<R*>(smd);
   const unsigned gt = team.gtid(), gn = team.gnth();
   const int tid = flat_tid(), nth = block_threads();
-  const bool staged = lu_sm && lu.m * lu.m <= lu_cap;
+  const bool staged = !lu.invd && lu_sm && lu.m * lu.m <= lu_cap;
   if (staged) {
     for (int i = tid; i < lu.m * lu.m; i += nth) lu_sm[i] = lu.lu[i];
     __syncthreads();
@@ -545,7 +562,36 @@ __device__ void coarse_cycle(Team& team, const LevelDev<C>* Ls, int nlev, const 
     const LevelDev<C>& L = Ls[nlev - 1];
     const int m = lu.m, P = L.P, n = L.n;
     double2* yv = reinterpret_cast<double2*>(smd);  // m <= 144 complex values
-    if (team.rank() == 0) {
+    if (lu.invd) {
+      // x = A^{-1} b: sixteen lanes per row (2 m dependent elimination steps on one warp
+      // would each take several 64-cycle FP64 instructions)
+      const int l16 = tid & 15;
+      for (int i = tid; i < m; i += nth) {
+        const int sx = i % n, sy = (i / n) % n, sz = dim == 3 ? i / (n * n) : 0;
+        yv[i] = to_d(L.b[pidx(sx, sy, sz, P)]);
+      }
+      __syncthreads();
+      for (int r0 = 0; r0 < m; r0 += nth / 16) {  // the same trips for every thread
+        const int row = r0 + (tid >> 4);
+        if (r0 + ((tid & ~31) >> 4) >= m) continue;  // uniform over the warp
+        double2 s = make_double2(0, 0);
+        if (row < m)
+          for (int q = l16; q < m; q += 16) s = cfma(__ldg(lu.invd + (size_t)row * m + q), yv[q], s);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+          s = cadd(s, make_double2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
+        if (row < m && l16 == 0) {
+          const int sx = row % n, sy = (row / n) % n, sz = dim == 3 ? row / (n * n) : 0;
+          L.xb[pidx(sx, sy, sz, P)] = from_d<C>(s);
+        }
+      }
+      const unsigned npts = cblock_npts(P, dim);
+      for (unsigned i = tid; i < npts; i += nth) {
+        int x, y, z;
+        cblock_coords(i, (unsigned)P, dim, x, y, z);
+        if (!inside(x, y, z, n)) L.xb[i] = czero<C>();
+      }
+    } else if (team.rank() == 0) {
       if (tid < 32) {
         for (int i = tid; i < m; i += 32) {
           const int src = lu.piv[i];

@@ -82,9 +82,10 @@ template <typename C, int J>
 static void arnoldi_J(int dim, const LevelDev<C>* levs, int grid, int ntiles, TileCfg cfg, bool r0_is_b,
                       bool store_p, cudaStream_t st) {
   if (dim == 2) {
-    const int t = tuned_tpc(TP_ARNOLDI, cfg.P, (int)sizeof(C), J, tiles_per_cta(k_arnoldi_t2<C, J>, ntiles));
-    pdl_launch(k_arnoldi_t2<C, J>, dim3(grid / ntiles * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t,
-               r0_is_b, store_p);
+    auto* const kern = tile2_q(cfg.P) == 1 ? k_arnoldi_t2<C, J, 1> : k_arnoldi_t2<C, J, 2>;
+    const int t = tuned_tpc(TP_ARNOLDI, cfg.P, (int)sizeof(C), J, tiles_per_cta(kern, ntiles));
+    pdl_launch(kern, dim3(grid / ntiles * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t, r0_is_b,
+               store_p);
   }
   else
     pdl_launch(k_arnoldi_t3<C, J>, dim3(grid), dim3(dim3(32, 8)), 0, st, levs, ntiles, cfg.rows, r0_is_b, store_p);
@@ -136,8 +137,9 @@ void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, Ti
     }
   }
   if (dim == 2) {
-    const int t = tuned_tpc(TP_RESTRICT, cfg.P, (int)sizeof(C), 0, tiles_per_cta(k_restrict_t2<C>, ntiles));
-    pdl_launch(k_restrict_t2<C>, dim3(nprob * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t, r0_is_b,
+    auto* const kern = tile2_q(cfg.P) == 1 ? k_restrict_t2<C, 1> : k_restrict_t2<C, 2>;
+    const int t = tuned_tpc(TP_RESTRICT, cfg.P, (int)sizeof(C), 0, tiles_per_cta(kern, ntiles));
+    pdl_launch(kern, dim3(nprob * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t, r0_is_b,
                x_from_zero, nosmooth);
   } else
     pdl_launch(k_restrict_t3<C>, dim3(nprob * ntiles), dim3(dim3(32, 8)), 0, st, levs, ntiles, cfg.rows, r0_is_b, x_from_zero, nosmooth);
@@ -161,8 +163,9 @@ void launch_prolong(int dim, bool with_residual, const LevelDev<C>* levs, int np
   if (!with_residual) {
     pdl_launch(k_prolong_flat<C>, dim3(nprob * ntiles), dim3(256), 0, st, levs, ntiles, dim);
   } else if (dim == 2) {
-    const int t = tuned_tpc(TP_PROLONG, cfg.P, (int)sizeof(C), 0, tiles_per_cta(k_prolong_t2<C>, ntiles));
-    pdl_launch(k_prolong_t2<C>, dim3(nprob * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t);
+    auto* const kern = tile2_q(cfg.P) == 1 ? k_prolong_t2<C, 1> : k_prolong_t2<C, 2>;
+    const int t = tuned_tpc(TP_PROLONG, cfg.P, (int)sizeof(C), 0, tiles_per_cta(kern, ntiles));
+    pdl_launch(kern, dim3(nprob * ceil_div(ntiles, t)), dim3(dim3(32, 8)), 0, st, levs, ntiles, t);
   } else {
     pdl_launch(k_prolong_t3<C>, dim3(nprob * ntiles), dim3(dim3(32, 8)), 0, st, levs, ntiles, cfg.rows);
   }
@@ -229,7 +232,7 @@ template <typename C, int J>
 static void record_arnoldi_J(PassSeq& q, int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg,
                              bool r0_is_b, bool store_p) {
   if (dim == 2) {
-    const int t = tuned_tpc(TP_ARNOLDI, cfg.P, (int)sizeof(C), J, tiles_per_cta(k_arnoldi_t2<C, J>, ntiles));
+    const int t = tuned_tpc(TP_ARNOLDI, cfg.P, (int)sizeof(C), J, tiles_per_cta(k_arnoldi_t2<C, J, 1>, ntiles));
     seq_push(q, levs, PK_ARNOLDI, J, ntiles, t, r0_is_b, store_p, 0, 0, nprob * ceil_div(ntiles, t));
   } else {
     seq_push(q, levs, PK_ARNOLDI, J, ntiles, cfg.rows, r0_is_b, store_p, 0, 0, nprob * ntiles);
@@ -251,7 +254,7 @@ template <typename C>
 void record_restrict(PassSeq& q, int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
                      bool x_from_zero, bool nosmooth) {
   if (dim == 2) {
-    const int t = tuned_tpc(TP_RESTRICT, cfg.P, (int)sizeof(C), 0, tiles_per_cta(k_restrict_t2<C>, ntiles));
+    const int t = tuned_tpc(TP_RESTRICT, cfg.P, (int)sizeof(C), 0, tiles_per_cta(k_restrict_t2<C, 1>, ntiles));
     seq_push(q, levs, PK_RESTRICT, 0, ntiles, t, r0_is_b, x_from_zero, nosmooth, 0, nprob * ceil_div(ntiles, t));
   } else {
     seq_push(q, levs, PK_RESTRICT, 0, ntiles, cfg.rows, r0_is_b, x_from_zero, nosmooth, 0, nprob * ntiles);
@@ -271,7 +274,7 @@ void record_prolong(PassSeq& q, int dim, bool with_residual, const LevelDev<C>* 
   if (!with_residual) {
     seq_push(q, levs, PK_PROLONG_FLAT, 0, ntiles, 0, 0, 0, 0, 0, nprob * ntiles);
   } else if (dim == 2) {
-    const int t = tuned_tpc(TP_PROLONG, cfg.P, (int)sizeof(C), 0, tiles_per_cta(k_prolong_t2<C>, ntiles));
+    const int t = tuned_tpc(TP_PROLONG, cfg.P, (int)sizeof(C), 0, tiles_per_cta(k_prolong_t2<C, 1>, ntiles));
     seq_push(q, levs, PK_PROLONG, 0, ntiles, t, 0, 0, 0, 0, nprob * ceil_div(ntiles, t));
   } else {
     seq_push(q, levs, PK_PROLONG, 0, ntiles, cfg.rows, 0, 0, 0, 0, nprob * ntiles);

@@ -82,3 +82,34 @@ def test_zero_and_degenerate_right_hand_sides(helm):
     h.precond_apply(bad, z1)
     h.precond_apply(good, z1)
     assert torch.equal(z0, z1)
+
+
+@pytest.mark.parametrize("dim,n,prec,s", [(2, 19, "c128", 3), (2, 23, "c128", 4), (2, 27, "c128", 1), (2, 39, "c128", 2),
+                                          (2, 95, "c128", 3), (2, 127, "c128", 4), (2, 639, "c128", 3),
+                                          (2, 767, "c128", 3), (3, 9, "c128", 4), (3, 23, "c128", 3),
+                                          (2, 111, "c64", 3), (2, 767, "c64", 3)])
+def test_tile_sizes_and_complex128_sweeps(helm, dim, n, prec, s):
+    """Both 2D tile sizes around their border (639 and 767), levels at the border of the
+    coarse kernel (23), and every sweep length of the complex128 algebra: V-cycle bounds of
+    tests/parity_check.py (c128 1e-11, c64 5e-5)."""
+    k = 0.2 * (n + 1)
+    r = I.random_source(dim, n, 900 + n)
+    h = helm.Handle(dim, n, 0.3, k=k, precision=prec, s=s, maxit=1)
+    rt = torch.from_numpy(r).cuda()
+    if prec == "c64":
+        rt = rt.to(torch.complex64)
+    zt = torch.empty_like(rt)
+    h.precond_apply(rt, zt)
+    assert_parity(zt, O.vcycle(O.build_hierarchy(dim, n, 0.3, k=k), r, 1, 1, s), ("vcycle", prec), f"n={n} s={s}")
+
+
+def test_complex128_breakdown(helm):
+    """An exact eigenvector of M: the first Arnoldi step breaks down in binary64 too."""
+    n, k = 63, 9.0
+    x = np.arange(1, n + 1) / (n + 1)
+    e = (np.sin(5 * np.pi * x)[:, None] * np.sin(3 * np.pi * x)[None, :]).astype(complex)
+    h = helm.Handle(2, n, 0.0, k=k, theta_gamma=0.0, precision="c128", maxit=1)
+    rt = torch.from_numpy(e).cuda()
+    zt = torch.empty_like(rt)
+    h.precond_apply(rt, zt)
+    assert_parity(zt, O.vcycle(O.build_hierarchy(2, n, 0.0, 0.0, k=k), e), ("vcycle", "c128"), "eigenvector")
