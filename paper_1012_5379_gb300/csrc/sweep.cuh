@@ -192,7 +192,7 @@ k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, 
   float2 phn[W];
   auto fetch = [&](int y, float4& v, float2& f) {
     const bool ok = in && (unsigned)y < (unsigned)n;
-    v = ok ? __ldg(reinterpret_cast<const float4*>(R0 + (size_t)y * P + x)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    v = ok ? *reinterpret_cast<const float4*>(R0 + (size_t)y * P + x) : make_float4(0.f, 0.f, 0.f, 0.f);
     if (PHI)  // some problem of the launch has a field; this one may not
       f = (ok && phi) ? __ldg(reinterpret_cast<const float2*>(phi + (size_t)y * P + x)) : make_float2(phir, phir);
   };
@@ -459,8 +459,8 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   float phn[W][2];
   auto fetch = [&](int z, float2 (&v)[2], float (&f)[2]) {
     const bool zin = (unsigned)z < (unsigned)n;
-    v[0] = (zin && in0) ? __ldg(R0 + (col + (long long)(z * PP))) : make_float2(0.f, 0.f);
-    v[1] = (zin && in1) ? __ldg(R0 + (col + P + (long long)(z * PP))) : make_float2(0.f, 0.f);
+    v[0] = (zin && in0) ? R0[col + (long long)(z * PP)] : make_float2(0.f, 0.f);
+    v[1] = (zin && in1) ? R0[col + P + (long long)(z * PP)] : make_float2(0.f, 0.f);
     if (PHI) {  // some problem of the launch has a field; this one may not
       f[0] = (phi && zin && in0) ? __ldg(phi + (col + (long long)(z * PP))) : phir;
       f[1] = (phi && zin && in1) ? __ldg(phi + (col + P + (long long)(z * PP))) : phir;

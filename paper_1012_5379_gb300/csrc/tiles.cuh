@@ -361,7 +361,7 @@ k_resid_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages) 
 #pragma unroll
     for (int q = 0; q < QY; ++q) {
       ph[q] = (u >= 2 && S.phi) ? __ldg(S.phi + pz + 8 * q * P) : S.phic;
-      bq[q] = u >= 2 ? __ldg(L.b + pz + 8 * q * P) : czero<C>();
+      bq[q] = u >= 2 ? L.b[pz + 8 * q * P] : czero<C>();
     }
     const bool mine = mbar_wait(&bar[cstage], cphase);
     const C* box = reinterpret_cast<const C*>(tsm + cstage * STRIDE);
@@ -1041,8 +1041,7 @@ namespace helm {
 // A virtual block does exactly what the block of the ordinary launch does (the same
 // body, the same partial-sum slot, the same last-block reduction), so the results are
 // bitwise those of the launch-per-pass schedule.  Vectors written earlier in the same
-// launch are read through the coherent path (NC = false: the read-only cache does not
-// see another SM's writes within a kernel); the barrier's fences order the passes.
+// launch are read by plain loads; the barrier's fences order the passes.
 // A CTA waits at most limit_ns (globaltimer) at a barrier; then it records the error
 // (the solve reports HELM_ETIMEOUT) and the whole launch returns: never a trap, never
 // an endless spin.

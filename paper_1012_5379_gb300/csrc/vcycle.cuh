@@ -18,12 +18,13 @@ __device__ __forceinline__ bool inside(int x, int y, int z, int n) {
 __device__ __forceinline__ size_t pidx(int x, int y, int z, int P) {
   return ((size_t)z * P + y) * (size_t)P + x;
 }
-// Bounds-checked load; NC = true uses the read-only path and is only for buffers no
-// thread writes during the kernel.
+// Bounds-checked load.  A plain load, not the read-only one: the compiler takes a read-only
+// load for invariant and may move it above the wait for the kernel that writes the buffer
+// (pdl_wait).  (NC names the launches outside the persistent segments.)
 template <typename C, bool NC = true>
 __device__ __forceinline__ C ldc(const C* p, int x, int y, int z, int n, int P) {
   if (!inside(x, y, z, n)) return czero<C>();
-  return NC ? __ldg(p + pidx(x, y, z, P)) : p[pidx(x, y, z, P)];
+  return p[pidx(x, y, z, P)];
 }
 
 // 1D coefficients of the axis at index i (zero outside)
@@ -227,10 +228,10 @@ k_update_flat(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, int mod
 }
 
 // Level-0 input: b <- src (natural layout, any precision), ||b||^2 starts the first
-// sweep.
+// sweep.  (src is not __restrict__: the compiler could then read it before the wait.)
 template <typename Cin, typename C>
 __global__ void __launch_bounds__(256)
-k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Cin* __restrict__ src) {
+k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Cin* src) {
   __shared__ typename CT<C>::R sm[64];
   const int prob = blockIdx.x / ntiles, tile = blockIdx.x - prob * ntiles;
   const LevelDev<C>& L = levs[prob];
