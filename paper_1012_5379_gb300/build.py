@@ -18,7 +18,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU = ["vcycle_c64.cu", "vcycle_c128.cu", "sweep.cu", "outer.cu", "convert.cu", "noalloc.cu"]
 CPP = ["engine.cpp", "geometry.cpp", "capi.cpp", "profiler.cpp", "serve.cpp", "tma.cpp", "tune.cpp", "autotune.cpp"]
 HEADERS = ["poly.h", "helm_internal.h", "device_common.cuh", "vcycle.cuh", "tiles.cuh", "vcycle_launch.cuh", "launch.cuh", "gram.cuh", "sweep.cuh",
-           "coarse.cuh", "dfloat.cuh", "engine.h", "geometry.h", "profiler.h"]
+           "coarse.cuh", "poly.cuh", "dfloat.cuh", "engine.h", "geometry.h", "profiler.h"]
 
 
 def _newest_input() -> float:

@@ -22,7 +22,8 @@ constexpr int CG_COARSE_POINTS = CG_THREADS * CG_PT;  // most interior points of
 constexpr int CG_INV = 1024;                          // entries of the inverse staged in shared memory
 constexpr int CG_COEF = 3 * 64;                       // 1D coefficients of all levels (31 + 15 + 7 + 3 per array)
 
-HELM_HD constexpr int cg_vectors(int S) { return 3 + (S > 1 ? S - 1 : 0); }  // b, x, r, k_1..k_{S-1}
+// b, x, r, k_1..k_{S-1}; S = 0 stands for the polynomial smoother
+HELM_HD constexpr int cg_vectors(int S) { return 3 + (S > 1 ? S - 1 : 0); }
 
 // One thread's points of a level and the level's vectors.
 template <int S, int DIM>
@@ -141,10 +142,39 @@ __device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2*
   }
 }
 
+// One sweep of the polynomial smoother (Sec. 4): x <- x + w_j (b - M x), j = 0, 1, 2, from
+// zero where `zero`.  x is published to V.x and V.r in turn (`tog`), one barrier a step.
+template <int S, int DIM>
+__device__ __forceinline__ void cg_poly(const CgLevel<S, DIM>& V, const float2 (&b)[CG_PT], float2 (&x)[CG_PT],
+                                        const float2* w, bool zero, int& tog) {
+  const float2 z0 = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int j = 0; j < 3; ++j) {
+    const float2 wj = w[j];
+    float2* buf = tog ? V.r : V.x;
+    if (!(zero && j == 0)) {
+#pragma unroll
+      for (int q = 0; q < CG_PT; ++q)
+        if (V.on[q]) buf[V.off[q]] = x[q];
+      __syncthreads();
+      tog ^= 1;
+    }
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) {
+      float2 r = b[q];
+      if (!(zero && j == 0) && V.on[q]) {
+        const float2 p = V.apply(buf, x[q], q, z0);
+        r = csub(r, make_float2(p.x * V.it, p.y * V.it));
+      }
+      x[q] = cfma(wj, r, x[q]);
+    }
+  }
+}
+
 template <int S, int DIM>
 __global__ void __launch_bounds__(CG_THREADS, 1)
 k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, const CoarseLU* __restrict__ lus,
-              int nu1, int nu2) {
+              const float2* __restrict__ pw, int nu1, int nu2) {
   extern __shared__ __align__(16) float2 cgsm[];
   __shared__ LevelDev<float2> Ls[MAX_COARSE_LEVELS_HOST];
   __shared__ int s_base[MAX_COARSE_LEVELS_HOST], s_cof[MAX_COARSE_LEVELS_HOST];
@@ -210,6 +240,26 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
       k0[q] = V.on[q] ? V.b[V.off[q]] : make_float2(0.f, 0.f);
       x[q] = make_float2(0.f, 0.f);
     }
+    if constexpr (S == 0) {
+      if (nu1 > 0) {
+        int tog = 0;
+        for (int sw = 0; sw < nu1; ++sw)
+          cg_poly<S, DIM>(V, k0, x, pw + 3 * ((size_t)prob * lev_stride + l), sw == 0, tog);
+        __syncthreads();  // the last step's readers of V.x are done
+#pragma unroll
+        for (int q = 0; q < CG_PT; ++q)
+          if (V.on[q]) V.x[V.off[q]] = x[q];
+        __syncthreads();
+        const float2 z0 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < CG_PT; ++q)
+          if (V.on[q]) {
+            const float2 p = V.apply(V.x, x[q], q, z0);
+            V.r[V.off[q]] = csub(k0[q], make_float2(p.x * V.it, p.y * V.it));
+          }
+        __syncthreads();
+      }
+    } else {
     const float2* R0 = V.b;
     for (int sw = 0; sw < nu1; ++sw) {
       float2 sg[S];
@@ -220,6 +270,7 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
       for (int q = 0; q < CG_PT; ++q)
         if (V.on[q]) V.r[V.off[q]] = k0[q];
       __syncthreads();
+    }
     }
     const float2* rr = nu1 > 0 ? V.r : V.b;
 #pragma unroll
@@ -319,7 +370,21 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
     for (int q = 0; q < CG_PT; ++q)
       if (V.on[q]) V.x[V.off[q]] = x[q];
     __syncthreads();
-    if (nu2 > 0) {
+    if constexpr (S == 0) {
+      if (nu2 > 0) {
+        float2 b[CG_PT];
+#pragma unroll
+        for (int q = 0; q < CG_PT; ++q) b[q] = V.on[q] ? V.b[V.off[q]] : make_float2(0.f, 0.f);
+        int tog = 1;  // V.x has just been written with x
+        for (int sw = 0; sw < nu2; ++sw)
+          cg_poly<S, DIM>(V, b, x, pw + 3 * ((size_t)prob * lev_stride + l), false, tog);
+        __syncthreads();  // the last step's readers of V.x are done
+#pragma unroll
+        for (int q = 0; q < CG_PT; ++q)
+          if (V.on[q]) V.x[V.off[q]] = x[q];
+        __syncthreads();
+      }
+    } else if (nu2 > 0) {
       float2 z0 = make_float2(0.f, 0.f);
 #pragma unroll
       for (int q = 0; q < CG_PT; ++q) {

@@ -510,6 +510,7 @@ struct Group {
   int nlev_c = 0;
   size_t coarse_smem = 0;          // dynamic shared memory of the staged coarse kernel (0: global)
   CoarseLU* dlu = nullptr;
+  C* pwc = nullptr;                // polynomial smoother: weights of the coarse levels [prob][level][3]
   struct Sub {
     int n = 0, cnt = 0, ntiles = 0, chunks = 1, m = 1;
     TileCfg cfg{8};
@@ -594,9 +595,9 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   // the split depends on the level sizes only, never on the other problems: a problem
   // whose finest level is already coarse runs its whole cycle in the coarse kernel
   g->tc = std::min(tthr, g->Lmax - 1);
-  // the polynomial smoother runs every level but the coarsest grid-wide; the coarse
-  // kernel then only solves the coarsest level
-  if (g->smoother == HELM_SMOOTHER_POLY) g->tc = g->Lmax - 1;
+  // in complex128 the polynomial smoother runs every level but the coarsest grid-wide; the
+  // coarse kernel then only solves the coarsest level
+  if (g->smoother == HELM_SMOOTHER_POLY && sizeof(C) == 16) g->tc = g->Lmax - 1;
   g->nlev_c = g->Lmax - g->tc;
   (void)maxoff;
   {
@@ -608,7 +609,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     if (sizeof(C) == 8) {
       std::vector<int> ns;
       for (int t = g->tc; t < g->Lmax; ++t) ns.push_back(big->lev[t].n);
-      bytes = coarse_gram_smem(g->dim, g->s, ns.data(), (int)ns.size());
+      bytes = coarse_gram_smem(g->dim, g->smoother == HELM_SMOOTHER_POLY ? 0 : g->s, ns.data(), (int)ns.size());
     }
     g->coarse_smem = (g->nlev_c <= MAX_COARSE_LEVELS_HOST && bytes <= 200 * 1024) ? bytes : 0;
   }
@@ -648,13 +649,23 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   }
   std::vector<LevelDev<C>> coarse;
   std::vector<CoarseLU> lus;
+  std::vector<C> pwc;  // polynomial smoother: three weights per coarse level (complex64)
   for (int p = 0; p < count; ++p) {
     // the problem's coarse levels (depths t0 .. Lmax-1) first, then padding up to the stride
     const int t0 = std::max(g->tc, off[p]);
     const int coarsest = (int)hs[p]->lev.size() - 1;
     for (int k = 0; k < g->nlev_c; ++k) {
       const int t = t0 + k;
-      coarse.push_back(make_leveldev<C>(*hs[p], t < g->Lmax ? t - off[p] : coarsest));
+      const int l = t < g->Lmax ? t - off[p] : coarsest;
+      coarse.push_back(make_leveldev<C>(*hs[p], l));
+      if (g->smoother == HELM_SMOOTHER_POLY)
+        for (int j = 0; j < 3; ++j) {
+          const cplx wj = l < coarsest ? hs[p]->polyw[l][j] : cplx(0.0);
+          C v;
+          v.x = (decltype(v.x))wj.real();
+          v.y = (decltype(v.y))wj.imag();
+          pwc.push_back(v);
+        }
     }
     CoarseLU c;
     c.nlev = g->Lmax - t0;
@@ -693,7 +704,8 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   // one device allocation for every descriptor array
   size_t bytes = 0;
   for (int t = 0; t < g->tc; ++t) bytes += dep[t].size() * sizeof(LevelDev<C>) + pws[t].size() * sizeof(C) + 64;
-  bytes += coarse.size() * sizeof(LevelDev<C>) + lus.size() * sizeof(CoarseLU) + lev0.size() * sizeof(LevelDev<C>);
+  bytes += coarse.size() * sizeof(LevelDev<C>) + lus.size() * sizeof(CoarseLU) + lev0.size() * sizeof(LevelDev<C>) +
+           pwc.size() * sizeof(C) + 64;
   for (auto& v : subs) bytes += v.size() * sizeof(OuterDev<C>);
   bytes += 64 * (g->tc + subs.size() + 4);
   if (arena) {
@@ -744,6 +756,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     if (!pws[t].empty()) g->depth[t].pw = (C*)put(pws[t].data(), pws[t].size() * sizeof(C));
   g->dcoarse = (LevelDev<C>*)put(coarse.data(), coarse.size() * sizeof(LevelDev<C>));
   g->dlu = (CoarseLU*)put(lus.data(), lus.size() * sizeof(CoarseLU));
+  if (!pwc.empty()) g->pwc = (C*)put(pwc.data(), pwc.size() * sizeof(C));
   g->lev0 = (LevelDev<C>*)put(lev0.data(), lev0.size() * sizeof(LevelDev<C>));
   for (size_t q = 0; q < subs.size(); ++q) g->outer[q].d = (OuterDev<C>*)put(subs[q].data(), subs[q].size() * sizeof(OuterDev<C>));
   const GridBar gb0{0u, 0u};
@@ -766,7 +779,8 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
 template <typename C>
 static void launch_coarse_part(const Group<C>& g, cudaStream_t st) {
   if constexpr (sizeof(C) == 8)
-    launch_coarse_gram(g.dim, g.s, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
+    launch_coarse_gram(g.dim, g.smoother == HELM_SMOOTHER_POLY ? 0 : g.s, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.pwc,
+                       g.nu1, g.nu2, g.coarse_smem, st);
   else
     launch_coarse_smem<C>(g.dim, g.dcoarse, g.nlev_c, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
 }
@@ -793,10 +807,25 @@ static void run_vcycle_poly(const Group<C>& g, cudaStream_t st) {
       launch_poly_step<C>(dim, D.d, D.pw, D.cnt, D.nflat, src, dst, k % 3, st);
     }
   };
+  // 2D complex64: every sweep in one pass, with the transfers beside it.  Successive sweeps
+  // go through p_0 and p_1 in turn (a pass reads its source beyond the points it writes).
+  constexpr bool C64 = sizeof(C) == 8;
+  const bool fused = C64 && dim == 2;
   for (int t = 0; t < g.tc; ++t) {
     const auto& D = g.depth[t];
     const double pts = (double)D.cnt * (dim == 3 ? (double)(D.n + 1) * (D.n + 1) * (D.n + 1) : (double)(D.n + 1) * (D.n + 1));
     const bool fine = (t == 0);
+    if constexpr (C64) {
+      if (fused && g.nu1 > 0) {
+        for (int sw = 0; sw < g.nu1; ++sw) {
+          const bool last = sw == g.nu1 - 1;
+          Launch L(fine ? "vc.poly.l0" : "vc.poly.lc", st, pts * E * (sw == 0 ? 2.0 : 3.0) + (last ? pts * E * cf : 0.0), 0);
+          launch_poly2(D.d, D.pw, D.cnt, D.n, sw == 0 ? POLY_FROM_ZERO : POLY_FROM_VEC, sw % 2 ? POLY_P0 : POLY_P1,
+                       last ? POLY_XA : sw % 2 ? POLY_P1 : POLY_P0, last, st);
+        }
+        continue;
+      }
+    }
     if (g.nu1 == 0) {
       Launch L(fine ? "vc.poly.l0" : "vc.poly.lc", st, pts * E, 0);
       launch_poly_step<C>(dim, D.d, D.pw, D.cnt, D.nflat, POLY_NONE, POLY_XA, -1, st);  // x_a = 0
@@ -814,6 +843,16 @@ static void run_vcycle_poly(const Group<C>& g, cudaStream_t st) {
     const auto& D = g.depth[t];
     const double pts = (double)D.cnt * (dim == 3 ? (double)(D.n + 1) * (D.n + 1) * (D.n + 1) : (double)(D.n + 1) * (D.n + 1));
     const bool fine = (t == 0);
+    if constexpr (C64) {
+      if (fused && g.nu2 > 0) {
+        for (int sw = 0; sw < g.nu2; ++sw) {
+          Launch L(fine ? "vc.poly.l0" : "vc.poly.lc", st, pts * E * (3.0 + (sw == 0 ? cf : 0.0)), 0);
+          launch_poly2(D.d, D.pw, D.cnt, D.n, sw == 0 ? POLY_FROM_COARSE : POLY_FROM_VEC, sw % 2 ? POLY_P0 : POLY_P1,
+                       sw == g.nu2 - 1 ? POLY_XB : sw % 2 ? POLY_P1 : POLY_P0, false, st);
+        }
+        continue;
+      }
+    }
     {
       Launch L(fine ? "vc.prolong.l0" : "vc.prolong.lc", st, pts * E * (2.0 + cf), 0);
       launch_prolong<C>(dim, false, D.d, D.cnt, D.nflat, D.cfg, false, st);  // x_b = x_a + P e_c

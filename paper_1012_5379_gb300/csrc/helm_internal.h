@@ -241,9 +241,10 @@ void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const
                   bool store_last, bool phi, cudaStream_t st);
 void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
                   bool store_last);
-// the complex64 coarse sub-cycle; smem from coarse_gram_smem over its level sizes
+// the complex64 coarse sub-cycle (S = 0: polynomial smoother, weights pw[prob][level][3]); smem
+// from coarse_gram_smem over its level sizes
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                        int nu1, int nu2, size_t smem, cudaStream_t st);
+                        const float2* pw, int nu1, int nu2, size_t smem, cudaStream_t st);
 size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev);
 template <typename C>
 void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,

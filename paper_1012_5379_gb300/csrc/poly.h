@@ -20,4 +20,11 @@ void launch_poly_step(int dim, const LevelDev<C>* levs, const C* pw, int nprob, 
 template <typename C>
 void launch_poly_restrict(int dim, const LevelDev<C>* levs, int nprob, int nflat, int src, cudaStream_t st);
 
+// A whole sweep of the 2D complex64 smoother in one pass (poly.cuh): from zero, from the
+// vector `src`, or from x_a + P e_c; dst receives x, and with restrict_end the coarser
+// level's b receives the full weighting of b - M x.  dst must differ from src.
+constexpr int POLY_FROM_ZERO = 0, POLY_FROM_VEC = 1, POLY_FROM_COARSE = 2;
+void launch_poly2(const LevelDev<float2>* levs, const float2* pw, int nprob, int n, int from, int src, int dst,
+                  bool restrict_end, cudaStream_t st);
+
 }  // namespace helm

@@ -2,6 +2,8 @@
 // (coarse.cuh).
 #include "sweep.cuh"
 #include "coarse.cuh"
+#include "poly.cuh"
+#include "poly.h"
 #include "launch.cuh"
 
 #include <algorithm>
@@ -125,29 +127,51 @@ size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {
 
 template <int S, int DIM>
 static void launch_coarse_gram_sd(const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                                  int nu1, int nu2, size_t smem, cudaStream_t st) {
+                                  const float2* pw, int nu1, int nu2, size_t smem, cudaStream_t st) {
   thread_local size_t configured = 0;
   if (configured < smem) {
     cudaFuncSetAttribute(k_coarse_gram<S, DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     configured = smem;
   }
-  pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, nu1, nu2);
+  pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, pw, nu1, nu2);
 }
 
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                        int nu1, int nu2, size_t smem, cudaStream_t st) {
+                        const float2* pw, int nu1, int nu2, size_t smem, cudaStream_t st) {
 #define HELM_CG(SS)                                                                                   \
   case SS:                                                                                            \
-    if (dim == 2) launch_coarse_gram_sd<SS, 2>(levs, lev_stride, lus, nprob, nu1, nu2, smem, st);     \
-    else launch_coarse_gram_sd<SS, 3>(levs, lev_stride, lus, nprob, nu1, nu2, smem, st);              \
+    if (dim == 2) launch_coarse_gram_sd<SS, 2>(levs, lev_stride, lus, nprob, pw, nu1, nu2, smem, st); \
+    else launch_coarse_gram_sd<SS, 3>(levs, lev_stride, lus, nprob, pw, nu1, nu2, smem, st);          \
     break;
   switch (S) {
+    HELM_CG(0)
     HELM_CG(1)
     HELM_CG(2)
     HELM_CG(3)
     HELM_CG(4)
   }
 #undef HELM_CG
+}
+
+template <int SRC, int END>
+static void poly2(const LevelDev<float2>* levs, const float2* pw, int nprob, int n, int src, int dst, cudaStream_t st) {
+  // regions of 16 rows while 32-row ones would leave SMs idle (1023^2: 1849 of the larger)
+  if (n <= 300) {
+    const int units = po_units(2, SRC, END, n);
+    pdl_launch(k_poly2<2, SRC, END>, dim3(nprob * units), dim3(32, SW2_NW), 0, st, levs, pw, units, src, dst);
+  } else {
+    const int units = po_units(4, SRC, END, n);
+    pdl_launch(k_poly2<4, SRC, END>, dim3(nprob * units), dim3(32, SW2_NW), 0, st, levs, pw, units, src, dst);
+  }
+}
+
+void launch_poly2(const LevelDev<float2>* levs, const float2* pw, int nprob, int n, int from, int src, int dst,
+                  bool restrict_end, cudaStream_t st) {
+  if (from == POLY_FROM_COARSE) poly2<2, 0>(levs, pw, nprob, n, src, dst, st);
+  else if (from == POLY_FROM_ZERO && restrict_end) poly2<0, 1>(levs, pw, nprob, n, src, dst, st);
+  else if (from == POLY_FROM_ZERO) poly2<0, 0>(levs, pw, nprob, n, src, dst, st);
+  else if (restrict_end) poly2<1, 1>(levs, pw, nprob, n, src, dst, st);
+  else poly2<1, 0>(levs, pw, nprob, n, src, dst, st);
 }
 
 }  // namespace helm
