@@ -44,29 +44,195 @@ __global__ void k_scatter_phi(int dim, int n, int stride, int nf, const float* _
   }
 }
 
-template <typename C>
-__global__ void k_apply_dense(int dim, int n, const double2* __restrict__ ca, const double2* __restrict__ cd,
-                              const double2* __restrict__ cc, const float* __restrict__ phi, double phic,
-                              const C* __restrict__ v, C* __restrict__ w) {
-  const size_t npts = dim == 3 ? (size_t)n * n * n : (size_t)n * n;
-  auto at = [&](int x, int y, int z) -> C {
-    return inside(x, y, z, n) ? v[((size_t)z * n + y) * n + x] : czero<C>();
-  };
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < npts; i += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % n), y = (int)((i / n) % n), z = dim == 3 ? (int)(i / ((size_t)n * n)) : 0;
-    C diag = cadd(from_d<C>(cd[x]), from_d<C>(cd[y]));
-    C p = czero<C>();
-    p = cfma(from_d<C>(ca[x]), at(x - 1, y, z), p);
-    p = cfma(from_d<C>(cc[x]), at(x + 1, y, z), p);
-    p = cfma(from_d<C>(ca[y]), at(x, y - 1, z), p);
-    p = cfma(from_d<C>(cc[y]), at(x, y + 1, z), p);
-    if (dim == 3) {
-      diag = cadd(diag, from_d<C>(cd[z]));
-      p = cfma(from_d<C>(ca[z]), at(x, y, z - 1), p);
-      p = cfma(from_d<C>(cc[z]), at(x, y, z + 1), p);
+// w = A v in the natural layout.  A warp holds 32 neighbouring x positions of one row and
+// marches along the last axis (z in 3D, y in 2D): its coefficients of the other axes and
+// three values of the march stay in registers, the remaining neighbours come from L1.
+//
+// complex128 is bound by the FP64 pipe (one instruction per warp and 64 cycles, comparisons
+// and predicated-off ones too): seven complex products, the diagonal's sums and phi's
+// conversion are 34 instructions a point.  Outside the absorbing layers H's coefficients are
+// real, and almost everywhere a node's two neighbours on an axis share one coefficient, so
+// an axis takes four instructions (AX_REAL), six (AX_SAME: the neighbours are added first)
+// or eight (AX_ANY), and three axes that share one coefficient fourteen (EVEN).  The cases
+// are uniform over a warp; each is a body of its own behind a switch, as bodies of one axis
+// would be predicated and all of them paid.  Coefficients are compared on their bits and phi
+// is widened on the integer pipes.  H at 255^3: 961 -> 633 us, M 959 -> 760; 2047^2 H 168 -> 118.
+//
+// complex64 is bound by HBM (its coefficients are narrowed on the integer pipes, those of the
+// march once for a warp's rows: converting six a point on the FP64 pipe bound it): 255^3 with
+// a field 488 -> 158 us, 2047^2 88 -> 21.
+__device__ __forceinline__ float narrow(double v) {  // round to nearest even
+  const unsigned hi = __double2hiint(v), lo = __double2loint(v), e = (hi >> 20) & 0x7ffu;
+  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);  // +-0
+  if (e - 897u >= 254u) return (float)v;                   // subnormal, huge, infinite, NaN
+  unsigned u = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  u += rest > 0x10000000u || (rest == 0x10000000u && (u & 1u));  // a carry moves the exponent up
+  return __uint_as_float(u);
+}
+template <typename C> __device__ __forceinline__ C dense_coef(const double2* p);
+template <> __device__ __forceinline__ double2 dense_coef<double2>(const double2* p) { return __ldg(p); }
+template <> __device__ __forceinline__ float2 dense_coef<float2>(const double2* p) {
+  const double2 v = __ldg(p);
+  return make_float2(narrow(v.x), narrow(v.y));
+}
+enum { AX_REAL, AX_SAME, AX_ANY };
+enum { EVEN = 12, GENERAL = 13 };
+__device__ __forceinline__ int axis_case(double2 a, double2 c) {
+  const long long dx = __double_as_longlong(a.x) ^ __double_as_longlong(c.x);
+  const long long dy = __double_as_longlong(a.y) ^ __double_as_longlong(c.y);
+  if (((__double_as_longlong(a.y) | __double_as_longlong(c.y)) << 1) == 0) return AX_REAL;
+  return (dx | dy) == 0 ? AX_SAME : AX_ANY;
+}
+template <int CASE, typename C>
+__device__ __forceinline__ C axis_terms(C p, C a, C c, C vm, C vp) {
+  if (CASE == AX_REAL) {
+    p.x = fma(a.x, vm.x, p.x);
+    p.y = fma(a.x, vm.y, p.y);
+    p.x = fma(c.x, vp.x, p.x);
+    p.y = fma(c.x, vp.y, p.y);
+    return p;
+  }
+  if (CASE == AX_SAME) return cfma(a, cadd(vm, vp), p);
+  return cfma(c, vp, cfma(a, vm, p));
+}
+// One value of w: axis terms by case, then the diagonal dxy + dz - f.
+template <int CX, int CY, int CZ, int DIM, typename C, typename R>
+__device__ __forceinline__ C dense_point(C ax, C qx, C ay, C qy, C az, C qz, C dxy, C dz, R f, C xm, C xp, C ym, C yp,
+                                         C vm, C vp, C v0) {
+  constexpr bool real = CX == AX_REAL && CY == AX_REAL && CZ == AX_REAL;
+  C p = axis_terms<CX>(czero<C>(), ax, qx, xm, xp);
+  if (DIM == 3) p = axis_terms<CY>(p, ay, qy, ym, yp);
+  p = axis_terms<CZ>(p, az, qz, vm, vp);
+  C d = dxy;
+  d.x += dz.x;
+  d.x -= f;
+  if (real) {
+    p.x = fma(d.x, v0.x, p.x);
+    p.y = fma(d.x, v0.y, p.y);
+    return p;
+  }
+  d.y += dz.y;
+  return cfma(d, v0, p);
+}
+
+template <typename C, int DIM>
+__global__ void __launch_bounds__(256, 3)
+k_apply_dense(int n, int rows, const double2* __restrict__ ca, const double2* __restrict__ cd,
+              const double2* __restrict__ cc, const float* __restrict__ phi, double phic,
+              const C* __restrict__ v, C* __restrict__ w) {
+  typedef typename CT<C>::R R;
+  const int ntx = (n + 31) / 32, nty = DIM == 3 ? (n + 7) / 8 : 1;
+  const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, bz = blockIdx.x / (ntx * nty);
+  const int x = bx * 32 + threadIdx.x;
+  const int y = DIM == 3 ? by * 8 + threadIdx.y : 0;              // the middle axis (3D)
+  const int m0 = (DIM == 3 ? bz : bz * 8 + threadIdx.y) * rows;   // the marched axis
+  const int m1 = min(m0 + rows, n);
+  const bool on = x < n && y < n;
+  const C zero = czero<C>();
+  auto coef = [&](const double2* p, int i) { return dense_coef<C>(p + i); };
+  C ax = zero, qx = zero, ay = zero, qy = zero, dxy = zero;
+  if (on) {
+    ax = coef(ca, x);
+    qx = coef(cc, x);
+    dxy = coef(cd, x);
+    if (DIM == 3) {
+      ay = coef(ca, y);
+      qy = coef(cc, y);
+      dxy = cadd(dxy, coef(cd, y));
     }
-    diag.x -= phi ? (typename CT<C>::R)phi[pidx(x, y, z, n + 1)] : (typename CT<C>::R)phic;
-    w[i] = cfma(diag, v[i], p);
+  }
+  int cx = GENERAL, cy = 0;
+  bool even = false;
+  if constexpr (sizeof(C) == 16) {  // uniform over the warp: lanes past the edge agree with any case
+    const unsigned full = 0xffffffffu;
+    const int lx = on ? axis_case(ax, qx) : -1;
+    cx = __all_sync(full, lx <= AX_REAL) ? AX_REAL : __all_sync(full, lx < 0 || lx == AX_SAME) ? AX_SAME : AX_ANY;
+    if (DIM == 3) {
+      const int ly = on ? axis_case(ay, qy) : -1;
+      cy = __all_sync(full, ly <= AX_REAL) ? AX_REAL : __all_sync(full, ly < 0 || ly == AX_SAME) ? AX_SAME : AX_ANY;
+      const long long dx = __double_as_longlong(ax.x) ^ __double_as_longlong(ay.x);
+      const long long dy = __double_as_longlong(ax.y) ^ __double_as_longlong(ay.y);
+      even = cx == AX_SAME && cy == AX_SAME && __all_sync(full, !on || (dx | dy) == 0);
+    }
+  }
+  const size_t plane = DIM == 3 ? (size_t)n * n : (size_t)n;      // one step of the march
+  const size_t col = (size_t)y * n + x;
+  const C* vc = v + col;
+  auto at = [&](int m) { return on && (unsigned)m < (unsigned)n ? vc[m * plane] : zero; };
+  if (m0 >= n) return;
+  C la = zero, ld = zero, lc = zero;  // complex64: lane i's are those of row m0 + i (rows <= 32)
+  if (sizeof(C) == 8 && m0 + (int)threadIdx.x < m1) {
+    la = coef(ca, m0 + threadIdx.x);
+    ld = coef(cd, m0 + threadIdx.x);
+    lc = coef(cc, m0 + threadIdx.x);
+  }
+  C vm = at(m0 - 1), v0 = at(m0);
+  for (int m = m0; m < m1; ++m) {
+    const C vp = at(m + 1);
+    C az, qz, dz;
+    if constexpr (sizeof(C) == 8) {
+      auto row = [&](C c) {
+        return make_float2(__shfl_sync(0xffffffffu, c.x, m - m0), __shfl_sync(0xffffffffu, c.y, m - m0));
+      };
+      az = row(la), qz = row(lc), dz = row(ld);
+    } else {
+      az = coef(ca, m), qz = coef(cc, m), dz = coef(cd, m);
+    }
+    if (on) {
+      const C* q = vc + m * plane;
+      const C xm = x > 0 ? q[-1] : zero, xp = x < n - 1 ? q[1] : zero;
+      C ym = zero, yp = zero;
+      if (DIM == 3) {
+        ym = y > 0 ? q[-n] : zero;
+        yp = y < n - 1 ? q[n] : zero;
+      }
+      const size_t pp = (DIM == 3 ? ((size_t)m * (n + 1) + y) : (size_t)m) * (n + 1) + x;  // padded
+      R f;
+      if constexpr (sizeof(C) == 16) f = phi ? widen(__ldg(phi + pp)) : phic;
+      else f = phi ? __ldg(phi + pp) : (R)phic;
+      C p;
+#define DENSE(X, Y, Z) dense_point<X, Y, Z, DIM>(ax, qx, ay, qy, az, qz, dxy, dz, f, xm, xp, ym, yp, vm, vp, v0)
+      if constexpr (sizeof(C) == 16) {
+        const int cz = axis_case(az, qz);  // of the row: uniform
+        int mode = cy == AX_ANY || cz == AX_ANY ? GENERAL : (cx * 2 + cy) * 2 + cz;
+        if (DIM == 3 && even && cz == AX_SAME) {
+          const long long dx = __double_as_longlong(ax.x) ^ __double_as_longlong(az.x);
+          const long long dy = __double_as_longlong(ax.y) ^ __double_as_longlong(az.y);
+          if (__all_sync(__activemask(), (dx | dy) == 0)) mode = EVEN;
+        }
+        switch (mode) {
+          case 0: p = DENSE(AX_REAL, AX_REAL, AX_REAL); break;
+          case 1: p = DENSE(AX_REAL, AX_REAL, AX_SAME); break;
+          case 4: p = DENSE(AX_SAME, AX_REAL, AX_REAL); break;
+          case 5: p = DENSE(AX_SAME, AX_REAL, AX_SAME); break;
+          case 8: p = DENSE(AX_ANY, AX_REAL, AX_REAL); break;
+          case 9: p = DENSE(AX_ANY, AX_REAL, AX_SAME); break;
+          case 2: if (DIM == 3) { p = DENSE(AX_REAL, AX_SAME, AX_REAL); break; }
+          case 3: if (DIM == 3) { p = DENSE(AX_REAL, AX_SAME, AX_SAME); break; }
+          case 6: if (DIM == 3) { p = DENSE(AX_SAME, AX_SAME, AX_REAL); break; }
+          case 7: if (DIM == 3) { p = DENSE(AX_SAME, AX_SAME, AX_SAME); break; }
+          case 10: if (DIM == 3) { p = DENSE(AX_ANY, AX_SAME, AX_REAL); break; }
+          case 11: if (DIM == 3) { p = DENSE(AX_ANY, AX_SAME, AX_SAME); break; }
+          case EVEN:
+            if (DIM == 3) {
+              const C s = cadd(cadd(cadd(xm, xp), cadd(ym, yp)), cadd(vm, vp));
+              p = cmul(az, s);
+              C d = cadd(dxy, dz);
+              d.x -= f;
+              p = cfma(d, v0, p);
+              break;
+            }
+          default: p = DENSE(AX_ANY, AX_ANY, AX_ANY); break;
+        }
+      } else {
+        p = DENSE(AX_ANY, AX_ANY, AX_ANY);
+      }
+#undef DENSE
+      w[col + m * plane] = p;
+    }
+    vm = v0;
+    v0 = vp;
   }
 }
 
@@ -84,12 +250,24 @@ void scatter_phi(int dim, int n_level, int stride, int n_fine, const float* phi_
 }
 void apply_operator_dense(int dim, int n, const double2* ca, const double2* cd, const double2* cc,
                           const float* phi_pad, double phic, const void* v, void* w, int prec, cudaStream_t st) {
-  const size_t nn = n;
-  const int grid = grid_for(dim == 3 ? nn * nn * nn : nn * nn);
-  if (prec == HELM_C128)
-    k_apply_dense<double2><<<grid, 256, 0, st>>>(dim, n, ca, cd, cc, phi_pad, phic, (const double2*)v, (double2*)w);
-  else
-    k_apply_dense<float2><<<grid, 256, 0, st>>>(dim, n, ca, cd, cc, phi_pad, phic, (const float2*)v, (float2*)w);
+  // rows per march: 8 (a plane is read from L2 1.25 times), fewer while that leaves fewer
+  // than eight warps on each SM sub-partition
+  const int ntx = (n + 31) / 32, lines = dim == 3 ? ntx * ((n + 7) / 8) * 8 : ntx;
+  int rows = 8;
+  while (rows > 1 && (long long)lines * ((n + rows - 1) / rows) < 152LL * 32) rows /= 2;
+  const int chunks = (n + rows - 1) / rows;
+  const dim3 block(32, 8);
+  const int grid = dim == 3 ? ntx * ((n + 7) / 8) * chunks : ntx * ((chunks + 7) / 8);
+  if (dim == 3) {
+    if (prec == HELM_C128)
+      k_apply_dense<double2, 3><<<grid, block, 0, st>>>(n, rows, ca, cd, cc, phi_pad, phic, (const double2*)v, (double2*)w);
+    else
+      k_apply_dense<float2, 3><<<grid, block, 0, st>>>(n, rows, ca, cd, cc, phi_pad, phic, (const float2*)v, (float2*)w);
+  } else if (prec == HELM_C128) {
+    k_apply_dense<double2, 2><<<grid, block, 0, st>>>(n, rows, ca, cd, cc, phi_pad, phic, (const double2*)v, (double2*)w);
+  } else {
+    k_apply_dense<float2, 2><<<grid, block, 0, st>>>(n, rows, ca, cd, cc, phi_pad, phic, (const float2*)v, (float2*)w);
+  }
 }
 
 }  // namespace helm
