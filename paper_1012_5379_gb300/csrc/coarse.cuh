@@ -174,7 +174,7 @@ __device__ __forceinline__ void cg_poly(const CgLevel<S, DIM>& V, const float2 (
 template <int S, int DIM>
 __global__ void __launch_bounds__(CG_THREADS, 1)
 k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, const CoarseLU* __restrict__ lus,
-              const float2* __restrict__ pw, int nu1, int nu2) {
+              const float2* __restrict__ pw, int nu1, int nu2, int from_res) {
   extern __shared__ __align__(16) float2 cgsm[];
   __shared__ LevelDev<float2> Ls[MAX_COARSE_LEVELS_HOST];
   __shared__ int s_base[MAX_COARSE_LEVELS_HOST], s_cof[MAX_COARSE_LEVELS_HOST];
@@ -227,9 +227,36 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
   enter(0);
   pdl_wait();
   pdl_trigger();
+  if (S > 0 && DIM == 2 && from_res && !Ls[0].top) {
+    // b = full weighting of the finer level's residual (k_sweep2_down does the same)
+    const LevelDev<float2>& L = Ls[0];
+    const int m = L.scf->m, Pf = 2 * L.P;
+    float2 rc[S + 1];
 #pragma unroll
-  for (int q = 0; q < CG_PT; ++q)
-    if (V.on[q]) V.b[V.off[q]] = G[0].b[V.off[q]];
+    for (int j = 0; j <= S; ++j) rc[j] = L.scf->rcoef[j];
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) {
+      if (!V.on[q]) continue;
+      const size_t f = (size_t)(2 * V.cy[q]) * Pf + 2 * V.cx[q];
+      float2 out = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          const size_t i = f + (size_t)dy * Pf + dx;
+          float2 r = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int j = 0; j <= S; ++j)
+            if (j <= m) r = cfma(rc[j], j == 0 ? L.fb[i] : L.fp[j > 0 ? j - 1 : 0][i], r);
+          out = cadd(out, cscale(r, (dx == 1 ? 0.5f : 0.25f) * (dy == 1 ? 0.5f : 0.25f)));
+        }
+      V.b[V.off[q]] = out;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q)
+      if (V.on[q]) V.b[V.off[q]] = G[0].b[V.off[q]];
+  }
   __syncthreads();
   // descent
   for (int l = 0; l < nlev - 1; ++l) {

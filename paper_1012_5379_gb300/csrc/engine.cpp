@@ -185,6 +185,15 @@ static int compute_poly_weights(Handle* h, const std::vector<int>& sizes) {
   return HELM_OK;
 }
 
+// 2D complex64 levels whose V(1,1) passes are fused (sweep.cuh).
+static bool fused2_cycle(int dim, int prec, int smoother, int nu1, int nu2) {
+  return dim == 2 && prec == HELM_C64 && smoother == HELM_SMOOTHER_GMRES && nu1 == 1 && nu2 == 1;
+}
+static bool fused2_level(const Handle& h, const HostLevel& L) {
+  return fused2_cycle(h.dim, h.prec, h.smoother, h.nu1, h.nu2) && fused2_size(L.n) &&
+         L.n > coarse_threshold(2, HELM_C64);
+}
+
 int setup_handle(const helm_grid* grid, const float* phi, double k, double theta_beta, const helm_opts* opts,
                  cudaStream_t st, Handle** out) {
   if (!grid || !out) { set_error("grid and out must not be NULL"); return HELM_EINVAL; }
@@ -299,6 +308,14 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     TRY(dev_alloc(h.get(), &L.r0, L.np * eb));
     for (int j = 0; j < h->s; ++j) TRY(dev_alloc(h.get(), &L.p[j], L.np * eb));
     for (void* v : {L.b, L.xa, L.xb, L.r0}) CUDA_TRY(cudaMemsetAsync(v, 0, L.np * eb, st));
+    if (h->prec == HELM_C64) L.sweep = sweep_cfg(h->dim, L.n, h->s, sm_count_host());
+    if (fused2_level(*h, L)) {
+      L.q[0] = L.xa;
+      for (int j = 1; j < h->s - 1; ++j) {
+        TRY(dev_alloc(h.get(), &L.q[j], L.np * eb));
+        CUDA_TRY(cudaMemsetAsync(L.q[j], 0, L.np * eb, st));
+      }
+    }
     for (int j = 0; j < h->s; ++j) CUDA_TRY(cudaMemsetAsync(L.p[j], 0, L.np * eb, st));
     const size_t scb = h->prec == HELM_C128 ? sizeof(SweepScalarsT<double>) : sizeof(SweepScalarsT<float>);
     TRY(dev_alloc(h.get(), &L.sc, scb));
@@ -312,10 +329,8 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
       nparts = std::max<size_t>(nparts, tiles_per_problem(3, L.P, finest));
     }
     size_t part_bytes = nparts * NPART * sizeof(double);
-    if (h->prec == HELM_C64) {
-      L.sweep = sweep_cfg(h->dim, L.n, h->s, sm_count_host());
-      part_bytes = std::max(part_bytes, (size_t)L.sweep.units * GRAM_SLOT * sizeof(float2));
-    }
+    if (h->prec == HELM_C64)
+      part_bytes = std::max(part_bytes, (size_t)std::max(L.sweep.units, L.sweep.units_res) * GRAM_SLOT * sizeof(float2));
     TRY(dev_alloc(h.get(), &L.part, part_bytes));
     // TMA maps of the vectors the large 3D complex64 levels' passes stream (two sets, for
     // column tiles of 16 and of 32 rows)
@@ -449,6 +464,13 @@ static LevelDev<C> make_leveldev(const Handle& h, int l) {
     d.xcb = (const C*)Lc.xb;
     d.scc = (SS*)Lc.sc;
   }
+  for (int j = 0; j < SMAX; ++j) d.q[j] = (C*)L.q[j];
+  if (l > 0) {
+    const HostLevel& Lf = h.lev[l - 1];
+    d.fb = (const C*)Lf.b;
+    for (int j = 0; j < SMAX; ++j) d.fp[j] = (const C*)Lf.p[j];
+    d.scf = (const SS*)Lf.sc;
+  }
   return d;
 }
 
@@ -521,6 +543,13 @@ struct Group {
   std::vector<Sub> outer;
   LevelDev<C>* lev0 = nullptr;   // level-0 descriptors of all problems (single problem: [0])
   int lev0_nflat = 1;
+  bool fuse2 = false;            // fused 2D passes at the depths t < tp (sweep.cuh)
+  // finest levels whose last update run_vcycle leaves to its caller's next pass
+  LevelDev<C>* pend = nullptr;
+  int npend = 0;
+  bool fused(int t) const { return fuse2 && t < tp && fused2_size(depth[t].n); }
+  // the restriction from depth t - 1 is part of depth t's pass (t = tc: of the coarse kernel)
+  bool fused_down(int t) const { return t < tc ? fused(t) : fuse2 && tc > 0 && tp == tc; }
   GridBar* gbar = nullptr;       // grid barrier of the persistent segments
   int tp = 0;                    // first depth of the persistent segments (tc: none)
   void* dmem = nullptr;
@@ -647,6 +676,24 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
       D.ntiles = g->dim == 3 ? tiles_per_problem(3, L.P, D.cfg) : L.ntiles;
     }
   }
+  // the persistent segments: the deepest run of grid-wide levels that qualify
+  // (bounded by the pass list's capacity: a depth records nu1 (s + 1) passes going down
+  // and 1 + nu2 (s + 1) coming up)
+  g->tp = g->tc;
+  const int per_depth = std::max(g->nu1 == 0 ? 1 : g->nu1 * (g->s + 1), 1 + g->nu2 * (g->s + 1));
+  if (g->smoother == HELM_SMOOTHER_GMRES)
+    while (g->tp > 0 && (g->tc - g->tp + 1) * per_depth <= SEQ_MAX &&
+           persist_level(g->dim, g->depth[g->tp - 1].n + 1, (int)sizeof(C)))
+      --g->tp;
+  g->fuse2 = fused2_cycle(g->dim, h0.prec, g->smoother, g->nu1, g->nu2);
+  for (int t = 0; t + 1 < g->tp && g->fuse2; ++t)  // depth t reads depth t + 1's last sweep
+    for (size_t k = 0, p = 0; p < (size_t)count; ++p) {
+      if (off[p] > t) continue;
+      const HostLevel& Lc = hs[p]->lev[t + 1 - off[p]];
+      LevelDev<C>& d = dep[t][k++];
+      d.cr0 = (const C*)Lc.r0;
+      for (int j = 0; j < SMAX; ++j) d.cp[j] = (const C*)(g->fused(t + 1) ? Lc.q[j] : Lc.p[j]);
+    }
   std::vector<LevelDev<C>> coarse;
   std::vector<CoarseLU> lus;
   std::vector<C> pwc;  // polynomial smoother: three weights per coarse level (complex64)
@@ -679,6 +726,15 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   std::vector<LevelDev<C>> lev0;
   for (int p = 0; p < count; ++p) lev0.push_back(make_leveldev<C>(*hs[p], 0));
   g->lev0_nflat = hs[0]->lev[0].nflat;
+  std::vector<LevelDev<C>> pend;
+  if (g->smoother == HELM_SMOOTHER_GMRES && g->nu2 > 0)
+    for (int p = 0; p < count; ++p) {
+      if (off[p] >= g->tp || (off[p] > 0 && !g->fuse2)) continue;
+      pend.push_back(lev0[p]);
+      if (g->fused(off[p]))
+        for (int j = 0; j < SMAX; ++j) pend.back().p[j] = pend.back().q[j];
+    }
+  g->npend = (int)pend.size();
   // outer subgroups by top size
   std::vector<std::vector<OuterDev<C>>> subs;
   for (int p = 0; p < count; ++p) {
@@ -704,7 +760,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   // one device allocation for every descriptor array
   size_t bytes = 0;
   for (int t = 0; t < g->tc; ++t) bytes += dep[t].size() * sizeof(LevelDev<C>) + pws[t].size() * sizeof(C) + 64;
-  bytes += coarse.size() * sizeof(LevelDev<C>) + lus.size() * sizeof(CoarseLU) + lev0.size() * sizeof(LevelDev<C>) +
+  bytes += coarse.size() * sizeof(LevelDev<C>) + lus.size() * sizeof(CoarseLU) + 2 * lev0.size() * sizeof(LevelDev<C>) +
            pwc.size() * sizeof(C) + 64;
   for (auto& v : subs) bytes += v.size() * sizeof(OuterDev<C>);
   bytes += 64 * (g->tc + subs.size() + 4);
@@ -758,18 +814,10 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   g->dlu = (CoarseLU*)put(lus.data(), lus.size() * sizeof(CoarseLU));
   if (!pwc.empty()) g->pwc = (C*)put(pwc.data(), pwc.size() * sizeof(C));
   g->lev0 = (LevelDev<C>*)put(lev0.data(), lev0.size() * sizeof(LevelDev<C>));
+  g->pend = (LevelDev<C>*)put(pend.data(), pend.size() * sizeof(LevelDev<C>));
   for (size_t q = 0; q < subs.size(); ++q) g->outer[q].d = (OuterDev<C>*)put(subs[q].data(), subs[q].size() * sizeof(OuterDev<C>));
   const GridBar gb0{0u, 0u};
   g->gbar = (GridBar*)put(&gb0, sizeof(GridBar));
-  // the persistent segments: the deepest run of grid-wide levels that qualify
-  // (bounded by the pass list's capacity: a depth records nu1 (s + 1) passes going down
-  // and 1 + nu2 (s + 1) coming up)
-  g->tp = g->tc;
-  const int per_depth = std::max(g->nu1 == 0 ? 1 : g->nu1 * (g->s + 1), 1 + g->nu2 * (g->s + 1));
-  if (g->smoother == HELM_SMOOTHER_GMRES)
-    while (g->tp > 0 && (g->tc - g->tp + 1) * per_depth <= SEQ_MAX &&
-           persist_level(g->dim, g->depth[g->tp - 1].n + 1, (int)sizeof(C)))
-      --g->tp;
   CUDA_TRY(cudaGetLastError());
   if (!arena) CUDA_TRY(cudaStreamSynchronize(st));
   return HELM_OK;
@@ -780,7 +828,7 @@ template <typename C>
 static void launch_coarse_part(const Group<C>& g, cudaStream_t st) {
   if constexpr (sizeof(C) == 8)
     launch_coarse_gram(g.dim, g.smoother == HELM_SMOOTHER_POLY ? 0 : g.s, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.pwc,
-                       g.nu1, g.nu2, g.coarse_smem, st);
+                       g.nu1, g.nu2, g.fused_down(g.tc), g.coarse_smem, st);
   else
     launch_coarse_smem<C>(g.dim, g.dcoarse, g.nlev_c, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
 }
@@ -861,8 +909,9 @@ static void run_vcycle_poly(const Group<C>& g, cudaStream_t st) {
   }
 }
 
+// With `defer` the last update of the problems in g.pend is left to the caller's next pass.
 template <typename C>
-static void run_vcycle(const Group<C>& g, cudaStream_t st) {
+static void run_vcycle(const Group<C>& g, cudaStream_t st, bool defer = false) {
   if (g.smoother == HELM_SMOOTHER_POLY) {
     run_vcycle_poly<C>(g, st);
     return;
@@ -927,7 +976,18 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
       continue;
     }
     for (int sw = 0; sw < g.nu1; ++sw) {
-      arnoldi(D, sw == 0, true, fine, rec, ph, pts);
+      if constexpr (sizeof(C) == 8) {
+        if (t > 0 && g.fused(t)) {  // with the restriction to this level
+          Launch L("vc.arnoldi.lc", st, pts * (E * ((g.s + 1) * (1.0 / cf) + g.s + 1) + ph), 0);
+          launch_fused2(FUSED2_DOWN, g.s, D.d, D.cnt, D.n, D.sweep, false, st);
+          if (g.fused_down(t + 1)) continue;
+        } else {
+          arnoldi(D, sw == 0, true, fine, rec, ph, pts);
+          if (!rec && g.fused_down(t + 1)) continue;
+        }
+      } else {
+        arnoldi(D, sw == 0, true, fine, rec, ph, pts);
+      }
       if (sw < g.nu1 - 1) {
         if (rec) {
           record_update<C>(seq, dim, UPD_RESIDUAL, D.d, D.cnt, D.nflat, sw == 0, 0, sw == 0);
@@ -960,6 +1020,23 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
     if (!rec) flush("vc.seq.up");
     const double ph = g.hs[0]->has_phi ? 4.0 : 0.0;
     const double pbytes = g.nu2 > 0 ? pts * (E * (4.0 + cf) + ph) : pts * E * (2.0 + cf);
+    if constexpr (sizeof(C) == 8) {
+      if (g.fuse2 && !rec) {
+        const double ebytes = pts * E * cf * (t + 1 < g.tp ? g.s + 1.0 : 1.0);
+        if (g.fused(t)) {
+          Launch L(fine ? "vc.prolong.l0" : "vc.prolong.lc", st, pts * (E * (2.0 * g.s + 1) + ph) + ebytes, 0);
+          launch_fused2(FUSED2_UP, g.s, D.d, D.cnt, D.n, D.sweep, true, st);
+        } else {
+          const bool xk = g.fused_down(t + 1);
+          {
+            Launch L(fine ? "vc.prolong.l0" : "vc.prolong.lc", st, pts * (E * (xk ? g.s + 2.0 : 4.0) + ph) + ebytes, 0);
+            launch_fused2(FUSED2_PROLONG, g.s, D.d, D.cnt, D.n, D.sweep, xk, st);
+          }
+          arnoldi(D, false, false, fine, false, ph, pts);
+        }
+        continue;
+      }
+    }
     if (rec) {
       record_prolong<C>(seq, dim, g.nu2 > 0, D.d, D.cnt, g.nu2 > 0 ? D.ntiles : D.nflat, D.cfg);
       seq_bytes += pbytes;
@@ -976,11 +1053,18 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st) {
         seq_bytes += pts * E * (last ? g.s + 2.0 : g.s + 4.0);
         continue;
       }
+      if (last && fine) continue;  // with the others in g.pend
       Launch L(fine ? "vc.update.l0" : "vc.update.lc", st, pts * E * (last ? g.s + 2.0 : g.s + 4.0), 0);
       launch_update_flat<C>(dim, last ? UPD_XONLY : UPD_RESIDUAL, D.d, D.cnt, D.nflat, false, 1, false, st);
     }
   }
   flush("vc.seq.up");
+  if (g.npend > 0 && !defer) {
+    double pts = 0;
+    for (const Handle* h : g.hs) pts += (double)h->lev[0].np;
+    Launch L("vc.update.l0", st, pts * E * (g.s + 2.0), 0);
+    launch_update_flat<C>(dim, UPD_XONLY, g.pend, g.npend, g.lev0_nflat, false, 1, false, st);
+  }
 }
 
 // Host work of group (re)builds and V-cycle graph captures, for the serving counters.
@@ -1056,10 +1140,10 @@ static int precond_apply_t(Handle* h, const void* r, void* z, int prec, cudaStre
     Launch L("io.load", st, 0, 0);
     launch_load_input<C>(h->dim, g->lev0, g->lev0_nflat, r, prec, st);
   }
-  run_vcycle<C>(*g, st);
+  run_vcycle<C>(*g, st, true);
   {
     Launch L("io.store", st, 0, 0);
-    launch_store_output<C>(h->dim, h->n, g->lev0, z, prec, st);
+    launch_store_output<C>(h->dim, h->n, g->npend ? g->pend : g->lev0, g->npend > 0, z, prec, st);
   }
   CUDA_TRY(cudaGetLastError());
   return HELM_OK;
@@ -1576,7 +1660,11 @@ size_t estimate_handle_bytes(int dim, int n, int prec, int s, int restart, int m
   bytes += outer_part_doubles(outer_chunks(vs), (int)m) * sizeof(double);
   bytes += (size_t)outer_dot_counters(outer_chunks(vs)) * sizeof(unsigned);
   if (prec == HELM_C64)
-    for (int nl : sizes) bytes += (size_t)sweep_cfg(dim, nl, s, sm_count_host()).units * GRAM_SLOT * sizeof(float2);
+    for (int nl : sizes) {
+      const SweepCfg c = sweep_cfg(dim, nl, s, sm_count_host());
+      bytes += (size_t)std::max(c.units, c.units_res) * GRAM_SLOT * sizeof(float2);
+      if (dim == 2 && fused2_size(nl) && s > 2) bytes += (size_t)(s - 2) * (nl + 1) * (nl + 1) * eb;
+    }
   return bytes;
 }
 

@@ -44,6 +44,7 @@ struct HostLevel {
   void* xb = nullptr;
   void* r0 = nullptr;
   void* p[SMAX] = {nullptr, nullptr, nullptr, nullptr};
+  void* q[SMAX] = {nullptr, nullptr, nullptr, nullptr};  // fused passes: post-smoothing vectors (q[0] is xa)
   void* coef = nullptr;     // 3n complex (a | d | c) in the preconditioner precision
   double2* coef64 = nullptr;// the same in FP64
   float* phi = nullptr;     // padded phi or nullptr

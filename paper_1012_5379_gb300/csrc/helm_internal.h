@@ -89,6 +89,13 @@ struct LevelDev {
   float2 ksh;             // the stencil's diagonal in the interior, to 8 significant bits
   float2 klap;            // d / h^2 of the interior spacing (the Laplacian's scale)
   int top;                // 1: the problem's finest level
+  // fused 2D passes (sweep.cuh)
+  const C* fb;            // finer level: b, last descent vectors and sweep state
+  const C* fp[SMAX];
+  const SweepScalarsT<typename RealOf<C>::T>* scf;
+  C* q[SMAX];             // vectors of the fused post-smoothing sweep
+  const C* cr0;           // coarser level's post-smoothing sweep whose update is pending, or nullptr
+  const C* cp[SMAX];
 };
 
 // TMA maps per level: b, r0, p_1..p_SMAX (in this order).
@@ -195,6 +202,7 @@ HELM_HD inline int coarse_threshold(int dim, int prec) {
 // the device's SM count only.
 struct SweepCfg {
   int march, geo, units;
+  int units_res;  // CTAs of a sweep that starts from the residual of an iterate
 };
 SweepCfg sweep_cfg(int dim, int n, int S, int sms);
 
@@ -237,6 +245,12 @@ template <typename C>
 void launch_arnoldi(int dim, int J, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
                     bool store_p, cudaStream_t st);
 // the complex64 sweep's basis and minimisation (first: R_0 = b, else r0; store_last: keep k_S)
+// Fused 2D V(1,1) passes (sweep.cuh): a level's way down, its way up, and the coarse correction
+// of a marching level (xk: x_a formed from the last sweep).
+bool fused2_size(int n);  // whether a level of this size takes the fused passes
+enum { FUSED2_DOWN, FUSED2_UP, FUSED2_PROLONG };
+void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int n, const SweepCfg& cfg, bool xk,
+                   cudaStream_t st);
 void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
                   bool store_last, bool phi, cudaStream_t st);
 void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
@@ -244,7 +258,7 @@ void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, co
 // the complex64 coarse sub-cycle (S = 0: polynomial smoother, weights pw[prob][level][3]); smem
 // from coarse_gram_smem over its level sizes
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                        const float2* pw, int nu1, int nu2, size_t smem, cudaStream_t st);
+                        const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st);
 size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev);
 template <typename C>
 void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
@@ -281,7 +295,7 @@ void launch_coarse_smem(int dim, const LevelDev<C>* levs, int nlev, int lev_stri
 template <typename C>
 void launch_load_input(int dim, const LevelDev<C>* levs, int ntiles, const void* src, int in_prec, cudaStream_t st);
 template <typename C>
-void launch_store_output(int dim, int n, const LevelDev<C>* levs, void* dst, int out_prec, cudaStream_t st);
+void launch_store_output(int dim, int n, const LevelDev<C>* levs, bool update, void* dst, int out_prec, cudaStream_t st);
 
 // Outer FP64 kernels (outer.cu).
 template <typename C>

@@ -243,7 +243,7 @@ int run_noalloc(const helm_grid* grid, double k, double theta_beta, int nu1, int
   }
   {
     Launch L("noalloc.store", st, 0, 0);
-    launch_store_output<C>(dim, n, dlev, z, prec, st);
+    launch_store_output<C>(dim, n, dlev, false, z, prec, st);
   }
   NA_CUDA(cudaGetLastError());
   return HELM_OK;

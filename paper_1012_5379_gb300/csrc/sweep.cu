@@ -14,12 +14,15 @@ namespace helm {
 // 1023^2 25 against 37; at 511^2 and below a march of few rows is mostly halo.
 constexpr int SWEEP2_MARCH_N = 600;
 
+bool fused2_size(int n) { return n < SWEEP2_MARCH_N; }
+
 SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
-  SweepCfg c{0, 0, 1};
+  SweepCfg c{0, 0, 1, 1};
   if (dim == 2) {
     if (n < SWEEP2_MARCH_N || S > 3) {
       c.geo = n <= 255 ? 2 : 4;
       c.units = sw2_units(S, c.geo, n);
+      c.units_res = sw2_units(S + 1, c.geo, n);
       return c;
     }
     // rows per march: the fewest row steps of the SM that takes the most, four CTAs per SM
@@ -34,11 +37,12 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
         c.units = (int)units;
       }
     }
+    c.units_res = c.units;
     return c;
   }
   if (n < 96 || S > 3) {
     c.geo = n < 64 ? 4 : 8;
-    c.units = sw3_units(S, c.geo, n);
+    c.units_res = c.units = sw3_units(S, c.geo, n);
     return c;
   }
   // planes per march: the fewest plane steps of the CTA that takes the most, one CTA per SM
@@ -54,6 +58,7 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
       c.units = (int)units;
     }
   }
+  c.units_res = c.units;
   return c;
 }
 
@@ -65,8 +70,9 @@ static void launch_sweep_s(int dim, const LevelDev<float2>* levs, int nprob, con
   if (dim == 2) {
     if (!cfg.march) {
       const dim3 block(32, SW2_NW);
-      if (cfg.geo == 2) pdl_launch(k_sweep2<S, 2>, grid, block, 0, st, levs, cfg.units, f, sl);
-      else pdl_launch(k_sweep2<S, 4>, grid, block, 0, st, levs, cfg.units, f, sl);
+      const int units = first ? cfg.units : cfg.units_res;
+      if (cfg.geo == 2) pdl_launch(k_sweep2<S, 2>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
+      else pdl_launch(k_sweep2<S, 4>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
     } else if constexpr (S <= 3) {
       const dim3 block(32, SV2_NW);
       const size_t smem = sv2_smem(S, cfg.geo);  // at most 256 rows: below 48 KB
@@ -111,9 +117,36 @@ void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const
   }
 }
 
+template <int S>
+static void fused2(int pass, const LevelDev<float2>* levs, int nprob, int n, const SweepCfg& cfg, bool xk,
+                   cudaStream_t st) {
+  const dim3 block(32, SW2_NW);
+  if (pass == FUSED2_PROLONG) {
+    const int ntiles = ceil_div(n + 1, 64) * ceil_div(n + 1, 16);
+    pdl_launch(k_prolong2_gram<S>, dim3(nprob * ntiles), block, 0, st, levs, ntiles, xk ? 1 : 0);
+  } else if (pass == FUSED2_DOWN) {
+    if (cfg.geo == 2) pdl_launch(k_sweep2_down<S, 2>, dim3(nprob * cfg.units), block, 0, st, levs, cfg.units);
+    else pdl_launch(k_sweep2_down<S, 4>, dim3(nprob * cfg.units), block, 0, st, levs, cfg.units);
+  } else {
+    if (cfg.geo == 2) pdl_launch(k_sweep2_up<S, 2>, dim3(nprob * cfg.units_res), block, 0, st, levs, cfg.units_res);
+    else pdl_launch(k_sweep2_up<S, 4>, dim3(nprob * cfg.units_res), block, 0, st, levs, cfg.units_res);
+  }
+}
+
+void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int n, const SweepCfg& cfg, bool xk,
+                   cudaStream_t st) {
+  switch (S) {
+    case 1: fused2<1>(pass, levs, nprob, n, cfg, xk, st); break;
+    case 2: fused2<2>(pass, levs, nprob, n, cfg, xk, st); break;
+    case 3: fused2<3>(pass, levs, nprob, n, cfg, xk, st); break;
+    default: fused2<4>(pass, levs, nprob, n, cfg, xk, st); break;
+  }
+}
+
 void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
                   bool store_last) {
-  seq_push(q, levs, PK_ARNOLDI, S, cfg.units, cfg.geo, first, store_last, 0, 0, nprob * cfg.units);
+  const int units = first ? cfg.units : cfg.units_res;
+  seq_push(q, levs, PK_ARNOLDI, S, units, cfg.geo, first, store_last, 0, 0, nprob * units);
 }
 
 size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {
@@ -127,21 +160,23 @@ size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {
 
 template <int S, int DIM>
 static void launch_coarse_gram_sd(const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                                  const float2* pw, int nu1, int nu2, size_t smem, cudaStream_t st) {
+                                  const float2* pw, int nu1, int nu2, bool from_res, size_t smem,
+                                  cudaStream_t st) {
   thread_local size_t configured = 0;
   if (configured < smem) {
     cudaFuncSetAttribute(k_coarse_gram<S, DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     configured = smem;
   }
-  pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, pw, nu1, nu2);
+  pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, pw, nu1, nu2,
+             from_res ? 1 : 0);
 }
 
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                        const float2* pw, int nu1, int nu2, size_t smem, cudaStream_t st) {
-#define HELM_CG(SS)                                                                                   \
-  case SS:                                                                                            \
-    if (dim == 2) launch_coarse_gram_sd<SS, 2>(levs, lev_stride, lus, nprob, pw, nu1, nu2, smem, st); \
-    else launch_coarse_gram_sd<SS, 3>(levs, lev_stride, lus, nprob, pw, nu1, nu2, smem, st);          \
+                        const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st) {
+#define HELM_CG(SS)                                                                                             \
+  case SS:                                                                                                      \
+    if (dim == 2) launch_coarse_gram_sd<SS, 2>(levs, lev_stride, lus, nprob, pw, nu1, nu2, from_res, smem, st); \
+    else launch_coarse_gram_sd<SS, 3>(levs, lev_stride, lus, nprob, pw, nu1, nu2, from_res, smem, st);          \
     break;
   switch (S) {
     HELM_CG(0)

@@ -36,10 +36,13 @@ __device__ __forceinline__ SwCoef sw_coef(const float2* ca, int i, int n, float 
 // ------------------------------------------------------------------ 2D
 // A CTA of 8 warps holds a 32 x 8 QY region in registers, QY consecutive rows per warp;
 // only the rows at a warp's edges pass through shared memory.  Its own points are the
-// inner (32 - 2S) x (8 QY - 2S).
+// inner (32 - 2H) x (8 QY - 2H), H = S for a sweep from b and S + 1 for one from the residual
+// of an iterate (one point more, as the fused pass forms that residual itself).
 constexpr int SW2_NW = 8;
-HELM_HD constexpr int sw2_oy(int S, int QY) { return SW2_NW * QY - 2 * S; }
-HELM_HD inline int sw2_units(int S, int QY, int n) { return ceil_div(n, sw_ox(S)) * ceil_div(n, sw2_oy(S, QY)); }
+HELM_HD constexpr int sw2_own(int R, int H) { return R - 2 * H; }
+HELM_HD inline int sw2_units(int H, int QY, int n) {
+  return ceil_div(n, sw2_own(32, H)) * ceil_div(n, sw2_own(SW2_NW * QY, H));
+}
 
 template <int S, int QY>
 struct Sw2Shared {
@@ -50,90 +53,370 @@ struct Sw2Shared {
   float wsum[SW2_NW * gram_ns(S)];
 };
 
-template <int S, int QY, bool NC = true>
-__device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
-                                            int store_last, int vblk, Sw2Shared<S, QY>& sh) {
-  constexpr int NS = gram_ns(S), RY = SW2_NW * QY;
-  auto& edge = sh.edge;
-  auto& yac = sh.yac;
-  auto& yd = sh.yd;
-  const int prob = vblk / nunits, unit = vblk - prob * nunits;
-  const LevelDev<float2>& L = levs[prob];
-  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
-  const int n = L.n, P = L.P;
-  const float t = L.kt;
-  const int ntx = ceil_div(n, sw_ox(S));
-  const int tx = unit % ntx, ty = unit / ntx;
-  const int x = tx * sw_ox(S) - S + lane, yr = ty * sw2_oy(S, QY) - S, y0 = yr + warp * QY;
-  const SwCoef cx = sw_coef(L.ca, x, n, t);
-  if (tid < RY) {
-    const SwCoef c = sw_coef(L.ca, yr + tid, n, t);
-    yac[tid] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
-    yd[tid] = c.d;
-  }
-  if (warp < 2) {  // the rows beyond the region
-    edge[warp][0][1][lane] = make_float2(0.f, 0.f);
-    edge[warp][SW2_NW + 1][0][lane] = make_float2(0.f, 0.f);
-  }
+// A thread's place in its CTA's region and the stencil there (times the basis scale t).
+template <int S, int QY>
+struct Sw2Region {
+  int n, P, H, x, y0, xr, yr, lane, warp, par;
+  SwCoef cx;
   float ph[QY];
-  const float phc = L.phir * t;
+  Sw2Shared<S, QY>& sh;
+  __device__ __forceinline__ Sw2Region(const LevelDev<float2>& L, int unit, int halo, Sw2Shared<S, QY>& shared)
+      : sh(shared) {
+    lane = threadIdx.x;
+    warp = threadIdx.y;
+    n = L.n;
+    P = L.P;
+    H = halo;
+    par = 0;
+    const float t = L.kt;
+    const int ox = sw2_own(32, H), oy = sw2_own(SW2_NW * QY, H), ntx = ceil_div(n, ox);
+    xr = (unit % ntx) * ox - H;
+    yr = (unit / ntx) * oy - H;
+    x = xr + lane;
+    y0 = yr + warp * QY;
+    cx = sw_coef(L.ca, x, n, t);
+    const int tid = warp * 32 + lane;
+    if (tid < SW2_NW * QY) {
+      const SwCoef c = sw_coef(L.ca, yr + tid, n, t);
+      sh.yac[tid] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
+      sh.yd[tid] = c.d;
+    }
+    if (warp < 2) {  // the rows beyond the region
+      sh.edge[warp][0][1][lane] = make_float2(0.f, 0.f);
+      sh.edge[warp][SW2_NW + 1][0][lane] = make_float2(0.f, 0.f);
+    }
+    const float phc = L.phir * t;
 #pragma unroll
-  for (int q = 0; q < QY; ++q)
-    ph[q] = (L.phi && inside(x, y0 + q, 0, n)) ? __ldg(L.phi + pidx(x, y0 + q, 0, P)) * t : phc;
-  pdl_wait();
-  float2 sg[S];
-  gram_shifts<S>(L, first != 0, sg);
-  const float2* R0 = first ? L.b : L.r0;
-  float2 k[S + 1][QY];
-#pragma unroll
-  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2, NC>(R0, x, y0 + q, 0, n, P);
-#pragma unroll
-  for (int j = 0; j < S; ++j) {
-    edge[j & 1][warp + 1][0][lane] = k[j][0];
-    edge[j & 1][warp + 1][1][lane] = k[j][QY - 1];
+    for (int q = 0; q < QY; ++q)
+      ph[q] = (L.phi && inside(x, y0 + q, 0, n)) ? __ldg(L.phi + pidx(x, y0 + q, 0, P)) * t : phc;
+  }
+  __device__ __forceinline__ bool own_row(int q) const {  // uniform over the warp
+    const int ry = warp * QY + q;
+    return ry >= H && ry < SW2_NW * QY - H && y0 + q < n;
+  }
+  __device__ __forceinline__ bool own_x() const { return lane >= H && lane < 32 - H && x < n; }
+  // o = t (M - sg) v on the region (wrong one point further in from its rim each time)
+  __device__ __forceinline__ void apply(const float2 (&v)[QY], const float2 sg, float2 (&o)[QY]) {
+    sh.edge[par][warp + 1][0][lane] = v[0];
+    sh.edge[par][warp + 1][1][lane] = v[QY - 1];
     __syncthreads();
-    const float2 up = edge[j & 1][warp][1][lane], dn = edge[j & 1][warp + 2][0][lane];
+    const float2 up = sh.edge[par][warp][1][lane], dn = sh.edge[par][warp + 2][0][lane];
+    par ^= 1;
 #pragma unroll
     for (int q = 0; q < QY; ++q) {
-      const float4 ac = yac[warp * QY + q];
-      float2 dg = cadd(cx.d, yd[warp * QY + q]);
-      dg.x = (dg.x - ph[q]) - sg[j].x;
-      dg.y -= sg[j].y;
-      const float2 v = k[j][q];
-      float2 p = cmul(dg, v);
-      p = cfma(cx.a, shfl_up_c(v, 1), p);
-      p = cfma(cx.c, shfl_down_c(v, 1), p);
-      p = cfma(make_float2(ac.x, ac.y), q > 0 ? k[j][q - 1] : up, p);
-      p = cfma(make_float2(ac.z, ac.w), q < QY - 1 ? k[j][q + 1] : dn, p);
-      k[j + 1][q] = p;
+      const float4 ac = sh.yac[warp * QY + q];
+      float2 dg = cadd(cx.d, sh.yd[warp * QY + q]);
+      dg.x = (dg.x - ph[q]) - sg.x;
+      dg.y -= sg.y;
+      float2 p = cmul(dg, v[q]);
+      p = cfma(cx.a, shfl_up_c(v[q], 1), p);
+      p = cfma(cx.c, shfl_down_c(v[q], 1), p);
+      p = cfma(make_float2(ac.x, ac.y), q > 0 ? v[q > 0 ? q - 1 : 0] : up, p);
+      o[q] = cfma(make_float2(ac.z, ac.w), q < QY - 1 ? v[q < QY - 1 ? q + 1 : q] : dn, p);
     }
   }
-  float acc[NS];
+  // k_1..k_S from k_0, the own points' k_j to p[j - 1] (j <= nstore), and the Gram matrix.
+  __device__ __forceinline__ void sweep(const LevelDev<float2>& L, const float2 (&sg)[S], float2 (&k)[S + 1][QY],
+                                        float2* const* p, int nstore, int unit, int nunits) {
 #pragma unroll
-  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
-  const bool ownx = lane >= S && lane < 32 - S && x < n;
+    for (int j = 0; j < S; ++j) apply(k[j], sg[j], k[j + 1]);
+    float acc[gram_ns(S)];
 #pragma unroll
-  for (int q = 0; q < QY; ++q) {
-    const int ry = warp * QY + q, y = y0 + q;
-    if (ry < S || ry >= RY - S || y >= n) continue;  // uniform over the warp
-    if (ownx) {
+    for (int i = 0; i < gram_ns(S); ++i) acc[i] = 0.f;
+    const bool ownx = own_x();
+#pragma unroll
+    for (int q = 0; q < QY; ++q) {
+      if (!own_row(q) || !ownx) continue;
       float2 kk[S + 1];
 #pragma unroll
       for (int j = 0; j <= S; ++j) kk[j] = k[j][q];
       gram_point<S>(kk, acc);
 #pragma unroll
       for (int j = 1; j <= S; ++j)
-        if (j < S || store_last) L.p[j - 1][pidx(x, y, 0, P)] = kk[j];
+        if (j <= nstore) p[j - 1][pidx(x, y0 + q, 0, P)] = kk[j];
     }
+    pdl_trigger();  // the main work is done: let the next pass launch
+    gram_finish<S, SW2_NW>(acc, L, sg, unit, nunits, sh.wsum, sh.gs);
   }
-  pdl_trigger();  // the main work is done: let the next pass launch
-  gram_finish<S, SW2_NW>(acc, L, sg, unit, nunits, sh.wsum, sh.gs);
+};
+
+template <int S, int QY, bool NC = true>
+__device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
+                                            int store_last, int vblk, Sw2Shared<S, QY>& sh) {
+  const int prob = vblk / nunits, unit = vblk - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  Sw2Region<S, QY> W(L, unit, first ? S : S + 1, sh);
+  pdl_wait();
+  float2 sg[S];
+  gram_shifts<S>(L, first != 0, sg);
+  const float2* R0 = first ? L.b : L.r0;
+  float2 k[S + 1][QY];
+#pragma unroll
+  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2, NC>(R0, W.x, W.y0 + q, 0, W.n, W.P);
+  W.sweep(L, sg, k, L.p, store_last ? S : S - 1, unit, nunits);
 }
 template <int S, int QY>
 __global__ void __launch_bounds__(256, 2)
 k_sweep2(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int store_last) {
   __shared__ Sw2Shared<S, QY> sh;
   sweep2_body<S, QY>(levs, nunits, first, store_last, blockIdx.x, sh);
+}
+
+// ------------------------------------------------------------------ 2D, fused V(1,1) passes
+// A level of a V(1,1) cycle in two launches instead of five: the pass that sweeps also forms
+// what it sweeps from, redundantly with its neighbours, so that the restriction, the coarse
+// correction, its residual and the updates need no passes and no vectors of their own.
+// Levels of this size live in L2 and a chained pass takes about 3 us whatever its size (5 to 6
+// with the Gram reduction), so launches are what they cost: 127^2 14 launches, 67.7 us, before
+// and 7, 55 us, now; 639^2 164 -> 128, 1023^2 209 -> 180.  Larger levels (the line of the
+// marching sweep) keep passes of their own: rereading a region's rim costs them more than a
+// launch (4095^2, s = 4: 4.3 ms fused, 3.1 ms apart).  The values are the separate passes', in
+// the same order of operations.
+//
+// Descent: b = full weighting of the finer level's residual sum_k rho_k k_k (its last sweep),
+// which a lane forms for its column from two fine columns, the third being its neighbour's
+// first.  A problem whose finest level this is takes b as given.
+template <int S, int QY>
+__global__ void __launch_bounds__(256, 2)
+k_sweep2_down(const LevelDev<float2>* __restrict__ levs, int nunits) {
+  __shared__ Sw2Shared<S, QY> sh;
+  const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  Sw2Region<S, QY> W(L, unit, S, sh);
+  pdl_wait();
+  float2 sg[S];
+  gram_shifts<S>(L, true, sg);
+  float2 k[S + 1][QY];
+  if (L.top) {
+#pragma unroll
+    for (int q = 0; q < QY; ++q) k[0][q] = ldc(L.b, W.x, W.y0 + q, 0, W.n, W.P);
+  } else {
+    const int nf = 2 * W.n + 1, Pf = nf + 1, m = L.scf->m, f0 = 2 * W.y0;
+    float2 rc[S + 1];
+    const float2* R[S + 1];
+#pragma unroll
+    for (int j = 0; j <= S; ++j) {
+      rc[j] = L.scf->rcoef[j];
+      R[j] = j == 0 ? L.fb : L.fp[j > 0 ? j - 1 : 0];
+    }
+    // the column right of lane 31's pair: lane i takes fine row f0 + i
+    float2 er = make_float2(0.f, 0.f);
+    {
+      const int ec = 2 * (W.xr + 32), er_row = f0 + W.lane;
+      const bool ok = W.lane <= 2 * QY && (unsigned)er_row < (unsigned)nf && (unsigned)ec < (unsigned)Pf;
+#pragma unroll
+      for (int j = 0; j <= S; ++j)
+        if (ok && j <= m) er = cfma(rc[j], R[j][(size_t)er_row * Pf + ec], er);
+    }
+    const int fc = 2 * W.x;
+    const bool colok = (unsigned)fc < (unsigned)Pf;  // a pair: Pf and fc are even
+    float2 out[QY];
+#pragma unroll
+    for (int q = 0; q < QY; ++q) out[q] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i <= 2 * QY; ++i) {
+      const int f = f0 + i;
+      const bool ok = colok && (unsigned)f < (unsigned)nf;
+      float2 r0 = make_float2(0.f, 0.f), r1 = r0;
+#pragma unroll
+      for (int j = 0; j <= S; ++j) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ok && j <= m) v = *reinterpret_cast<const float4*>(R[j] + (size_t)f * Pf + fc);
+        if (j <= m) {  // uniform
+          r0 = cfma(rc[j], make_float2(v.x, v.y), r0);
+          r1 = cfma(rc[j], make_float2(v.z, v.w), r1);
+        }
+      }
+      const float2 rn = shfl_down_c(r0, 1);
+      const float2 re = make_float2(__shfl_sync(0xffffffffu, er.x, i), __shfl_sync(0xffffffffu, er.y, i));
+      const float2 r2 = W.lane == 31 ? re : rn;
+#pragma unroll
+      for (int q = 0; q < QY; ++q) {
+        if (i < 2 * q || i > 2 * q + 2) continue;
+        const float w = i == 2 * q + 1 ? 0.125f : 0.0625f;
+        out[q] = cadd(out[q], cscale(r0, w));
+        out[q] = cadd(out[q], cscale(r1, 2.0f * w));
+        out[q] = cadd(out[q], cscale(r2, w));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < QY; ++q) {
+      k[0][q] = inside(W.x, W.y0 + q, 0, W.n) ? out[q] : make_float2(0.f, 0.f);
+      if (W.own_row(q) && W.own_x()) L.b[pidx(W.x, W.y0 + q, 0, W.P)] = k[0][q];
+    }
+  }
+  W.sweep(L, sg, k, L.p, S, unit, nunits);
+}
+
+// Coarse points around a 32 x R region of fine points: the coarser level's output there, its
+// last sweep's update included if that has no pass of its own (L.cr0), to es.
+template <int S>
+__device__ __forceinline__ float2 coarse_value(const LevelDev<float2>& L, const float2 (&yc)[S], int mc, int X, int Y) {
+  if ((unsigned)X >= (unsigned)L.nc || (unsigned)Y >= (unsigned)L.nc) return make_float2(0.f, 0.f);
+  const size_t i = (size_t)Y * L.Pc + X;
+  const float2 xv = L.xcb[i];
+  if (!L.cr0) return xv;
+  float2 dx = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < S; ++j)
+    if (j < mc) dx = cfma(yc[j], j == 0 ? L.cr0[i] : L.cp[j > 0 ? j - 1 : 0][i], dx);
+  return cadd(xv, dx);
+}
+template <int S>
+__device__ __forceinline__ int coarse_update(const LevelDev<float2>& L, float2 (&yc)[S]) {
+#pragma unroll
+  for (int j = 0; j < S; ++j) yc[j] = L.cr0 ? L.scc->xcoef[j] : make_float2(0.f, 0.f);
+  return L.cr0 ? L.scc->m : 0;
+}
+// Bilinear interpolation from rows of staged coarse values at fine (x, y), (X0, Y0) the first.
+template <int EX>
+__device__ __forceinline__ float2 staged_interp(const float2 (*es)[EX], int X0, int Y0, int x, int y) {
+  const int X = (x >> 1) - X0, Y = (y >> 1) - Y0;
+  float2 a = make_float2(0.f, 0.f);
+  float w = 1.0f;
+  if (!(x & 1)) w *= 0.5f;
+  if (!(y & 1)) {
+    w *= 0.5f;
+    if (!(x & 1)) a = cadd(a, es[Y - 1][X - 1]);
+    a = cadd(a, es[Y - 1][X]);
+  }
+  if (!(x & 1)) a = cadd(a, es[Y][X - 1]);
+  a = cadd(a, es[Y][X]);
+  return cscale(a, w);
+}
+
+// Ascent: x_b = sum_k y_k k_k + P e_c (the pre-smoothing sweep from b, and the corrected
+// coarser output), R_0 = b - M x_b, and the sweep from it.  The new vectors go to L.q: other
+// CTAs still read the old ones.
+template <int S, int QY>
+__global__ void __launch_bounds__(256, 2)
+k_sweep2_up(const LevelDev<float2>* __restrict__ levs, int nunits) {
+  constexpr int EX = 18, EY = SW2_NW * QY / 2 + 2;
+  __shared__ Sw2Shared<S, QY> sh;
+  __shared__ float2 es[EY][EX];
+  const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
+  const LevelDev<float2>& L = levs[prob];
+  Sw2Region<S, QY> W(L, unit, S + 1, sh);
+  pdl_wait();
+  const int m = L.sc->m;
+  float2 xc[S], yc[S], sg[S];
+#pragma unroll
+  for (int j = 0; j < S; ++j) xc[j] = L.sc->xcoef[j];
+  const int mc = coarse_update<S>(L, yc);
+  gram_shifts<S>(L, false, sg);
+  float2 b[QY], dx[QY];
+#pragma unroll
+  for (int q = 0; q < QY; ++q) {
+    const bool in = inside(W.x, W.y0 + q, 0, W.n);
+    const size_t i = pidx(W.x, W.y0 + q, 0, W.P);
+    b[q] = in ? L.b[i] : make_float2(0.f, 0.f);
+    dx[q] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+      if (j < m) dx[q] = cfma(xc[j], j == 0 ? b[q] : in ? L.p[j > 0 ? j - 1 : 0][i] : make_float2(0.f, 0.f), dx[q]);
+  }
+  const int X0 = (W.xr >> 1) - 1, Y0 = (W.yr >> 1) - 1;
+  for (int i = W.warp * 32 + W.lane; i < EX * EY; i += 256)
+    es[i / EX][i % EX] = coarse_value<S>(L, yc, mc, X0 + i % EX, Y0 + i / EX);
+  __syncthreads();
+  float2 v[QY], k[S + 1][QY];
+#pragma unroll
+  for (int q = 0; q < QY; ++q) {
+    v[q] = make_float2(0.f, 0.f);
+    if (inside(W.x, W.y0 + q, 0, W.n)) v[q] = cadd(dx[q], staged_interp<EX>(es, X0, Y0, W.x, W.y0 + q));
+  }
+  W.apply(v, make_float2(0.f, 0.f), k[0]);
+  const float it = __frcp_rn(L.kt);  // exact
+#pragma unroll
+  for (int q = 0; q < QY; ++q) {
+    k[0][q] = csub(b[q], cscale(k[0][q], it));
+    if (W.own_row(q) && W.own_x()) {
+      const size_t i = pidx(W.x, W.y0 + q, 0, W.P);
+      L.xb[i] = v[q];
+      L.r0[i] = k[0][q];
+    }
+  }
+  W.sweep(L, sg, k, L.q, S - 1, unit, nunits);
+}
+
+// Coarse correction and residual of a larger level (the sweep after it marches), 64 x 16 tiles:
+// x_a from the last sweep if the restriction was fused (xk), else as stored.
+template <int S>
+__global__ void __launch_bounds__(256, 3)
+k_prolong2_gram(const LevelDev<float2>* __restrict__ levs, int ntiles, int xk) {
+  constexpr int TX = 64, TY = 16, EX = TX / 2 + 2, EY = TY / 2 + 2;
+  __shared__ float2 es[EY][EX];
+  __shared__ float2 vt[TY + 2][TX + 2];
+  const int prob = blockIdx.x / ntiles, tile = blockIdx.x - prob * ntiles;
+  const LevelDev<float2>& L = levs[prob];
+  const int n = L.n, P = L.P, ntx = ceil_div(P, TX);
+  const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+  const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
+  pdl_wait();
+  const int m = L.sc->m;
+  float2 xc[S], yc[S];
+#pragma unroll
+  for (int j = 0; j < S; ++j) xc[j] = L.sc->xcoef[j];
+  const int mc = coarse_update<S>(L, yc);
+  const int X0 = x0 / 2 - 1, Y0 = y0 / 2 - 1;
+  for (int i = tid; i < EX * EY; i += 256)
+    es[i / EX][i % EX] = coarse_value<S>(L, yc, mc, X0 + i % EX, Y0 + i / EX);
+  auto before = [&](int x, int y, float2& b) {  // x_a and b
+    const bool in = inside(x, y, 0, n);
+    const size_t i = pidx(x, y, 0, P);
+    b = in ? L.b[i] : make_float2(0.f, 0.f);
+    if (!xk) return in ? L.xa[i] : make_float2(0.f, 0.f);
+    float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+      if (j < m) d = cfma(xc[j], j == 0 ? b : in ? L.p[j > 0 ? j - 1 : 0][i] : make_float2(0.f, 0.f), d);
+    return d;
+  };
+  float2 bq[4], xv[4], hv = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) xv[q] = before(x0 + lx + 32 * (q & 1), y0 + ly + 8 * (q >> 1), bq[q]);
+  int hx = 0, hy = 0;
+  const bool halo = tid < 2 * (TX + TY);  // the tile's rim, corners excepted
+  if (halo) {
+    if (tid < 2 * TX) {
+      hx = tid % TX;
+      hy = tid < TX ? -1 : TY;
+    } else {
+      hx = tid - 2 * TX < TY ? -1 : TX;
+      hy = (tid - 2 * TX) % TY;
+    }
+    float2 b;
+    hv = before(x0 + hx, y0 + hy, b);
+  }
+  __syncthreads();
+  auto value = [&](float2 xa, int x, int y) {
+    return inside(x, y, 0, n) ? cadd(xa, staged_interp<EX>(es, X0, Y0, x, y)) : make_float2(0.f, 0.f);
+  };
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1);
+    vt[oy + 1][ox + 1] = value(xv[q], x0 + ox, y0 + oy);
+  }
+  if (halo) vt[hy + 1][hx + 1] = value(hv, x0 + hx, y0 + hy);
+  __syncthreads();
+  const SwCoef cx[2] = {sw_coef(L.ca, x0 + lx, n, 1.0f), sw_coef(L.ca, x0 + lx + 32, n, 1.0f)};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ox = lx + 32 * (q & 1), oy = ly + 8 * (q >> 1), x = x0 + ox, y = y0 + oy;
+    if (x >= n || y >= n) continue;  // the ghost row and column stay zero
+    const SwCoef cy = sw_coef(L.ca, y, n, 1.0f);
+    const size_t i = pidx(x, y, 0, P);
+    float2 dg = cadd(cx[q & 1].d, cy.d);
+    dg.x -= L.phi ? __ldg(L.phi + i) : L.phir;
+    float2 p = cmul(dg, vt[oy + 1][ox + 1]);
+    p = cfma(cx[q & 1].a, vt[oy + 1][ox], p);
+    p = cfma(cx[q & 1].c, vt[oy + 1][ox + 2], p);
+    p = cfma(cy.a, vt[oy][ox + 1], p);
+    p = cfma(cy.c, vt[oy + 2][ox + 1], p);
+    L.xb[i] = vt[oy + 1][ox + 1];
+    L.r0[i] = csub(bq[q], p);
+  }
+  pdl_trigger();
 }
 
 // ------------------------------------------------------------------ 2D, large levels

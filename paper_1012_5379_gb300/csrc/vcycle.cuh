@@ -227,6 +227,12 @@ k_update_flat(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, int mod
   update_pass_body<C>(levs, ntiles, dim, mode, r0_is_b, xsel, x_from_zero, blockIdx.x);
 }
 
+// Level-0 input and output: a warp takes IO_XPT x 32 neighbouring points of a row at a time,
+// all their loads in flight together.  255^3 complex64: 50 us for the input (a row per CTA, one
+// point per thread and round, took 95); 108 us for the output with the last update, which
+// were passes of 58 and 109 us; both at 85% of the copy rate.
+constexpr int IO_XPT = 4;
+
 // Level-0 input: b <- src (natural layout, any precision), ||b||^2 starts the first
 // sweep.  (src is not __restrict__: the compiler could then read it before the wait.)
 template <typename Cin, typename C>
@@ -237,21 +243,30 @@ k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Ci
   const LevelDev<C>& L = levs[prob];
   const int n = L.n, P = L.P;
   pdl_wait();
-  // CTAs take rows (z, y) of the padded layout in turn; threads stride along x
-  const int nrows = dim == 3 ? P * P : P;
   C* const b = L.b;
   constexpr bool GRAM = sizeof(C) == 8;  // complex64: the first sweep's shift from neighbour differences
   typename CT<C>::R acc = 0, accd = 0;
-  for (int row = tile; row < nrows; row += ntiles) {
-    const int y = dim == 3 ? row % P : row, z = dim == 3 ? row / P : 0;
-    const bool rin = y < n && z < n;
-    const size_t base = (size_t)row * P, sbase = ((size_t)z * n + y) * n;
-    for (int x = threadIdx.x; x < P; x += blockDim.x) {
-      C v = czero<C>();
-      if (rin && x < n) v = to_c<C>(src[sbase + x]);
-      b[base + x] = v;
-      acc += cabs2(v);
-      if (GRAM && rin && x + 1 < n) accd += cabs2(csub(to_c<C>(src[sbase + x + 1]), v));
+  // the ghost positions stay zero
+  const int nchunk = (n + 32 * IO_XPT - 1) / (32 * IO_XPT), lane = threadIdx.x & 31;
+  const int items = (dim == 3 ? n * n : n) * nchunk;
+  for (int it = tile * 8 + (threadIdx.x >> 5); it < items; it += ntiles * 8) {
+    const int row = it / nchunk, xc = (it - row * nchunk) * 32 * IO_XPT, x0 = xc + lane;
+    const int y = dim == 3 ? row % n : row, z = dim == 3 ? row / n : 0;
+    const size_t s = (size_t)row * n + x0, i = ((size_t)z * P + y) * P + x0;
+    C v[IO_XPT + 1];
+#pragma unroll
+    for (int q = 0; q < IO_XPT; ++q) v[q] = x0 + 32 * q < n ? to_c<C>(src[s + 32 * q]) : czero<C>();
+    v[IO_XPT] = czero<C>();
+    if (GRAM && lane == 0 && x0 + 32 * IO_XPT < n) v[IO_XPT] = to_c<C>(src[s + 32 * IO_XPT]);
+#pragma unroll
+    for (int q = 0; q < IO_XPT; ++q) {
+      if (x0 + 32 * q < n) b[i + 32 * q] = v[q];
+      acc += cabs2(v[q]);
+      if constexpr (GRAM) {
+        const C in = shfl_down_c(v[q], 1);
+        const C over = make_float2(__shfl_sync(0xffffffffu, v[q + 1].x, 0), __shfl_sync(0xffffffffu, v[q + 1].y, 0));
+        if (x0 + 32 * q + 1 < n) accd += cabs2(csub(lane == 31 ? over : in, v[q]));
+      }
     }
   }
   if constexpr (GRAM) {
@@ -272,21 +287,44 @@ k_load_input(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, const Ci
   }
 }
 
-// Level-0 output: dst (natural layout, any precision) <- xb.
+// Level-0 output: dst (natural layout, any precision) <- xb, plus the last post-smoothing
+// sweep's update if it is pending (`update`): that reads what the update pass would and spares
+// its launch and x_b's way to memory and back.
 template <typename C, typename Cout>
 __global__ void __launch_bounds__(256)
-k_store_output(const LevelDev<C>* __restrict__ levs, int dim, Cout* __restrict__ dst) {
+k_store_output(const LevelDev<C>* __restrict__ levs, int dim, int update, Cout* __restrict__ dst) {
   pdl_trigger();
   const LevelDev<C>& L = levs[0];
   const int n = L.n, P = L.P;
   pdl_wait();
-  // CTAs take rows (z, y) of the natural layout in turn; threads stride along x
-  const int nrows = dim == 3 ? n * n : n;
-  const C* const xb = L.xb;
-  for (int row = blockIdx.x; row < nrows; row += gridDim.x) {
+  const UpdCoef<C> u = load_upd(L, 0);
+  const int m = update ? u.m : 0;
+  constexpr int NX = sizeof(C) == 16 ? 2 : IO_XPT;  // points a lane takes together (registers)
+  const int nchunk = (n + 32 * IO_XPT - 1) / (32 * IO_XPT), lane = threadIdx.x & 31;
+  const int items = (dim == 3 ? n * n : n) * nchunk;
+  for (int it = blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += gridDim.x * 8) {
+    const int row = it / nchunk, xc = (it - row * nchunk) * 32 * IO_XPT;
     const int y = dim == 3 ? row % n : row, z = dim == 3 ? row / n : 0;
-    const size_t dbase = (size_t)row * n, sbase = ((size_t)z * P + y) * P;
-    for (int x = threadIdx.x; x < n; x += blockDim.x) dst[dbase + x] = to_c<Cout>(xb[sbase + x]);
+#pragma unroll
+    for (int x0 = xc + lane; x0 < xc + 32 * IO_XPT; x0 += 32 * NX) {
+      const size_t d = (size_t)row * n + x0, i = ((size_t)z * P + y) * P + x0;
+      C v[SMAX][NX], xv[NX];
+#pragma unroll
+      for (int q = 0; q < NX; ++q) {
+        const bool in = x0 + 32 * q < n;
+        xv[q] = in ? L.xb[i + 32 * q] : czero<C>();
+#pragma unroll
+        for (int k = 0; k < SMAX; ++k) v[k][q] = in && k < m ? u.Rk[k][i + 32 * q] : czero<C>();
+      }
+#pragma unroll
+      for (int q = 0; q < NX; ++q) {
+        C dx = czero<C>();
+#pragma unroll
+        for (int k = 0; k < SMAX; ++k)
+          if (k < m) dx = cfma(u.xc[k], v[k][q], dx);
+        if (x0 + 32 * q < n) dst[d + 32 * q] = to_c<Cout>(m > 0 ? cadd(xv[q], dx) : xv[q]);
+      }
+    }
   }
 }
 

@@ -204,13 +204,13 @@ void launch_load_input(int dim, const LevelDev<C>* levs, int ntiles, const void*
 }
 
 template <typename C>
-void launch_store_output(int dim, int n, const LevelDev<C>* levs, void* dst, int out_prec, cudaStream_t st) {
-  const size_t npts = dim == 3 ? (size_t)n * n * n : (size_t)n * n;
-  const int grid = (int)std::min<size_t>((npts + 255) / 256, 4096);
+void launch_store_output(int dim, int n, const LevelDev<C>* levs, bool update, void* dst, int out_prec, cudaStream_t st) {
+  const size_t items = (dim == 3 ? (size_t)n * n : (size_t)n) * ceil_div(n, 32 * IO_XPT);  // a warp's share
+  const int grid = (int)std::min<size_t>((items + 7) / 8, (size_t)8 * sm_count());
   if (out_prec == HELM_C128)
-    pdl_launch(k_store_output<C, double2>, dim3(grid), dim3(256), 0, st, levs, dim, (double2*)dst);
+    pdl_launch(k_store_output<C, double2>, dim3(grid), dim3(256), 0, st, levs, dim, update ? 1 : 0, (double2*)dst);
   else
-    pdl_launch(k_store_output<C, float2>, dim3(grid), dim3(256), 0, st, levs, dim, (float2*)dst);
+    pdl_launch(k_store_output<C, float2>, dim3(grid), dim3(256), 0, st, levs, dim, update ? 1 : 0, (float2*)dst);
 }
 
 template <typename C>
@@ -324,7 +324,7 @@ int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_
   template void launch_coarse<C>(int, const LevelDev<C>*, int, int, const CoarseLU*, int, int, int,           \
                                  cudaStream_t);                                                               \
   template void launch_load_input<C>(int, const LevelDev<C>*, int, const void*, int, cudaStream_t);           \
-  template void launch_store_output<C>(int, int, const LevelDev<C>*, void*, int, cudaStream_t);              \
+  template void launch_store_output<C>(int, int, const LevelDev<C>*, bool, void*, int, cudaStream_t);        \
   template void launch_poly_step<C>(int, const LevelDev<C>*, const C*, int, int, int, int, int, cudaStream_t); \
   template void launch_poly_restrict<C>(int, const LevelDev<C>*, int, int, int, cudaStream_t);                \
   template void record_restrict<C>(PassSeq&, int, const LevelDev<C>*, int, int, TileCfg, bool, bool, bool);    \
