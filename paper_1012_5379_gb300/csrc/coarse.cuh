@@ -247,7 +247,10 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
           float2 r = make_float2(0.f, 0.f);
 #pragma unroll
           for (int j = 0; j <= S; ++j)
-            if (j <= m) r = cfma(rc[j], j == 0 ? L.fb[i] : L.fp[j > 0 ? j - 1 : 0][i], r);
+          {
+            const float2 v = j == 0 ? L.fb[i] : L.fp[j > 0 ? j - 1 : 0][i];
+            if (j <= m) r = cfma(rc[j], v, r);
+          }
           out = cadd(out, cscale(r, (dx == 1 ? 0.5f : 0.25f) * (dy == 1 ? 0.5f : 0.25f)));
         }
       V.b[V.off[q]] = out;

@@ -202,7 +202,7 @@ HELM_HD inline int coarse_threshold(int dim, int prec) {
 // the device's SM count only.
 struct SweepCfg {
   int march, geo, units;
-  int units_res;  // CTAs of a sweep that starts from the residual of an iterate
+  int geo_res, units_res;  // shape and CTAs of a sweep that starts from the residual of an iterate
 };
 SweepCfg sweep_cfg(int dim, int n, int S, int sms);
 

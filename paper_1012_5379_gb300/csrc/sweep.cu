@@ -17,12 +17,25 @@ constexpr int SWEEP2_MARCH_N = 600;
 bool fused2_size(int n) { return n < SWEEP2_MARCH_N; }
 
 SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
-  SweepCfg c{0, 0, 1, 1};
+  SweepCfg c{0, 0, 1, 0, 1};
   if (dim == 2) {
     if (n < SWEEP2_MARCH_N || S > 3) {
-      c.geo = n <= 255 ? 2 : 4;
-      c.units = sw2_units(S, c.geo, n);
-      c.units_res = sw2_units(S + 1, c.geo, n);
+      // rows per warp: the fewest rounds of resident CTAs, each a fixed latency and its rows
+      // (511^2: one round at 6 rows; two at 4, 21 us against 12 on the way up)
+      auto pick = [&](int H, int& geo, int& units) {
+        int best = -1;
+        for (int qy = 2; qy <= 6; qy += 2) {
+          const int u = sw2_units(H, qy, n), slots = (qy == 2 ? 3 : 2) * sms;
+          const int cost = (u + slots - 1) / slots * (4 + qy);
+          if (best < 0 || cost < best) {
+            best = cost;
+            geo = qy;
+            units = u;
+          }
+        }
+      };
+      pick(S, c.geo, c.units);
+      pick(S + 1, c.geo_res, c.units_res);
       return c;
     }
     // rows per march: the fewest row steps of the SM that takes the most, four CTAs per SM
@@ -38,11 +51,13 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
       }
     }
     c.units_res = c.units;
+    c.geo_res = c.geo;
     return c;
   }
   if (n < 96 || S > 3) {
     c.geo = n < 64 ? 4 : 8;
     c.units_res = c.units = sw3_units(S, c.geo, n);
+    c.geo_res = c.geo;
     return c;
   }
   // planes per march: the fewest plane steps of the CTA that takes the most, one CTA per SM
@@ -58,6 +73,7 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
       c.units = (int)units;
     }
   }
+  c.geo_res = c.geo;
   c.units_res = c.units;
   return c;
 }
@@ -70,9 +86,10 @@ static void launch_sweep_s(int dim, const LevelDev<float2>* levs, int nprob, con
   if (dim == 2) {
     if (!cfg.march) {
       const dim3 block(32, SW2_NW);
-      const int units = first ? cfg.units : cfg.units_res;
-      if (cfg.geo == 2) pdl_launch(k_sweep2<S, 2>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
-      else pdl_launch(k_sweep2<S, 4>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
+      const int units = first ? cfg.units : cfg.units_res, qy = first ? cfg.geo : cfg.geo_res;
+      if (qy == 2) pdl_launch(k_sweep2<S, 2>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
+      else if (qy == 4) pdl_launch(k_sweep2<S, 4>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
+      else pdl_launch(k_sweep2<S, 6>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
     } else if constexpr (S <= 3) {
       const dim3 block(32, SV2_NW);
       const size_t smem = sv2_smem(S, cfg.geo);  // at most 256 rows: below 48 KB
@@ -125,11 +142,15 @@ static void fused2(int pass, const LevelDev<float2>* levs, int nprob, int n, con
     const int ntiles = ceil_div(n + 1, 64) * ceil_div(n + 1, 16);
     pdl_launch(k_prolong2_gram<S>, dim3(nprob * ntiles), block, 0, st, levs, ntiles, xk ? 1 : 0);
   } else if (pass == FUSED2_DOWN) {
-    if (cfg.geo == 2) pdl_launch(k_sweep2_down<S, 2>, dim3(nprob * cfg.units), block, 0, st, levs, cfg.units);
-    else pdl_launch(k_sweep2_down<S, 4>, dim3(nprob * cfg.units), block, 0, st, levs, cfg.units);
+    const dim3 grid(nprob * cfg.units);
+    if (cfg.geo == 2) pdl_launch(k_sweep2_down<S, 2>, grid, block, 0, st, levs, cfg.units);
+    else if (cfg.geo == 4) pdl_launch(k_sweep2_down<S, 4>, grid, block, 0, st, levs, cfg.units);
+    else pdl_launch(k_sweep2_down<S, 6>, grid, block, 0, st, levs, cfg.units);
   } else {
-    if (cfg.geo == 2) pdl_launch(k_sweep2_up<S, 2>, dim3(nprob * cfg.units_res), block, 0, st, levs, cfg.units_res);
-    else pdl_launch(k_sweep2_up<S, 4>, dim3(nprob * cfg.units_res), block, 0, st, levs, cfg.units_res);
+    const dim3 grid(nprob * cfg.units_res);
+    if (cfg.geo_res == 2) pdl_launch(k_sweep2_up<S, 2>, grid, block, 0, st, levs, cfg.units_res);
+    else if (cfg.geo_res == 4) pdl_launch(k_sweep2_up<S, 4>, grid, block, 0, st, levs, cfg.units_res);
+    else pdl_launch(k_sweep2_up<S, 6>, grid, block, 0, st, levs, cfg.units_res);
   }
 }
 
@@ -146,7 +167,7 @@ void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int
 void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
                   bool store_last) {
   const int units = first ? cfg.units : cfg.units_res;
-  seq_push(q, levs, PK_ARNOLDI, S, units, cfg.geo, first, store_last, 0, 0, nprob * units);
+  seq_push(q, levs, PK_ARNOLDI, S, units, first ? cfg.geo : cfg.geo_res, first, store_last, 0, 0, nprob * units);
 }
 
 size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {

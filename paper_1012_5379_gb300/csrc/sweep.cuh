@@ -168,7 +168,7 @@ k_sweep2(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int s
 // correction, its residual and the updates need no passes and no vectors of their own.
 // Levels of this size live in L2 and a chained pass takes about 3 us whatever its size (5 to 6
 // with the Gram reduction), so launches are what they cost: 127^2 14 launches, 67.7 us, before
-// and 7, 55 us, now; 639^2 164 -> 128, 1023^2 209 -> 180.  Larger levels (the line of the
+// and 7, 53 us, now; 639^2 164 -> 121, 1023^2 209 -> 159.  Larger levels (the line of the
 // marching sweep) keep passes of their own: rereading a region's rim costs them more than a
 // launch (4095^2, s = 4: 4.3 ms fused, 3.1 ms apart).  The values are the separate passes', in
 // the same order of operations.
@@ -206,7 +206,10 @@ k_sweep2_down(const LevelDev<float2>* __restrict__ levs, int nunits) {
       const bool ok = W.lane <= 2 * QY && (unsigned)er_row < (unsigned)nf && (unsigned)ec < (unsigned)Pf;
 #pragma unroll
       for (int j = 0; j <= S; ++j)
-        if (ok && j <= m) er = cfma(rc[j], R[j][(size_t)er_row * Pf + ec], er);
+        {
+          const float2 v = ok ? R[j][(size_t)er_row * Pf + ec] : make_float2(0.f, 0.f);
+          if (j <= m) er = cfma(rc[j], v, er);
+        }
     }
     const int fc = 2 * W.x;
     const bool colok = (unsigned)fc < (unsigned)Pf;  // a pair: Pf and fc are even
@@ -221,7 +224,7 @@ k_sweep2_down(const LevelDev<float2>* __restrict__ levs, int nunits) {
 #pragma unroll
       for (int j = 0; j <= S; ++j) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ok && j <= m) v = *reinterpret_cast<const float4*>(R[j] + (size_t)f * Pf + fc);
+        if (ok) v = *reinterpret_cast<const float4*>(R[j] + (size_t)f * Pf + fc);  // not after m: its load is in flight
         if (j <= m) {  // uniform
           r0 = cfma(rc[j], make_float2(v.x, v.y), r0);
           r1 = cfma(rc[j], make_float2(v.z, v.w), r1);
@@ -259,7 +262,10 @@ __device__ __forceinline__ float2 coarse_value(const LevelDev<float2>& L, const 
   float2 dx = make_float2(0.f, 0.f);
 #pragma unroll
   for (int j = 0; j < S; ++j)
-    if (j < mc) dx = cfma(yc[j], j == 0 ? L.cr0[i] : L.cp[j > 0 ? j - 1 : 0][i], dx);
+  {
+    const float2 v = j == 0 ? L.cr0[i] : L.cp[j > 0 ? j - 1 : 0][i];
+    if (j < mc) dx = cfma(yc[j], v, dx);
+  }
   return cadd(xv, dx);
 }
 template <int S>
@@ -313,7 +319,10 @@ k_sweep2_up(const LevelDev<float2>* __restrict__ levs, int nunits) {
     dx[q] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < S; ++j)
-      if (j < m) dx[q] = cfma(xc[j], j == 0 ? b[q] : in ? L.p[j > 0 ? j - 1 : 0][i] : make_float2(0.f, 0.f), dx[q]);
+    {  // loaded whatever m is: m's own load is in flight
+      const float2 v = j == 0 ? b[q] : in ? L.p[j > 0 ? j - 1 : 0][i] : make_float2(0.f, 0.f);
+      if (j < m) dx[q] = cfma(xc[j], v, dx[q]);
+    }
   }
   const int X0 = (W.xr >> 1) - 1, Y0 = (W.yr >> 1) - 1;
   for (int i = W.warp * 32 + W.lane; i < EX * EY; i += 256)
@@ -369,7 +378,10 @@ k_prolong2_gram(const LevelDev<float2>* __restrict__ levs, int ntiles, int xk) {
     float2 d = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < S; ++j)
-      if (j < m) d = cfma(xc[j], j == 0 ? b : in ? L.p[j > 0 ? j - 1 : 0][i] : make_float2(0.f, 0.f), d);
+      {
+        const float2 v = j == 0 ? b : in ? L.p[j > 0 ? j - 1 : 0][i] : make_float2(0.f, 0.f);
+        if (j < m) d = cfma(xc[j], v, d);
+      }
     return d;
   };
   float2 bq[4], xv[4], hv = make_float2(0.f, 0.f);

@@ -288,7 +288,7 @@ int launch_seq(int dim, const PassSeq& q, GridBar* gb, unsigned long long limit_
   if (q.npass == 0) return 0;
   void (*kern)(const PassSeq, GridBar*, unsigned long long) = dim == 2 ? k_vcycle_seq<C, 2> : k_vcycle_seq<C, 3>;
   // shared memory of the complex64 sweep pass
-  const size_t smem = sizeof(C) != 8 ? 0 : dim == 3 ? sw3_smem(SMAX, SEQ_O3) : sizeof(Sw2Shared<SMAX, 4>);
+  const size_t smem = sizeof(C) != 8 ? 0 : dim == 3 ? sw3_smem(SMAX, SEQ_O3) : sizeof(Sw2Shared<SMAX, 6>);
   thread_local void (*last)(const PassSeq, GridBar*, unsigned long long) = nullptr;
   thread_local int occ = 1;
   if (kern != last) {
