@@ -683,6 +683,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   const int per_depth = std::max(g->nu1 == 0 ? 1 : g->nu1 * (g->s + 1), 1 + g->nu2 * (g->s + 1));
   if (g->smoother == HELM_SMOOTHER_GMRES)
     while (g->tp > 0 && (g->tc - g->tp + 1) * per_depth <= SEQ_MAX &&
+           !(g->dim == 3 && g->depth[g->tp - 1].sweep.march) &&  // (sweeps of a CTA shape of their own)
            persist_level(g->dim, g->depth[g->tp - 1].n + 1, (int)sizeof(C)))
       --g->tp;
   g->fuse2 = fused2_cycle(g->dim, h0.prec, g->smoother, g->nu1, g->nu2);

@@ -21,6 +21,21 @@ static inline int sm_count() {
   }();
   return n;
 }
+// Allow a kernel the largest dynamic shared memory the device offers beside its static part,
+// once per host thread.  The limit belongs to the kernel, not to the thread: every thread must
+// set the same value, or one would take back what another counts on.
+template <auto Kern>
+static inline void allow_smem() {
+  thread_local bool done = false;
+  if (done) return;
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (cudaFuncGetAttributes(&fa, Kern) == cudaSuccess && optin > (int)fa.sharedSizeBytes)
+    cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+  done = true;
+}
 template <typename... KArgs, typename... Args>
 static inline void pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args... args) {

@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "device_common.cuh"
+#include "launch.cuh"
 #include "dfloat.cuh"
 #include "vcycle.cuh"
 
@@ -1042,11 +1043,7 @@ static int resident_grid(K kernel, int threads, size_t smem) {
 template <typename C, int VB>
 static void launch_dots(const OuterDev<C>* od, int nprob, int chunks, int m, cudaStream_t s) {
   const size_t smem = (size_t)(DOT_THREADS / 32) * 2 * (m + 1) * sizeof(double);
-  thread_local size_t configured = 0;  // per host thread and block size; setting it again is harmless
-  if (smem > 48 * 1024 && smem > configured) {
-    cudaFuncSetAttribute(k_dots<C, VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
+  if (smem > 48 * 1024) allow_smem<k_dots<C, VB>>();
   thread_local size_t res_smem = 0;
   thread_local int resident = 0;
   if (resident == 0 || res_smem != smem) {
@@ -1079,16 +1076,9 @@ void outer_vnew(const OuterDev<C>* od, int nprob, int chunks, int m, bool start,
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     pad = (size_t)per_sm / 5 + 1024;
-    cudaFuncSetAttribute(k_vnew<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(pad, 160 * 1024));
   }
+  allow_smem<k_vnew<C>>();
   const size_t need = vnew_smem_bytes(m);
-  if (need > 160 * 1024) {
-    thread_local size_t configured = 0;
-    if (need > configured) {
-      cudaFuncSetAttribute(k_vnew<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-      configured = need;
-    }
-  }
   if (start) {
     thread_local int vres = 0;
     if (vres == 0) vres = resident_grid(k_vstart<C>, 256, 0);
@@ -1106,11 +1096,7 @@ void outer_backsolve(const OuterDev<C>* od, int nprob, cudaStream_t s) {
 template <typename C>
 void outer_solution(const OuterDev<C>* od, int nprob, int chunks, int m, cudaStream_t s) {
   const size_t smem = 2 * (size_t)(m + 1) * sizeof(double2);
-  thread_local size_t configured = 0;  // per host thread; setting the attribute again is harmless
-  if (smem > 48 * 1024 && smem > configured) {
-    cudaFuncSetAttribute(k_solution<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
+  if (smem > 48 * 1024) allow_smem<k_solution<C>>();
   k_solution<C><<<nprob * chunks, 256, smem, s>>>(od, chunks);
 }
 

@@ -13,6 +13,7 @@ namespace helm {
 // 2D levels from this size on march: 639^2 20 us a sweep against 21.7 in register regions,
 // 1023^2 25 against 37; at 511^2 and below a march of few rows is mostly halo.
 constexpr int SWEEP2_MARCH_N = 600;
+constexpr int SWEEP3_MARCH_N = 40;
 
 bool fused2_size(int n) { return n < SWEEP2_MARCH_N; }
 
@@ -54,8 +55,10 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
     c.geo_res = c.geo;
     return c;
   }
-  if (n < 96 || S > 3) {
-    c.geo = n < 64 ? 4 : 8;
+  // 3D levels from this size on march: 47^3 12 us a sweep, 63^3 14.5 against 25 in regions, 95^3
+  // 23 against 42; at 31^3 both take 10
+  if (n < SWEEP3_MARCH_N || S > 3) {
+    c.geo = S <= 3 || n < 64 ? 4 : 8;
     c.units_res = c.units = sw3_units(S, c.geo, n);
     c.geo_res = c.geo;
     return c;
@@ -100,25 +103,22 @@ static void launch_sweep_s(int dim, const LevelDev<float2>* levs, int nprob, con
   }
   if (!cfg.march) {
     const dim3 block(32, SW3_NW);
-    thread_local bool configured = false;  // per host thread; setting the attribute again is harmless
-    if (!configured) {
-      cudaFuncSetAttribute(k_sweep3<S, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw3_smem(S, 4));
-      cudaFuncSetAttribute(k_sweep3<S, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw3_smem(S, 8));
-      configured = true;
+    if constexpr (S > 3) {
+      if (cfg.geo == 8) {
+        allow_smem<k_sweep3<S, 8>>();
+        pdl_launch(k_sweep3<S, 8>, grid, block, sw3_smem(S, 8), st, levs, cfg.units, f, sl);
+        return;
+      }
     }
-    if (cfg.geo == 4) pdl_launch(k_sweep3<S, 4>, grid, block, sw3_smem(S, 4), st, levs, cfg.units, f, sl);
-    else pdl_launch(k_sweep3<S, 8>, grid, block, sw3_smem(S, 8), st, levs, cfg.units, f, sl);
+    allow_smem<k_sweep3<S, 4>>();
+    pdl_launch(k_sweep3<S, 4>, grid, block, sw3_smem(S, 4), st, levs, cfg.units, f, sl);
     return;
   }
   if constexpr (S <= 3) {
     const dim3 block(32, SM3_NW);
     const size_t smem = sm3_smem(S, cfg.geo);
-    thread_local size_t configured = 0;
-    if (configured < smem) {
-      cudaFuncSetAttribute(k_sweep3_march<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(k_sweep3_march<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      configured = smem;
-    }
+    if (phi) allow_smem<k_sweep3_march<S, true>>();
+    else allow_smem<k_sweep3_march<S, false>>();
     if (phi) pdl_launch(k_sweep3_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
     else pdl_launch(k_sweep3_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
   }
@@ -183,11 +183,7 @@ template <int S, int DIM>
 static void launch_coarse_gram_sd(const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
                                   const float2* pw, int nu1, int nu2, bool from_res, size_t smem,
                                   cudaStream_t st) {
-  thread_local size_t configured = 0;
-  if (configured < smem) {
-    cudaFuncSetAttribute(k_coarse_gram<S, DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
+  allow_smem<k_coarse_gram<S, DIM>>();
   pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, pw, nu1, nu2,
              from_res ? 1 : 0);
 }

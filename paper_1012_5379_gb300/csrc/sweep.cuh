@@ -695,8 +695,12 @@ k_sweep3(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int s
 // A CTA of 16 warps holds a 32 x 32 column of the level (two rows per warp) and marches in
 // z.  In the step that loads plane z of R_0 it forms k_j of plane z - j for every j: the z
 // neighbours are in registers (four planes of each vector), the x and y neighbours were
-// published to shared memory in the previous step, so one barrier per step suffices.  R_0
-// of the next planes is loaded ahead.  Own points: (32 - 2S)^2 columns of `zc` planes.
+// published to shared memory in the previous step, so one barrier per step suffices.  Planes
+// of R_0 (and phi) arrive in a ring of four by asynchronous copies issued two steps ahead
+// (loaded to registers ahead, their waits fell together and the field's variant spilled).
+// Bound by issue (61% active, 16 warps at 128 registers).  255^3, s = 3: 205 us a sweep, 238
+// with a field; 248 and 311 with the loads in registers.
+// Own points: (32 - 2S)^2 columns of `zc` planes.
 constexpr int SM3_NW = 16, SM3_R = 32;
 HELM_HD inline int sm3_units(int S, int n, int zc) {
   return ceil_div(n, sw_ox(S)) * ceil_div(n, sw_ox(S)) * ceil_div(n, zc);
@@ -704,7 +708,22 @@ HELM_HD inline int sm3_units(int S, int n, int zc) {
 // published planes: [parity][vector][row][lane], one guard row at either end
 HELM_HD constexpr unsigned sm3_plane() { return (SM3_R + 2) * 32; }
 HELM_HD constexpr unsigned sm3_smem(int S, int zc) {
-  return 2u * S * sm3_plane() * 8u + (unsigned)(zc + 2 * S) * 24u;
+  return (4u + 2u * (S - 1)) * sm3_plane() * 8u + 4u * SM3_R * 32u * 4u + (unsigned)(zc + 2 * S) * 24u;
+}
+// Asynchronous copies to shared memory; with ok false they fill zeros and read nothing.
+__device__ __forceinline__ void copy8_async(float2* dst, const float2* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 8 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copy4_async(float* dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copies_wait() {  // all but the N newest groups
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 template <int S, bool PHI>
@@ -725,8 +744,10 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   const int x = (unit % nt) * sw_ox(S) - S + lane;
   const int ry = 2 * warp, y = ((unit / nt) % nt) * sw_ox(S) - S + ry;  // rows y, y + 1
   const int zb = (unit / (nt * nt)) * zc, ze = min(zb + zc, n);
-  float2* const pub = swsm;                                              // 2 S planes
-  float4* const zac = reinterpret_cast<float4*>(swsm + 2 * S * sm3_plane());
+  float2* const ring = swsm;                                             // R_0: plane i in slot i & 3
+  float2* const pub = ring + 4 * sm3_plane();                            // [parity][k_1 .. k_{S-1}]
+  float* const phring = reinterpret_cast<float*>(pub + 2 * (S - 1) * sm3_plane());
+  float4* const zac = reinterpret_cast<float4*>(phring + 4 * SM3_R * 32);
   float2* const zd = reinterpret_cast<float2*>(zac + (zc + 2 * S));
   const SwCoef cx = sw_coef(L.ca, x, n, t), cy0 = sw_coef(L.ca, y, n, t), cy1 = sw_coef(L.ca, y + 1, n, t);
   const float2 dxy[2] = {cadd(cx.d, cy0.d), cadd(cx.d, cy1.d)};
@@ -735,7 +756,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
     zac[i] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
     zd[i] = c.d;
   }
-  for (int i = tid; i < 2 * S * (int)sm3_plane(); i += SM3_NW * 32) pub[i] = make_float2(0.f, 0.f);
+  for (int i = tid; i < (4 + 2 * (S - 1)) * (int)sm3_plane(); i += SM3_NW * 32) ring[i] = make_float2(0.f, 0.f);
   pdl_wait();
   float2 sg[S];
   gram_shifts<S>(L, first != 0, sg);
@@ -750,15 +771,18 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
 #pragma unroll
     for (int w = 0; w < W; ++w) win[j][w][0] = win[j][w][1] = make_float2(0.f, 0.f);
   float phw[W][2];
-  float2 nxt[W][2];
-  float phn[W][2];
-  auto fetch = [&](int z, float2 (&v)[2], float (&f)[2]) {
-    const bool zin = (unsigned)z < (unsigned)n;
-    v[0] = (zin && in0) ? R0[col + (long long)(z * PP)] : make_float2(0.f, 0.f);
-    v[1] = (zin && in1) ? R0[col + P + (long long)(z * PP)] : make_float2(0.f, 0.f);
-    if (PHI) {  // some problem of the launch has a field; this one may not
-      f[0] = (phi && zin && in0) ? __ldg(phi + (col + (long long)(z * PP))) : phir;
-      f[1] = (phi && zin && in1) ? __ldg(phi + (col + P + (long long)(z * PP))) : phir;
+  const bool field = PHI && phi;  // some problem of the launch has a field; this one may not
+  const int at0 = (ry + 1) * 32 + lane;
+  auto fetch = [&](int z, int slot) {
+    const bool zin = (unsigned)z < (unsigned)n, ok0 = zin && in0, ok1 = zin && in1;
+    const long long i = col + (long long)(z * PP);
+    float2* const d = ring + slot * sm3_plane() + at0;
+    copy8_async(d, ok0 ? R0 + i : R0, ok0);
+    copy8_async(d + 32, ok1 ? R0 + i + P : R0, ok1);
+    if (PHI && field) {
+      float* const f = phring + slot * SM3_R * 32 + ry * 32 + lane;
+      copy4_async(f, ok0 ? phi + i : phi, ok0);
+      copy4_async(f + 32, ok1 ? phi + i + P : phi, ok1);
     }
   };
   float acc[NS];
@@ -768,12 +792,17 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   const bool own0 = ox && ry >= S && ry < SM3_R - S && y < n;
   const bool own1 = ox && ry + 1 >= S && ry + 1 < SM3_R - S && y + 1 < n;
   const int zf = zb - S, zl = ze + S;  // planes loaded: zf .. zl - 1
-  constexpr int AHEAD = 2;             // planes of loads in flight beyond the current one
+  constexpr int AHEAD = 2;             // planes of copies in flight beyond the current one
+  __syncthreads();                     // the ring is cleared before copies land in it
 #pragma unroll
-  for (int u = 0; u < AHEAD; ++u) fetch(zf + u, nxt[u], phn[u]);
+  for (int u = 0; u < AHEAD; ++u) {
+    fetch(zf + u, u);
+    copies_commit();
+  }
+  copies_wait<AHEAD - 1>();
   __syncthreads();
-  // step i loads plane zf + i; slots are indexed by i & 3, which the unrolling by four
-  // makes static
+  // step i takes plane zf + i; slots are indexed by i & 3, which the unrolling by four
+  // makes static.  Its copies overwrite plane i - 2, last read in the step before.
 #pragma unroll 1
   for (int i0 = 0; i0 < zl - zf; i0 += W) {
 #pragma unroll
@@ -781,20 +810,18 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
       const int i = i0 + u;
       if (i >= zl - zf) break;  // uniform
       const int z = zf + i;
-      float2 k0[2];
-      k0[0] = nxt[u][0];
-      k0[1] = nxt[u][1];
+      if (z + AHEAD < zl) fetch(z + AHEAD, (u + AHEAD) & 3);
+      copies_commit();
+      const float2* const r0 = ring + u * sm3_plane() + at0;
+      win[0][u][0] = r0[0];
+      win[0][u][1] = r0[32];
       if (PHI) {
-        phw[u][0] = phn[u][0] * t;
-        phw[u][1] = phn[u][1] * t;
+        const float* const f = phring + u * SM3_R * 32 + ry * 32 + lane;
+        phw[u][0] = field ? f[0] * t : phc;
+        phw[u][1] = field ? f[32] * t : phc;
       }
-      if (z + AHEAD < zl) fetch(z + AHEAD, nxt[(u + AHEAD) & 3], phn[(u + AHEAD) & 3]);
-      const float2* rd = pub + (size_t)((u & 1) ^ 1) * S * sm3_plane() + (ry + 1) * 32 + lane;
-      float2* wr = pub + (size_t)(u & 1) * S * sm3_plane() + (ry + 1) * 32 + lane;
-      win[0][u][0] = k0[0];
-      win[0][u][1] = k0[1];
-      wr[0] = k0[0];
-      wr[32] = k0[1];
+      const float2* rd = pub + (size_t)((u & 1) ^ 1) * (S - 1) * sm3_plane() + at0;
+      float2* wr = pub + (size_t)(u & 1) * (S - 1) * sm3_plane() + at0;
       float2 last[2];
 #pragma unroll
       for (int j = 1; j <= S; ++j) {
@@ -805,7 +832,8 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
         if (iz >= 0) {         // uniform
           const float4 za = zac[iz];
           const float2 zdd = zd[iz];
-          const float2* s = rd + (size_t)(j - 1) * sm3_plane();
+          // k_{j-1} of plane z - j as published
+          const float2* s = j == 1 ? ring + ((u + 3) & 3) * sm3_plane() + at0 : rd + (size_t)(j > 1 ? j - 2 : 0) * sm3_plane();
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             float2 dg = dxy[q];
@@ -827,8 +855,8 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
         if (j < S) {
           win[j][c][0] = r[0];
           win[j][c][1] = r[1];
-          wr[(size_t)j * sm3_plane()] = r[0];
-          wr[(size_t)j * sm3_plane() + 32] = r[1];
+          wr[(size_t)(j - 1) * sm3_plane()] = r[0];
+          wr[(size_t)(j - 1) * sm3_plane() + 32] = r[1];
         } else {
           last[0] = r[0];
           last[1] = r[1];
@@ -852,6 +880,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
           }
         }
       }
+      copies_wait<AHEAD - 1>();
       __syncthreads();
     }
   }

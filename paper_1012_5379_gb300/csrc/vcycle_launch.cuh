@@ -40,14 +40,8 @@ static int tiles_per_cta(K kernel, int ntiles, size_t smem = 0) {
 template <int QY>
 static void resid_tma3(const LevelDev<float2>* levs, int nprob, int P, const Tma3Params& tp, cudaStream_t st) {
   const size_t smem = tma3_smem(1, QY, tp.stages);
-  // per host thread: the largest dynamic shared memory set so far, and the residency
-  // of the last configuration
-  thread_local size_t configured = 0;
-  thread_local int occ_stages = -1, occ = 1;
-  if (configured < smem) {
-    cudaFuncSetAttribute(k_resid_tma3<QY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
+  thread_local int occ_stages = -1, occ = 1;  // per host thread: the residency of the last configuration
+  allow_smem<k_resid_tma3<QY>>();
   if (occ_stages != tp.stages) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_resid_tma3<QY>, 256, smem) != cudaSuccess || occ < 1)
       occ = 1;
@@ -108,12 +102,8 @@ static void restrict_tma3(const LevelDev<float2>* levs, int nprob, int P, bool r
                           bool nosmooth, int nraw, cudaStream_t st) {
   const Tma3Params tp = tma3_params(TP_RESTRICT, P);
   const size_t smem = (size_t)tp.stages * nraw * tm3_box_stride(2);
-  thread_local size_t configured = 0;
   thread_local int occ_key = -1, occ = 1;
-  if (configured < smem) {
-    cudaFuncSetAttribute(k_restrict_tma3<SMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
+  allow_smem<k_restrict_tma3<SMAX>>();
   const int key = tp.stages * 16 + nraw;
   if (occ_key != key) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_restrict_tma3<SMAX>, 256, smem) != cudaSuccess || occ < 1)
@@ -180,18 +170,7 @@ void launch_coarse(int dim, const LevelDev<C>* levs, int nlev, int lev_stride, c
 template <typename C>
 void launch_coarse_smem(int dim, const LevelDev<C>* levs, int nlev, int lev_stride, const CoarseLU* lus, int nprob,
                         int nu1, int nu2, size_t smem_bytes, cudaStream_t st) {
-  // the static part (descriptors, sweep scalars) counts against the same limit: allow
-  // the largest dynamic part the device offers, once per host thread
-  thread_local bool configured = false;
-  if (!configured) {
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (cudaFuncGetAttributes(&fa, k_coarse_smem<C>) == cudaSuccess && optin > (int)fa.sharedSizeBytes)
-      cudaFuncSetAttribute(k_coarse_smem<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-    configured = true;
-  }
+  allow_smem<k_coarse_smem<C>>();
   pdl_launch(k_coarse_smem<C>, dim3(nprob), dim3(512), smem_bytes, st, levs, nlev, lev_stride, lus, nu1, nu2, dim);
 }
 
