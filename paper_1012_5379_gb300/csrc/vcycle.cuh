@@ -81,6 +81,23 @@ __device__ __forceinline__ C interp(const C* xcb, int n, int nc, int Pc, int x, 
   typedef typename CT<C>::R R;
   C acc = czero<C>();
   if (!inside(x, y, z, n)) return acc;
+  if constexpr (sizeof(C) == 8) {
+    // every load in flight before the first is used (complex128 keeps the loop below: its
+    // additions of zeros would cost more than the loads)
+    const int X = x >> 1, Y = y >> 1, Z = z >> 1;
+    const bool ex = !(x & 1), ey = !(y & 1), ez = dim == 3 && !(z & 1);
+    C v[2][2][2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int a = i & 1, b = (i >> 1) & 1, c = i >> 2;  // 0: the lower neighbour of an even position
+      const bool use = (a || ex) && (b || ey) && (c || ez);
+      const int p = X - 1 + a, q = Y - 1 + b, r = dim == 3 ? Z - 1 + c : 0;
+      v[c][b][a] = use && inside(p, q, r, nc) ? xcb[pidx(p, q, r, Pc)] : czero<C>();
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc = cadd(acc, v[i >> 2][(i >> 1) & 1][i & 1]);
+    return cscale(acc, (ex ? 0.5f : 1.0f) * (ey ? 0.5f : 1.0f) * (ez ? 0.5f : 1.0f));
+  }
   int ix[2], iy[2], iz[2];
   R wx, wy, wz;
   int nx, ny, nz;
