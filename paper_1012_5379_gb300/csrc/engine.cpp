@@ -1423,7 +1423,6 @@ struct ActiveSet {
       for (Handle* m : o.members) o.sum_j1 += m->last_j + 1;
     }
     TRY(run_iteration<C>(*g, st));
-    run_cycle_end<C>(*g, st);
     CUDA_TRY(cudaGetLastError());
     graph_pending = g;
     if (pin_cap < members.size()) {
@@ -1432,12 +1431,16 @@ struct ActiveSet {
       pin_cap = std::max<size_t>(2 * members.size(), 16);
       CUDA_TRY(cudaMallocHost(&pin, sizeof(OuterState) * pin_cap));
     }
+    n_read = members.size();
+    return read_states(st);
+  }
+  // Gather the states of the n_read members to pinned host memory.
+  int read_states(cudaStream_t st) {
     {
       Launch L("io.state", st, 0, 0);
-      gather_states(d_src, d_stage, (int)members.size(), st);
+      gather_states(d_src, d_stage, (int)n_read, st);
     }
-    CUDA_TRY(cudaMemcpyAsync(pin, d_stage, members.size() * sizeof(OuterState), cudaMemcpyDeviceToHost, st));
-    n_read = members.size();
+    CUDA_TRY(cudaMemcpyAsync(pin, d_stage, n_read * sizeof(OuterState), cudaMemcpyDeviceToHost, st));
     return HELM_OK;
   }
   // Wait for the last iterate() (synchronises st); finished members move to `done`.
@@ -1445,6 +1448,17 @@ struct ActiveSet {
   int collect(cudaStream_t st, std::vector<std::pair<Handle*, OuterState>>* done) {
     if (n_read == 0) return HELM_OK;
     CUDA_TRY(cudaStreamSynchronize(st));
+    // Cycle ends (four passes per size) run only when some problem's cycle has ended, an
+    // iteration in restart or so; enqueued every time they found nothing to do in 30 to 120 us
+    // of launches and CTAs (a batch of eight 2D problems 134.6 -> 130 ms, 255^3 210 -> 205).
+    bool ended = false;
+    for (size_t p = 0; p < n_read; ++p) ended = ended || pin[p].cycle_end;
+    if (ended) {
+      run_cycle_end<C>(*g, st);
+      TRY(read_states(st));
+      CUDA_TRY(cudaGetLastError());
+      CUDA_TRY(cudaStreamSynchronize(st));
+    }
     if (graph_pending) {
       harvest(graph_pending->vrecs);  // timed V-cycle launches of the replay just completed
       graph_pending = nullptr;
