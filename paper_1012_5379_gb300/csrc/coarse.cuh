@@ -234,26 +234,37 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
     float2 rc[S + 1];
 #pragma unroll
     for (int j = 0; j <= S; ++j) rc[j] = L.scf->rcoef[j];
+    // a warp per coarse row (n <= 31), fine points in pairs, each row read once per coarse row:
+    // nine single loads a point and vector took 2 us more at n = 31
+    const int lane = tid & 31, n = L.n;
+    for (int y = tid >> 5; y < n; y += CG_NW) {
+      float4 v[3][S + 1];
+      const bool ok = lane <= n;
 #pragma unroll
-    for (int q = 0; q < CG_PT; ++q) {
-      if (!V.on[q]) continue;
-      const size_t f = (size_t)(2 * V.cy[q]) * Pf + 2 * V.cx[q];
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j <= S; ++j) {
+          const float2* R = j == 0 ? L.fb : L.fp[j > 0 ? j - 1 : 0];
+          v[i][j] = ok ? *reinterpret_cast<const float4*>(R + (size_t)(2 * y + i) * Pf + 2 * lane)
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       float2 out = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int dy = 0; dy < 3; ++dy)
+      for (int i = 0; i < 3; ++i) {
+        float2 r0 = make_float2(0.f, 0.f), r1 = r0;
 #pragma unroll
-        for (int dx = 0; dx < 3; ++dx) {
-          const size_t i = f + (size_t)dy * Pf + dx;
-          float2 r = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int j = 0; j <= S; ++j)
-          {
-            const float2 v = j == 0 ? L.fb[i] : L.fp[j > 0 ? j - 1 : 0][i];
-            if (j <= m) r = cfma(rc[j], v, r);
+        for (int j = 0; j <= S; ++j)
+          if (j <= m) {  // uniform
+            r0 = cfma(rc[j], make_float2(v[i][j].x, v[i][j].y), r0);
+            r1 = cfma(rc[j], make_float2(v[i][j].z, v[i][j].w), r1);
           }
-          out = cadd(out, cscale(r, (dx == 1 ? 0.5f : 0.25f) * (dy == 1 ? 0.5f : 0.25f)));
-        }
-      V.b[V.off[q]] = out;
+        const float2 r2 = shfl_down_c(r0, 1);
+        const float w = i == 1 ? 0.125f : 0.0625f;
+        out = cadd(out, cscale(r0, w));
+        out = cadd(out, cscale(r1, 2.0f * w));
+        out = cadd(out, cscale(r2, w));
+      }
+      if (lane < n) V.b[y * L.P + lane] = out;
     }
   } else {
 #pragma unroll
