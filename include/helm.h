@@ -376,7 +376,8 @@ int helm_tuning_load(const char* path);
  * step J (0 for the other passes): writes its 4 integers into v and returns 1, or
  * returns 0 when the table has none (the built-in default applies).  v: 2D passes
  * {tiles per CTA}; 3D restrict and prolong {TMA-fed pass on, plane slots, z pieces per
- * column (0: one share per resident CTA), points per thread in y}; "persist" {persistent segment on};
+ * column (0: one share per resident CTA), points per thread in y}; "persist" {persistent segment on
+ * (not used on 3D complex64 levels from 40^3 on, whose sweeps march)};
  * "zplanes" (3D levels without the TMA-fed passes) {planes each CTA marches: 2, 4, 8 or
  * 16}.  Host only. */
 int helm_tuning_get(const char* pass, int dim, int P, int prec, int J, int* v);

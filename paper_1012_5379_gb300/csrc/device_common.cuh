@@ -154,16 +154,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
 __device__ __forceinline__ void tmap_acquire(const CUtensorMap* tm) {
   asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tm) : "memory");
 }
-// 2D tiled TMA load of the box at element coordinates (c0, c1) into shared memory,
+// 3D tiled TMA load of the box at element coordinates (c0, c1, c2) into shared memory,
 // completing on `bar`.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int c0, int c1, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_addr(dst)), "l"(tm), "r"(c0), "r"(c1), "r"(smem_addr(bar))
-      : "memory");
-}
-
-// 3D tiled TMA load of the box at element coordinates (c0, c1, c2).
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"

@@ -302,21 +302,25 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     // flat passes: one wave of four CTAs per SM at most (their occupancy), so every CTA
     // streams an equal share and no partial second wave trails
     L.nflat = (int)std::max<size_t>(1, std::min<size_t>(std::min(1024, 4 * sm_count_host()), (L.np + 1023) / 1024));
-    TRY(dev_alloc(h.get(), &L.b, L.np * eb));
-    TRY(dev_alloc(h.get(), &L.xa, L.np * eb));
-    TRY(dev_alloc(h.get(), &L.xb, L.np * eb));
-    TRY(dev_alloc(h.get(), &L.r0, L.np * eb));
-    for (int j = 0; j < h->s; ++j) TRY(dev_alloc(h.get(), &L.p[j], L.np * eb));
-    for (void* v : {L.b, L.xa, L.xb, L.r0}) CUDA_TRY(cudaMemsetAsync(v, 0, L.np * eb, st));
     if (h->prec == HELM_C64) L.sweep = sweep_cfg(h->dim, L.n, h->s, sm_count_host());
-    if (fused2_level(*h, L)) {
-      L.q[0] = L.xa;
-      for (int j = 1; j < h->s - 1; ++j) {
-        TRY(dev_alloc(h.get(), &L.q[j], L.np * eb));
-        CUDA_TRY(cudaMemsetAsync(L.q[j], 0, L.np * eb, st));
-      }
-    }
-    for (int j = 0; j < h->s; ++j) CUDA_TRY(cudaMemsetAsync(L.p[j], 0, L.np * eb, st));
+    // the level's vectors in one allocation, cleared at once (a cudaMalloc and a memset each took
+    // most of a small problem's set-up)
+    const size_t vb = (L.np * eb + 255) / 256 * 256;
+    const int nq = fused2_level(*h, L) ? std::max(0, h->s - 2) : 0;
+    char* vecs = nullptr;
+    TRY(dev_alloc(h.get(), &vecs, (4 + h->s + nq) * vb));
+    CUDA_TRY(cudaMemsetAsync(vecs, 0, (4 + h->s + nq) * vb, st));
+    auto take = [&](void** v) {
+      *v = vecs;
+      vecs += vb;
+    };
+    take(&L.b);
+    take(&L.xa);
+    take(&L.xb);
+    take(&L.r0);
+    for (int j = 0; j < h->s; ++j) take(&L.p[j]);
+    if (fused2_level(*h, L)) L.q[0] = L.xa;
+    for (int j = 1; j <= nq; ++j) take(&L.q[j]);
     const size_t scb = h->prec == HELM_C128 ? sizeof(SweepScalarsT<double>) : sizeof(SweepScalarsT<float>);
     TRY(dev_alloc(h.get(), &L.sc, scb));
     CUDA_TRY(cudaMemsetAsync(L.sc, 0, scb, st));
@@ -1667,7 +1671,7 @@ size_t estimate_handle_bytes(int dim, int n, int prec, int s, int restart, int m
   size_t bytes = 0;
   for (int nl : sizes) {
     const size_t P = nl + 1, np = dim == 3 ? P * P * P : P * P;
-    bytes += (4 + (size_t)s) * np * eb + 3 * nl * (eb + sizeof(double2)) + 4096;
+    bytes += (4 + (size_t)s) * (np * eb + 255) + 3 * nl * (eb + sizeof(double2)) + 4096;
   }
   const size_t P0 = n + 1, vs = dim == 3 ? P0 * P0 * P0 : P0 * P0;
   const size_t m = restart > 0 ? std::min(restart, maxit) : maxit;
@@ -1678,7 +1682,7 @@ size_t estimate_handle_bytes(int dim, int n, int prec, int s, int restart, int m
     for (int nl : sizes) {
       const SweepCfg c = sweep_cfg(dim, nl, s, sm_count_host());
       bytes += (size_t)std::max(c.units, c.units_res) * GRAM_SLOT * sizeof(float2);
-      if (dim == 2 && fused2_size(nl) && s > 2) bytes += (size_t)(s - 2) * (nl + 1) * (nl + 1) * eb;
+      if (dim == 2 && fused2_size(nl) && s > 2) bytes += (size_t)(s - 2) * ((nl + 1) * (nl + 1) * eb + 255);
     }
   return bytes;
 }

@@ -766,7 +766,8 @@ __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__
   }
 }
 template <typename C, int Q>
-__global__ void __launch_bounds__(256, sizeof(C) == 16 ? 2 : 3)
+// (complex64 4095^2: 130 us at four CTAs per SM, 142 at three, 155 at five with spills)
+__global__ void __launch_bounds__(256, sizeof(C) == 16 ? 2 : 4)
 k_restrict_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int x_from_zero,
               int nosmooth) {
   restrict_t2_body<C, Q>(levs, ntiles, tpc, r0_is_b, x_from_zero, nosmooth, blockIdx.x);

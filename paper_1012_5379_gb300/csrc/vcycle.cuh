@@ -138,23 +138,6 @@ __device__ __forceinline__ UpdCoef<C> load_upd(const LevelDev<C>& L, int r0_is_b
   }
   return u;
 }
-// x-increment and residual at a point: dx = sum_{k<m} xc[k] R_k and, if want_r,
-// r = sum_{k<=m} rc[k] R_k.
-template <typename C, bool NC = true>
-__device__ __forceinline__ void upd_point(const UpdCoef<C>& u, int x, int y, int z, int n, int P,
-                                          C& dx, C& r, bool want_r = true) {
-  dx = czero<C>();
-  r = czero<C>();
-#pragma unroll
-  for (int k = 0; k <= SMAX; ++k) {
-    if (k < u.m || (want_r && k == u.m)) {
-      C v = ldc<C, NC>(u.Rk[k], x, y, z, n, P);
-      if (k < u.m) dx = cfma(u.xc[k], v, dx);
-      r = cfma(u.rc[k], v, r);
-    }
-  }
-}
-
 // Pointwise end of a sweep: x += dx (in place on xa or xb, or from zero) and, in
 // residual mode, r0 <- r (in place) with ||r||^2 starting the next sweep.  Every
 // vector is zero at the padding positions, so this is a plain stream over the padded
@@ -369,14 +352,12 @@ k_prolong_flat(const LevelDev<C>* __restrict__ levs, int ntiles, int dim) {
 }
 
 // ------------------------------------------------------------------ coarse levels
-// The sub-cycle of the coarse levels (sizes where a grid-wide launch is all latency)
-// runs on a "team" per problem: one CTA, or a thread-block cluster whose CTAs act as
-// one block.  Every pass is a team-wide loop over the level's points; sync() orders
-// all of the team's global-memory accesses; sum() totals per-thread values in a fixed
-// order and leaves the totals with thread 0 of every CTA, which then runs the small
-// sweep algebra on its CTA's own copy of the sweep scalars (bitwise the same in every
-// CTA, so no further exchange is needed).  The coarsest level is a dense FP64 LU solve
-// by one warp.
+// The sub-cycle of the coarse levels (sizes where a grid-wide launch is all latency) runs on
+// a "team" per problem, one CTA (complex64 levels that fit in shared memory: coarse.cuh).  Every
+// pass is a team-wide loop over the level's points; sync() orders all of the team's memory
+// accesses; sum() totals per-thread values in a fixed order and leaves the totals with thread 0,
+// which then runs the small sweep algebra.  The coarsest level is solved in FP64 by one warp or
+// by its inverse.
 struct CtaTeam {
   __device__ __forceinline__ int rank() const { return 0; }
   __device__ __forceinline__ unsigned gtid() const { return (unsigned)flat_tid(); }
