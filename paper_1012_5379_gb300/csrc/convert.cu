@@ -78,10 +78,12 @@ template <> __device__ __forceinline__ float2 dense_coef<float2>(const double2* 
 }
 enum { AX_REAL, AX_SAME, AX_ANY };
 enum { EVEN = 12, GENERAL = 13 };
-__device__ __forceinline__ int axis_case(double2 a, double2 c) {
+// (The complex shift of M is in the diagonals alone: an axis with real off-diagonals and a
+// complex diagonal is AX_SAME or AX_ANY.)
+__device__ __forceinline__ int axis_case(double2 a, double2 d, double2 c) {
   const long long dx = __double_as_longlong(a.x) ^ __double_as_longlong(c.x);
   const long long dy = __double_as_longlong(a.y) ^ __double_as_longlong(c.y);
-  if (((__double_as_longlong(a.y) | __double_as_longlong(c.y)) << 1) == 0) return AX_REAL;
+  if (((__double_as_longlong(a.y) | __double_as_longlong(d.y) | __double_as_longlong(c.y)) << 1) == 0) return AX_REAL;
   return (dx | dy) == 0 ? AX_SAME : AX_ANY;
 }
 template <int CASE, typename C>
@@ -131,25 +133,26 @@ k_apply_dense(int n, int rows, const double2* __restrict__ ca, const double2* __
   const bool on = x < n && y < n;
   const C zero = czero<C>();
   auto coef = [&](const double2* p, int i) { return dense_coef<C>(p + i); };
-  C ax = zero, qx = zero, ay = zero, qy = zero, dxy = zero;
+  C ax = zero, qx = zero, ay = zero, qy = zero, dx0 = zero, dy0 = zero;
   if (on) {
     ax = coef(ca, x);
     qx = coef(cc, x);
-    dxy = coef(cd, x);
+    dx0 = coef(cd, x);
     if (DIM == 3) {
       ay = coef(ca, y);
       qy = coef(cc, y);
-      dxy = cadd(dxy, coef(cd, y));
+      dy0 = coef(cd, y);
     }
   }
+  const C dxy = DIM == 3 ? cadd(dx0, dy0) : dx0;
   int cx = GENERAL, cy = 0;
   bool even = false;
   if constexpr (sizeof(C) == 16) {  // uniform over the warp: lanes past the edge agree with any case
     const unsigned full = 0xffffffffu;
-    const int lx = on ? axis_case(ax, qx) : -1;
+    const int lx = on ? axis_case(ax, dx0, qx) : -1;
     cx = __all_sync(full, lx <= AX_REAL) ? AX_REAL : __all_sync(full, lx < 0 || lx == AX_SAME) ? AX_SAME : AX_ANY;
     if (DIM == 3) {
-      const int ly = on ? axis_case(ay, qy) : -1;
+      const int ly = on ? axis_case(ay, dy0, qy) : -1;
       cy = __all_sync(full, ly <= AX_REAL) ? AX_REAL : __all_sync(full, ly < 0 || ly == AX_SAME) ? AX_SAME : AX_ANY;
       const long long dx = __double_as_longlong(ax.x) ^ __double_as_longlong(ay.x);
       const long long dy = __double_as_longlong(ax.y) ^ __double_as_longlong(ay.y);
@@ -194,7 +197,7 @@ k_apply_dense(int n, int rows, const double2* __restrict__ ca, const double2* __
       C p;
 #define DENSE(X, Y, Z) dense_point<X, Y, Z, DIM>(ax, qx, ay, qy, az, qz, dxy, dz, f, xm, xp, ym, yp, vm, vp, v0)
       if constexpr (sizeof(C) == 16) {
-        const int cz = axis_case(az, qz);  // of the row: uniform
+        const int cz = axis_case(az, dz, qz);  // of the row: uniform
         int mode = cy == AX_ANY || cz == AX_ANY ? GENERAL : (cx * 2 + cy) * 2 + cz;
         if (DIM == 3 && even && cz == AX_SAME) {
           const long long dx = __double_as_longlong(ax.x) ^ __double_as_longlong(az.x);

@@ -46,3 +46,23 @@ def test_operator_cases(helm, dim, n, tb, field, prec, tol):
         h.apply_operator(vt, wt, which)
         got = wt.cpu().numpy().astype(np.complex128)
         assert np.linalg.norm(got - want) <= tol * np.linalg.norm(want), which
+
+
+@pytest.mark.parametrize("prec,tol", [("c128", 1e-13), ("c64", 1e-6)])
+@pytest.mark.parametrize("dim,n,tb,eps", [(2, 127, 0.0, 0.5), (2, 255, 0.0, 0.1), (2, 255, 0.3, 0.5), (3, 95, 0.0, 0.5),
+                                          (3, 63, 0.25, 0.3)])
+def test_complex_shift(helm, dim, n, tb, eps, prec, tol):
+    """M with the complex shift in its diagonal (csl_eps), at sizes where whole warps lie between
+    the absorbing layers and every off-diagonal there is real (theta_beta = 0): the worst point
+    too, as a term lost in part of the grid is a step at the edge of that part."""
+    k = 0.3 * (n + 1)
+    L = O.build_hierarchy(dim, n, tb, TG, WF, k=k, csl_eps=eps)[0]
+    h = helm.Handle(dim, n, tb, k=k, precision=prec, csl_eps=eps)
+    v = I.random_source(dim, n, 5)
+    vt = torch.from_numpy(np.ascontiguousarray(v)).to("cuda", torch.complex128 if prec == "c128" else torch.complex64)
+    for which, want in (("M", L.apply(v)), ("H", L.apply_h(v))):
+        wt = torch.empty_like(vt)
+        h.apply_operator(vt, wt, which)
+        got = wt.cpu().numpy().astype(np.complex128)
+        assert np.linalg.norm(got - want) <= tol * np.linalg.norm(want), which
+        assert np.max(np.abs(got - want)) <= tol * np.max(np.abs(want)), which
