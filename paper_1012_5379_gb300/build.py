@@ -15,9 +15,9 @@ LIB = os.path.join(PKG, "libhelm.so")
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU = ["vcycle_c64.cu", "vcycle_c128.cu", "sweep.cu", "outer.cu", "convert.cu", "noalloc.cu"]
+CU = ["vcycle_c64.cu", "vcycle_c128.cu", "sweep.cu", "sweep_wide.cu", "outer.cu", "convert.cu", "noalloc.cu"]
 CPP = ["engine.cpp", "geometry.cpp", "capi.cpp", "profiler.cpp", "serve.cpp", "tma.cpp", "tune.cpp", "autotune.cpp"]
-HEADERS = ["poly.h", "helm_internal.h", "device_common.cuh", "vcycle.cuh", "tiles.cuh", "vcycle_launch.cuh", "launch.cuh", "gram.cuh", "sweep.cuh",
+HEADERS = ["poly.h", "helm_internal.h", "device_common.cuh", "vcycle.cuh", "tiles.cuh", "vcycle_launch.cuh", "launch.cuh", "gram.cuh", "sweep.cuh", "sweep_launch.cuh",
            "coarse.cuh", "poly.cuh", "dfloat.cuh", "engine.h", "geometry.h", "profiler.h"]
 
 

@@ -88,7 +88,7 @@ struct CgLevel {
 };
 
 struct CgShared {
-  float wsum[CG_NW * 32];
+  float2 wsum[CG_NW * 32];
   float2 gs[gram_nv(SMAX)];
   float2 xc[SMAX], rc[SMAX + 1];
 };
@@ -97,7 +97,7 @@ struct CgShared {
 // the CTA) -> x += dx and k0 = the new residual.
 template <int S, int DIM>
 __device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2* R0, float2 (&k0)[CG_PT],
-                                         float2 (&x)[CG_PT], const float2 (&sg)[S], CgShared& sh) {
+                                         float2 (&x)[CG_PT], const float2 (&sg)[S], bool wide, CgShared& sh) {
   constexpr int NS = gram_ns(S);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float2 k[CG_PT][S + 1];
@@ -119,13 +119,22 @@ __device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2*
   float acc[NS];
 #pragma unroll
   for (int i = 0; i < NS; ++i) acc[i] = 0.f;
+  if (wide) {
+    float c[NS];
 #pragma unroll
-  for (int q = 0; q < CG_PT; ++q) gram_point<S>(k[q], acc);
-  gram_block_sum<S, CG_NW>(acc, sh.wsum, sh.gs);
+    for (int i = 0; i < NS; ++i) c[i] = 0.f;
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) gram_point_wide<S>(k[q], acc, c);
+    gram_block_sum_wide<S, CG_NW>(acc, c, sh.wsum, sh.gs);
+  } else {
+#pragma unroll
+    for (int q = 0; q < CG_PT; ++q) gram_point<S>(k[q], acc);
+    gram_block_sum<S, CG_NW>(acc, sh.wsum, sh.gs);
+  }
   __syncthreads();
   if (warp == 0) {
     float2 xk, rk;
-    gram_solve<S>(sh.gs, sg[0], sg[S > 1 ? 1 : 0], V.t, lane, xk, rk);
+    gram_solve<S>(sh.gs, sg, wide, V.t, lane, xk, rk);
     if (lane < S) sh.xc[lane] = xk;
     if (lane <= S) sh.rc[lane] = rk;
   }
@@ -171,7 +180,7 @@ __device__ __forceinline__ void cg_poly(const CgLevel<S, DIM>& V, const float2 (
   }
 }
 
-template <int S, int DIM>
+template <int S, int DIM, int WIDE>  // 1: some level of the problem's is wide
 __global__ void __launch_bounds__(CG_THREADS, 1)
 k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, const CoarseLU* __restrict__ lus,
               const float2* __restrict__ pw, int nu1, int nu2, int from_res) {
@@ -304,8 +313,9 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
     const float2* R0 = V.b;
     for (int sw = 0; sw < nu1; ++sw) {
       float2 sg[S];
-      gram_shifts<S>(Ls[l], sw == 0, sg);
-      cg_sweep<S, DIM>(V, R0, k0, x, sg, sh);
+      const bool wide = WIDE && Ls[l].wide;
+      gram_shifts<S>(Ls[l], sw == 0, wide, sg);
+      cg_sweep<S, DIM>(V, R0, k0, x, sg, wide, sh);
       R0 = V.r;
 #pragma unroll
       for (int q = 0; q < CG_PT; ++q)
@@ -439,8 +449,9 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
       __syncthreads();
       for (int sw = 0; sw < nu2; ++sw) {
         float2 sg[S];
-        gram_shifts<S>(Ls[l], false, sg);
-        cg_sweep<S, DIM>(V, V.r, k0, x, sg, sh);
+        const bool wide = WIDE && Ls[l].wide;
+        gram_shifts<S>(Ls[l], false, wide, sg);
+        cg_sweep<S, DIM>(V, V.r, k0, x, sg, wide, sh);
         if (sw + 1 < nu2) {
 #pragma unroll
           for (int q = 0; q < CG_PT; ++q)

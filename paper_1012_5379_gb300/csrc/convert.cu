@@ -4,6 +4,7 @@
 #include "vcycle.cuh"
 #include "../../include/helm.h"
 #include <algorithm>
+#include <cstring>
 
 namespace helm {
 
@@ -41,6 +42,29 @@ __global__ void k_scatter_phi(int dim, int n, int stride, int nf, const float* _
       v = phi_f[(fz * nf + fy) * nf + fx];
     }
     dst[i] = v;
+  }
+}
+
+// Largest and smallest finite value of a level's field: out[0] the largest as bits ordered like
+// the values, out[1] the smallest as their complement (both zero before, and if there is none).
+__global__ void __launch_bounds__(256) k_phi_range(int dim, int n, const float* __restrict__ phi, unsigned* out) {
+  const int P = n + 1, rows = dim == 3 ? n * n : n;
+  unsigned hi = 0u, lo = 0u;
+  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += gridDim.x * 8) {
+    const float* r = phi + (dim == 3 ? ((size_t)(row / n) * P + row % n) * P : (size_t)row * P);
+    for (int x = threadIdx.x & 31; x < n; x += 32) {
+      const float v = r[x];
+      if (!isfinite(v)) continue;
+      const unsigned b = __float_as_uint(v), o = b & 0x80000000u ? ~b : b | 0x80000000u;
+      hi = max(hi, o);
+      lo = max(lo, ~o);
+    }
+  }
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  lo = __reduce_max_sync(0xffffffffu, lo);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(out, hi);
+    atomicMax(out + 1, lo);
   }
 }
 
@@ -250,6 +274,20 @@ void convert_padded_to_dense_c128(int dim, int n, const double2* src, double2* d
 void scatter_phi(int dim, int n_level, int stride, int n_fine, const float* phi_f, float* dst, cudaStream_t st) {
   const size_t P = n_level + 1;
   k_scatter_phi<<<grid_for(dim == 3 ? P * P * P : P * P), 256, 0, st>>>(dim, n_level, stride, n_fine, phi_f, dst);
+}
+void phi_range(int dim, int n, const float* phi_pad, unsigned* out, cudaStream_t st) {
+  const int rows = dim == 3 ? n * n : n;
+  k_phi_range<<<std::min((rows + 7) / 8, 1024), 256, 0, st>>>(dim, n, phi_pad, out);
+}
+void phi_range_values(const unsigned* bits, double* lo, double* hi) {
+  auto value = [](unsigned o) {
+    const unsigned b = o & 0x80000000u ? o & 0x7fffffffu : ~o;
+    float v;
+    std::memcpy(&v, &b, sizeof v);
+    return (double)v;
+  };
+  *hi = bits[0] ? value(bits[0]) : 0.0;
+  *lo = bits[1] ? value(~bits[1]) : 0.0;
 }
 void apply_operator_dense(int dim, int n, const double2* ca, const double2* cd, const double2* cc,
                           const float* phi_pad, double phic, const void* v, void* w, int prec, cudaStream_t st) {

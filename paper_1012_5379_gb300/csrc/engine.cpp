@@ -78,18 +78,23 @@ static int upload_level_coefficients(Handle* h, int l, double theta_beta, cudaSt
     for (auto& v : d) v += per_axis;
   }
   if (h->prec == HELM_C64) {
-    // basis of the Gram sweeps (gram.cuh): the interior's Laplacian scale and diagonal, and a
+    // basis of the Gram sweeps (gram.cuh): the interior's Laplacian scale, the shifts, and a
     // power of two near the reciprocal of half the spectrum's width
     const int mid = L.n / 2;
     const cplx lap = -0.5 * (double)h->dim * (a[mid] + c[mid]);
-    const cplx diag = (double)h->dim * d[mid] - (L.phi ? 0.0 : L.phic);
+    const cplx diag = (double)h->dim * d[mid];
+    const double lo = L.phi ? L.philo : L.phic, hi = L.phi ? L.phihi : L.phic, mean = 0.5 * (lo + hi);
     auto bits8 = [](double v) {
       int e = 0;
       const double m = std::frexp(v, &e);
       return (float)std::ldexp(std::trunc(m * 256.0) / 256.0, e);
     };
     L.kt = (float)std::ldexp(1.0, -(int)std::lround(std::log2(2.0 * std::abs(lap))));
-    L.ksh = make_float2(bits8(diag.real()), bits8(diag.imag()));
+    // the diagonal at the middle of the field, or where the field dominates the stencil at its
+    // smallest value, middle and largest (the line: gram.cuh)
+    L.wide = hi - lo > GRAM_WIDE * std::abs(diag);
+    const cplx shift[3] = {diag - (L.wide ? lo : mean), L.wide ? diag - mean : 0.0, diag - (L.wide ? hi : mean)};
+    for (int j = 0; j < 3; ++j) L.ksh[j] = make_float2(bits8(shift[j].real()), bits8(shift[j].imag()));
     L.klap = make_float2((float)lap.real(), (float)lap.imag());
   }
   double2* c64 = reinterpret_cast<double2*>(h->stage + h->stage_coef[l]);
@@ -280,6 +285,8 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     off += r256((size_t)cm * sizeof(int));
     h->stage_inv = off;
     off += r256((size_t)cm * cm * sizeof(float4));
+    h->stage_phi = off;
+    off += r256(2 * nlev * sizeof(unsigned));
     h->stage_coef.resize(nlev);
     for (int l = 0; l < nlev; ++l) {
       h->stage_coef[l] = off;
@@ -296,6 +303,29 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     L.n = sizes[l];
     L.P = L.n + 1;
     L.np = h->dim == 3 ? (size_t)L.P * L.P * L.P : (size_t)L.P * L.P;
+    // phi sampled at this level's nodes (node x of level l is fine node (x+1) 2^l - 1)
+    if (phi) {
+      TRY(dev_alloc(h.get(), &L.phi, L.np * sizeof(float)));
+      scatter_phi(h->dim, L.n, 1 << l, h->n, phi, L.phi, st);
+      CUDA_TRY(cudaGetLastError());
+    } else {
+      L.phic = k * k;
+    }
+  }
+  if (phi && h->prec == HELM_C64) {  // the sweeps' shifts need every level's range
+    const size_t bytes = 2 * nlev * sizeof(unsigned);
+    unsigned* range = nullptr;
+    TRY(dev_alloc(h.get(), &range, bytes));
+    CUDA_TRY(cudaMemsetAsync(range, 0, bytes, st));
+    for (int l = 0; l < nlev; ++l) phi_range(h->dim, h->lev[l].n, h->lev[l].phi, range + 2 * l, st);
+    CUDA_TRY(cudaGetLastError());
+    unsigned* host = reinterpret_cast<unsigned*>(h->stage + h->stage_phi);
+    CUDA_TRY(cudaMemcpyAsync(host, range, bytes, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    for (int l = 0; l < nlev; ++l) phi_range_values(host + 2 * l, &h->lev[l].philo, &h->lev[l].phihi);
+  }
+  for (int l = 0; l < nlev; ++l) {
+    HostLevel& L = h->lev[l];
     const TileCfg cfg = default_tiles(h->dim, L.P);
     if (l == 0) h->cfg = cfg;
     L.ntiles = vtiles(h->dim, L.P);
@@ -356,15 +386,12 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     // coefficients of M on this level (rediscretisation with spacing 2^l h)
     TRY(dev_alloc(h.get(), &L.coef64, 3 * L.n * sizeof(double2)));
     TRY(dev_alloc(h.get(), &L.coef, 3 * L.n * eb));
-    // phi sampled at this level's nodes (node x of level l is fine node (x+1) 2^l - 1)
-    if (phi) {
-      TRY(dev_alloc(h.get(), &L.phi, L.np * sizeof(float)));
-      scatter_phi(h->dim, L.n, 1 << l, h->n, phi, L.phi, st);
-      CUDA_TRY(cudaGetLastError());
-    } else {
-      L.phic = k * k;
-    }
     TRY(upload_level_coefficients(h.get(), l, theta_beta, st));
+    if (L.wide && L.sweep.march) {  // runs as regions: their partial slots
+      L.sweep = sweep_cfg(h->dim, L.n, h->s, sm_count_host(), false);
+      const size_t need = (size_t)std::max(L.sweep.units, L.sweep.units_res) * GRAM_SLOT * sizeof(float2);
+      if (need > part_bytes) TRY(dev_alloc(h.get(), &L.part, need));
+    }
   }
   // ------------------------------------------------ coarsest LU (FP64)
   h->lu_m = cm;
@@ -457,7 +484,8 @@ static LevelDev<C> make_leveldev(const Handle& h, int l) {
   d.part = L.part;
   d.tm = L.tm;
   d.kt = L.kt;
-  d.ksh = L.ksh;
+  for (int j = 0; j < 3; ++j) d.ksh[j] = L.ksh[j];
+  d.wide = L.wide;
   d.klap = L.klap;
   d.top = l == 0;
   if (l + 1 < (int)h.lev.size()) {
@@ -525,7 +553,8 @@ struct Group {
   struct Depth {
     int n = 0, cnt = 0, ntiles = 0, nflat = 0;
     bool tma = true;  // every problem at this depth has TMA maps
-    SweepCfg sweep{}; // complex64: the sweep pass's launch choice
+    SweepCfg sweep{}, sweepw{};  // complex64: the sweep pass's launch choice (wide levels' own)
+    int nw = 0;       // problems whose level is wide, after the others
     bool phi = false; // some problem at this depth has a wavenumber field
     TileCfg cfg{8};
     LevelDev<C>* d = nullptr;
@@ -536,6 +565,7 @@ struct Group {
   int nlev_c = 0;
   size_t coarse_smem = 0;          // dynamic shared memory of the staged coarse kernel (0: global)
   CoarseLU* dlu = nullptr;
+  int nwc = 0;                     // problems with a wide level among the coarse ones, after the others
   C* pwc = nullptr;                // polynomial smoother: weights of the coarse levels [prob][level][3]
   struct Sub {
     int n = 0, cnt = 0, ntiles = 0, chunks = 1, m = 1;
@@ -653,9 +683,12 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
   std::vector<std::vector<LevelDev<C>>> dep(g->tc);
   std::vector<std::vector<C>> pws(g->tc);
   g->depth.resize(g->tc);
+  std::vector<std::vector<int>> order(g->tc);  // problems of a depth, those with wide levels last
   for (int t = 0; t < g->tc; ++t) {
-    for (int p = 0; p < count; ++p) {
-      if (off[p] > t) continue;
+    for (int wide = 0; wide < 2; ++wide)
+      for (int p = 0; p < count; ++p)
+        if (off[p] <= t && hs[p]->lev[t - off[p]].wide == wide) order[t].push_back(p);
+    for (int p : order[t]) {
       const int l = t - off[p];
       dep[t].push_back(make_leveldev<C>(*hs[p], l));
       if (g->smoother == HELM_SMOOTHER_POLY)
@@ -673,12 +706,14 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
       D.cnt += 1;
       D.tma = D.tma && L.tm != nullptr;
       D.nflat = L.nflat;
-      D.sweep = L.sweep;
+      (L.wide ? D.sweepw : D.sweep) = L.sweep;
+      D.nw += L.wide;
       D.phi = D.phi || L.phi != nullptr;
       D.cfg.rows = g->dim == 3 ? tuned_zchunk(L.P, (int)sizeof(C)) : zchunk(L.P);
       D.cfg.P = L.P;
       D.ntiles = g->dim == 3 ? tiles_per_problem(3, L.P, D.cfg) : L.ntiles;
     }
+    if (g->depth[t].nw == g->depth[t].cnt) g->depth[t].sweep = g->depth[t].sweepw;
   }
   // the persistent segments: the deepest run of grid-wide levels that qualify
   // (bounded by the pass list's capacity: a depth records nu1 (s + 1) passes going down
@@ -692,17 +727,28 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
       --g->tp;
   g->fuse2 = fused2_cycle(g->dim, h0.prec, g->smoother, g->nu1, g->nu2);
   for (int t = 0; t + 1 < g->tp && g->fuse2; ++t)  // depth t reads depth t + 1's last sweep
-    for (size_t k = 0, p = 0; p < (size_t)count; ++p) {
-      if (off[p] > t) continue;
+    for (size_t k = 0; k < order[t].size(); ++k) {
+      const int p = order[t][k];
       const HostLevel& Lc = hs[p]->lev[t + 1 - off[p]];
-      LevelDev<C>& d = dep[t][k++];
+      LevelDev<C>& d = dep[t][k];
       d.cr0 = (const C*)Lc.r0;
       for (int j = 0; j < SMAX; ++j) d.cp[j] = (const C*)(g->fused(t + 1) ? Lc.q[j] : Lc.p[j]);
     }
   std::vector<LevelDev<C>> coarse;
   std::vector<CoarseLU> lus;
   std::vector<C> pwc;  // polynomial smoother: three weights per coarse level (complex64)
-  for (int p = 0; p < count; ++p) {
+  auto wide_coarse = [&](int p) {
+    for (int t = std::max(g->tc, off[p]); t < g->Lmax; ++t)
+      if (hs[p]->lev[t - off[p]].wide) return true;
+    return false;
+  };
+  std::vector<int> corder;
+  for (int p = 0; p < count; ++p)
+    if (!wide_coarse(p)) corder.push_back(p);
+  g->nwc = count - (int)corder.size();
+  for (int p = 0; p < count; ++p)
+    if (wide_coarse(p)) corder.push_back(p);
+  for (int p : corder) {
     // the problem's coarse levels (depths t0 .. Lmax-1) first, then padding up to the stride
     const int t0 = std::max(g->tc, off[p]);
     const int coarsest = (int)hs[p]->lev.size() - 1;
@@ -832,7 +878,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
 template <typename C>
 static void launch_coarse_part(const Group<C>& g, cudaStream_t st) {
   if constexpr (sizeof(C) == 8)
-    launch_coarse_gram(g.dim, g.smoother == HELM_SMOOTHER_POLY ? 0 : g.s, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.pwc,
+    launch_coarse_gram(g.dim, g.smoother == HELM_SMOOTHER_POLY ? 0 : g.s, g.dcoarse, g.nlev_c, g.dlu, g.nprob, g.nwc, g.pwc,
                        g.nu1, g.nu2, g.fused_down(g.tc), g.coarse_smem, st);
   else
     launch_coarse_smem<C>(g.dim, g.dcoarse, g.nlev_c, g.nlev_c, g.dlu, g.nprob, g.nu1, g.nu2, g.coarse_smem, st);
@@ -949,7 +995,9 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st, bool defer = false) {
         return;
       }
       Launch L(name, st, bytes, pts * (8.0 * (2 * dim + 1) * g.s + 4.0 * (g.s + 1) * (g.s + 1)));
-      launch_sweep(dim, g.s, D.d, D.cnt, D.sweep, first, store_last, D.phi, st);
+      const int m = D.cnt - D.nw;
+      if (m > 0) launch_sweep(dim, g.s, D.d, m, D.sweep, first, store_last, D.phi, false, st);
+      if (D.nw > 0) launch_sweep(dim, g.s, D.d + m, D.nw, D.sweepw, first, store_last, true, true, st);
     } else {
       for (int J = 1; J <= g.s; ++J) {
         const bool store = J < g.s || store_last;
@@ -984,7 +1032,7 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st, bool defer = false) {
       if constexpr (sizeof(C) == 8) {
         if (t > 0 && g.fused(t)) {  // with the restriction to this level
           Launch L("vc.arnoldi.lc", st, pts * (E * ((g.s + 1) * (1.0 / cf) + g.s + 1) + ph), 0);
-          launch_fused2(FUSED2_DOWN, g.s, D.d, D.cnt, D.n, D.sweep, false, st);
+          launch_fused2(FUSED2_DOWN, g.s, D.d, D.cnt, D.nw, D.n, D.sweep, false, st);
           if (g.fused_down(t + 1)) continue;
         } else {
           arnoldi(D, sw == 0, true, fine, rec, ph, pts);
@@ -1030,12 +1078,12 @@ static void run_vcycle(const Group<C>& g, cudaStream_t st, bool defer = false) {
         const double ebytes = pts * E * cf * (t + 1 < g.tp ? g.s + 1.0 : 1.0);
         if (g.fused(t)) {
           Launch L(fine ? "vc.prolong.l0" : "vc.prolong.lc", st, pts * (E * (2.0 * g.s + 1) + ph) + ebytes, 0);
-          launch_fused2(FUSED2_UP, g.s, D.d, D.cnt, D.n, D.sweep, true, st);
+          launch_fused2(FUSED2_UP, g.s, D.d, D.cnt, D.nw, D.n, D.sweep, true, st);
         } else {
           const bool xk = g.fused_down(t + 1);
           {
             Launch L(fine ? "vc.prolong.l0" : "vc.prolong.lc", st, pts * (E * (xk ? g.s + 2.0 : 4.0) + ph) + ebytes, 0);
-            launch_fused2(FUSED2_PROLONG, g.s, D.d, D.cnt, D.n, D.sweep, xk, st);
+            launch_fused2(FUSED2_PROLONG, g.s, D.d, D.cnt, 0, D.n, D.sweep, xk, st);
           }
           arnoldi(D, false, false, fine, false, ph, pts);
         }

@@ -49,10 +49,12 @@ struct HostLevel {
   double2* coef64 = nullptr;// the same in FP64
   float* phi = nullptr;     // padded phi or nullptr
   double phic = 0.0;
+  double philo = 0.0, phihi = 0.0;  // range of the level's field (complex64)
   void* sc = nullptr;          // SweepScalarsT<R> of the preconditioner precision
   const CUtensorMap* tm = nullptr;  // TMA maps (3D complex64 grid-wide levels), device memory
   float kt = 0;                // Gram sweeps (complex64): basis scale, shift, Laplacian scale
-  float2 ksh{}, klap{};
+  float2 ksh[3] = {}, klap{};
+  int wide = 0;                // 1: the field dominates the stencil here (gram.cuh)
   SweepCfg sweep{};            // the sweep pass's launch choice
   double* part = nullptr;
 };
@@ -103,7 +105,7 @@ struct Handle {
   // the outer state, the coarsest LU and pivots, each level's coefficients (FP64 and
   // the preconditioner precision), at fixed offsets
   char* stage = nullptr;
-  size_t stage_lu = 0, stage_piv = 0, stage_inv = 0;
+  size_t stage_lu = 0, stage_piv = 0, stage_inv = 0, stage_phi = 0;
   std::vector<size_t> stage_coef;  // per level: FP64 block, then the level-precision block
   ~Handle();
 };

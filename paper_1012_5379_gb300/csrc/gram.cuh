@@ -15,16 +15,25 @@
 // Accuracy.  Errors of G are amplified by the square of the basis's condition number, so
 // the sums beyond a warp, the factorisation and the Schur complements are held as pairs of
 // binary32 numbers (dfloat.cuh); the warp sums' binary32 roundings are independent and
-// average out over the level.  The shifts keep the basis well conditioned: sigma_1 is the
-// stencil's diagonal (the middle of the spectrum), sigma_0 = 0, so that k_1 carries M k_0
-// to full relative accuracy when k_0 is smooth, where M k_0 is small and a shifted k_1
-// would lose it.  The first sweep on the finest level meets arbitrary right-hand sides:
-// there sigma_0 is the Rayleigh quotient estimated from the differences of neighbouring
-// values (taken by the pass that writes the right-hand side).  Shifts carry 8 significant
-// bits, so that subtracting one from a binary32 diagonal is exact.  Measured over whole
-// V-cycles on the CPU in complex64, relative to 64 bits: 3.4e-7 / 2.2e-7 on white noise
-// (step-by-step orthogonalisation in binary32: 3.3e-7 / 2.0e-7), 2.4-5e-7 on a point source
-// (8.1e-7), 2.5e-7 on the Gaussian model's source (3.4e-7).
+// average out over the level.  The shifts keep the basis well conditioned: sigma_1 = sigma_3
+// is the middle of the spectrum (the stencil's diagonal at the middle of the field's range),
+// sigma_0 = sigma_2 = 0, so that k_1 carries M k_0 to full relative accuracy when k_0 is smooth,
+// where M k_0 is small and a shifted k_1 would lose it.  The first sweep on the finest level
+// meets arbitrary right-hand sides: there sigma_0 is the Rayleigh quotient estimated from the
+// differences of neighbouring values (taken by the pass that writes the right-hand side).
+// Shifts carry 8 significant bits.
+//
+// Wide levels.  Where a wavenumber field's range exceeds the diagonal (GRAM_WIDE; the coarse
+// levels of media with a contrast of three or more, where phi h^2 is large), the spectrum falls
+// into clusters at the field's values and the k_j become dependent to 1e-4 and less: G and its
+// solution then need all of double-float's digits.  There the warp sums are double-float too
+// (ten instructions a product instead of one, 0.5 to 2 us a sweep), a pivot counts down to
+// GRAM_TAU_WIDE, and the shifts are 0 and the diagonal at the field's smallest value, middle and
+// largest.  Whole V-cycles with layers and discs of contrast 3 to 27, against 64 bits, norm: at
+// most 1.8 times and in the mean 0.4 times the error of step-by-step orthogonalisation in
+// binary32; with binary32 sums and shifts that ignore the field up to 1e5 times (6e-2 instead of
+// 6e-6 for discs of 12 at 255^2, s = 3).  On the CPU, lines from 0.25 to 2 diagonals gave the
+// same errors; at one, media within +-30% keep the binary32 sums on all levels but the smallest.
 #pragma once
 #include "device_common.cuh"
 #include "dfloat.cuh"
@@ -60,6 +69,26 @@ __device__ __forceinline__ void gram_point(const float2 (&k)[S + 1], float (&acc
   }
 }
 
+// The same in double-float, sums s + c: the products are exact (TwoProduct) and so is every
+// addition into s (TwoSum).
+template <int S>
+__device__ __forceinline__ void gram_point_wide(const float2 (&k)[S + 1], float (&s)[gram_ns(S)], float (&c)[gram_ns(S)]) {
+  auto mac = [&](int i, float a, float b) { df_mac1(s[i], c[i], a, 0.f, b); };
+#pragma unroll
+  for (int i = 0; i <= S; ++i) {
+    mac(gram_at(S, i, i), k[i].x, k[i].x);
+    mac(gram_at(S, i, i), k[i].y, k[i].y);
+#pragma unroll
+    for (int j = i + 1; j <= S; ++j) {
+      const int re = gram_at(S, i, j), im = re + 1;
+      mac(re, k[i].x, k[j].x);
+      mac(re, k[i].y, k[j].y);
+      mac(im, k[i].x, k[j].y);
+      mac(im, -k[i].y, k[j].x);
+    }
+  }
+}
+
 // Sum NS (16 or 32) per-lane binary32 values over the warp by butterflies that halve the
 // values kept; lane L ends with the total of value L (NS = 32) or L >> 1 (NS = 16).
 template <int NS>
@@ -84,6 +113,34 @@ __device__ __forceinline__ float2 df_fast2(float s, float c) {
   return make_float2(t, __fsub_rn(c, __fsub_rn(t, s)));
 }
 
+// warp_transpose_sum_f in double-float.
+template <int NS>
+__device__ __forceinline__ float2 warp_transpose_sum_df(float (&s)[NS], float (&c)[NS], int lane) {
+  int o = 16;
+  auto add = [](float& s, float& c, float s2, float c2) {
+    float t, r;
+    df_two_sum(s, s2, t, r);
+    c = (c + c2) + r;
+    s = t;
+  };
+#pragma unroll
+  for (int n = NS / 2; n >= 1; n >>= 1, o >>= 1) {
+    const bool hi = lane & o;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const float s2 = __shfl_xor_sync(0xffffffffu, hi ? s[k] : s[k + n], o);
+      const float c2 = __shfl_xor_sync(0xffffffffu, hi ? c[k] : c[k + n], o);
+      if (hi) {
+        s[k] = s[k + n];
+        c[k] = c[k + n];
+      }
+      add(s[k], c[k], s2, c2);
+    }
+  }
+  if (NS == 16) add(s[0], c[0], __shfl_xor_sync(0xffffffffu, s[0], 1), __shfl_xor_sync(0xffffffffu, c[0], 1));
+  return make_float2(s[0], c[0]);
+}
+
 // ------------------------------------------------------------------ the minimisation
 // min ||K_{s+1} rho|| over rho = e_0 - B y.  B's left null vector c (c_0 = 1, c_{j+1} =
 // -t sigma_j c_j: the basis polynomials' values at zero) makes the constraint c^T rho = 1,
@@ -101,6 +158,7 @@ __device__ __forceinline__ float2 df_fast2(float s, float c) {
 // earlier vectors (to the rounding of binary32 vectors and of their Gram sums): rho is then
 // that combination, m = i Krylov steps.
 constexpr float GRAM_TAU = 1e-7f;
+constexpr float GRAM_TAU_WIDE = 1e-13f;  // double-float sums: a few 2^-45
 
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
@@ -118,13 +176,15 @@ __device__ __forceinline__ float2 df_fms2x2(float2 s, float2 a, float2 b, float2
   return df_fast2(v, ((s.y - e) - f) + (x + y));
 }
 
-// g: the NV double-float sums; sg0 = t sigma_0, sg1 = t sigma_1 = t sigma_3 (sigma_2 = 0).
+// g: the NV double-float sums; sg: t sigma_j (sigma_2 = 0 and sigma_3 = sigma_1, or on wide
+// levels sigma_0 = 0: in both cases c_j = 0 from j = 3 on).
 // Lane k < S returns x's coefficient xk of k_k (x += sum_{k<m} x_k k_k), lane k <= S the
 // residual's rk (r = sum_{k<=m} r_k k_k); every lane returns m.  The whole warp calls it.
 template <int S>
-__device__ __forceinline__ int gram_solve(const float2* g, float2 sg0, float2 sg1, float t, int lane, float2& xk,
-                                          float2& rk) {
+__device__ __forceinline__ int gram_solve(const float2* g, const float2 (&sg)[S], bool wide, float t, int lane,
+                                          float2& xk, float2& rk) {
   constexpr int NC = S + 2, N = S + 1;
+  const float2 sg0 = sg[0], sg1 = sg[S > 1 ? 1 : 0];
   const unsigned full = 0xffffffffu;
   xk = make_float2(0.f, 0.f);
   rk = make_float2(lane == 0 ? 1.f : 0.f, 0.f);
@@ -154,7 +214,7 @@ __device__ __forceinline__ int gram_solve(const float2* g, float2 sg0, float2 sg
       im = make_float2(-c.y, 0.f);
     }
   }
-  const float tau = re.x * GRAM_TAU;  // lanes (i, i): the threshold of pivot i
+  const float tau = re.x * (wide ? GRAM_TAU_WIDE : GRAM_TAU);  // lanes (i, i): the threshold of pivot i
   int m = N, ii = 0, ji = j * NC, ik = k;
   float dinv = 0.f;                   // lane i: 1 / d_i
 #pragma unroll 1
@@ -200,22 +260,32 @@ __device__ __forceinline__ int gram_solve(const float2* g, float2 sg0, float2 sg
   // y_j = -rho_{j+1} - sg_{j+1} y_{j+1}: sg_2 = 0, so odd j end there and even j take one more
   const float2 r1 = make_float2(__shfl_down_sync(full, rk.x, 1), __shfl_down_sync(full, rk.y, 1));
   const float2 r2 = make_float2(__shfl_down_sync(full, rk.x, 2), __shfl_down_sync(full, rk.y, 2));
-  const float2 y = csub(cmul((lane & 1) ? make_float2(0.f, 0.f) : sg1, r2), r1);
+  float2 y = csub(cmul((lane & 1) ? make_float2(0.f, 0.f) : sg1, r2), r1);
+  if (wide) {  // all the way down: y_{S-1} = -rho_S, y_{j-1} = -rho_j - sg_j y_j
+    float2 yj = make_float2(0.f, 0.f);
+    y = yj;
+#pragma unroll
+    for (int j = S; j >= 1; --j) {
+      const float2 rj = make_float2(__shfl_sync(full, rk.x, j), __shfl_sync(full, rk.y, j));
+      yj = j < S ? csub(make_float2(-rj.x, -rj.y), cmul(sg[j < S ? j : 0], yj)) : make_float2(-rj.x, -rj.y);
+      if (lane == j - 1) y = yj;
+    }
+  }
   xk = make_float2(t * y.x, t * y.y);
   return m;
 }
 
 // The (scaled) shifts of a sweep on level L: sigma_0 = 0, or the estimate left by the pass
-// that wrote the right-hand side (finest level, first sweep), sigma_1 = sigma_3 = the
-// stencil's diagonal, sigma_2 = 0.
+// that wrote the right-hand side (finest level, first sweep; not on a wide level), then the
+// level's own.
 template <int S>
-__device__ __forceinline__ void gram_shifts(const LevelDev<float2>& L, bool first, float2 (&sg)[S]) {
+__device__ __forceinline__ void gram_shifts(const LevelDev<float2>& L, bool first, bool wide, float2 (&sg)[S]) {
   const float t = L.kt;
 #pragma unroll
   for (int j = 0; j < S; ++j) {
     float2 s = make_float2(0.f, 0.f);
-    if (j & 1) s = L.ksh;
-    else if (j == 0 && first && L.top) s = L.sc->sig0;
+    if (j > 0) s = L.ksh[j > 0 ? j - 1 : 0];
+    else if (first && L.top && !wide) s = L.sc->sig0;
     sg[j] = make_float2(s.x * t, s.y * t);
   }
 }
@@ -237,9 +307,10 @@ __device__ __forceinline__ float2 df_group_sum(float2 a) {
 // The warps' sums of a CTA of NW warps, combined: gs[0..NV-1].  Every thread calls it (it
 // starts with a barrier; another must precede the reads of gs).
 template <int S, int NW>
-__device__ __forceinline__ void gram_block_sum(float (&acc)[gram_ns(S)], float* wsum, float2* gs) {
+__device__ __forceinline__ void gram_block_sum(float (&acc)[gram_ns(S)], float2* wsum2, float2* gs) {
   constexpr int NV = gram_nv(S), NS = gram_ns(S);
   const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5;
+  float* const wsum = reinterpret_cast<float*>(wsum2);
   const float tot = warp_transpose_sum_f<NS>(acc, lane);
   if (NS == 32) wsum[warp * NS + lane] = tot;
   else if ((lane & 1) == 0) wsum[warp * NS + (lane >> 1)] = tot;
@@ -251,18 +322,34 @@ __device__ __forceinline__ void gram_block_sum(float (&acc)[gram_ns(S)], float* 
   }
 }
 
-// End of a sweep pass: every thread's Gram sums `acc` are reduced over its warp (binary32),
-// the CTA and the level (double-float, fixed order); the last CTA of the problem solves the
-// minimisation and writes the sweep's coefficients.  Every thread of the block calls it.
-// `wsum` is NW * NS floats, `gs` gram_nv(S) * (NW + 1) float2 of shared memory.
+// The same from double-float sums.
 template <int S, int NW>
-__device__ __forceinline__ void gram_finish(float (&acc)[gram_ns(S)], const LevelDev<float2>& L, const float2 (&sg)[S],
-                                            int unit, int nunits, float* wsum, float2* gs) {
+__device__ __forceinline__ void gram_block_sum_wide(float (&s)[gram_ns(S)], float (&c)[gram_ns(S)], float2* wsum,
+                                                    float2* gs) {
+  constexpr int NV = gram_nv(S), NS = gram_ns(S);
+  const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5;
+  const float2 tot = warp_transpose_sum_df<NS>(s, c, lane);
+  if (NS == 32) wsum[warp * NS + lane] = tot;
+  else if ((lane & 1) == 0) wsum[warp * NS + (lane >> 1)] = tot;
+  __syncthreads();
+  const int v = tid / NW, w = tid % NW;
+  if (warp * 32 < NV * NW) {  // uniform over the warp
+    const float2 a = df_group_sum<NW>(v < NV ? wsum[w * NS + v] : make_float2(0.f, 0.f));
+    if (w == 0 && v < NV) gs[v] = a;
+  }
+}
+
+// End of a sweep pass, after the CTA's sums (gram_block_sum): they are added over the level
+// (double-float, fixed order); the last CTA of the problem solves the minimisation and writes
+// the sweep's coefficients.  Every thread of the block calls it.  (The block sum's `wsum` is
+// NW * NS float2, `gs` gram_nv(S) * (NW + 1) float2 of shared memory.)
+template <int S, int NW>
+__device__ __forceinline__ void gram_finish(const LevelDev<float2>& L, const float2 (&sg)[S], bool wide, int unit,
+                                            int nunits, float2* gs) {
   constexpr int NV = gram_nv(S), NS = gram_ns(S);
   constexpr int H = NS == 16 ? 2 : 1;  // slots a warp reads at a time
   __shared__ int s_last;
   const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5;
-  gram_block_sum<S, NW>(acc, wsum, gs);
   __syncthreads();
   auto* sc = L.sc;
   if (nunits > 1) {
@@ -315,7 +402,7 @@ __device__ __forceinline__ void gram_finish(float (&acc)[gram_ns(S)], const Leve
   }
   if (warp == 0) {
     float2 xk, rk;
-    const int m = gram_solve<S>(gs, sg[0], sg[S > 1 ? 1 : 0], L.kt, lane, xk, rk);
+    const int m = gram_solve<S>(gs, sg, wide, L.kt, lane, xk, rk);
     if (lane < S) sc->xcoef[lane] = xk;
     if (lane <= S) sc->rcoef[lane] = rk;
     if (lane == 0) {

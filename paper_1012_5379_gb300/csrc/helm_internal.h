@@ -25,6 +25,7 @@ namespace helm {
 constexpr int SMAX = 4;            // max GMRES(s) steps per smoothing sweep
 constexpr int NPART = 2 * SMAX + 4;  // doubles per partial-sum slot of a sweep pass
 constexpr int GRAM_SLOT = 32;        // double-floats per partial slot of a Gram sweep pass (gram.cuh)
+constexpr double GRAM_WIDE = 1.0;    // a level is wide when its field's range exceeds this many diagonals (gram.cuh)
 
 // Real and complex scalar types of a preconditioner precision.
 template <typename C> struct RealOf;
@@ -86,7 +87,8 @@ struct LevelDev {
   const CUtensorMap* tm;  // 3D complex64 levels: TMA maps of b, r0, p_1..p_SMAX, xb (else nullptr)
   // Gram sweeps (complex64, gram.cuh)
   float kt;               // basis scale: a power of two near 1 / (spectral half width)
-  float2 ksh;             // the stencil's diagonal in the interior, to 8 significant bits
+  float2 ksh[3];          // shifts of the steps after the first, to 8 significant bits
+  int wide;               // 1: a field dominates the stencil (double-float Gram sums)
   float2 klap;            // d / h^2 of the interior spacing (the Laplacian's scale)
   int top;                // 1: the problem's finest level
   // fused 2D passes (sweep.cuh)
@@ -204,7 +206,8 @@ struct SweepCfg {
   int march, geo, units;
   int geo_res, units_res;  // shape and CTAs of a sweep that starts from the residual of an iterate
 };
-SweepCfg sweep_cfg(int dim, int n, int S, int sms);
+// (march false: the kernels whose CTAs hold a region, whatever the size)
+SweepCfg sweep_cfg(int dim, int n, int S, int sms, bool march = true);
 
 // Marching FP64 stencil of the outer solve: 2D warps march cfg.rows rows, 3D CTAs
 // march cfg.rows planes.
@@ -249,16 +252,17 @@ void launch_arnoldi(int dim, int J, const LevelDev<C>* levs, int nprob, int ntil
 // of a marching level (xk: x_a formed from the last sweep).
 bool fused2_size(int n);  // whether a level of this size takes the fused passes
 enum { FUSED2_DOWN, FUSED2_UP, FUSED2_PROLONG };
-void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int n, const SweepCfg& cfg, bool xk,
-                   cudaStream_t st);
+// (the last nwide problems' levels are wide; launch_sweep: all of them or none)
+void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int nwide, int n, const SweepCfg& cfg,
+                   bool xk, cudaStream_t st);
 void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
-                  bool store_last, bool phi, cudaStream_t st);
+                  bool store_last, bool phi, bool wide, cudaStream_t st);
 void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
                   bool store_last);
 // the complex64 coarse sub-cycle (S = 0: polynomial smoother, weights pw[prob][level][3]); smem
-// from coarse_gram_smem over its level sizes
+// from coarse_gram_smem over its level sizes; the last nwide problems have wide levels
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                        const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st);
+                        int nwide, const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st);
 size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev);
 template <typename C>
 void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
@@ -384,6 +388,10 @@ void convert_dense_to_padded_c128(int dim, int n, const double2* src, double2* d
 void convert_padded_to_dense_c128(int dim, int n, const double2* src, double2* dst, cudaStream_t st);
 void scatter_phi(int dim, int n_level, int stride, int n_fine, const float* phi_dense_fine, float* phi_pad_level,
                  cudaStream_t st);
+// Range of the finite values of a padded field: two ordered-bit words to out (zero before), and
+// what they stand for (0 if there are none).
+void phi_range(int dim, int n, const float* phi_pad, unsigned* out, cudaStream_t st);
+void phi_range_values(const unsigned* bits, double* lo, double* hi);
 // w = A v on the finest level, A given by 1D coefficients (prec: HELM_C64/HELM_C128),
 // natural layout in and out.
 void apply_operator_dense(int dim, int n, const double2* ca, const double2* cd, const double2* cc,

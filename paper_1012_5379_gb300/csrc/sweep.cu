@@ -1,10 +1,8 @@
 // Launchers of the complex64 sweep passes (sweep.cuh) and of the complex64 coarse sub-cycle
 // (coarse.cuh).
-#include "sweep.cuh"
-#include "coarse.cuh"
+#include "sweep_launch.cuh"
 #include "poly.cuh"
 #include "poly.h"
-#include "launch.cuh"
 
 #include <algorithm>
 
@@ -17,10 +15,10 @@ constexpr int SWEEP3_MARCH_N = 40;
 
 bool fused2_size(int n) { return n < SWEEP2_MARCH_N; }
 
-SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
+SweepCfg sweep_cfg(int dim, int n, int S, int sms, bool march) {
   SweepCfg c{0, 0, 1, 0, 1};
   if (dim == 2) {
-    if (n < SWEEP2_MARCH_N || S > 3) {
+    if (n < SWEEP2_MARCH_N || S > 3 || !march) {
       // rows per warp: the fewest rounds of resident CTAs, each a fixed latency and its rows
       // (511^2: one round at 6 rows; two at 4, 21 us against 12 on the way up)
       auto pick = [&](int H, int& geo, int& units) {
@@ -57,7 +55,7 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
   }
   // 3D levels from this size on march: 47^3 12 us a sweep, 63^3 14.5 against 25 in regions, 95^3
   // 23 against 42; at 31^3 both take 10
-  if (n < SWEEP3_MARCH_N || S > 3) {
+  if (n < SWEEP3_MARCH_N || S > 3 || !march) {
     c.geo = S <= 3 || n < 64 ? 4 : 8;
     c.units_res = c.units = sw3_units(S, c.geo, n);
     c.geo_res = c.geo;
@@ -82,85 +80,57 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms) {
 }
 
 template <int S>
-static void launch_sweep_s(int dim, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
-                           bool store_last, bool phi, cudaStream_t st) {
+static void launch_march(int dim, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, int first,
+                         int store_last, bool phi, cudaStream_t st) {
   const dim3 grid(nprob * cfg.units);
-  const int f = first ? 1 : 0, sl = store_last ? 1 : 0;
   if (dim == 2) {
-    if (!cfg.march) {
-      const dim3 block(32, SW2_NW);
-      const int units = first ? cfg.units : cfg.units_res, qy = first ? cfg.geo : cfg.geo_res;
-      if (qy == 2) pdl_launch(k_sweep2<S, 2>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
-      else if (qy == 4) pdl_launch(k_sweep2<S, 4>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
-      else pdl_launch(k_sweep2<S, 6>, dim3(nprob * units), block, 0, st, levs, units, f, sl);
-    } else if constexpr (S <= 3) {
-      const dim3 block(32, SV2_NW);
-      const size_t smem = sv2_smem(S, cfg.geo);  // at most 256 rows: below 48 KB
-      if (phi) pdl_launch(k_sweep2_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
-      else pdl_launch(k_sweep2_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
-    }
+    const dim3 block(32, SV2_NW);
+    const size_t smem = sv2_smem(S, cfg.geo);  // at most 256 rows: below 48 KB
+    if (phi) pdl_launch(k_sweep2_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
+    else pdl_launch(k_sweep2_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
     return;
   }
-  if (!cfg.march) {
-    const dim3 block(32, SW3_NW);
-    if constexpr (S > 3) {
-      if (cfg.geo == 8) {
-        allow_smem<k_sweep3<S, 8>>();
-        pdl_launch(k_sweep3<S, 8>, grid, block, sw3_smem(S, 8), st, levs, cfg.units, f, sl);
-        return;
-      }
-    }
-    allow_smem<k_sweep3<S, 4>>();
-    pdl_launch(k_sweep3<S, 4>, grid, block, sw3_smem(S, 4), st, levs, cfg.units, f, sl);
-    return;
-  }
-  if constexpr (S <= 3) {
-    const dim3 block(32, SM3_NW);
-    const size_t smem = sm3_smem(S, cfg.geo);
-    if (phi) allow_smem<k_sweep3_march<S, true>>();
-    else allow_smem<k_sweep3_march<S, false>>();
-    if (phi) pdl_launch(k_sweep3_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
-    else pdl_launch(k_sweep3_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, f, sl);
-  }
+  const dim3 block(32, SM3_NW);
+  const size_t smem = sm3_smem(S, cfg.geo);
+  if (phi) allow_smem<k_sweep3_march<S, true>>();
+  else allow_smem<k_sweep3_march<S, false>>();
+  if (phi) pdl_launch(k_sweep3_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
+  else pdl_launch(k_sweep3_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
 }
 
 void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
-                  bool store_last, bool phi, cudaStream_t st) {
-  switch (S) {
-    case 1: launch_sweep_s<1>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
-    case 2: launch_sweep_s<2>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
-    case 3: launch_sweep_s<3>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
-    default: launch_sweep_s<4>(dim, levs, nprob, cfg, first, store_last, phi, st); break;
+                  bool store_last, bool phi, bool wide, cudaStream_t st) {
+  const int f = first ? 1 : 0, sl = store_last ? 1 : 0;
+  if (!cfg.march) {
+    if (wide) launch_regions_wide(dim, S, levs, nprob, cfg, f, sl, st);
+    else launch_regions<W_NO>(dim, S, levs, nprob, cfg, f, sl, st);
+    return;
+  }
+  switch (S) {  // (S <= 3: sweep_cfg)
+    case 1: launch_march<1>(dim, levs, nprob, cfg, f, sl, phi, st); break;
+    case 2: launch_march<2>(dim, levs, nprob, cfg, f, sl, phi, st); break;
+    default: launch_march<3>(dim, levs, nprob, cfg, f, sl, phi, st); break;
   }
 }
 
 template <int S>
-static void fused2(int pass, const LevelDev<float2>* levs, int nprob, int n, const SweepCfg& cfg, bool xk,
-                   cudaStream_t st) {
-  const dim3 block(32, SW2_NW);
-  if (pass == FUSED2_PROLONG) {
-    const int ntiles = ceil_div(n + 1, 64) * ceil_div(n + 1, 16);
-    pdl_launch(k_prolong2_gram<S>, dim3(nprob * ntiles), block, 0, st, levs, ntiles, xk ? 1 : 0);
-  } else if (pass == FUSED2_DOWN) {
-    const dim3 grid(nprob * cfg.units);
-    if (cfg.geo == 2) pdl_launch(k_sweep2_down<S, 2>, grid, block, 0, st, levs, cfg.units);
-    else if (cfg.geo == 4) pdl_launch(k_sweep2_down<S, 4>, grid, block, 0, st, levs, cfg.units);
-    else pdl_launch(k_sweep2_down<S, 6>, grid, block, 0, st, levs, cfg.units);
-  } else {
-    const dim3 grid(nprob * cfg.units_res);
-    if (cfg.geo_res == 2) pdl_launch(k_sweep2_up<S, 2>, grid, block, 0, st, levs, cfg.units_res);
-    else if (cfg.geo_res == 4) pdl_launch(k_sweep2_up<S, 4>, grid, block, 0, st, levs, cfg.units_res);
-    else pdl_launch(k_sweep2_up<S, 6>, grid, block, 0, st, levs, cfg.units_res);
-  }
+static void prolong2(const LevelDev<float2>* levs, int nprob, int n, bool xk, cudaStream_t st) {
+  const int ntiles = ceil_div(n + 1, 64) * ceil_div(n + 1, 16);
+  pdl_launch(k_prolong2_gram<S>, dim3(nprob * ntiles), dim3(32, SW2_NW), 0, st, levs, ntiles, xk ? 1 : 0);
 }
 
-void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int n, const SweepCfg& cfg, bool xk,
-                   cudaStream_t st) {
+void launch_fused2(int pass, int S, const LevelDev<float2>* levs, int nprob, int nwide, int n, const SweepCfg& cfg,
+                   bool xk, cudaStream_t st) {
+  if (pass != FUSED2_PROLONG) {
+    if (nprob > nwide) launch_fused_regions<W_NO>(pass, S, levs, nprob - nwide, cfg, st);
+    if (nwide > 0) launch_fused_regions_wide(pass, S, levs + (nprob - nwide), nwide, cfg, st);
+    return;
+  }
   switch (S) {
-    case 1: fused2<1>(pass, levs, nprob, n, cfg, xk, st); break;
-    case 2: fused2<2>(pass, levs, nprob, n, cfg, xk, st); break;
-    case 3: fused2<3>(pass, levs, nprob, n, cfg, xk, st); break;
-    default: fused2<4>(pass, levs, nprob, n, cfg, xk, st); break;
+    case 1: prolong2<1>(levs, nprob, n, xk, st); break;
+    case 2: prolong2<2>(levs, nprob, n, xk, st); break;
+    case 3: prolong2<3>(levs, nprob, n, xk, st); break;
+    default: prolong2<4>(levs, nprob, n, xk, st); break;
   }
 }
 
@@ -179,30 +149,19 @@ size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {
   return total * sizeof(float2);
 }
 
-template <int S, int DIM>
-static void launch_coarse_gram_sd(const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                                  const float2* pw, int nu1, int nu2, bool from_res, size_t smem,
-                                  cudaStream_t st) {
-  allow_smem<k_coarse_gram<S, DIM>>();
-  pdl_launch(k_coarse_gram<S, DIM>, dim3(nprob), dim3(CG_THREADS), smem, st, levs, lev_stride, lus, pw, nu1, nu2,
-             from_res ? 1 : 0);
-}
-
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
-                        const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st) {
-#define HELM_CG(SS)                                                                                             \
-  case SS:                                                                                                      \
-    if (dim == 2) launch_coarse_gram_sd<SS, 2>(levs, lev_stride, lus, nprob, pw, nu1, nu2, from_res, smem, st); \
-    else launch_coarse_gram_sd<SS, 3>(levs, lev_stride, lus, nprob, pw, nu1, nu2, from_res, smem, st);          \
-    break;
-  switch (S) {
-    HELM_CG(0)
-    HELM_CG(1)
-    HELM_CG(2)
-    HELM_CG(3)
-    HELM_CG(4)
+                        int nwide, const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st) {
+  const int m = nprob - nwide;
+  const CoarseArgs a{lev_stride, pw, nu1, nu2, from_res ? 1 : 0, smem};
+  if (m > 0) {
+    if (S == 0) {
+      if (dim == 2) launch_coarse_sd<0, 2, W_NO>(levs, lus, m, a, st);
+      else launch_coarse_sd<0, 3, W_NO>(levs, lus, m, a, st);
+    } else {
+      launch_coarse_s<W_NO>(dim, S, levs, lus, m, a, st);
+    }
   }
-#undef HELM_CG
+  if (nwide > 0) launch_coarse_wide(dim, S, levs + (size_t)m * lev_stride, lus + m, nwide, a, st);
 }
 
 template <int SRC, int END>

@@ -50,7 +50,7 @@ struct Sw2Shared {
   float2 yd[SW2_NW * QY];
   float2 edge[2][SW2_NW + 2][2][32];      // [parity][warp + 1][first / last row][lane]
   float2 gs[(SW2_NW + 1) * gram_nv(S)];
-  float wsum[SW2_NW * gram_ns(S)];
+  float2 wsum[SW2_NW * gram_ns(S)];
 };
 
 // A thread's place in its CTA's region and the stencil there (times the basis scale t).
@@ -116,50 +116,68 @@ struct Sw2Region {
     }
   }
   // k_1..k_S from k_0, the own points' k_j to p[j - 1] (j <= nstore), and the Gram matrix.
-  __device__ __forceinline__ void sweep(const LevelDev<float2>& L, const float2 (&sg)[S], float2 (&k)[S + 1][QY],
-                                        float2* const* p, int nstore, int unit, int nunits) {
+  __device__ __forceinline__ void sweep(const LevelDev<float2>& L, const float2 (&sg)[S], bool wide,
+                                        float2 (&k)[S + 1][QY], float2* const* p, int nstore, int unit, int nunits) {
 #pragma unroll
     for (int j = 0; j < S; ++j) apply(k[j], sg[j], k[j + 1]);
+    const bool ownx = own_x();
+    auto own_points = [&](auto sum) {
+#pragma unroll
+      for (int q = 0; q < QY; ++q) {
+        if (!own_row(q) || !ownx) continue;
+        float2 kk[S + 1];
+#pragma unroll
+        for (int j = 0; j <= S; ++j) kk[j] = k[j][q];
+        sum(kk);
+#pragma unroll
+        for (int j = 1; j <= S; ++j)
+          if (j <= nstore) p[j - 1][pidx(x, y0 + q, 0, P)] = kk[j];
+      }
+      pdl_trigger();  // the main work is done: let the next pass launch
+    };
     float acc[gram_ns(S)];
 #pragma unroll
     for (int i = 0; i < gram_ns(S); ++i) acc[i] = 0.f;
-    const bool ownx = own_x();
+    if (wide) {
+      float c[gram_ns(S)];
 #pragma unroll
-    for (int q = 0; q < QY; ++q) {
-      if (!own_row(q) || !ownx) continue;
-      float2 kk[S + 1];
-#pragma unroll
-      for (int j = 0; j <= S; ++j) kk[j] = k[j][q];
-      gram_point<S>(kk, acc);
-#pragma unroll
-      for (int j = 1; j <= S; ++j)
-        if (j <= nstore) p[j - 1][pidx(x, y0 + q, 0, P)] = kk[j];
+      for (int i = 0; i < gram_ns(S); ++i) c[i] = 0.f;
+      own_points([&](const float2 (&kk)[S + 1]) { gram_point_wide<S>(kk, acc, c); });
+      gram_block_sum_wide<S, SW2_NW>(acc, c, sh.wsum, sh.gs);
+    } else {
+      own_points([&](const float2 (&kk)[S + 1]) { gram_point<S>(kk, acc); });
+      gram_block_sum<S, SW2_NW>(acc, sh.wsum, sh.gs);
     }
-    pdl_trigger();  // the main work is done: let the next pass launch
-    gram_finish<S, SW2_NW>(acc, L, sg, unit, nunits, sh.wsum, sh.gs);
+    gram_finish<S, SW2_NW>(L, sg, wide, unit, nunits, sh.gs);
   }
 };
 
-template <int S, int QY, bool NC = true>
+// W: whether the problems' levels are wide (their sums need more registers, so that is a kernel
+// of its own), or W_ANY: each problem's own flag.
+enum { W_NO, W_YES, W_ANY };
+__device__ __forceinline__ bool wide_level(const LevelDev<float2>& L, int W) { return W == W_ANY ? L.wide != 0 : W == W_YES; }
+
+template <int S, int QY, int W, bool NC = true>
 __device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
                                             int store_last, int vblk, Sw2Shared<S, QY>& sh) {
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
-  Sw2Region<S, QY> W(L, unit, first ? S : S + 1, sh);
+  const bool wide = wide_level(L, W);
+  Sw2Region<S, QY> G(L, unit, first ? S : S + 1, sh);
   pdl_wait();
   float2 sg[S];
-  gram_shifts<S>(L, first != 0, sg);
+  gram_shifts<S>(L, first != 0, wide, sg);
   const float2* R0 = first ? L.b : L.r0;
   float2 k[S + 1][QY];
 #pragma unroll
-  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2, NC>(R0, W.x, W.y0 + q, 0, W.n, W.P);
-  W.sweep(L, sg, k, L.p, store_last ? S : S - 1, unit, nunits);
+  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2, NC>(R0, G.x, G.y0 + q, 0, G.n, G.P);
+  G.sweep(L, sg, wide, k, L.p, store_last ? S : S - 1, unit, nunits);
 }
-template <int S, int QY>
+template <int S, int QY, int W>
 __global__ void __launch_bounds__(256, 2)
 k_sweep2(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int store_last) {
   __shared__ Sw2Shared<S, QY> sh;
-  sweep2_body<S, QY>(levs, nunits, first, store_last, blockIdx.x, sh);
+  sweep2_body<S, QY, W>(levs, nunits, first, store_last, blockIdx.x, sh);
 }
 
 // ------------------------------------------------------------------ 2D, fused V(1,1) passes
@@ -176,7 +194,7 @@ k_sweep2(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int s
 // Descent: b = full weighting of the finer level's residual sum_k rho_k k_k (its last sweep),
 // which a lane forms for its column from two fine columns, the third being its neighbour's
 // first.  A problem whose finest level this is takes b as given.
-template <int S, int QY>
+template <int S, int QY, int WIDE>
 __global__ void __launch_bounds__(256, 2)
 k_sweep2_down(const LevelDev<float2>* __restrict__ levs, int nunits) {
   __shared__ Sw2Shared<S, QY> sh;
@@ -185,7 +203,7 @@ k_sweep2_down(const LevelDev<float2>* __restrict__ levs, int nunits) {
   Sw2Region<S, QY> W(L, unit, S, sh);
   pdl_wait();
   float2 sg[S];
-  gram_shifts<S>(L, true, sg);
+  gram_shifts<S>(L, true, WIDE, sg);
   float2 k[S + 1][QY];
   if (L.top) {
 #pragma unroll
@@ -248,7 +266,7 @@ k_sweep2_down(const LevelDev<float2>* __restrict__ levs, int nunits) {
       if (W.own_row(q) && W.own_x()) L.b[pidx(W.x, W.y0 + q, 0, W.P)] = k[0][q];
     }
   }
-  W.sweep(L, sg, k, L.p, S, unit, nunits);
+  W.sweep(L, sg, WIDE, k, L.p, S, unit, nunits);
 }
 
 // Coarse points around a 32 x R region of fine points: the coarser level's output there, its
@@ -294,7 +312,7 @@ __device__ __forceinline__ float2 staged_interp(const float2 (*es)[EX], int X0, 
 // Ascent: x_b = sum_k y_k k_k + P e_c (the pre-smoothing sweep from b, and the corrected
 // coarser output), R_0 = b - M x_b, and the sweep from it.  The new vectors go to L.q: other
 // CTAs still read the old ones.
-template <int S, int QY>
+template <int S, int QY, int WIDE>
 __global__ void __launch_bounds__(256, 2)
 k_sweep2_up(const LevelDev<float2>* __restrict__ levs, int nunits) {
   constexpr int EX = 18, EY = SW2_NW * QY / 2 + 2;
@@ -309,7 +327,7 @@ k_sweep2_up(const LevelDev<float2>* __restrict__ levs, int nunits) {
 #pragma unroll
   for (int j = 0; j < S; ++j) xc[j] = L.sc->xcoef[j];
   const int mc = coarse_update<S>(L, yc);
-  gram_shifts<S>(L, false, sg);
+  gram_shifts<S>(L, false, WIDE, sg);
   float2 b[QY], dx[QY];
 #pragma unroll
   for (int q = 0; q < QY; ++q) {
@@ -345,7 +363,7 @@ k_sweep2_up(const LevelDev<float2>* __restrict__ levs, int nunits) {
       L.r0[i] = k[0][q];
     }
   }
-  W.sweep(L, sg, k, L.q, S - 1, unit, nunits);
+  W.sweep(L, sg, WIDE, k, L.q, S - 1, unit, nunits);
 }
 
 // Coarse correction and residual of a larger level (the sweep after it marches), 64 x 16 tiles:
@@ -452,7 +470,7 @@ k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, 
   constexpr int NS = gram_ns(S), NV = gram_nv(S), W = 4;
   static_assert(S <= 3, "register windows hold four rows");
   extern __shared__ __align__(16) float2 swsm[];
-  __shared__ float wsum[SV2_NW * NS];
+  __shared__ float2 wsum[SV2_NW * NS];
   __shared__ float2 gs[(SV2_NW + 1) * NV];
   const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
@@ -474,7 +492,7 @@ k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, 
   pdl_wait();
   __syncthreads();
   float2 sg[S];
-  gram_shifts<S>(L, first != 0, sg);
+  gram_shifts<S>(L, first != 0, false, sg);
   const float2* R0 = first ? L.b : L.r0;
   const bool in = (unsigned)x < (unsigned)P;  // the pair lies in the row (P is even, x too)
   float2 win[S][W][2];  // k_j of the last rows, slot = step & 3
@@ -564,7 +582,8 @@ k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, 
     }
   }
   pdl_trigger();  // the main work is done: let the next pass launch
-  gram_finish<S, SV2_NW>(acc, L, sg, unit, nunits, wsum, gs);
+  gram_block_sum<S, SV2_NW>(acc, wsum, gs);
+  gram_finish<S, SV2_NW>(L, sg, false, unit, nunits, gs);
 }
 
 // ------------------------------------------------------------------ 3D, small levels
@@ -612,13 +631,13 @@ __device__ __forceinline__ float2 sw3_row(const float2* sm, const SwCoef& cx, co
   return cfma(make_float2(za.z, za.w), vt, p);
 }
 
-template <int S, int O, bool NC = true>
+template <int S, int O, int W, bool NC = true>
 __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
                                             int store_last, int vblk, float2* sm) {
   constexpr int NS = gram_ns(S), NV = gram_nv(S), R = O + 2 * S;
   __shared__ float4 yac[R], zac[R];
   __shared__ float2 yd[R], zd[R];
-  __shared__ float wsum[SW3_NW * NS];
+  __shared__ float2 wsum[SW3_NW * NS];
   __shared__ float2 gs[(SW3_NW + 1) * NV];
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
@@ -638,7 +657,8 @@ __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__
   }
   pdl_wait();
   float2 sg[S];
-  gram_shifts<S>(L, first != 0, sg);
+  const bool wide = wide_level(L, W);
+  gram_shifts<S>(L, first != 0, wide, sg);
   const float2* R0 = first ? L.b : L.r0;
 #pragma unroll 4
   for (int r = warp; r < R * R; r += SW3_NW)
@@ -661,34 +681,46 @@ __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__
   if constexpr (S >= 2) stage(std::integral_constant<int, 1>());
   if constexpr (S >= 3) stage(std::integral_constant<int, 2>());
   if constexpr (S >= 4) stage(std::integral_constant<int, 3>());
+  const bool ownx = lane >= S && lane < 32 - S && x < n;
+  auto own_points = [&](auto sum) {
+    for (int r = warp; r < O * O; r += SW3_NW) {
+      const int ry = r % O, rz = r / O, y = y0 + ry + S, z = z0 + rz + S;
+      if (y >= n || z >= n) continue;  // uniform over the warp
+      float2 kk[S + 1];
+      kk[S] = sw3_row<S, O, S>(sm, cx, yac, yd, zac, zd, sg[S - 1], phi_of(y, z), ry, rz, lane);
+      kk[0] = sm[((rz + S) * R + ry + S) * 32 + lane];
+      if constexpr (S >= 2) kk[1] = sm[(sw3_base<S, O, 1>() + (rz + S - 1) * (R - 2) + ry + S - 1) * 32 + lane];
+      if constexpr (S >= 3) kk[2] = sm[(sw3_base<S, O, 2>() + (rz + S - 2) * (R - 4) + ry + S - 2) * 32 + lane];
+      if constexpr (S >= 4) kk[3] = sm[(sw3_base<S, O, 3>() + (rz + S - 3) * (R - 6) + ry + S - 3) * 32 + lane];
+      if (ownx) {
+        sum(kk);
+#pragma unroll
+        for (int j = 1; j <= S; ++j)
+          if (j < S || store_last) L.p[j - 1][pidx(x, y, z, P)] = kk[j];
+      }
+    }
+    pdl_trigger();  // the main work is done: let the next pass launch
+  };
   float acc[NS];
 #pragma unroll
   for (int i = 0; i < NS; ++i) acc[i] = 0.f;
-  const bool ownx = lane >= S && lane < 32 - S && x < n;
-  for (int r = warp; r < O * O; r += SW3_NW) {
-    const int ry = r % O, rz = r / O, y = y0 + ry + S, z = z0 + rz + S;
-    if (y >= n || z >= n) continue;  // uniform over the warp
-    float2 kk[S + 1];
-    kk[S] = sw3_row<S, O, S>(sm, cx, yac, yd, zac, zd, sg[S - 1], phi_of(y, z), ry, rz, lane);
-    kk[0] = sm[((rz + S) * R + ry + S) * 32 + lane];
-    if constexpr (S >= 2) kk[1] = sm[(sw3_base<S, O, 1>() + (rz + S - 1) * (R - 2) + ry + S - 1) * 32 + lane];
-    if constexpr (S >= 3) kk[2] = sm[(sw3_base<S, O, 2>() + (rz + S - 2) * (R - 4) + ry + S - 2) * 32 + lane];
-    if constexpr (S >= 4) kk[3] = sm[(sw3_base<S, O, 3>() + (rz + S - 3) * (R - 6) + ry + S - 3) * 32 + lane];
-    if (ownx) {
-      gram_point<S>(kk, acc);
+  if (wide) {
+    float c[NS];
 #pragma unroll
-      for (int j = 1; j <= S; ++j)
-        if (j < S || store_last) L.p[j - 1][pidx(x, y, z, P)] = kk[j];
-    }
+    for (int i = 0; i < NS; ++i) c[i] = 0.f;
+    own_points([&](const float2 (&kk)[S + 1]) { gram_point_wide<S>(kk, acc, c); });
+    gram_block_sum_wide<S, SW3_NW>(acc, c, wsum, gs);
+  } else {
+    own_points([&](const float2 (&kk)[S + 1]) { gram_point<S>(kk, acc); });
+    gram_block_sum<S, SW3_NW>(acc, wsum, gs);
   }
-  pdl_trigger();  // the main work is done: let the next pass launch
-  gram_finish<S, SW3_NW>(acc, L, sg, unit, nunits, wsum, gs);
+  gram_finish<S, SW3_NW>(L, sg, wide, unit, nunits, gs);
 }
-template <int S, int O>
+template <int S, int O, int W>
 __global__ void __launch_bounds__(256)
 k_sweep3(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int store_last) {
   extern __shared__ __align__(16) float2 swsm[];
-  sweep3_body<S, O>(levs, nunits, first, store_last, blockIdx.x, swsm);
+  sweep3_body<S, O, W>(levs, nunits, first, store_last, blockIdx.x, swsm);
 }
 
 // ------------------------------------------------------------------ 3D, large levels
@@ -732,7 +764,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   constexpr int NS = gram_ns(S), NV = gram_nv(S), W = 4;
   static_assert(S <= 3, "register windows hold four planes");
   extern __shared__ __align__(16) float2 swsm[];
-  __shared__ float wsum[SM3_NW * NS];
+  __shared__ float2 wsum[SM3_NW * NS];
   __shared__ float2 gs[(SM3_NW + 1) * NV];
   const int prob = blockIdx.x / nunits, unit = blockIdx.x - prob * nunits;
   const LevelDev<float2>& L = levs[prob];
@@ -759,7 +791,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   for (int i = tid; i < (4 + 2 * (S - 1)) * (int)sm3_plane(); i += SM3_NW * 32) ring[i] = make_float2(0.f, 0.f);
   pdl_wait();
   float2 sg[S];
-  gram_shifts<S>(L, first != 0, sg);
+  gram_shifts<S>(L, first != 0, false, sg);
   const float2* R0 = first ? L.b : L.r0;
   const bool in0 = (unsigned)x < (unsigned)n && (unsigned)y < (unsigned)n;
   const bool in1 = (unsigned)x < (unsigned)n && (unsigned)(y + 1) < (unsigned)n;
@@ -885,7 +917,8 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
     }
   }
   pdl_trigger();  // the main work is done: let the next pass launch
-  gram_finish<S, SM3_NW>(acc, L, sg, unit, nunits, wsum, gs);
+  gram_block_sum<S, SM3_NW>(acc, wsum, gs);
+  gram_finish<S, SM3_NW>(L, sg, false, unit, nunits, gs);
 }
 
 }  // namespace helm

@@ -1083,11 +1083,11 @@ constexpr int SEQ_O3 = 4;  // own rows of the 3D sweep pass on levels the segmen
 template <typename C, int DIM, int J>
 __device__ __noinline__ void seq_arnoldi(const PassDesc d, const LevelDev<C>* levs, int v, float2* sm) {
   if constexpr (sizeof(C) == 8 && DIM == 2) {
-    if (d.geo == 2) sweep2_body<J, 2, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 2>*>(sm));
-    else if (d.geo == 4) sweep2_body<J, 4, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 4>*>(sm));
-    else sweep2_body<J, 6, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 6>*>(sm));
+    if (d.geo == 2) sweep2_body<J, 2, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 2>*>(sm));
+    else if (d.geo == 4) sweep2_body<J, 4, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 4>*>(sm));
+    else sweep2_body<J, 6, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 6>*>(sm));
   } else if constexpr (sizeof(C) == 8) {
-    sweep3_body<J, SEQ_O3, false>(levs, d.ntiles, d.f0, d.f1, v, sm);
+    sweep3_body<J, SEQ_O3, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, sm);
   } else if constexpr (DIM == 2) {
     arnoldi_t2_body<C, J, 1, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
   } else {
