@@ -543,9 +543,11 @@ __device__ __forceinline__ float bits8(float v) { return __uint_as_float(__float
 // The finest level's first shift from diff2 = sum |b_{x+1} - b_x|^2 over the pairs of
 // neighbours counted and norm2 = sum |b|^2: the Rayleigh quotient of the Laplacian's
 // isotropic estimate, minus the constant wavenumber term.  klap = (d / h^2) e^{-2 i theta}.
+// 0 stands for a smooth b (e below 1/5; white noise and points have 2), whose sweep takes no
+// shifts at all (gram_shifts).
 __device__ __forceinline__ float2 sweep_first_shift(float2 klap, float phic, float diff2, float norm2) {
   const float e = norm2 > 0.0f ? fminf(diff2 / norm2, 2.0f) : 0.0f;
-  if (!isfinite(e)) return make_float2(0.f, 0.f);
+  if (!(e >= 0.2f) || !isfinite(e)) return make_float2(0.f, 0.f);
   return make_float2(bits8(klap.x * e - phic), bits8(klap.y * e));
 }
 
