@@ -298,34 +298,12 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
   }
   // ------------------------------------------------ levels
   h->lev.resize(nlev);
+  std::vector<size_t> part_bytes(nlev);
   for (int l = 0; l < nlev; ++l) {
     HostLevel& L = h->lev[l];
     L.n = sizes[l];
     L.P = L.n + 1;
     L.np = h->dim == 3 ? (size_t)L.P * L.P * L.P : (size_t)L.P * L.P;
-    // phi sampled at this level's nodes (node x of level l is fine node (x+1) 2^l - 1)
-    if (phi) {
-      TRY(dev_alloc(h.get(), &L.phi, L.np * sizeof(float)));
-      scatter_phi(h->dim, L.n, 1 << l, h->n, phi, L.phi, st);
-      CUDA_TRY(cudaGetLastError());
-    } else {
-      L.phic = k * k;
-    }
-  }
-  if (phi && h->prec == HELM_C64) {  // the sweeps' shifts need every level's range
-    const size_t bytes = 2 * nlev * sizeof(unsigned);
-    unsigned* range = nullptr;
-    TRY(dev_alloc(h.get(), &range, bytes));
-    CUDA_TRY(cudaMemsetAsync(range, 0, bytes, st));
-    for (int l = 0; l < nlev; ++l) phi_range(h->dim, h->lev[l].n, h->lev[l].phi, range + 2 * l, st);
-    CUDA_TRY(cudaGetLastError());
-    unsigned* host = reinterpret_cast<unsigned*>(h->stage + h->stage_phi);
-    CUDA_TRY(cudaMemcpyAsync(host, range, bytes, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    for (int l = 0; l < nlev; ++l) phi_range_values(host + 2 * l, &h->lev[l].philo, &h->lev[l].phihi);
-  }
-  for (int l = 0; l < nlev; ++l) {
-    HostLevel& L = h->lev[l];
     const TileCfg cfg = default_tiles(h->dim, L.P);
     if (l == 0) h->cfg = cfg;
     L.ntiles = vtiles(h->dim, L.P);
@@ -362,10 +340,10 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
       finest.rows = 2;
       nparts = std::max<size_t>(nparts, tiles_per_problem(3, L.P, finest));
     }
-    size_t part_bytes = nparts * NPART * sizeof(double);
+    part_bytes[l] = nparts * NPART * sizeof(double);
     if (h->prec == HELM_C64)
-      part_bytes = std::max(part_bytes, (size_t)std::max(L.sweep.units, L.sweep.units_res) * GRAM_SLOT * sizeof(float2));
-    TRY(dev_alloc(h.get(), &L.part, part_bytes));
+      part_bytes[l] = std::max(part_bytes[l], (size_t)std::max(L.sweep.units, L.sweep.units_res) * GRAM_SLOT * sizeof(float2));
+    TRY(dev_alloc(h.get(), &L.part, part_bytes[l]));
     // TMA maps of the vectors the large 3D complex64 levels' passes stream (two sets, for
     // column tiles of 16 and of 32 rows)
     if (h->prec == HELM_C64 && h->dim == 3 && L.P >= 64 && L.P % 32 == 0) {
@@ -386,11 +364,34 @@ int setup_handle(const helm_grid* grid, const float* phi, double k, double theta
     // coefficients of M on this level (rediscretisation with spacing 2^l h)
     TRY(dev_alloc(h.get(), &L.coef64, 3 * L.n * sizeof(double2)));
     TRY(dev_alloc(h.get(), &L.coef, 3 * L.n * eb));
+    // phi sampled at this level's nodes (node x of level l is fine node (x+1) 2^l - 1)
+    if (phi) {
+      TRY(dev_alloc(h.get(), &L.phi, L.np * sizeof(float)));
+      scatter_phi(h->dim, L.n, 1 << l, h->n, phi, L.phi, st);
+      CUDA_TRY(cudaGetLastError());
+    } else {
+      L.phic = k * k;
+    }
+  }
+  if (phi && h->prec == HELM_C64) {  // the sweeps' shifts need every level's range
+    const size_t bytes = 2 * nlev * sizeof(unsigned);
+    unsigned* range = nullptr;
+    TRY(dev_alloc(h.get(), &range, bytes));
+    CUDA_TRY(cudaMemsetAsync(range, 0, bytes, st));
+    for (int l = 0; l < nlev; ++l) phi_range(h->dim, h->lev[l].n, h->lev[l].phi, range + 2 * l, st);
+    CUDA_TRY(cudaGetLastError());
+    unsigned* host = reinterpret_cast<unsigned*>(h->stage + h->stage_phi);
+    CUDA_TRY(cudaMemcpyAsync(host, range, bytes, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    for (int l = 0; l < nlev; ++l) phi_range_values(host + 2 * l, &h->lev[l].philo, &h->lev[l].phihi);
+  }
+  for (int l = 0; l < nlev; ++l) {
+    HostLevel& L = h->lev[l];
     TRY(upload_level_coefficients(h.get(), l, theta_beta, st));
     if (L.wide && L.sweep.march) {  // runs as regions: their partial slots
       L.sweep = sweep_cfg(h->dim, L.n, h->s, sm_count_host(), false);
       const size_t need = (size_t)std::max(L.sweep.units, L.sweep.units_res) * GRAM_SLOT * sizeof(float2);
-      if (need > part_bytes) TRY(dev_alloc(h.get(), &L.part, need));
+      if (need > part_bytes[l]) TRY(dev_alloc(h.get(), &L.part, need));
     }
   }
   // ------------------------------------------------ coarsest LU (FP64)

@@ -289,7 +289,10 @@ __device__ __forceinline__ void gram_shifts(const LevelDev<float2>& L, bool firs
   const float tj = est && s0.x == 0.0f && s0.y == 0.0f ? 0.0f : t;
   sg[0] = make_float2(s0.x * t, s0.y * t);
 #pragma unroll
-  for (int j = 1; j < S; ++j) sg[j] = make_float2(L.ksh[j - 1].x * tj, L.ksh[j - 1].y * tj);
+  for (int j = 1; j < S; ++j) {  // (ordinary levels: sigma_2 = 0, sigma_3 = sigma_1)
+    const float2 k = wide ? L.ksh[j - 1] : j == 2 ? make_float2(0.f, 0.f) : L.ksh[0];
+    sg[j] = make_float2(k.x * tj, k.y * tj);
+  }
 }
 
 // Sum of NW double-floats per value, gs-style: thread v NW + w holds part w of value v (NW a

@@ -55,8 +55,8 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms, bool march) {
   }
   // 3D levels from this size on march: 47^3 12 us a sweep, 63^3 14.5 against 25 in regions, 95^3
   // 23 against 42; at 31^3 both take 10
-  if (n < SWEEP3_MARCH_N || S > 3 || !march) {
-    c.geo = S <= 3 || n < 64 ? 4 : 8;
+  if (n < SWEEP3_MARCH_N || !march) {
+    c.geo = 4;
     c.units_res = c.units = sw3_units(S, c.geo, n);
     c.geo_res = c.geo;
     return c;
@@ -80,6 +80,16 @@ SweepCfg sweep_cfg(int dim, int n, int S, int sms, bool march) {
 }
 
 template <int S>
+static void launch_march3(const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, int first, int store_last,
+                          bool phi, cudaStream_t st) {
+  const dim3 grid(nprob * cfg.units), block(32, SM3_NW);
+  const size_t smem = sm3_smem(S, cfg.geo);
+  if (phi) allow_smem<k_sweep3_march<S, true>>();
+  else allow_smem<k_sweep3_march<S, false>>();
+  if (phi) pdl_launch(k_sweep3_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
+  else pdl_launch(k_sweep3_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
+}
+template <int S>
 static void launch_march(int dim, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, int first,
                          int store_last, bool phi, cudaStream_t st) {
   const dim3 grid(nprob * cfg.units);
@@ -90,12 +100,7 @@ static void launch_march(int dim, const LevelDev<float2>* levs, int nprob, const
     else pdl_launch(k_sweep2_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
     return;
   }
-  const dim3 block(32, SM3_NW);
-  const size_t smem = sm3_smem(S, cfg.geo);
-  if (phi) allow_smem<k_sweep3_march<S, true>>();
-  else allow_smem<k_sweep3_march<S, false>>();
-  if (phi) pdl_launch(k_sweep3_march<S, true>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
-  else pdl_launch(k_sweep3_march<S, false>, grid, block, smem, st, levs, cfg.units, cfg.geo, first, store_last);
+  launch_march3<S>(levs, nprob, cfg, first, store_last, phi, st);
 }
 
 void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const SweepCfg& cfg, bool first,
@@ -106,10 +111,11 @@ void launch_sweep(int dim, int S, const LevelDev<float2>* levs, int nprob, const
     else launch_regions<W_NO>(dim, S, levs, nprob, cfg, f, sl, st);
     return;
   }
-  switch (S) {  // (S <= 3: sweep_cfg)
+  switch (S) {
     case 1: launch_march<1>(dim, levs, nprob, cfg, f, sl, phi, st); break;
     case 2: launch_march<2>(dim, levs, nprob, cfg, f, sl, phi, st); break;
-    default: launch_march<3>(dim, levs, nprob, cfg, f, sl, phi, st); break;
+    case 3: launch_march<3>(dim, levs, nprob, cfg, f, sl, phi, st); break;
+    default: launch_march3<4>(levs, nprob, cfg, f, sl, phi, st); break;  // (2D: sweep_cfg marches to S = 3)
   }
 }
 

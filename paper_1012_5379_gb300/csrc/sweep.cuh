@@ -717,7 +717,7 @@ __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__
   gram_finish<S, SW3_NW>(L, sg, wide, unit, nunits, gs);
 }
 template <int S, int O, int W>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, W == W_NO && S <= 3 ? 4 : 1)
 k_sweep3(const LevelDev<float2>* __restrict__ levs, int nunits, int first, int store_last) {
   extern __shared__ __align__(16) float2 swsm[];
   sweep3_body<S, O, W>(levs, nunits, first, store_last, blockIdx.x, swsm);
@@ -739,8 +739,10 @@ HELM_HD inline int sm3_units(int S, int n, int zc) {
 }
 // published planes: [parity][vector][row][lane], one guard row at either end
 HELM_HD constexpr unsigned sm3_plane() { return (SM3_R + 2) * 32; }
+// planes of R_0 and phi kept: four, or eight where the registers hold no window of k_0 (S = 4)
+HELM_HD constexpr int sm3_ring(int S) { return S > 3 ? 8 : 4; }
 HELM_HD constexpr unsigned sm3_smem(int S, int zc) {
-  return (4u + 2u * (S - 1)) * sm3_plane() * 8u + 4u * SM3_R * 32u * 4u + (unsigned)(zc + 2 * S) * 24u;
+  return (sm3_ring(S) + 2u * (S - 1)) * sm3_plane() * 8u + sm3_ring(S) * SM3_R * 32u * 4u + (unsigned)(zc + 2 * S) * 24u;
 }
 // Asynchronous copies to shared memory; with ok false they fill zeros and read nothing.
 __device__ __forceinline__ void copy8_async(float2* dst, const float2* src, bool ok) {
@@ -762,7 +764,8 @@ template <int S, bool PHI>
 __global__ void __launch_bounds__(SM3_NW * 32, 1)
 k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, int first, int store_last) {
   constexpr int NS = gram_ns(S), NV = gram_nv(S), W = 4;
-  static_assert(S <= 3, "register windows hold four planes");
+  constexpr int RING = sm3_ring(S);
+  constexpr bool K0 = RING == W;  // k_0 and phi of the last planes in registers too
   extern __shared__ __align__(16) float2 swsm[];
   __shared__ float2 wsum[SM3_NW * NS];
   __shared__ float2 gs[(SM3_NW + 1) * NV];
@@ -776,10 +779,10 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   const int x = (unit % nt) * sw_ox(S) - S + lane;
   const int ry = 2 * warp, y = ((unit / nt) % nt) * sw_ox(S) - S + ry;  // rows y, y + 1
   const int zb = (unit / (nt * nt)) * zc, ze = min(zb + zc, n);
-  float2* const ring = swsm;                                             // R_0: plane i in slot i & 3
-  float2* const pub = ring + 4 * sm3_plane();                            // [parity][k_1 .. k_{S-1}]
+  float2* const ring = swsm;                                             // R_0: plane i in slot i & (RING - 1)
+  float2* const pub = ring + RING * sm3_plane();                         // [parity][k_1 .. k_{S-1}]
   float* const phring = reinterpret_cast<float*>(pub + 2 * (S - 1) * sm3_plane());
-  float4* const zac = reinterpret_cast<float4*>(phring + 4 * SM3_R * 32);
+  float4* const zac = reinterpret_cast<float4*>(phring + RING * SM3_R * 32);
   float2* const zd = reinterpret_cast<float2*>(zac + (zc + 2 * S));
   const SwCoef cx = sw_coef(L.ca, x, n, t), cy0 = sw_coef(L.ca, y, n, t), cy1 = sw_coef(L.ca, y + 1, n, t);
   const float2 dxy[2] = {cadd(cx.d, cy0.d), cadd(cx.d, cy1.d)};
@@ -788,7 +791,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
     zac[i] = make_float4(c.a.x, c.a.y, c.c.x, c.c.y);
     zd[i] = c.d;
   }
-  for (int i = tid; i < (4 + 2 * (S - 1)) * (int)sm3_plane(); i += SM3_NW * 32) ring[i] = make_float2(0.f, 0.f);
+  for (int i = tid; i < (RING + 2 * (S - 1)) * (int)sm3_plane(); i += SM3_NW * 32) ring[i] = make_float2(0.f, 0.f);
   pdl_wait();
   float2 sg[S];
   gram_shifts<S>(L, first != 0, false, sg);
@@ -799,7 +802,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   const size_t PP = (size_t)P * P;
   float2 win[S][W][2];  // k_j of the last planes, slot = plane & 3
 #pragma unroll
-  for (int j = 0; j < S; ++j)
+  for (int j = K0 ? 0 : 1; j < S; ++j)
 #pragma unroll
     for (int w = 0; w < W; ++w) win[j][w][0] = win[j][w][1] = make_float2(0.f, 0.f);
   float phw[W][2];
@@ -842,12 +845,19 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
       const int i = i0 + u;
       if (i >= zl - zf) break;  // uniform
       const int z = zf + i;
-      if (z + AHEAD < zl) fetch(z + AHEAD, (u + AHEAD) & 3);
+      auto slot = [&](int d) { return K0 ? (u + d) & 3 : (i + d) & (RING - 1); };  // of plane i + d
+      auto k0 = [&](int d, int q) { return ring[slot(d) * (int)sm3_plane() + at0 + 32 * q]; };
+      auto ph = [&](int d, int q) {
+        return field ? phring[slot(d) * SM3_R * 32 + (ry + q) * 32 + lane] * t : phc;
+      };
+      if (z + AHEAD < zl) fetch(z + AHEAD, slot(AHEAD));
       copies_commit();
       const float2* const r0 = ring + u * sm3_plane() + at0;
-      win[0][u][0] = r0[0];
-      win[0][u][1] = r0[32];
-      if (PHI) {
+      if (K0) {
+        win[0][u][0] = r0[0];
+        win[0][u][1] = r0[32];
+      }
+      if (PHI && K0) {
         const float* const f = phring + u * SM3_R * 32 + ry * 32 + lane;
         phw[u][0] = field ? f[0] * t : phc;
         phw[u][1] = field ? f[32] * t : phc;
@@ -865,22 +875,23 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
           const float4 za = zac[iz];
           const float2 zdd = zd[iz];
           // k_{j-1} of plane z - j as published
-          const float2* s = j == 1 ? ring + ((u + 3) & 3) * sm3_plane() + at0 : rd + (size_t)(j > 1 ? j - 2 : 0) * sm3_plane();
+          const float2* s = j == 1 ? ring + slot(-1) * sm3_plane() + at0 : rd + (size_t)(j > 1 ? j - 2 : 0) * sm3_plane();
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
+            const bool reg = K0 || j > 1;
             float2 dg = dxy[q];
-            dg.x = (dg.x - (PHI ? phw[c][q] : phc)) - sg[j - 1].x;
+            dg.x = (dg.x - (PHI ? (K0 ? phw[c][q] : ph(-j, q)) : phc)) - sg[j - 1].x;
             dg.y -= sg[j - 1].y;
-            const float2 v = win[j - 1][c][q];
+            const float2 v = reg ? win[j - 1][c][q] : k0(-1, q);
             float2 p = cmul(dg, v);
             p = cfma(zdd, v, p);
             p = cfma(cx.a, s[32 * q - 1], p);
             p = cfma(cx.c, s[32 * q + 1], p);
             const SwCoef& cy = q ? cy1 : cy0;
-            p = cfma(cy.a, q ? win[j - 1][c][0] : s[-32], p);
-            p = cfma(cy.c, q ? s[64] : win[j - 1][c][1], p);
-            p = cfma(make_float2(za.x, za.y), win[j - 1][b][q], p);
-            p = cfma(make_float2(za.z, za.w), win[j - 1][f][q], p);
+            p = cfma(cy.a, q ? (reg ? win[j - 1][c][0] : s[0]) : s[-32], p);
+            p = cfma(cy.c, q ? s[64] : (reg ? win[j - 1][c][1] : s[32]), p);
+            p = cfma(make_float2(za.x, za.y), reg ? win[j - 1][b][q] : k0(-2, q), p);
+            p = cfma(make_float2(za.z, za.w), reg ? win[j - 1][f][q] : k0(0, q), p);
             r[q] = p;
           }
         }
@@ -902,8 +913,9 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
         for (int q = 0; q < 2; ++q) {
           if (q ? own1 : own0) {
             float2 kk[S + 1];
+            kk[0] = K0 ? win[0][c][q] : k0(-S, q);
 #pragma unroll
-            for (int j = 0; j < S; ++j) kk[j] = win[j][c][q];
+            for (int j = 1; j < S; ++j) kk[j] = win[j][c][q];
             kk[S] = last[q];
             gram_point<S>(kk, acc);
 #pragma unroll

@@ -20,13 +20,6 @@ static void launch_regions_s(int dim, const LevelDev<float2>* levs, int nprob, c
     else pdl_launch(k_sweep2<S, 6, W>, grid, block, 0, st, levs, units, first, store_last);
     return;
   }
-  if constexpr (S > 3) {
-    if (geo == 8) {
-      allow_smem<k_sweep3<S, 8, W>>();
-      pdl_launch(k_sweep3<S, 8, W>, grid, block, sw3_smem(S, 8), st, levs, units, first, store_last);
-      return;
-    }
-  }
   allow_smem<k_sweep3<S, 4, W>>();
   pdl_launch(k_sweep3<S, 4, W>, grid, block, sw3_smem(S, 4), st, levs, units, first, store_last);
 }
