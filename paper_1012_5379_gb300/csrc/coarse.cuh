@@ -22,8 +22,8 @@ constexpr int CG_COARSE_POINTS = CG_THREADS * CG_PT;  // most interior points of
 constexpr int CG_INV = 1024;                          // entries of the inverse staged in shared memory
 constexpr int CG_COEF = 3 * 64;                       // 1D coefficients of all levels (31 + 15 + 7 + 3 per array)
 
-// b, x, r, k_1..k_{S-1}; S = 0 stands for the polynomial smoother
-HELM_HD constexpr int cg_vectors(int S) { return 3 + (S > 1 ? S - 1 : 0); }
+// b, x, r, k_1..k_{S-1} and, where a level is wide, k_S; S = 0 stands for the polynomial smoother
+HELM_HD constexpr int cg_vectors(int S, bool wide = false) { return 3 + (S > 1 ? S - 1 : 0) + (wide ? 1 : 0); }
 
 // One thread's points of a level and the level's vectors.
 template <int S, int DIM>
@@ -31,6 +31,8 @@ struct CgLevel {
   int n, P;
   float t, it;                         // basis scale and its reciprocal
   float2 *b, *x, *r, *k[S > 1 ? S - 1 : 1];
+  float2* kv;                          // k_1 .. (at strides of np)
+  int np;                              // padded points
   int off[CG_PT], cx[CG_PT], cy[CG_PT], cz[CG_PT];
   bool on[CG_PT];
   float2 ax[CG_PT], qx[CG_PT], ay[CG_PT], qy[CG_PT], az[CG_PT], qz[CG_PT], dg[CG_PT], dz[CG_PT];
@@ -88,10 +90,37 @@ struct CgLevel {
 };
 
 struct CgShared {
-  float2 wsum[CG_NW * 32];
+  float2 wsum[CG_NW * 16];
   float2 gs[gram_nv(SMAX)];
   float2 xc[SMAX], rc[SMAX + 1];
 };
+
+// The Gram matrix of a wide level in double-float: a warp per value, all of the level's points
+// from shared memory (k_0 at R0, k_j at kv + (j - 1) np; ghosts are zero).  A loop of a few
+// instructions: as thread sums of both points and a transposed butterfly it was 14 KB of
+// straight-line code, fetched from L2 for every launch (a 3D sub-cycle took 31 us, 16 without).
+template <int S>
+__device__ __forceinline__ void cg_gram_wide(const float2* R0, const float2* kv, int np, float2* gs) {
+  const int lane = threadIdx.x & 31;
+  for (int v = threadIdx.x >> 5; v < gram_nv(S); v += CG_NW) {
+    int i = 0, e = v;  // row i, entry e of it: the diagonal, then re and im of each column
+    while (e > 2 * (S - i)) {
+      e -= 1 + 2 * (S - i);
+      ++i;
+    }
+    const int j = i + (e + 1) / 2;
+    const bool im = e > 0 && !(e & 1);
+    const float2 *A = i == 0 ? R0 : kv + (size_t)(i - 1) * np, *B = j == 0 ? R0 : kv + (size_t)(j - 1) * np;
+    float s = 0.f, c = 0.f;
+    for (int p = lane; p < np; p += 32) {
+      const float2 a = A[p], b = B[p];
+      df_mac1(s, c, a.x, 0.f, im ? b.y : b.x);
+      df_mac1(s, c, a.y, 0.f, im ? -b.x : b.y);
+    }
+    const float2 tot = df_group_sum<32>(make_float2(s, c));
+    if (lane == 0) gs[v] = tot;
+  }
+}
 
 // One sweep: k0 (this thread's values of R_0, already in shared memory at R0 and visible to
 // the CTA) -> x += dx and k0 = the new residual.
@@ -112,21 +141,18 @@ __device__ __forceinline__ void cg_sweep(const CgLevel<S, DIM>& V, const float2*
       if (V.on[q]) {
         k[q][j] = V.apply(src, k[q][j - 1], q, sg[j - 1]);
         if (j < S) V.k[j >= 1 && j < S ? j - 1 : 0][V.off[q]] = k[q][j];
+        else if (wide) V.kv[(S - 1) * V.np + V.off[q]] = k[q][j];
       }
     }
     if (j < S) __syncthreads();
   }
-  float acc[NS];
-#pragma unroll
-  for (int i = 0; i < NS; ++i) acc[i] = 0.f;
   if (wide) {
-    float c[NS];
-#pragma unroll
-    for (int i = 0; i < NS; ++i) c[i] = 0.f;
-#pragma unroll
-    for (int q = 0; q < CG_PT; ++q) gram_point_wide<S>(k[q], acc, c);
-    gram_block_sum_wide<S, CG_NW>(acc, c, sh.wsum, sh.gs);
+    __syncthreads();
+    cg_gram_wide<S>(R0, V.kv, V.np, sh.gs);
   } else {
+    float acc[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) acc[i] = 0.f;
 #pragma unroll
     for (int q = 0; q < CG_PT; ++q) gram_point<S>(k[q], acc);
     gram_block_sum<S, CG_NW>(acc, sh.wsum, sh.gs);
@@ -190,7 +216,7 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
   __shared__ float2 coef[CG_COEF];
   __shared__ float4 inv_sm[CG_INV];
   __shared__ CgShared sh;
-  constexpr int NVEC = cg_vectors(S);
+  constexpr int NVEC = cg_vectors(S, WIDE);
   const int tid = threadIdx.x, prob = blockIdx.x;
   const LevelDev<float2>* G = levs_all + (size_t)prob * lev_stride;
   const CoarseLU lu = lus[prob];
@@ -229,8 +255,10 @@ k_coarse_gram(const LevelDev<float2>* __restrict__ levs_all, int lev_stride, con
     V.b = v;
     V.x = v + np;
     V.r = v + 2 * np;
+    V.kv = v + 3 * np;
+    V.np = np;
 #pragma unroll
-    for (int j = 0; j + 1 < S; ++j) V.k[j] = v + (3 + j) * np;
+    for (int j = 0; j + 1 < S; ++j) V.k[j] = V.kv + j * np;
     V.stencil_setup(Ls[l], coef + s_cof[l], tid);
   };
   enter(0);

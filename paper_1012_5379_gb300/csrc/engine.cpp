@@ -673,7 +673,7 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
     if (sizeof(C) == 8) {
       std::vector<int> ns;
       for (int t = g->tc; t < g->Lmax; ++t) ns.push_back(big->lev[t].n);
-      bytes = coarse_gram_smem(g->dim, g->smoother == HELM_SMOOTHER_POLY ? 0 : g->s, ns.data(), (int)ns.size());
+      bytes = coarse_gram_smem(g->dim, g->smoother == HELM_SMOOTHER_POLY ? 0 : g->s, ns.data(), (int)ns.size(), true);
     }
     g->coarse_smem = (g->nlev_c <= MAX_COARSE_LEVELS_HOST && bytes <= 200 * 1024) ? bytes : 0;
   }

@@ -263,7 +263,7 @@ void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, co
 // from coarse_gram_smem over its level sizes; the last nwide problems have wide levels
 void launch_coarse_gram(int dim, int S, const LevelDev<float2>* levs, int lev_stride, const CoarseLU* lus, int nprob,
                         int nwide, const float2* pw, int nu1, int nu2, bool from_res, size_t smem, cudaStream_t st);
-size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev);
+size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev, bool wide = false);
 template <typename C>
 void launch_restrict(int dim, const LevelDev<C>* levs, int nprob, int ntiles, TileCfg cfg, bool r0_is_b,
                      bool x_from_zero, bool nosmooth, cudaStream_t st, bool tma = false, int nraw = SMAX + 1);

@@ -146,11 +146,11 @@ void record_sweep(PassSeq& q, int S, const LevelDev<float2>* levs, int nprob, co
   seq_push(q, levs, PK_ARNOLDI, S, units, first ? cfg.geo : cfg.geo_res, first, store_last, 0, 0, nprob * units);
 }
 
-size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev) {
+size_t coarse_gram_smem(int dim, int S, const int* sizes, int nlev, bool wide) {
   size_t total = 0;
   for (int l = 0; l < nlev; ++l) {
     const size_t P = sizes[l] + 1, np = dim == 3 ? P * P * P : P * P;
-    total += np / P + cg_vectors(S) * np;
+    total += np / P + cg_vectors(S, wide) * np;
   }
   return total * sizeof(float2);
 }
