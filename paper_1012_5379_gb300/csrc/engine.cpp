@@ -130,32 +130,23 @@ static int factor_coarsest(Handle* h, double theta_beta, cudaStream_t st) {
         for (int x = 0; x < Lc.n; ++x) phic[(z * Lc.n + y) * Lc.n + x] = pad[((size_t)z * Lc.P + y) * Lc.P + x];
   }
   std::vector<cplx> A = dense_operator(h->dim, Lc.n, a, d, c, phic, cplx(1.0, h->csl_eps));
+  const std::vector<cplx> A0 = A;
   std::vector<int> perm;
   if (!lu_factor(A, cm, perm)) { set_error("coarsest operator is singular"); return HELM_ENUMERIC; }
-  {  // the inverse, column by column from the factors (binary64); complex64: as double-floats
+  {  // the inverse (binary64); complex64: as double-floats
     double2* ivd = reinterpret_cast<double2*>(h->stage + h->stage_inv);
     float4* iv = reinterpret_cast<float4*>(ivd);
-    std::vector<cplx> y(cm);
     auto split = [](double v, float* hi, float* lo) {
       *hi = (float)v;
       *lo = (float)(v - (double)*hi);
     };
-    for (int j = 0; j < cm; ++j) {
-      for (int i = 0; i < cm; ++i) y[i] = perm[i] == j ? 1.0 : 0.0;
-      for (int i = 0; i < cm; ++i)
-        for (int q = 0; q < i; ++q) y[i] -= A[(size_t)i * cm + q] * y[q];
-      for (int i = cm - 1; i >= 0; --i) {
-        for (int q = i + 1; q < cm; ++q) y[i] -= A[(size_t)i * cm + q] * y[q];
-        y[i] /= A[(size_t)i * cm + i];
-      }
-      for (int i = 0; i < cm; ++i) {
-        const size_t at = (size_t)i * cm + j;
-        if (h->prec == HELM_C128) {
-          ivd[at] = make_double2(y[i].real(), y[i].imag());
-        } else {
-          split(y[i].real(), &iv[at].x, &iv[at].y);
-          split(y[i].imag(), &iv[at].z, &iv[at].w);
-        }
+    const std::vector<cplx> X = lu_inverse(A0, A, cm, perm);
+    for (size_t at = 0; at < X.size(); ++at) {
+      if (h->prec == HELM_C128) {
+        ivd[at] = make_double2(X[at].real(), X[at].imag());
+      } else {
+        split(X[at].real(), &iv[at].x, &iv[at].y);
+        split(X[at].imag(), &iv[at].z, &iv[at].w);
       }
     }
     static_assert(sizeof(float4) == sizeof(double2), "one staging block for either form");

@@ -100,6 +100,77 @@ bool lu_factor(std::vector<cplx>& A, int m, std::vector<int>& perm) {
   return true;
 }
 
+// s + c += a b exactly up to the rounding of c (TwoProduct, TwoSum)
+static void mac2(double a, double b, double& s, double& c) {
+  const double p = a * b, e = std::fma(a, b, -p), t = s + p, z = t - s;
+  c += ((s - (t - z)) + (p - z)) + e;
+  s = t;
+}
+
+// sum_{q0 <= q < q1} LU[i][q] y[q] (written out: std::complex products test for NaN every time)
+static cplx row_product(const std::vector<cplx>& LU, int m, int i, int q0, int q1, const std::vector<cplx>& y) {
+  double re = 0.0, im = 0.0;
+  for (int q = q0; q < q1; ++q) {
+    const cplx a = LU[(size_t)i * m + q], b = y[q];
+    re += a.real() * b.real() - a.imag() * b.imag();
+    im += a.real() * b.imag() + a.imag() * b.real();
+  }
+  return cplx(re, im);
+}
+
+// The inverse X of A: from its factors LU by substitution, then X += X (I - A X) with the
+// residual in twice the working precision until that no longer counts.  The entries are then
+// correct to a rounding whatever the condition number (short of 1 / eps), where substitution
+// alone leaves cond(A) eps and a product with X would add as much again.
+std::vector<cplx> lu_inverse(const std::vector<cplx>& A, const std::vector<cplx>& LU, int m, const std::vector<int>& perm) {
+  std::vector<cplx> X((size_t)m * m), R((size_t)m * m), y(m), dx(m);
+  for (int j = 0; j < m; ++j) {
+    int first = m;  // the unit vector's leading zeros stay zero
+    for (int i = 0; i < m; ++i) {
+      y[i] = perm[i] == j ? 1.0 : 0.0;
+      if (perm[i] == j) first = i;
+      if (i > first) y[i] -= row_product(LU, m, i, first, i, y);
+    }
+    for (int i = m - 1; i >= 0; --i) y[i] = (y[i] - row_product(LU, m, i, i + 1, m, y)) / LU[(size_t)i * m + i];
+    for (int i = 0; i < m; ++i) X[(size_t)i * m + j] = y[i];
+  }
+  for (int step = 0; step < 4; ++step) {
+    double rho = 0.0;
+    for (int i = 0; i < m; ++i) {
+      std::vector<int> col;  // A's few entries in this row
+      for (int q = 0; q < m; ++q)
+        if (A[(size_t)i * m + q] != cplx(0.0)) col.push_back(q);
+      for (int j = 0; j < m; ++j) {
+        double sr = i == j ? 1.0 : 0.0, cr = 0.0, si = 0.0, ci = 0.0;
+        for (int q : col) {
+          const cplx a = A[(size_t)i * m + q], x = X[(size_t)q * m + j];
+          mac2(-a.real(), x.real(), sr, cr);
+          mac2(a.imag(), x.imag(), sr, cr);
+          mac2(-a.real(), x.imag(), si, ci);
+          mac2(-a.imag(), x.real(), si, ci);
+        }
+        R[(size_t)i * m + j] = cplx(sr + cr, si + ci);
+        rho = std::max({rho, std::abs(sr + cr), std::abs(si + ci)});
+      }
+    }
+    for (int i = 0; i < m; ++i) {
+      std::fill(dx.begin(), dx.end(), cplx(0.0));
+      double* const d = reinterpret_cast<double*>(dx.data());
+      for (int q = 0; q < m; ++q) {
+        const double xr = X[(size_t)i * m + q].real(), xi = X[(size_t)i * m + q].imag();
+        const double* const r = reinterpret_cast<const double*>(R.data() + (size_t)q * m);
+        for (int j = 0; j < m; ++j) {
+          d[2 * j] += xr * r[2 * j] - xi * r[2 * j + 1];
+          d[2 * j + 1] += xr * r[2 * j + 1] + xi * r[2 * j];
+        }
+      }
+      for (int j = 0; j < m; ++j) X[(size_t)i * m + j] += dx[j];
+    }
+    if (!(rho > 1e-9)) break;  // the next step's correction would be rho^2
+  }
+  return X;
+}
+
 std::vector<int> level_sizes(int n, int coarsest) {
   std::vector<int> s{n};
   while (s.back() > coarsest && (s.back() + 1) % 2 == 0) s.push_back((s.back() + 1) / 2 - 1);
