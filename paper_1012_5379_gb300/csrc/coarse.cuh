@@ -21,6 +21,10 @@ constexpr int CG_THREADS = 512, CG_NW = CG_THREADS / 32, CG_PT = 2;
 constexpr int CG_COARSE_POINTS = CG_THREADS * CG_PT;  // most interior points of a level
 constexpr int CG_INV = 1024;                          // entries of the inverse staged in shared memory
 constexpr int CG_COEF = 3 * 64;                       // 1D coefficients of all levels (31 + 15 + 7 + 3 per array)
+static_assert(coarse_threshold(2, 1) * coarse_threshold(2, 1) <= CG_COARSE_POINTS &&
+                  coarse_threshold(3, 1) * coarse_threshold(3, 1) * coarse_threshold(3, 1) <= CG_COARSE_POINTS &&
+                  2 * coarse_threshold(2, 1) <= CG_COEF / 3,
+              "a thread holds CG_PT points of a level; the levels halve");
 
 // b, x, r, k_1..k_{S-1} and, where a level is wide, k_S; S = 0 stands for the polynomial smoother
 HELM_HD constexpr int cg_vectors(int S, bool wide = false) { return 3 + (S > 1 ? S - 1 : 0) + (wide ? 1 : 0); }

@@ -555,7 +555,7 @@ struct Group {
   std::vector<Depth> depth;      // t < tc
   LevelDev<C>* dcoarse = nullptr;  // [prob][Lmax - tc]
   int nlev_c = 0;
-  size_t coarse_smem = 0;          // dynamic shared memory of the staged coarse kernel (0: global)
+  size_t coarse_smem = 0;          // dynamic shared memory of the coarse kernel
   CoarseLU* dlu = nullptr;
   int nwc = 0;                     // problems with a wide level among the coarse ones, after the others
   C* pwc = nullptr;                // polynomial smoother: weights of the coarse levels [prob][level][3]
@@ -666,7 +666,11 @@ static int build_group(Handle* const* hs, int count, cudaStream_t st, Group<C>* 
       for (int t = g->tc; t < g->Lmax; ++t) ns.push_back(big->lev[t].n);
       bytes = coarse_gram_smem(g->dim, g->smoother == HELM_SMOOTHER_POLY ? 0 : g->s, ns.data(), (int)ns.size(), true);
     }
-    g->coarse_smem = (g->nlev_c <= MAX_COARSE_LEVELS_HOST && bytes <= 200 * 1024) ? bytes : 0;
+    if (g->nlev_c > MAX_COARSE_LEVELS_HOST || bytes > 200 * 1024) {  // (coarse_threshold keeps it below)
+      set_error("coarse levels do not fit in shared memory");
+      return HELM_EINVAL;
+    }
+    g->coarse_smem = bytes;
   }
   // tile config of a group: the first problem's
   for (int p = 0; p < count; ++p)

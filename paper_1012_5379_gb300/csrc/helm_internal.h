@@ -194,7 +194,7 @@ HELM_HD inline int vtiles(int dim, int P) {
 // Largest level size run by the coarse sub-cycle kernel (one CTA per problem) instead of
 // grid-wide launches.  Complex128 is bound by the FP64 pipe (2 lanes per SM and cycle): a
 // 31^2 Arnoldi step takes one SM 29,000 cycles, more than its launches on four.
-HELM_HD inline int coarse_threshold(int dim, int prec) {
+HELM_HD constexpr int coarse_threshold(int dim, int prec) {
   return dim == 3 ? 7 : prec == 2 /* HELM_C128 */ ? 23 : 31;
 }
 
