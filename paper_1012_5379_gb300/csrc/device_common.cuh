@@ -186,8 +186,9 @@ __device__ __forceinline__ void warp_rows_total(const double* sm, int nw, double
   for (int i = 0; i < NV; ++i) tot[i] = __shfl_sync(0xffffffffu, s, i);
 }
 
-// Sum NV values over the block in a fixed order; thread 0 ends with the totals.
-// `sm` needs 32 * NV values.  Every thread of the block must call it.
+// Sum NV values over the block in a fixed order; thread 0 ends with the totals.  `sm` needs
+// 32 NV values: binary64 takes sum_vp(NV) < 2 NV per warp, and a block has at most 16 warps.
+// Every thread of the block must call it.
 template <int NV, typename T>
 __device__ __forceinline__ void block_sum(T (&v)[NV], T* sm) {
   const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5, nw = (block_threads() + 31) >> 5;
@@ -196,6 +197,7 @@ __device__ __forceinline__ void block_sum(T (&v)[NV], T* sm) {
     // the warp halves the values kept at every butterfly (VP - 1 + 5 - log2 VP additions,
     // 9 for seven values, instead of 5 NV = 35) and the cross-warp sum takes four more
     constexpr int VP = sum_vp(NV);
+    static_assert(16 * VP <= 32 * NV, "scratch of 16 warps");
     double a[VP];
 #pragma unroll
     for (int i = 0; i < VP; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : 0.0;
