@@ -295,7 +295,7 @@ void apply_operator_dense(int dim, int n, const double2* ca, const double2* cd, 
   // than eight warps on each SM sub-partition
   const int ntx = (n + 31) / 32, lines = dim == 3 ? ntx * ((n + 7) / 8) * 8 : ntx;
   int rows = 8;
-  while (rows > 1 && (long long)lines * ((n + rows - 1) / rows) < 152LL * 32) rows /= 2;
+  while (rows > 1 && (long long)lines * ((n + rows - 1) / rows) < 32LL * GB300_SMS) rows /= 2;
   const int chunks = (n + rows - 1) / rows;
   const dim3 block(32, 8);
   const int grid = dim == 3 ? ntx * ((n + 7) / 8) * chunks : ntx * ((chunks + 7) / 8);

@@ -39,7 +39,7 @@ static int sm_count_host() {
 static TileCfg default_tiles(int dim, int P) {
   TileCfg c;
   if (dim == 2) {
-    int rows = (int)((long long)P * P / (32LL * WARPS2 * 608));
+    int rows = (int)((long long)P * P / (32LL * WARPS2 * 4 * GB300_SMS));
     rows = std::max(2, std::min(32, rows & ~1));
     c.rows = rows;
   } else {

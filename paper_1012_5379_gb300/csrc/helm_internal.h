@@ -22,6 +22,8 @@
 
 namespace helm {
 
+constexpr int GB300_SMS = 152;     // the device this is for: lines between kernels, which must not move with the
+                                   // device at hand (grids and shares follow its own count)
 constexpr int SMAX = 4;            // max GMRES(s) steps per smoothing sweep
 constexpr int NPART = 2 * SMAX + 4;  // doubles per partial-sum slot of a sweep pass
 constexpr int GRAM_SLOT = 32;        // double-floats per partial slot of a Gram sweep pass (gram.cuh)
@@ -185,7 +187,8 @@ HELM_HD inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 // of 7.6; at 1023^2 and above the larger tile's thinner halo wins.
 HELM_HD inline int zchunk(int P) { return P >= 128 ? 32 : (P >= 64 ? 4 : 2); }
 // (The persistent segments' levels, P <= 512, have Q = 1.)
-HELM_HD inline int tile2_q(int P) { return ceil_div(P, 64) * ceil_div(P, 16) < 608 ? 1 : 2; }
+HELM_HD constexpr int tile2_q(int P) { return ((P + 63) / 64) * ((P + 15) / 16) < 4 * GB300_SMS ? 1 : 2; }
+static_assert(tile2_q(512) == 1, "the persistent segments are compiled for Q = 1");
 HELM_HD inline int vtiles(int dim, int P) {
   const int q = tile2_q(P);
   return dim == 2 ? ceil_div(P, 32 * q) * ceil_div(P, 8 * q) : ceil_div(P, 32) * ceil_div(P, 8) * ceil_div(P, zchunk(P));
