@@ -186,7 +186,7 @@ HELM_HD inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 // CTAs of 1024 points hold 16 SMs' FP64 pipes for 13 us), a complex64 restriction 6.9 instead
 // of 7.6; at 1023^2 and above the larger tile's thinner halo wins.
 HELM_HD inline int zchunk(int P) { return P >= 128 ? 32 : (P >= 64 ? 4 : 2); }
-// (The persistent segments' levels, P <= 512, have Q = 1.)
+// (The persistent segments: levels of P <= 512.)
 HELM_HD constexpr int tile2_q(int P) { return ((P + 63) / 64) * ((P + 15) / 16) < 4 * GB300_SMS ? 1 : 2; }
 static_assert(tile2_q(512) == 1, "the persistent segments are compiled for Q = 1");
 HELM_HD inline int vtiles(int dim, int P) {
