@@ -5,8 +5,9 @@
 // coordinate descent from the built-in defaults, finest level first.  A candidate
 // replaces the current choice when the V-cycle gets faster by more than 0.5%, which
 // keeps run-to-run noise from deciding.  Choices:
-//   2D levels: tiles per CTA of the residual + restriction pass, of the prolongation pass
-//     and (complex128) of the Arnoldi passes of each step J (1, 2, 4, 8);
+//   2D levels: tiles per CTA of the residual + restriction pass and of the prolongation pass
+//     where the cycle launches them (the fused complex64 V(1,1) passes take their shape from
+//     the level size), and (complex128) of the Arnoldi passes of each step J (1, 2, 4, 8);
 //   3D levels without the TMA-fed passes (pitch below 128, or complex128): the planes
 //     each CTA of the plain passes marches (2, 4, 8, 16);
 //   3D complex64 levels of pitch 128..1024: the TMA-fed restriction and post-smoothing
@@ -120,7 +121,8 @@ int autotune(const helm_grid* grid, const float* phi, double k, double theta_bet
   // the choices of this hierarchy's grid-wide levels
   const int thr = coarse_threshold(dim, h->prec);
   std::vector<Knob> knobs;
-  for (const HostLevel& L : h->lev) {
+  for (int l = 0; l < (int)h->lev.size(); ++l) {
+    const HostLevel& L = h->lev[l];
     if (L.n <= thr) continue;
     const int P = L.P;
     if (dim == 3 && !(eb == 8 && L.tm && P >= 128 && P <= 1024 && P % 32 == 0)) {
@@ -133,8 +135,8 @@ int autotune(const helm_grid* grid, const float* phi, double k, double theta_bet
     if (dim == 2) {
       if (eb == 16)
         for (int J = 1; J <= h->s; ++J) knobs.push_back({TP_ARNOLDI, 2, P, eb, J, {tc(1), tc(2), tc(4), tc(8)}});
-      knobs.push_back({TP_RESTRICT, 2, P, eb, 0, {tc(1), tc(2), tc(4), tc(8)}});
-      knobs.push_back({TP_PROLONG, 2, P, eb, 0, {tc(1), tc(2), tc(4), tc(8)}});
+      for (TunePass ps : {TP_RESTRICT, TP_PROLONG})
+        if (tiled_transfer(*h, l, ps)) knobs.push_back({ps, 2, P, eb, 0, {tc(1), tc(2), tc(4), tc(8)}});
     } else if (eb == 8 && L.tm && P >= 128 && P <= 1024 && P % 32 == 0) {
       Knob kr{TP_RESTRICT, 3, P, eb, 0, {tc(0, 2, 0, 2)}};
       for (int stg : {2, 3, 4})

@@ -190,6 +190,14 @@ static bool fused2_level(const Handle& h, const HostLevel& L) {
          L.n > coarse_threshold(2, HELM_C64);
 }
 
+bool tiled_transfer(const Handle& h, int l, int pass) {
+  const int eb = h.prec == HELM_C128 ? 16 : 8;
+  if (pass == TP_PROLONG && h.nu2 == 0) return false;
+  if (!fused2_cycle(h.dim, h.prec, h.smoother, h.nu1, h.nu2) || persist_level(h.dim, h.lev[l].P, eb)) return true;
+  // fused: only above a level whose sweep marches does the restriction have a pass of its own
+  return pass == TP_RESTRICT && l + 1 < (int)h.lev.size() && !fused2_size(h.lev[l + 1].n);
+}
+
 int setup_handle(const helm_grid* grid, const float* phi, double k, double theta_beta, const helm_opts* opts,
                  cudaStream_t st, Handle** out) {
   if (!grid || !out) { set_error("grid and out must not be NULL"); return HELM_EINVAL; }

@@ -110,6 +110,10 @@ struct Handle {
   ~Handle();
 };
 
+// Whether the handle's V-cycle launches the tiled residual + restriction pass (TP_RESTRICT) below
+// level l, or the tiled coarse correction (TP_PROLONG) on it: the fused 2D cycles do without.
+bool tiled_transfer(const Handle& h, int l, int pass);
+
 int setup_handle(const helm_grid* grid, const float* phi, double k, double theta_beta, const helm_opts* opts,
                  cudaStream_t st, Handle** out);
 int precond_apply(Handle* h, const void* r, void* z, int prec, cudaStream_t st);

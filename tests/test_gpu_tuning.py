@@ -132,3 +132,13 @@ def test_autotune_writes_a_table_and_keeps_parity(helm, table, tmp_path, cube127
     zt = torch.empty_like(rt)
     h.precond_apply(rt, zt)
     assert_parity(zt, want, ("vcycle", "c64"), "after autotune")
+
+
+@pytest.mark.parametrize("n,prec,choices", [(639, "c64", 0), (1279, "c64", 1), (63, "c128", 10)])
+def test_autotune_times_only_passes_the_cycle_launches(helm, table, tmp_path, n, prec, choices):
+    """2D complex64 V(1,1): no tiled transfer on fused levels (below 600), the restriction alone
+    above a marching one; complex128: both and three Arnoldi steps on each of two levels."""
+    table([])
+    path = str(tmp_path / "tuned.json")
+    helm.autotune(2, n, 0.3, k=0.2 * (n + 1), precision=prec, reps=1, path=path)
+    assert json.load(open(path))["runs"][-1]["choices"] == choices
