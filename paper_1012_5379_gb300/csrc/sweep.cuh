@@ -157,7 +157,7 @@ struct Sw2Region {
 enum { W_NO, W_YES, W_ANY };
 __device__ __forceinline__ bool wide_level(const LevelDev<float2>& L, int W) { return W == W_ANY ? L.wide != 0 : W == W_YES; }
 
-template <int S, int QY, int W, bool NC = true>
+template <int S, int QY, int W>
 __device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
                                             int store_last, int vblk, Sw2Shared<S, QY>& sh) {
   const int prob = vblk / nunits, unit = vblk - prob * nunits;
@@ -170,7 +170,7 @@ __device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__
   const float2* R0 = first ? L.b : L.r0;
   float2 k[S + 1][QY];
 #pragma unroll
-  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2, NC>(R0, G.x, G.y0 + q, 0, G.n, G.P);
+  for (int q = 0; q < QY; ++q) k[0][q] = ldc<float2>(R0, G.x, G.y0 + q, 0, G.n, G.P);
   G.sweep(L, sg, wide, k, L.p, store_last ? S : S - 1, unit, nunits);
 }
 template <int S, int QY, int W>
@@ -631,7 +631,7 @@ __device__ __forceinline__ float2 sw3_row(const float2* sm, const SwCoef& cx, co
   return cfma(make_float2(za.z, za.w), vt, p);
 }
 
-template <int S, int O, int W, bool NC = true>
+template <int S, int O, int W>
 __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
                                             int store_last, int vblk, float2* sm) {
   constexpr int NS = gram_ns(S), NV = gram_nv(S), R = O + 2 * S;
@@ -662,7 +662,7 @@ __device__ __forceinline__ void sweep3_body(const LevelDev<float2>* __restrict__
   const float2* R0 = first ? L.b : L.r0;
 #pragma unroll 4
   for (int r = warp; r < R * R; r += SW3_NW)
-    sm[r * 32 + lane] = ldc<float2, NC>(R0, x, y0 + r % R, z0 + r / R, n, P);
+    sm[r * 32 + lane] = ldc<float2>(R0, x, y0 + r % R, z0 + r / R, n, P);
   __syncthreads();
   auto phi_of = [&](int y, int z) -> float {
     return phi ? (inside(x, y, z, n) ? __ldg(phi + pidx(x, y, z, P)) * t : 0.f) : phc;

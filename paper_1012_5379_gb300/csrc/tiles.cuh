@@ -52,7 +52,7 @@ __device__ __forceinline__ C stencil5(const Coef3<C>& cx, const Coef3<C>& cy, ty
 
 // ------------------------------------------------------------------ Arnoldi step J
 // Complex128 holds twice the registers per raw vector: two CTAs per SM.
-template <typename C, int J, int Q, bool NC = true>
+template <typename C, int J, int Q>
 __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int store_p, int vblk) {
   typedef typename CT<C>::R R;
   __shared__ C vt[t2y(Q) + 2][t2x(Q) + 2];
@@ -90,7 +90,7 @@ __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ 
       C v = czero<C>();
 #pragma unroll
       for (int k = 0; k < J; ++k) {
-        raw[q][k] = ldc<C, NC>(Rk[k], x0 + ox, y0 + oy, 0, n, P);
+        raw[q][k] = ldc<C>(Rk[k], x0 + ox, y0 + oy, 0, n, P);
         v = cfma(cf[k], raw[q][k], v);
       }
       vt[oy + 1][ox + 1] = v;
@@ -100,7 +100,7 @@ __device__ __forceinline__ void arnoldi_t2_body(const LevelDev<C>* __restrict__ 
       halo_coord<t2x(Q), t2y(Q)>(tid, hx, hy);
       C v = czero<C>();
 #pragma unroll
-      for (int k = 0; k < J; ++k) v = cfma(cf[k], ldc<C, NC>(Rk[k], x0 + hx, y0 + hy, 0, n, P), v);
+      for (int k = 0; k < J; ++k) v = cfma(cf[k], ldc<C>(Rk[k], x0 + hx, y0 + hy, 0, n, P), v);
       vt[hy + 1][hx + 1] = v;
     }
     __syncthreads();
@@ -136,7 +136,7 @@ k_arnoldi_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_i
   arnoldi_t2_body<C, J, Q>(levs, ntiles, tpc, r0_is_b, store_p, blockIdx.x);
 }
 
-template <typename C, int J, bool NC = true>
+template <typename C, int J>
 __device__ __forceinline__ void arnoldi_t3_body(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_is_b, int store_p, int vblk) {
   typedef typename CT<C>::R R;
   __shared__ C vb[4][T3Y + 2][T3X + 2];
@@ -169,8 +169,8 @@ __device__ __forceinline__ void arnoldi_t3_body(const LevelDev<C>* __restrict__ 
   auto fetch = [&](int z, C* raw, C* hraw) {
 #pragma unroll
     for (int k = 0; k < J; ++k) {
-      raw[k] = ldc<C, NC>(Rk[k], x, y, z, n, P);
-      hraw[k] = halo ? ldc<C, NC>(Rk[k], x0 + hx, y0 + hy, z, n, P) : czero<C>();
+      raw[k] = ldc<C>(Rk[k], x, y, z, n, P);
+      hraw[k] = halo ? ldc<C>(Rk[k], x0 + hx, y0 + hy, z, n, P) : czero<C>();
     }
   };
   auto store_plane = [&](int z, const C* raw, const C* hraw) {
@@ -666,7 +666,7 @@ k_prolong3_rows(const LevelDev<C>* __restrict__ levs, int nblk) {
 // The tiles of one CTA with the sweep's raw-vector count M fixed, so that every load
 // of a tile (M + 1 raw vectors and x at four points per thread) is issued before the
 // first is used.
-template <typename C, int M, int Q, bool NC = true>
+template <typename C, int M, int Q>
 __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCoef<C>& u, int unit, int tpc,
                                                int ntiles, int x_from_zero, C (*rt)[t2x(Q) + 1],
                                                typename CT<C>::R& acc) {
@@ -689,7 +689,7 @@ __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCo
         const int q = q0 + b;
         const int x = x0 + lx + 32 * (q % Q), y = y0 + ly + 8 * (q / Q);
 #pragma unroll
-        for (int k = 0; k <= M; ++k) v[b][k] = ldc<C, NC>(u.Rk[k], x, y, 0, n, P);
+        for (int k = 0; k <= M; ++k) v[b][k] = ldc<C>(u.Rk[k], x, y, 0, n, P);
         xv[b] = (x_from_zero || x >= n || y >= n) ? czero<C>() : xa[pidx(x, y, 0, P)];
       }
 #pragma unroll
@@ -711,7 +711,7 @@ __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCo
       const int hy = tid < t2x(Q) + 1 ? t2y(Q) : tid - (t2x(Q) + 1);
       C r = czero<C>();
 #pragma unroll
-      for (int k = 0; k <= M; ++k) r = cfma(u.rc[k], ldc<C, NC>(u.Rk[k], x0 + hx, y0 + hy, 0, n, P), r);
+      for (int k = 0; k <= M; ++k) r = cfma(u.rc[k], ldc<C>(u.Rk[k], x0 + hx, y0 + hy, 0, n, P), r);
       rt[hy][hx] = r;
     }
     __syncthreads();
@@ -735,7 +735,7 @@ __device__ __forceinline__ void restrict_tiles(const LevelDev<C>& L, const UpdCo
   }
 }
 
-template <typename C, int Q, bool NC = true>
+template <typename C, int Q>
 __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_is_b, int x_from_zero,
               int nosmooth, int vblk) {
   typedef typename CT<C>::R R;
@@ -749,11 +749,11 @@ __device__ __forceinline__ void restrict_t2_body(const LevelDev<C>* __restrict__
   if (nosmooth) { u.m = 0; u.rc[0] = CT<C>::make(1, 0); }
   R acc = 0;
   switch (u.m) {  // uniform over the grid
-    case 0: restrict_tiles<C, 0, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 1: restrict_tiles<C, 1, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 2: restrict_tiles<C, 2, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 3: restrict_tiles<C, 3, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
-    case 4: restrict_tiles<C, 4, Q, NC>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 0: restrict_tiles<C, 0, Q>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 1: restrict_tiles<C, 1, Q>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 2: restrict_tiles<C, 2, Q>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 3: restrict_tiles<C, 3, Q>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
+    case 4: restrict_tiles<C, 4, Q>(L, u, unit, tpc, ntiles, x_from_zero, rt, acc); break;
     default: break;
   }
   static_assert(SMAX == 4, "restrict_tiles is instantiated for m = 0..4");
@@ -776,7 +776,7 @@ k_restrict_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int r0_
 // The z-march of one 3D restriction tile with the sweep's raw-vector count M fixed:
 // the next plane's raw values (own point and halo point) and x are loaded before the
 // current plane is processed, so each plane's loads overlap the previous plane's work.
-template <typename C, int M, bool NC = true>
+template <typename C, int M>
 __device__ __forceinline__ void restrict3_march(const LevelDev<C>& L, const UpdCoef<C>& u, int x0, int y0, int zbeg,
                                                 int zend, int x_from_zero, C (*rb)[T3Y + 1][T3X + 1],
                                                 typename CT<C>::R& acc) {
@@ -794,11 +794,11 @@ __device__ __forceinline__ void restrict3_march(const LevelDev<C>& L, const UpdC
   C vn[M + 1], hn[M + 1], xn;
   auto load = [&](int z) {
 #pragma unroll
-    for (int k = 0; k <= M; ++k) vn[k] = ldc<C, NC>(u.Rk[k], x, y, z, n, P);
+    for (int k = 0; k <= M; ++k) vn[k] = ldc<C>(u.Rk[k], x, y, z, n, P);
     xn = (x_from_zero || !inside(x, y, z, n)) ? czero<C>() : xa[pidx(x, y, z, P)];
     if (halo) {
 #pragma unroll
-      for (int k = 0; k <= M; ++k) hn[k] = ldc<C, NC>(u.Rk[k], x0 + hx, y0 + hy, z, n, P);
+      for (int k = 0; k <= M; ++k) hn[k] = ldc<C>(u.Rk[k], x0 + hx, y0 + hy, z, n, P);
     }
   };
   load(zbeg);
@@ -844,7 +844,7 @@ __device__ __forceinline__ void restrict3_march(const LevelDev<C>& L, const UpdC
   }
 }
 
-template <typename C, bool NC = true>
+template <typename C>
 __device__ __forceinline__ void restrict_t3_body(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_is_b, int x_from_zero, int nosmooth, int vblk) {
   typedef typename CT<C>::R R;
   __shared__ C rb[4][T3Y + 1][T3X + 1];
@@ -861,11 +861,11 @@ __device__ __forceinline__ void restrict_t3_body(const LevelDev<C>* __restrict__
   R acc = 0;
   if (zbeg < P) {
     switch (u.m) {  // uniform over the grid
-      case 0: restrict3_march<C, 0, NC>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
-      case 1: restrict3_march<C, 1, NC>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
-      case 2: restrict3_march<C, 2, NC>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
-      case 3: restrict3_march<C, 3, NC>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
-      case 4: restrict3_march<C, 4, NC>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
+      case 0: restrict3_march<C, 0>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
+      case 1: restrict3_march<C, 1>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
+      case 2: restrict3_march<C, 2>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
+      case 3: restrict3_march<C, 3>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
+      case 4: restrict3_march<C, 4>(L, u, x0, y0, zbeg, zend, x_from_zero, rb, acc); break;
       default: break;
     }
   }
@@ -885,7 +885,7 @@ k_restrict_t3(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int r0_i
 
 // ------------------------------------------------------------------ coarse correction
 // x_b = x_a + P e_c, r0 = b - M x_b, ||r0||^2 starts post-smoothing.
-template <typename C, int Q, bool NC = true>
+template <typename C, int Q>
 __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc, int vblk) {
   typedef typename CT<C>::R R;
   __shared__ C vt[t2y(Q) + 2][t2x(Q) + 2];
@@ -905,7 +905,7 @@ __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ 
   C* const r0 = L.r0;
   const int nc = L.nc, Pc = L.Pc;
   auto form = [&](int xx, int yy) -> C {
-    return cadd(ldc<C, NC>(xa, xx, yy, 0, n, P), interp<C, NC>(xcb, n, nc, Pc, xx, yy, 0, 2));
+    return cadd(ldc<C>(xa, xx, yy, 0, n, P), interp<C>(xcb, n, nc, Pc, xx, yy, 0, 2));
   };
   R acc = 0;
   const int t_end = min(ntiles, (unit + 1) * tpc);
@@ -916,7 +916,7 @@ __device__ __forceinline__ void prolong_t2_body(const LevelDev<C>* __restrict__ 
 #pragma unroll
     for (int q = 0; q < Q * Q; ++q) {
       const int ox = lx + 32 * (q % Q), oy = ly + 8 * (q / Q);
-      bq[q] = ldc<C, NC>(bv, x0 + ox, y0 + oy, 0, n, P);
+      bq[q] = ldc<C>(bv, x0 + ox, y0 + oy, 0, n, P);
       vt[oy + 1][ox + 1] = form(x0 + ox, y0 + oy);
     }
     if (tid < halo2(Q)) {
@@ -961,7 +961,7 @@ k_prolong_t2(const LevelDev<C>* __restrict__ levs, int ntiles, int tpc) {
   prolong_t2_body<C, Q>(levs, ntiles, tpc, blockIdx.x);
 }
 
-template <typename C, bool NC = true>
+template <typename C>
 __device__ __forceinline__ void prolong_t3_body(const LevelDev<C>* __restrict__ levs, int ntiles, int zc, int vblk) {
   typedef typename CT<C>::R R;
   __shared__ C vb[4][T3Y + 2][T3X + 2];
@@ -979,7 +979,7 @@ __device__ __forceinline__ void prolong_t3_body(const LevelDev<C>* __restrict__ 
   int hx = 0, hy = 0;
   if (halo) halo_coord<T3X, T3Y>(tid, hx, hy);
   auto form = [&](int xx, int yy, int zz) -> C {
-    return cadd(ldc<C, NC>((const C*)L.xa, xx, yy, zz, n, P), interp<C, NC>(L, xx, yy, zz, 3));
+    return cadd(ldc<C>((const C*)L.xa, xx, yy, zz, n, P), interp<C>(L, xx, yy, zz, 3));
   };
   auto load_plane = [&](int z) {
     vb[z & 3][ly + 1][lx + 1] = form(x, y, z);
@@ -990,11 +990,11 @@ __device__ __forceinline__ void prolong_t3_body(const LevelDev<C>* __restrict__ 
   if (zbeg < P) {
     load_plane(zbeg - 1);
     load_plane(zbeg);
-    C bnext = ldc<C, NC>((const C*)L.b, x, y, zbeg, n, P);  // b of the next plane, loaded a plane ahead
+    C bnext = ldc<C>((const C*)L.b, x, y, zbeg, n, P);  // b of the next plane, loaded a plane ahead
     for (int z = zbeg; z < zend; ++z) {
       const C bcur = bnext;
       load_plane(z + 1);
-      if (z + 1 < zend) bnext = ldc<C, NC>((const C*)L.b, x, y, z + 1, n, P);
+      if (z + 1 < zend) bnext = ldc<C>((const C*)L.b, x, y, z + 1, n, P);
       __syncthreads();
       const int s0 = z & 3;
       if (x < P && y < P) {
@@ -1083,26 +1083,26 @@ constexpr int SEQ_O3 = 4;  // own rows of the 3D sweep pass on levels the segmen
 template <typename C, int DIM, int J>
 __device__ __noinline__ void seq_arnoldi(const PassDesc d, const LevelDev<C>* levs, int v, float2* sm) {
   if constexpr (sizeof(C) == 8 && DIM == 2) {
-    if (d.geo == 2) sweep2_body<J, 2, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 2>*>(sm));
-    else if (d.geo == 4) sweep2_body<J, 4, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 4>*>(sm));
-    else sweep2_body<J, 6, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 6>*>(sm));
+    if (d.geo == 2) sweep2_body<J, 2, W_ANY>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 2>*>(sm));
+    else if (d.geo == 4) sweep2_body<J, 4, W_ANY>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 4>*>(sm));
+    else sweep2_body<J, 6, W_ANY>(levs, d.ntiles, d.f0, d.f1, v, *reinterpret_cast<Sw2Shared<J, 6>*>(sm));
   } else if constexpr (sizeof(C) == 8) {
-    sweep3_body<J, SEQ_O3, W_ANY, false>(levs, d.ntiles, d.f0, d.f1, v, sm);
+    sweep3_body<J, SEQ_O3, W_ANY>(levs, d.ntiles, d.f0, d.f1, v, sm);
   } else if constexpr (DIM == 2) {
-    arnoldi_t2_body<C, J, 1, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
+    arnoldi_t2_body<C, J, 1>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
   } else {
-    arnoldi_t3_body<C, J, false>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
+    arnoldi_t3_body<C, J>(levs, d.ntiles, d.geo, d.f0, d.f1, v);
   }
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_restrict(const PassDesc d, const LevelDev<C>* levs, int v) {
-  if constexpr (DIM == 2) restrict_t2_body<C, 1, false>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
-  else restrict_t3_body<C, false>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
+  if constexpr (DIM == 2) restrict_t2_body<C, 1>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
+  else restrict_t3_body<C>(levs, d.ntiles, d.geo, d.f0, d.f1, d.f2, v);
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_prolong(const PassDesc d, const LevelDev<C>* levs, int v) {
-  if constexpr (DIM == 2) prolong_t2_body<C, 1, false>(levs, d.ntiles, d.geo, v);
-  else prolong_t3_body<C, false>(levs, d.ntiles, d.geo, v);
+  if constexpr (DIM == 2) prolong_t2_body<C, 1>(levs, d.ntiles, d.geo, v);
+  else prolong_t3_body<C>(levs, d.ntiles, d.geo, v);
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_update(const PassDesc d, const LevelDev<C>* levs, int v) {
@@ -1110,7 +1110,7 @@ __device__ __noinline__ void seq_update(const PassDesc d, const LevelDev<C>* lev
 }
 template <typename C, int DIM>
 __device__ __noinline__ void seq_prolong_flat(const PassDesc d, const LevelDev<C>* levs, int v) {
-  prolong_flat_body<C, false>(levs, d.ntiles, DIM, v);
+  prolong_flat_body<C>(levs, d.ntiles, DIM, v);
 }
 
 // flags: arnoldi f0 = R_0 is b, f1 = store p_J; restrict f0 = R_0 is b, f1 = x from zero,

@@ -20,8 +20,8 @@ __device__ __forceinline__ size_t pidx(int x, int y, int z, int P) {
 }
 // Bounds-checked load.  A plain load, not the read-only one: the compiler takes a read-only
 // load for invariant and may move it above the wait for the kernel that writes the buffer
-// (pdl_wait).  (NC names the launches outside the persistent segments.)
-template <typename C, bool NC = true>
+// (pdl_wait).
+template <typename C>
 __device__ __forceinline__ C ldc(const C* p, int x, int y, int z, int n, int P) {
   if (!inside(x, y, z, n)) return czero<C>();
   return p[pidx(x, y, z, P)];
@@ -76,7 +76,7 @@ struct StencilRegs {
 // ------------------------------------------------------------------ prolongation
 // Vertex-centred bi/trilinear interpolation of the coarser output at fine node i:
 // odd i -> coarse (i-1)/2 with weight 1; even i -> coarse i/2-1 and i/2 with 1/2.
-template <typename C, bool NC = true>
+template <typename C>
 __device__ __forceinline__ C interp(const C* xcb, int n, int nc, int Pc, int x, int y, int z, int dim) {
   typedef typename CT<C>::R R;
   C acc = czero<C>();
@@ -109,12 +109,12 @@ __device__ __forceinline__ C interp(const C* xcb, int n, int nc, int Pc, int x, 
   const R w = wx * wy * wz;
   for (int c = 0; c < nz; ++c)
     for (int b = 0; b < ny; ++b)
-      for (int a = 0; a < nx; ++a) acc = cadd(acc, ldc<C, NC>(xcb, ix[a], iy[b], iz[c], nc, Pc));
+      for (int a = 0; a < nx; ++a) acc = cadd(acc, ldc<C>(xcb, ix[a], iy[b], iz[c], nc, Pc));
   return cscale(acc, w);
 }
-template <typename C, bool NC = true>
+template <typename C>
 __device__ __forceinline__ C interp(const LevelDev<C>& L, int x, int y, int z, int dim) {
-  return interp<C, NC>(L.xcb, L.n, L.nc, L.Pc, x, y, z, dim);
+  return interp<C>(L.xcb, L.n, L.nc, L.Pc, x, y, z, dim);
 }
 
 // ------------------------------------------------------------------ sweep end
@@ -330,7 +330,7 @@ k_store_output(const LevelDev<C>* __restrict__ levs, int dim, int update, Cout* 
 
 // ------------------------------------------------------------------ coarse correction
 // Coarse correction without post-smoothing (nu2 = 0): x_b = x_a + P e_c, pointwise.
-template <typename C, bool NC = true>
+template <typename C>
 __device__ __forceinline__ void prolong_flat_body(const LevelDev<C>* __restrict__ levs, int ntiles, int dim, int vblk) {
   pdl_trigger();
   const int prob = vblk / ntiles, tile = vblk - prob * ntiles;
@@ -341,7 +341,7 @@ __device__ __forceinline__ void prolong_flat_body(const LevelDev<C>* __restrict_
   for (size_t i = (size_t)tile * block_threads() + flat_tid(); i < npts; i += (size_t)ntiles * block_threads()) {
     const int x = (int)(i % P), y = (int)((i / P) % P), z = dim == 3 ? (int)(i / ((size_t)P * P)) : 0;
     C v = czero<C>();
-    if (inside(x, y, z, n)) v = cadd(L.xa[i], interp<C, NC>(L, x, y, z, dim));
+    if (inside(x, y, z, n)) v = cadd(L.xa[i], interp<C>(L, x, y, z, dim));
     L.xb[i] = v;
   }
 }
@@ -376,15 +376,15 @@ __device__ void cblock_stencil_apply(const LevelDev<C>& L, const C* v, int x, in
   C v0 = v[pidx(x, y, z, P)];
   C diag = cadd(cx.d, cy.d);
   C p = czero<C>();
-  p = cfma(cx.a, ldc<C, false>(v, x - 1, y, z, n, P), p);
-  p = cfma(cx.c, ldc<C, false>(v, x + 1, y, z, n, P), p);
-  p = cfma(cy.a, ldc<C, false>(v, x, y - 1, z, n, P), p);
-  p = cfma(cy.c, ldc<C, false>(v, x, y + 1, z, n, P), p);
+  p = cfma(cx.a, ldc<C>(v, x - 1, y, z, n, P), p);
+  p = cfma(cx.c, ldc<C>(v, x + 1, y, z, n, P), p);
+  p = cfma(cy.a, ldc<C>(v, x, y - 1, z, n, P), p);
+  p = cfma(cy.c, ldc<C>(v, x, y + 1, z, n, P), p);
   if (dim == 3) {
     const Coef3<C> cz = ldcoef(L, z);
     diag = cadd(diag, cz.d);
-    p = cfma(cz.a, ldc<C, false>(v, x, y, z - 1, n, P), p);
-    p = cfma(cz.c, ldc<C, false>(v, x, y, z + 1, n, P), p);
+    p = cfma(cz.a, ldc<C>(v, x, y, z - 1, n, P), p);
+    p = cfma(cz.c, ldc<C>(v, x, y, z + 1, n, P), p);
   }
   diag.x -= phi_at(L, x, y, z);
   out = cfma(diag, v0, p);
@@ -580,7 +580,7 @@ __device__ void coarse_cycle(Team& team, const LevelDev<C>* Ls, int nlev, const 
             for (int dy = -1; dy <= 1; ++dy)
               for (int dx = -1; dx <= 1; ++dx) {
                 R wgt = (R)((dx == 0 ? 0.5 : 0.25) * (dy == 0 ? 0.5 : 0.25) * (dim == 3 ? (dz == 0 ? 0.5 : 0.25) : 1.0));
-                out[u] = cadd(out[u], cscale(ldc<C, false>((const C*)L.xb, fx + dx, fy + dy, fz + dz, L.n, P), wgt));
+                out[u] = cadd(out[u], cscale(ldc<C>((const C*)L.xb, fx + dx, fy + dy, fz + dz, L.n, P), wgt));
               }
           acc += cabs2(out[u]);
         }
@@ -682,7 +682,7 @@ __device__ void coarse_cycle(Team& team, const LevelDev<C>* Ls, int nlev, const 
         if (i >= npts) continue;
         int x, y, z;
         cblock_coords(i, (unsigned)P, dim, x, y, z);
-        if (inside(x, y, z, n)) xv[u] = cadd(L.xa[i], interp<C, false>(L, x, y, z, dim));
+        if (inside(x, y, z, n)) xv[u] = cadd(L.xa[i], interp<C>(L, x, y, z, dim));
       }
 #pragma unroll
       for (int u = 0; u < CB_U; ++u)
@@ -824,7 +824,7 @@ k_poly_fw(const LevelDev<C>* __restrict__ levs, int ntiles, int dim) {
         for (int dy = -1; dy <= 1; ++dy)
           for (int dx = -1; dx <= 1; ++dx) {
             const R wgt = (R)((dx == 0 ? 0.5 : 0.25) * (dy == 0 ? 0.5 : 0.25) * (dim == 3 ? (dz == 0 ? 0.5 : 0.25) : 1.0));
-            out = cadd(out, cscale(ldc<C, false>((const C*)L.r0, fx + dx, fy + dy, fz + dz, n, P), wgt));
+            out = cadd(out, cscale(ldc<C>((const C*)L.r0, fx + dx, fy + dy, fz + dz, n, P), wgt));
           }
     }
     L.bc[i] = out;
