@@ -118,3 +118,20 @@ def test_barrier_timeout_reports_etimeout_and_recovers(helm, table):
     assert np.linalg.norm(b.cpu().numpy() - levels[0].apply_h(xs)) / np.linalg.norm(b.cpu().numpy()) <= 1.05e-6
     with pytest.raises(helm.HelmError):
         helm.set_barrier_timeout(-1.0)
+
+
+@pytest.mark.parametrize("dim,n,s", [(2, 255, 3), (2, 511, 4), (3, 31, 3), (3, 63, 2)])
+def test_persistent_segments_with_levels_a_field_dominates(helm, table, dim, n, s):
+    """A disc of contrast 12: its coarse levels take double-float sums, in the segments by each
+    problem's own flag; bit for bit the launch-per-pass cycle."""
+    x = np.arange(1, n + 1) / (n + 1)
+    r2 = sum((a - 0.5) ** 2 for a in np.meshgrid(*([x] * dim), indexing="ij"))
+    phi = torch.from_numpy(((np.where(r2 < 0.09, 0.05, 1.2) * (n + 1)) ** 2).astype(np.float32)).cuda()
+    rt = torch.from_numpy(I.random_source(dim, n, 9)).cuda().to(torch.complex64)
+    outs = []
+    for entries in (persist_on(dim, "c64"), []):
+        table(entries)
+        h = helm.Handle(dim, n, 0.3, phi=phi, precision="c64", s=s, maxit=1)
+        outs.append(torch.empty_like(rt))
+        h.precond_apply(rt, outs[-1])
+    assert torch.equal(*outs) and torch.isfinite(torch.view_as_real(outs[0])).all()
