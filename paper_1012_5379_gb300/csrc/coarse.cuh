@@ -78,18 +78,17 @@ struct CgLevel {
     float2 d = dg[q];
     d.x -= sg.x;
     d.y -= sg.y;
-    float2 p = cmul(d, v0);
     const float2* s = v + off[q];
-    p = cfma(ax[q], s[-1], p);
+    float2 p = cmul(ax[q], s[-1]);
     p = cfma(qx[q], s[1], p);
     p = cfma(ay[q], s[-P], p);
     p = cfma(qy[q], s[P], p);
     if (DIM == 3) {
-      p = cfma(dz[q], v0, p);  // apart: the sum of the three diagonals would be rounded
       p = cfma(az[q], s[-P * P], p);
       p = cfma(qz[q], s[P * P], p);
+      p = cfma(dz[q], v0, p);  // apart: the sum of the three diagonals would be rounded
     }
-    return p;
+    return cfma(d, v0, p);
   }
 };
 

@@ -24,8 +24,8 @@ HELM_HD inline int po_units(int QY, int SRC, int END, int n) {
 
 // SRC 0: from zero, 1: from `src`, 2: from x_a + P e_c; END 0: x only, 1: and the coarse
 // right-hand side.
-template <int QY, int SRC, int END>
-__global__ void __launch_bounds__(256, 2)
+template <int QY, int SRC, int END>  // (three CTAs per SM: 1023^2 81 us a V-cycle, 88 at two)
+__global__ void __launch_bounds__(256, 3)
 k_poly2(const LevelDev<float2>* __restrict__ levs, const float2* __restrict__ pw, int nunits, int src, int dst) {
   constexpr int RY = SW2_NW * QY, OX = po_own(32, SRC, END), OY = po_own(RY, SRC, END);
   __shared__ float2 edge[2][SW2_NW + 2][2][32];
@@ -74,12 +74,11 @@ k_poly2(const LevelDev<float2>* __restrict__ levs, const float2* __restrict__ pw
       const float4 ac = yac[warp * QY + q];
       float2 dg = cadd(cx.d, yd[warp * QY + q]);
       dg.x -= ph;
-      float2 p = cmul(dg, v[q]);
-      p = cfma(cx.a, shfl_up_c(v[q], 1), p);
+      float2 p = cmul(cx.a, shfl_up_c(v[q], 1));
       p = cfma(cx.c, shfl_down_c(v[q], 1), p);
       p = cfma(make_float2(ac.x, ac.y), q > 0 ? v[q > 0 ? q - 1 : 0] : up, p);
       p = cfma(make_float2(ac.z, ac.w), q < QY - 1 ? v[q < QY - 1 ? q + 1 : q] : dn, p);
-      r[q] = csub(b[q], p);
+      r[q] = csub(b[q], cfma(dg, v[q], p));
     }
   };
 #pragma unroll

@@ -43,6 +43,13 @@ __device__ __forceinline__ C stencil5(const Coef3<C>& cx, const Coef3<C>& cy, ty
                                       C vr, C vs, C vn) {
   C diag = cadd(cx.d, cy.d);
   diag.x -= phi;
+  if constexpr (sizeof(C) == 8) {  // binary32: the largest term last, so that one rounding is its size
+    C p = cmul(cx.a, vl);
+    p = cfma(cx.c, vr, p);
+    p = cfma(cy.a, vs, p);
+    p = cfma(cy.c, vn, p);
+    return cfma(diag, v0, p);
+  }
   C p = cmul(diag, v0);
   p = cfma(cx.a, vl, p);
   p = cfma(cx.c, vr, p);
