@@ -204,7 +204,7 @@ __device__ __forceinline__ void cg_poly(const CgLevel<S, DIM>& V, const float2 (
         const float2 p = V.apply(buf, x[q], q, z0);
         r = csub(r, make_float2(p.x * V.it, p.y * V.it));
       }
-      x[q] = cfma(wj, r, x[q]);
+      x[q] = cadd(x[q], cmul(wj, r));
     }
   }
 }
