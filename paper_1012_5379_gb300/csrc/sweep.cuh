@@ -501,7 +501,7 @@ k_sweep2_march(const LevelDev<float2>* __restrict__ levs, int nunits, int rows, 
   for (int j = 0; j < S; ++j)
 #pragma unroll
     for (int w = 0; w < W; ++w) win[j][w][0] = win[j][w][1] = make_float2(0.f, 0.f);
-  float phw[W][2];
+  float phw[W][2] = {};
   float4 nxt[W];
   float2 phn[W];
   auto fetch = [&](int y, float4& v, float2& f) {
@@ -806,7 +806,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   for (int j = K0 ? 0 : 1; j < S; ++j)
 #pragma unroll
     for (int w = 0; w < W; ++w) win[j][w][0] = win[j][w][1] = make_float2(0.f, 0.f);
-  float phw[W][2];
+  float phw[W][2] = {};
   const bool field = PHI && phi;  // some problem of the launch has a field; this one may not
   const int at0 = (ry + 1) * 32 + lane;
   auto fetch = [&](int z, int slot) {

@@ -339,8 +339,18 @@ k_resid_tma3(const LevelDev<float2>* __restrict__ levs, int nunits, int stages) 
   int hx = 0, hy = 0;
   const bool halo = tid < HALO;
   if (halo) halo_coord<TM3_TX, TY>(tid, hx, hy);
-  C vprev[QY], vcur[QY];  // own points two planes and one plane back
+  // own points two planes and one plane back, and the column's coefficients.  Set before the loop
+  // although no stencil reads them before they are: the loop copies vcur to vprev from its first
+  // plane on, and a copy of an indeterminate value let the compiler drop the later ones (at 80
+  // registers the residual was wrong, at 125 it happened to be right).
+  C vprev[QY], vcur[QY];
   Coef3<C> cx, cy[QY];
+  cx.a = cx.d = cx.c = czero<C>();
+#pragma unroll
+  for (int q = 0; q < QY; ++q) {
+    vprev[q] = vcur[q] = czero<C>();
+    cy[q] = cx;
+  }
   int x0 = 0, y0 = 0;
   unsigned off = 0;       // padded index of the thread's first point in plane 0
   // consumer: walks the same planes
@@ -798,7 +808,7 @@ __device__ __forceinline__ void restrict3_march(const LevelDev<C>& L, const UpdC
   const int cx = tid % (T3X / 2), cy = tid / (T3X / 2);
   C* const xa = L.xa;
   C* const bc = L.bc;
-  C vn[M + 1], hn[M + 1], xn;
+  C vn[M + 1] = {}, hn[M + 1] = {}, xn = czero<C>();  // (hn stays zero off the halo: the loop copies it)
   auto load = [&](int z) {
 #pragma unroll
     for (int k = 0; k <= M; ++k) vn[k] = ldc<C>(u.Rk[k], x, y, z, n, P);
