@@ -327,13 +327,11 @@ __device__ __forceinline__ void gram_block_sum(float (&acc)[gram_ns(S)], float2*
   }
 }
 
-// The same from double-float sums.
+// The same from the warps' double-float totals (as warp_transpose_sum_f leaves them).
 template <int S, int NW>
-__device__ __forceinline__ void gram_block_sum_wide(float (&s)[gram_ns(S)], float (&c)[gram_ns(S)], float2* wsum,
-                                                    float2* gs) {
+__device__ __forceinline__ void gram_block_total(float2 tot, float2* wsum, float2* gs) {
   constexpr int NV = gram_nv(S), NS = gram_ns(S);
   const int tid = flat_tid(), lane = tid & 31, warp = tid >> 5;
-  const float2 tot = warp_transpose_sum_df<NS>(s, c, lane);
   if (NS == 32) wsum[warp * NS + lane] = tot;
   else if ((lane & 1) == 0) wsum[warp * NS + (lane >> 1)] = tot;
   __syncthreads();
@@ -342,6 +340,12 @@ __device__ __forceinline__ void gram_block_sum_wide(float (&s)[gram_ns(S)], floa
     const float2 a = df_group_sum<NW>(v < NV ? wsum[w * NS + v] : make_float2(0.f, 0.f));
     if (w == 0 && v < NV) gs[v] = a;
   }
+}
+// The same from every thread's double-float sums.
+template <int S, int NW>
+__device__ __forceinline__ void gram_block_sum_wide(float (&s)[gram_ns(S)], float (&c)[gram_ns(S)], float2* wsum,
+                                                    float2* gs) {
+  gram_block_total<S, NW>(warp_transpose_sum_df<gram_ns(S)>(s, c, flat_tid() & 31), wsum, gs);
 }
 
 // End of a sweep pass, after the CTA's sums (gram_block_sum): they are added over the level

@@ -767,6 +767,9 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
   constexpr int NS = gram_ns(S), NV = gram_nv(S), W = 4;
   constexpr int RING = sm3_ring(S);
   constexpr bool K0 = RING == W;  // k_0 and phi of the last planes in registers too
+  // s = 4: sums of four planes at a time to double-float (127^3 point source: error 3e-7, 1.5e-6
+  // with one binary32 chain a thread, 7% of the time; s <= 3 has the smaller error either way)
+  constexpr bool FOLD = S > 3;
   extern __shared__ __align__(16) float2 swsm[];
   __shared__ float2 wsum[SM3_NW * NS];
   __shared__ float2 gs[(SM3_NW + 1) * NV];
@@ -821,7 +824,7 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
       copy4_async(f + 32, ok1 ? phi + i + P : phi, ok1);
     }
   };
-  float acc[NS];
+  float acc[NS], gsum = 0.f, gerr = 0.f;
 #pragma unroll
   for (int i = 0; i < NS; ++i) acc[i] = 0.f;
   const bool ox = lane >= S && lane < 32 - S && x < n;
@@ -931,9 +934,19 @@ k_sweep3_march(const LevelDev<float2>* __restrict__ levs, int nunits, int zc, in
       copies_wait<AHEAD - 1>();
       __syncthreads();
     }
+    if (FOLD) {
+      const float tot = warp_transpose_sum_f<NS>(acc, lane);
+      float sum, e;
+      df_two_sum(gsum, tot, sum, e);
+      gsum = sum;
+      gerr += e;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) acc[k] = 0.f;
+    }
   }
   pdl_trigger();  // the main work is done: let the next pass launch
-  gram_block_sum<S, SM3_NW>(acc, wsum, gs);
+  if (FOLD) gram_block_total<S, SM3_NW>(make_float2(gsum, gerr), wsum, gs);
+  else gram_block_sum<S, SM3_NW>(acc, wsum, gs);
   gram_finish<S, SM3_NW>(L, sg, false, unit, nunits, gs);
 }
 

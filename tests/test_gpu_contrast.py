@@ -136,3 +136,17 @@ def test_smooth_source(helm, dim, n, kh, s, width, e_norm):
         z[prec] = torch.empty_like(rt)
         h.precond_apply(rt, z[prec])
     assert errors(z["c64"], z["c128"])[0] <= 4 * e_norm
+
+
+@pytest.mark.parametrize("n,kh,e_norm", [(127, 0.16, 3.0e-7), (127, 0.3, 2.6e-7)])
+def test_point_source_of_four_steps_3d(helm, n, kh, e_norm):
+    """s = 4 on a marching level, where a few planes hold all of a vector: against the complex128
+    V-cycle, four times the step-by-step error."""
+    z = {}
+    for prec, dt in (("c64", torch.complex64), ("c128", torch.complex128)):
+        h = helm.Handle(3, n, 0.3, k=kh * (n + 1), precision=prec, s=4, maxit=1)
+        r = torch.zeros((n,) * 3, dtype=dt, device="cuda")
+        r[(n // 2,) * 3] = 1.0
+        z[prec] = torch.empty_like(r)
+        h.precond_apply(r, z[prec])
+    assert errors(z["c64"], z["c128"])[0] <= 4 * e_norm
