@@ -354,7 +354,8 @@ int helm_precond_apply_noalloc(const helm_grid* grid, double k, double theta_bet
  * complex128 Arnoldi steps; the fused complex64 V(1,1) passes have none), and for 3D
  * complex64 levels of pitch 128..1024 the TMA-fed restriction and post-smoothing residual
  * (off, or on with 2..8 plane slots in flight, 2 or 4 points per thread in y, and the
- * level shared as one piece per resident CTA or as 1, 2 or 4 z pieces per column).  The complex64 smoothing sweeps have no tuned choice.
+ * level shared as one piece per resident CTA or as 1, 2 or 4 z pieces per column).
+ * The complex64 smoothing sweeps have no tuned choice.
  * Every candidate is timed over whole V-cycles (reps cycles, best of three trials) by
  * coordinate descent from the defaults, finest level first, and kept when it makes the
  * V-cycle more than 0.5% faster.  grid, phi, k, theta_beta, opts as for helm_setup

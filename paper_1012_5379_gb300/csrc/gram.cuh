@@ -30,9 +30,9 @@
 // levels of media with a contrast of three or more, where phi h^2 is large), the spectrum falls
 // into clusters at the field's values and the k_j become dependent to 1e-4 and less: G and its
 // solution then need all of double-float's digits.  There the warp sums are double-float too
-// (ten instructions a product instead of one; 255^2 with discs 75 us a V-cycle, 69 without), a pivot counts down to
-// GRAM_TAU_WIDE, and the shifts are 0 and the diagonal at the field's smallest value, middle and
-// largest.  Whole V-cycles with layers and discs of contrast 3 to 27, against 64 bits, norm: at
+// (ten instructions a product instead of one; 255^2 with discs 75 us a V-cycle, 69 without), a
+// pivot counts down to GRAM_TAU_WIDE, and the shifts are 0 and the diagonal at the field's
+// smallest value, middle and largest.  Whole V-cycles with layers and discs of contrast 3 to 27, against 64 bits, norm: at
 // most 1.8 times and in the mean 0.4 times the error of step-by-step orthogonalisation in
 // binary32; with binary32 sums and shifts that ignore the field up to 1e5 times (6e-2 instead of
 // 6e-6 for discs of 12 at 255^2, s = 3).  On the CPU, lines from 0.25 to 2 diagonals gave the

@@ -86,7 +86,7 @@ k_poly2(const LevelDev<float2>* __restrict__ levs, const float2* __restrict__ pw
     float2 r[QY];
     residual(r);
 #pragma unroll
-    for (int q = 0; q < QY; ++q) v[q] = cadd(v[q], cmul(w[j], r[q]));  // (as multiply-adds both products round at v's size)
+    for (int q = 0; q < QY; ++q) v[q] = cadd(v[q], cmul(w[j], r[q]));  // (a multiply-add rounds twice at v's size)
   }
   float2* const out = poly_vec(L, dst);
   const bool ownx = lane >= PO_H && lane < PO_H + OX && x < n;

@@ -156,7 +156,9 @@ struct Sw2Region {
 // W: whether the problems' levels are wide (their sums need more registers, so that is a kernel
 // of its own), or W_ANY: each problem's own flag.
 enum { W_NO, W_YES, W_ANY };
-__device__ __forceinline__ bool wide_level(const LevelDev<float2>& L, int W) { return W == W_ANY ? L.wide != 0 : W == W_YES; }
+__device__ __forceinline__ bool wide_level(const LevelDev<float2>& L, int W) {
+  return W == W_ANY ? L.wide != 0 : W == W_YES;
+}
 
 template <int S, int QY, int W>
 __device__ __forceinline__ void sweep2_body(const LevelDev<float2>* __restrict__ levs, int nunits, int first,
